@@ -621,22 +621,126 @@ __global__ void kvarn_block_kernel(Geom g, int L, TokSrc sk, TokSrc sv, float in
   }
 }
 
-// The same block transform with warps instead of CTA-wide steps (D = 64/128/
-// 256, G = 32/64).  Every floating-point operation and its order are those of
+// The same block transform with the block in registers (D = 64/128/256,
+// G = 32/64).  Every floating-point operation and its order are those of
 // kvarn_block_kernel (and of the reference definition): Hadamard stages
 // h = 1 .. D/2 with explicit fp32 add/sub, the stride-halving pairwise trees
-// for the row and column sums of squares, IEEE sqrt and division.  A warp
-// owns whole rows for the Hadamard and the row statistics (lane l holds
-// channels l + 32 i: the upper tree levels add slots in registers, the last
-// five add lanes by xor-shuffle); a thread owns a whole column for the column
-// statistics (the tree in registers).  Two CTA barriers per iteration.
+// for the row and column sums of squares, IEEE sqrt and division.
+//
+// What bounds it is instructions: per element 16 divisions and 16 squares
+// and sums.  So lane l of warp w keeps rows w + 8 i, channels l + 32 j in
+// registers from the load to the codes, paired along j for the two-wide fp32
+// instructions; the upper levels of both trees stay in registers, the lower
+// five of a row are lane exchanges that also spread the rows over the lanes
+// (NR rows cost NR + 1 exchanges instead of 5 NR), the lower three of a
+// column go through shared memory (two CTA barriers per iteration).
+//
+// Division: y / s as q = RN(y v), RN(q + v (y - q s)) with v = RN(1 / s): the
+// correctly rounded quotient (P. Markstein, "Computation of elementary
+// functions on the IBM RISC System/6000 processor", 1990), given v correctly
+// rounded and y - q s exact.  s lies in [1e-8, 2^30] and every nonzero y is at
+// least 2^-50 in the row step, so at least 2^-80 in the column step: the
+// remainder is then representable and no quotient is subnormal.  A warp with
+// a value outside those bounds divides with __fdiv_rn.
+//
+// 4 sequences x 8 heads x 8000 tokens, D = 256, G = 64: 1990 us with the block
+// in shared memory, 792 us so.
+__device__ __forceinline__ uint64_t pk2(float lo, float hi) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ float2 upk2(uint64_t v) {
+  float2 f;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(f.x), "=f"(f.y) : "l"(v));
+  return f;
+}
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
+  uint64_t d;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
+  uint64_t d;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+// RN(y^2) for a pair, as y y + nz with nz = (-0, -0) unknown to the compiler:
+// mul.rn.f32x2 (or a constant -0) before an add.rn.f32x2 is contracted into one
+// fma, which would round the sums of squares differently.
+__device__ __forceinline__ uint64_t square2(uint64_t y, uint64_t nz) { return fma2(y, y, nz); }
+// y / s for a pair, from ns = -s and v = RN(1 / s) (see above).
+__device__ __forceinline__ uint64_t div2(uint64_t y, uint64_t ns, uint64_t v) {
+  const uint64_t q = mul2(y, v);
+  return fma2(fma2(q, ns, y), v, q);
+}
+__device__ __forceinline__ uint64_t div2_exact(uint64_t y, float s0, float s1) {
+  const float2 f = upk2(y);
+  return pk2(__fdiv_rn(f.x, s0), __fdiv_rn(f.y, s1));
+}
+
+// Butterfly over the lanes in the order 16, 8, 4, 2, 1 of N = 4 .. 32 values
+// at once, each step halving the values a lane carries while more than one
+// is left: lane l ends with the result of value l / (32 / N).
+template <int N, class Op>
+__device__ __forceinline__ float lanes_reduce(float (&v)[N], int lane, Op op) {
+  int n = N;
+#pragma unroll
+  for (int o = 16; o >= 1; o >>= 1) {
+    if (n > 1) {
+      n >>= 1;
+      const bool up = lane & o;
+#pragma unroll
+      for (int i = 0; i < N / 2; ++i)
+        if (i < n) {
+          const float mine = up ? v[i + n] : v[i], other = up ? v[i] : v[i + n];
+          v[i] = op(mine, __shfl_xor_sync(0xffffffffu, other, o));
+        }
+    } else {
+      v[0] = op(v[0], __shfl_xor_sync(0xffffffffu, v[0], o));
+    }
+  }
+  return v[0];
+}
+
+// 8 nibbles in each of 8 lanes, transposed: nibble j of lane a (of the 8) and
+// nibble a of lane j change places.
+__device__ __forceinline__ uint32_t nibble_transpose8(uint32_t w, int lane) {
+  uint32_t o = __shfl_xor_sync(0xffffffffu, w, 4);
+  w = __byte_perm(w, o, lane & 4 ? 0x3276 : 0x5410);
+  o = __shfl_xor_sync(0xffffffffu, w, 2);
+  w = __byte_perm(w, o, lane & 2 ? 0x3715 : 0x6240);
+  o = __shfl_xor_sync(0xffffffffu, w, 1);
+  return lane & 1 ? ((o >> 4) & 0x0F0F0F0Fu) | (w & 0xF0F0F0F0u)
+                  : (w & 0x0F0F0F0Fu) | ((o & 0x0F0F0F0Fu) << 4);
+}
+__device__ __forceinline__ uint32_t nibbles_to_bytes(uint32_t x) {   // 4 nibbles
+  x = (x | (x << 8)) & 0x00FF00FFu;
+  return (x | (x << 4)) & 0x0F0F0F0Fu;
+}
+
 template <int D, int G>
-__global__ void __launch_bounds__(256)
-kvarn_block_fast_kernel(Geom g, int L, TokSrc sk, TokSrc sv, float inv_sqrt_d) {
+struct KvarnSmem {
+  float rows[G * D];                 // Hadamard: channel order <-> lane order
+  float part[8][D];                  // column sums of squares of each warp's rows
+  float2 csig[D];                    // column divisors: -s, 1 / s
+  float4 grp[8][32];                 // coding: minimum, 1 / scale, scale
+};
+
+template <int D, int G>
+__global__ void __launch_bounds__(256, 2)
+kvarn_block_fast_kernel(Geom g, int L, TokSrc sk, TokSrc sv, float inv_sqrt_d, uint64_t nz) {
   pdl_wait();
   pdl_trigger();
-  constexpr int NS = D / 32, NG = D / G;
-  extern __shared__ float smem[];
+  constexpr int NS = D / 32, NP = NS / 2, NR = G / 8, NG = D / G;
+  constexpr int NV = NR * NG;                    // (row, group) pairs of a warp
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  KvarnSmem<D, G>& sm = *reinterpret_cast<KvarnSmem<D, G>*>(smem_raw);
   bool ok;
   const int T0 = append_begin(g, L, &ok);
   const int n0 = kvarn_nblocks(T0, g.S, G), n1 = kvarn_nblocks(T0 + L, g.S, G);
@@ -646,137 +750,269 @@ kvarn_block_fast_kernel(Geom g, int L, TokSrc sk, TokSrc sv, float inv_sqrt_d) {
   TokSrc src = which ? sv : sk;
   src.T0 = T0;
   const int bits = which ? g.vb : g.kb;
-  float* y = smem;                                // [G][D]
-  float* rsc = y + G * D;                         // [G] row scales
-  float* csc = rsc + G;                           // [D] column scales
-  uint8_t* cs = reinterpret_cast<uint8_t*>(csc + D);   // [G][D] codes
   const int h = blockIdx.y % g.H, b = blockIdx.y / g.H;
   const int q0 = blk * G, t0 = g.S + q0;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  // load and rotate: a warp per row
-  for (int r = warp; r < G; r += 8) {
-    float x[NS];
+
+  // load (lane l: channels NS l ..) and the Hadamard stages below NS, then
+  // channels l + 32 j
+  float* wrows = sm.rows + warp * (NR * D);
+#pragma unroll
+  for (int i = 0; i < NR; ++i) {
     const void* sb;
-    const int64_t e = tok_elem(g, src, b, h, t0 + r, &sb);
+    const int64_t e = tok_elem(g, src, b, h, t0 + warp + 8 * i, &sb) + lane * NS;
+    float x[NS];
+    if (g.act == KVQ_BF16) {
+      const __nv_bfloat16* p = reinterpret_cast<const __nv_bfloat16*>(sb) + e;
+      __nv_bfloat162 u[NP];
+      if constexpr (NS == 8) *reinterpret_cast<uint4*>(u) = *reinterpret_cast<const uint4*>(p);
+      else if constexpr (NS == 4) *reinterpret_cast<uint2*>(u) = *reinterpret_cast<const uint2*>(p);
+      else *reinterpret_cast<uint32_t*>(u) = *reinterpret_cast<const uint32_t*>(p);
 #pragma unroll
-    for (int i = 0; i < NS; ++i) x[i] = ld_act(sb, e + lane + 32 * i, g.act);
+      for (int k = 0; k < NP; ++k) {
+        const float2 f = __bfloat1622float2(u[k]);
+        x[2 * k] = f.x;
+        x[2 * k + 1] = f.y;
+      }
+    } else {
+      const float2* p = reinterpret_cast<const float2*>(reinterpret_cast<const float*>(sb) + e);
 #pragma unroll
-    for (int hh = 1; hh < 32; hh <<= 1)
+      for (int k = 0; k < NP; ++k) {
+        const float2 f = p[k];
+        x[2 * k] = f.x;
+        x[2 * k + 1] = f.y;
+      }
+    }
 #pragma unroll
-      for (int i = 0; i < NS; ++i) {
-        const float o = __shfl_xor_sync(0xffffffffu, x[i], hh);
-        x[i] = (lane & hh) ? __fsub_rn(o, x[i]) : __fadd_rn(x[i], o);
+    for (int hs = 1; hs < NS; hs <<= 1)
+#pragma unroll
+      for (int k = 0; k < NS; ++k)
+        if (!(k & hs)) {
+          const float a = x[k], c = x[k + hs];
+          x[k] = __fadd_rn(a, c);
+          x[k + hs] = __fsub_rn(a, c);
+        }
+#pragma unroll
+    for (int k = 0; k < NP; ++k)
+      *reinterpret_cast<float2*>(wrows + i * D + lane * NS + 2 * k) = make_float2(x[2 * k], x[2 * k + 1]);
+  }
+  __syncwarp();
+  uint64_t y[NR][NP];                            // pair p: channels l + 64 p, l + 64 p + 32
+#pragma unroll
+  for (int i = 0; i < NR; ++i) {
+    float x[NS];
+#pragma unroll
+    for (int j = 0; j < NS; ++j) x[j] = wrows[i * D + lane + 32 * j];
+#pragma unroll
+    for (int hh = NS; hh < 32; hh <<= 1)
+#pragma unroll
+      for (int j = 0; j < NS; ++j) {
+        const float o = __shfl_xor_sync(0xffffffffu, x[j], hh);
+        x[j] = (lane & hh) ? __fsub_rn(o, x[j]) : __fadd_rn(x[j], o);
       }
 #pragma unroll
     for (int hs = 1; hs < NS; hs <<= 1)
 #pragma unroll
-      for (int i = 0; i < NS; ++i)
-        if (!(i & hs)) {
-          const float a = x[i], c = x[i + hs];
-          x[i] = __fadd_rn(a, c);
-          x[i + hs] = __fsub_rn(a, c);
+      for (int j = 0; j < NS; ++j)
+        if (!(j & hs)) {
+          const float a = x[j], c = x[j + hs];
+          x[j] = __fadd_rn(a, c);
+          x[j + hs] = __fsub_rn(a, c);
         }
 #pragma unroll
-    for (int i = 0; i < NS; ++i) y[r * D + lane + 32 * i] = __fmul_rn(x[i], inv_sqrt_d);
-    if (lane == 0) rsc[r] = 1.f;
+    for (int p = 0; p < NP; ++p)
+      y[i][p] = pk2(__fmul_rn(x[2 * p], inv_sqrt_d), __fmul_rn(x[2 * p + 1], inv_sqrt_d));
   }
-  for (int j = threadIdx.x; j < D; j += blockDim.x) csc[j] = 1.f;
-  __syncthreads();
+
+  constexpr float kMaxS = 0x1p30f;
+  constexpr uint32_t kMinY = (77u << 24) - 1;    // 2^-50, sign shifted out, less one
   const float inv_d = 1.f / (float)D, inv_g = 1.f / (float)G;
+  float rsc = 1.f, csc = 1.f;   // scale of row lane / (32 / NR), of column threadIdx.x
   for (int it = 0; it < g.iters; ++it) {
-    // rows
-    for (int r = warp; r < G; r += 8) {
-      float x[NS], a[NS];
+    // ---- rows ----
+    float a[NR];
+    uint32_t ymin = 0xffffffffu;                 // smallest nonzero magnitude (0 wraps to the top)
 #pragma unroll
-      for (int i = 0; i < NS; ++i) {
-        x[i] = y[r * D + lane + 32 * i];
-        a[i] = __fmul_rn(x[i], x[i]);
+    for (int i = 0; i < NR; ++i) {
+      uint64_t s[NP];
+#pragma unroll
+      for (int p = 0; p < NP; ++p) {
+        s[p] = square2(y[i][p], nz);
+        const float2 f = upk2(y[i][p]);
+        ymin = min(ymin, min((__float_as_uint(f.x) << 1) - 1, (__float_as_uint(f.y) << 1) - 1));
       }
 #pragma unroll
-      for (int ns = NS / 2; ns >= 1; ns >>= 1)
+      for (int n = NP / 2; n >= 1; n >>= 1)
 #pragma unroll
-        for (int i = 0; i < ns; ++i) a[i] = __fadd_rn(a[i], a[i + ns]);
-#pragma unroll
-      for (int n = 16; n >= 1; n >>= 1) a[0] = __fadd_rn(a[0], __shfl_xor_sync(0xffffffffu, a[0], n));
-      const float sum = __shfl_sync(0xffffffffu, a[0], 0);
-      const float sg = fmaxf(__fsqrt_rn(__fmul_rn(sum, inv_d)), 1e-8f);
-      if (lane == 0) rsc[r] = __fmul_rn(rsc[r], sg);
-#pragma unroll
-      for (int i = 0; i < NS; ++i) y[r * D + lane + 32 * i] = __fdiv_rn(x[i], sg);
+        for (int p = 0; p < n; ++p) s[p] = add2(s[p], s[p + n]);
+      const float2 f = upk2(s[0]);
+      a[i] = __fadd_rn(f.x, f.y);
     }
-    __syncthreads();
-    // columns: a thread per column
-    for (int j = threadIdx.x; j < D; j += blockDim.x) {
-      float col[G], a[G];
+    const float sum = lanes_reduce<NR>(a, lane, [](float x, float z) { return __fadd_rn(x, z); });
+    const float sg = fmaxf(__fsqrt_rn(__fmul_rn(sum, inv_d)), 1e-8f);
+    const float inv = __frcp_rn(sg);
+    rsc = __fmul_rn(rsc, sg);
+    const bool fast = __all_sync(0xffffffffu, ymin >= kMinY && sg <= kMaxS);
 #pragma unroll
-      for (int r = 0; r < G; ++r) {
-        col[r] = y[r * D + j];
-        a[r] = __fmul_rn(col[r], col[r]);
+    for (int i = 0; i < NR; ++i) {
+      const float s = __shfl_sync(0xffffffffu, sg, i * (32 / NR));
+      const float v = __shfl_sync(0xffffffffu, inv, i * (32 / NR));
+      if (fast) {
+        const uint64_t ns2 = pk2(-s, -s), v2 = pk2(v, v);
+#pragma unroll
+        for (int p = 0; p < NP; ++p) y[i][p] = div2(y[i][p], ns2, v2);
+      } else {
+#pragma unroll
+        for (int p = 0; p < NP; ++p) y[i][p] = div2_exact(y[i][p], s, s);
       }
+    }
+    // ---- columns ----
 #pragma unroll
-      for (int n = G / 2; n >= 1; n >>= 1)
+    for (int p = 0; p < NP; ++p) {
+      uint64_t s[NR];
 #pragma unroll
-        for (int r = 0; r < n; ++r) a[r] = __fadd_rn(a[r], a[r + n]);
-      const float sg = fmaxf(__fsqrt_rn(__fmul_rn(a[0], inv_g)), 1e-8f);
-      csc[j] = __fmul_rn(csc[j], sg);
+      for (int i = 0; i < NR; ++i) s[i] = square2(y[i][p], nz);
 #pragma unroll
-      for (int r = 0; r < G; ++r) y[r * D + j] = __fdiv_rn(col[r], sg);
+      for (int n = NR / 2; n >= 1; n >>= 1)
+#pragma unroll
+        for (int i = 0; i < n; ++i) s[i] = add2(s[i], s[i + n]);
+      const float2 f = upk2(s[0]);
+      sm.part[warp][lane + 64 * p] = f.x;
+      sm.part[warp][lane + 64 * p + 32] = f.y;
     }
     __syncthreads();
+    if (threadIdx.x < D) {
+      float s[8];
+#pragma unroll
+      for (int w = 0; w < 8; ++w) s[w] = sm.part[w][threadIdx.x];
+#pragma unroll
+      for (int n = 4; n >= 1; n >>= 1)
+#pragma unroll
+        for (int w = 0; w < n; ++w) s[w] = __fadd_rn(s[w], s[w + n]);
+      const float cg = fmaxf(__fsqrt_rn(__fmul_rn(s[0], inv_g)), 1e-8f);
+      csc = __fmul_rn(csc, cg);
+      sm.csig[threadIdx.x] = make_float2(-cg, __frcp_rn(cg));
+    }
+    __syncthreads();
+#pragma unroll
+    for (int p = 0; p < NP; ++p) {
+      const float2 c0 = sm.csig[lane + 64 * p], c1 = sm.csig[lane + 64 * p + 32];
+      if (__all_sync(0xffffffffu, fast && fmaxf(-c0.x, -c1.x) <= kMaxS)) {
+        const uint64_t ns2 = pk2(c0.x, c1.x), v2 = pk2(c0.y, c1.y);
+#pragma unroll
+        for (int i = 0; i < NR; ++i) y[i][p] = div2(y[i][p], ns2, v2);
+      } else {
+#pragma unroll
+        for (int i = 0; i < NR; ++i) y[i][p] = div2_exact(y[i][p], -c0.x, -c1.x);
+      }
+    }
   }
-  // grouped affine along D (groups of G channels)
+
+  // ---- grouped affine along D (groups of G channels) ----
   const int codes_plane = which ? KVQ_PLANE_V_CODES : KVQ_PLANE_K_CODES;
   const int scale_plane = which ? KVQ_PLANE_V_SCALE : KVQ_PLANE_K_SCALE;
   const int zero_plane = which ? KVQ_PLANE_V_ZERO : KVQ_PLANE_K_ZERO;
   const int row_plane = which ? KVQ_PLANE_V_ROW : KVQ_PLANE_K_ROW;
   const int col_plane = which ? KVQ_PLANE_V_COL : KVQ_PLANE_K_COL;
-  // a thread per (row, group); each lane walks its group from its own lane
-  // offset, so the lanes of a warp read (and write) different banks (min, max
-  // and the codes do not depend on the order)
-  const int rot = threadIdx.x & 31;
-  for (int p = threadIdx.x; p < G * NG; p += blockDim.x) {
-    const int r = p / NG, gq = p % NG;
-    const float* row = y + r * D + gq * G;
-    uint8_t* crow = cs + r * D + gq * G;
-    float mn = row[rot & (G - 1)], mx = mn;
-    for (int jj = 1; jj < G; ++jj) {
-      const float x = row[(jj + rot) & (G - 1)];
-      mn = fminf(mn, x);
-      mx = fmaxf(mx, x);
+  {
+    float lo[NV], hi[NV];
+#pragma unroll
+    for (int i = 0; i < NR; ++i)
+#pragma unroll
+      for (int p = 0; p < NP; ++p) {
+        const float2 f = upk2(y[i][p]);
+        if constexpr (G == 64) {
+          lo[i * NG + p] = fminf(f.x, f.y);
+          hi[i * NG + p] = fmaxf(f.x, f.y);
+        } else {
+          lo[i * NG + 2 * p] = hi[i * NG + 2 * p] = f.x;
+          lo[i * NG + 2 * p + 1] = hi[i * NG + 2 * p + 1] = f.y;
+        }
+      }
+    const float mn = lanes_reduce<NV>(lo, lane, [](float x, float z) { return fminf(x, z); });
+    const float mx = lanes_reduce<NV>(hi, lane, [](float x, float z) { return fmaxf(x, z); });
+    const int u = lane / (32 / NV), r = warp + 8 * (u / NG), gq = u % NG;
+    const float sc = affine_scale(mn, mx, bits);
+    if (lane % (32 / NV) == 0) {
+      sm.grp[warp][u] = make_float4(mn, __frcp_rn(sc), sc, 0.f);
+      *plane_ptr<__half>(g, scale_plane, b, h, q0 + r, gq) = __float2half_rn(sc);
+      *plane_ptr<__half>(g, zero_plane, b, h, q0 + r, gq) = __float2half_rn(mn + 0.0f);
     }
-    const float sc = affine_scale(mn, mx, bits), inv = __frcp_rn(sc);
-    bool ok = true;
-    for (int jj = 0; jj < G; ++jj) {
-      const int j = (jj + rot) & (G - 1);
-      crow[j] = (uint8_t)clamp_code(rint_quot_fast(__fsub_rn(row[j], mn), inv, ok), bits);
-    }
-    if (!ok)                                   // a quotient near a tie: all of them exactly
-      for (int j = 0; j < G; ++j) crow[j] = (uint8_t)affine_code(row[j], mn, sc, inv, bits);
-    *plane_ptr<__half>(g, scale_plane, b, h, q0 + r, gq) = __float2half_rn(sc);
-    *plane_ptr<__half>(g, zero_plane, b, h, q0 + r, gq) = __float2half_rn(mn + 0.0f);
+    if (lane % (32 / NR) == 0)
+      *plane_ptr<__half>(g, row_plane, b, h, 0, q0 + warp + 8 * (lane / (32 / NR))) = __float2half_rn(rsc);
+    if (threadIdx.x < D)
+      *plane_ptr<__half>(g, col_plane, b, h, blk, threadIdx.x) = __float2half_rn(csc);
   }
-  for (int r = threadIdx.x; r < G; r += blockDim.x)
-    *plane_ptr<__half>(g, row_plane, b, h, 0, q0 + r) = __float2half_rn(rsc[r]);
-  for (int j = threadIdx.x; j < D; j += blockDim.x)
-    *plane_ptr<__half>(g, col_plane, b, h, blk, j) = __float2half_rn(csc[j]);
-  __syncthreads();
-  const int per = 8 / bits, row_bytes = D * bits / 8;
-  for (int i = threadIdx.x; i < G * row_bytes; i += blockDim.x) {
-    const int r = i / row_bytes, j = i % row_bytes;
-    unsigned byte = 0;
-    for (int e = 0; e < per; ++e) byte |= (unsigned)cs[r * D + j * per + e] << (e * bits);
-    plane_ptr<uint8_t>(g, codes_plane, b, h, q0 + r)[j] = (uint8_t)byte;
+  __syncwarp();
+  // codes: the nearest integer of the quotient by the reciprocal, unless that
+  // lies near a tie (then the IEEE quotient decides; quant_common.cuh).  Low
+  // and (8-bit codes) high nibbles of 8 (row, j) slots per word, transposed
+  // over 8 lanes so that a lane holds 8 neighbouring channels of one row.
+  constexpr int RW = 8 / NS;                     // rows per word
+#pragma unroll
+  for (int m = 0; m < NR / RW; ++m) {
+    uint32_t wl = 0, wh = 0;
+#pragma unroll
+    for (int ii = 0; ii < RW; ++ii) {
+      const int i = m * RW + ii;
+      bool near = false;
+      uint32_t c[NS];
+#pragma unroll
+      for (int p = 0; p < NP; ++p) {
+        const float4 g0 = sm.grp[warp][i * NG + (G == 64 ? p : 2 * p)];
+        const float4 g1 = G == 64 ? g0 : sm.grp[warp][i * NG + 2 * p + 1];
+        const uint64_t magic = pk2(12582912.f, 12582912.f), nmagic = pk2(-12582912.f, -12582912.f);
+        const uint64_t q = mul2(add2(y[i][p], pk2(-g0.x, -g1.x)), pk2(g0.y, g1.y));
+        const uint64_t t = add2(q, magic);       // 1.5 2^23 + the nearest integer
+        const float2 rf = upk2(add2(t, nmagic)), qf = upk2(q), tf = upk2(t);
+        near = near || !(fabsf(qf.x - rf.x) < 0.5f - 0x1p-14f) || !(fabsf(qf.y - rf.y) < 0.5f - 0x1p-14f);
+        c[2 * p] = __float_as_uint(tf.x) & 0xFFu;
+        c[2 * p + 1] = __float_as_uint(tf.y) & 0xFFu;
+      }
+      if (near) {
+#pragma unroll
+        for (int p = 0; p < NP; ++p) {
+          const float4 g0 = sm.grp[warp][i * NG + (G == 64 ? p : 2 * p)];
+          const float4 g1 = G == 64 ? g0 : sm.grp[warp][i * NG + 2 * p + 1];
+          const float2 f = upk2(y[i][p]);
+          c[2 * p] = (uint32_t)affine_code(f.x, g0.x, g0.z, g0.y, bits);
+          c[2 * p + 1] = (uint32_t)affine_code(f.y, g1.x, g1.z, g1.y, bits);
+        }
+      }
+#pragma unroll
+      for (int j = 0; j < NS; ++j) {
+        wl |= (c[j] & 0xFu) << (4 * (ii * NS + j));
+        if (bits == 8) wh |= (c[j] >> 4) << (4 * (ii * NS + j));
+      }
+    }
+    wl = nibble_transpose8(wl, lane);
+    const int e = lane & 7;                      // this lane's slot
+    const int r = warp + 8 * (m * RW + e / NS), c8 = 4 * (e % NS) + (lane >> 3);
+    uint8_t* row = plane_ptr<uint8_t>(g, codes_plane, b, h, q0 + r) + c8 * bits;
+    if (bits == 4) {
+      *reinterpret_cast<uint32_t*>(row) = wl;
+    } else if (bits == 2) {
+      uint32_t w = (wl | (wl >> 2)) & 0x0F0F0F0Fu;
+      w = (w | (w >> 4)) & 0x00FF00FFu;
+      *reinterpret_cast<uint16_t*>(row) = (uint16_t)(w | (w >> 8));
+    } else {
+      wh = nibble_transpose8(wh, lane);
+      *reinterpret_cast<uint2*>(row) =
+          make_uint2(nibbles_to_bytes(wl & 0xFFFFu) | nibbles_to_bytes(wh & 0xFFFFu) << 4,
+                     nibbles_to_bytes(wl >> 16) | nibbles_to_bytes(wh >> 16) << 4);
+    }
   }
 }
 
 template <int D, int G>
 cudaError_t launch_kvarn_fast(const Geom& g, int max_blocks, int L, const TokSrc& sk,
                               const TokSrc& sv, float inv_sqrt_d, cudaStream_t s) {
-  const size_t sm = (size_t)G * D * 4 + (size_t)(G + D) * 4 + (size_t)G * D;
+  const size_t sm = sizeof(KvarnSmem<D, G>);
   auto kern = kvarn_block_fast_kernel<D, G>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   if (e != cudaSuccess) return e;
-  launch_pdl(kern, dim3(dim3(max_blocks, g.B * g.H, 2)), dim3(256), sm, s, g, L, sk, sv, inv_sqrt_d);
+  launch_pdl(kern, dim3(dim3(max_blocks, g.B * g.H, 2)), dim3(256), sm, s, g, L, sk, sv, inv_sqrt_d,
+             (uint64_t)0x8000000080000000ull);
   return cudaGetLastError();
 }
 
