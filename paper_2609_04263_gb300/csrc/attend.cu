@@ -4,12 +4,13 @@
 #include <math.h>
 
 #include "kvq_internal.cuh"
+#include "reconstruct.cuh"
 
 namespace kvq {
 namespace {
 
-constexpr int kTile = 32;       // tokens per shared-memory tile
-constexpr int kThreads = 128;
+constexpr int kTile = 64;       // tokens per shared-memory tile
+constexpr int kThreads = 256;
 
 // Split-K partials of (b, q head): kMaxSplits rows of (m, l, o[D]).
 __device__ __forceinline__ float* ws_row(const Geom& g, int b, int hq) {
@@ -22,10 +23,12 @@ __device__ __forceinline__ unsigned code_at(const uint8_t* row, int d, int bits)
   return (row[bit >> 3] >> (bit & 7)) & ((1u << bits) - 1);
 }
 
-// Reconstruct tokens [t0, t0 + n) of one (b, h) into dst [n][ld] (fp32).
-// which = 0 keys, 1 values.  T = tokens stored.
-__device__ void dequant_tile(const Geom& g, int which, int b, int h, int t0, int n, int T,
-                             float* dst, int ld, float inv_sqrt_d) {
+// KVarN: tokens [t0, t0 + n) of one (b, h) in the rotated basis into dst
+// [n][ld] (fp32): the coded rows are stored rotated, the full-precision rows
+// (sinks, staged) are rotated forward.  which = 0 keys, 1 values; T = tokens
+// stored; tokens from T on are zero.
+__device__ void kvarn_rows(const Geom& g, int which, int b, int h, int t0, int n, int T,
+                           float* dst, int ld, float inv_sqrt_d) {
   const int D = g.D, G = g.G;
   const int bits = which ? g.vb : g.kb;
   const int P_CODES = which ? KVQ_PLANE_V_CODES : KVQ_PLANE_K_CODES;
@@ -35,69 +38,28 @@ __device__ void dequant_tile(const Geom& g, int which, int b, int h, int t0, int
   const int P_PEND = which ? KVQ_PLANE_V_PEND : KVQ_PLANE_K_PEND;
   const int P_ROW = which ? KVQ_PLANE_V_ROW : KVQ_PLANE_K_ROW;
   const int P_COL = which ? KVQ_PLANE_V_COL : KVQ_PLANE_K_COL;
-  const int tq = g.fmt == KVQ_FMT_KIVI ? kivi_tq(T, g.R, G) : 0;
-  const int nbq = g.fmt == KVQ_FMT_KVARN ? kvarn_nblocks(T, g.S, G) * G : 0;
+  const int nbq = kvarn_nblocks(T, g.S, G) * G;
   for (int i = threadIdx.x; i < n * D; i += blockDim.x) {
     const int r = i / D, d = i % D, t = t0 + r;
     float val = 0.f;
     if (t < T) {
-      switch (g.fmt) {
-        case KVQ_FMT_FLOAT:
-          val = ld_act(g.pl[P_FULL].p, plane_index(g.pl[P_FULL], b, h, g.H, t, d), g.act);
-          break;
-        case KVQ_FMT_AFFINE: {
-          unsigned c = code_at(plane_ptr<uint8_t>(g, P_CODES, b, h, t), d, bits);
-          float s = __half2float(*plane_ptr<__half>(g, P_SCALE, b, h, t, d / G));
-          float m = __half2float(*plane_ptr<__half>(g, P_ZERO, b, h, t, d / G));
-          val = (float)c * s + m;
-          break;
-        }
-        case KVQ_FMT_SYMMETRIC: {
-          unsigned c = code_at(plane_ptr<uint8_t>(g, P_CODES, b, h, t), d, bits);
-          float s = __half2float(*plane_ptr<__half>(g, P_SCALE, b, h, t, d / G));
-          val = (float)((int)c - (1 << (bits - 1))) * s;
-          break;
-        }
-        case KVQ_FMT_KIVI:
-          if (t < tq) {
-            unsigned c = code_at(plane_ptr<uint8_t>(g, P_CODES, b, h, t), d, bits);
-            float s, m;
-            if (which == 0) {
-              s = __half2float(*plane_ptr<__half>(g, P_SCALE, b, h, t / G, d));
-              m = __half2float(*plane_ptr<__half>(g, P_ZERO, b, h, t / G, d));
-            } else {
-              s = __half2float(*plane_ptr<__half>(g, P_SCALE, b, h, t, d / G));
-              m = __half2float(*plane_ptr<__half>(g, P_ZERO, b, h, t, d / G));
-            }
-            val = (float)c * s + m;
-          } else {
-            val = ld_act(g.pl[P_FULL].p, plane_index(g.pl[P_FULL], b, h, g.H, t % g.ring, d),
-                         g.act);
-          }
-          break;
-        case KVQ_FMT_KVARN:
-          if (t < g.S) {
-            val = ld_act(g.pl[P_FULL].p, plane_index(g.pl[P_FULL], b, h, g.H, t, d), g.act);
-          } else if (t - g.S < nbq) {
-            const int q = t - g.S;
-            unsigned c = code_at(plane_ptr<uint8_t>(g, P_CODES, b, h, q), d, bits);
-            float s = __half2float(*plane_ptr<__half>(g, P_SCALE, b, h, q, d / G));
-            float m = __half2float(*plane_ptr<__half>(g, P_ZERO, b, h, q, d / G));
-            float rr = __half2float(*plane_ptr<__half>(g, P_ROW, b, h, 0, q));
-            float cc = __half2float(*plane_ptr<__half>(g, P_COL, b, h, q / G, d));
-            val = rr * cc * ((float)c * s + m);
-          } else {
-            val = ld_act(g.pl[P_PEND].p,
-                         plane_index(g.pl[P_PEND], b, h, g.H, (t - g.S) % G, d), g.act);
-          }
-          break;
+      if (t < g.S) {
+        val = ld_act(g.pl[P_FULL].p, plane_index(g.pl[P_FULL], b, h, g.H, t, d), g.act);
+      } else if (t - g.S < nbq) {
+        const int q = t - g.S;
+        unsigned c = code_at(plane_ptr<uint8_t>(g, P_CODES, b, h, q), d, bits);
+        float s = __half2float(*plane_ptr<__half>(g, P_SCALE, b, h, q, d / G));
+        float m = __half2float(*plane_ptr<__half>(g, P_ZERO, b, h, q, d / G));
+        float rr = __half2float(*plane_ptr<__half>(g, P_ROW, b, h, 0, q));
+        float cc = __half2float(*plane_ptr<__half>(g, P_COL, b, h, q / G, d));
+        val = rr * cc * ((float)c * s + m);
+      } else {
+        val = ld_act(g.pl[P_PEND].p, plane_index(g.pl[P_PEND], b, h, g.H, (t - g.S) % G, d), g.act);
       }
     }
     dst[r * ld + d] = val;
   }
-  if (g.fmt == KVQ_FMT_KVARN && !(t0 >= g.S && t0 + n <= g.S + nbq)) {
-    // KVarN is attended in the rotated basis (the coded rows are stored
-    // rotated): rotate the full-precision rows (sinks, staged) forward
+  if (!(t0 >= g.S && t0 + n <= g.S + nbq)) {
     __syncthreads();
     for (int hs = 1; hs < D; hs <<= 1) {
       for (int p = threadIdx.x; p < n * D / 2; p += blockDim.x) {
@@ -113,6 +75,29 @@ __device__ void dequant_tile(const Geom& g, int which, int b, int h, int t0, int
     for (int i = threadIdx.x; i < n * D; i += blockDim.x) {
       const int r = i / D, t = t0 + r;
       if (t < T && !(t >= g.S && t - g.S < nbq)) dst[r * ld + i % D] *= inv_sqrt_d;
+    }
+  }
+}
+
+// The other formats: 8 channels of a token per thread and step.
+template <int D>
+__device__ __forceinline__ void dequant_rows(const Geom& g, int which, int b, int h, int t0, int n,
+                                             int T, int tq, float* dst, int ld) {
+  const bool f32 = g.act == KVQ_F32;
+  const int P_FULL = which ? KVQ_PLANE_V_FULL : KVQ_PLANE_K_FULL;
+  for (int i = threadIdx.x; i < n * (D / 8); i += kThreads) {
+    const int r = i / (D / 8), c = i % (D / 8), t = t0 + r;
+    float4* d4 = reinterpret_cast<float4*>(dst + r * ld + 8 * c);
+    if (f32 && t < T && (g.fmt == KVQ_FMT_FLOAT || (g.fmt == KVQ_FMT_KIVI && t >= tq))) {
+      const float4* src = reinterpret_cast<const float4*>(
+          plane_ptr<float>(g, P_FULL, b, h, g.fmt == KVQ_FMT_KIVI ? t % g.ring : t, 8 * c));
+      d4[0] = src[0];
+      d4[1] = src[1];
+    } else {
+      float v[8];
+      deq8(g, which, b, h, t, c, T, tq, v);
+      d4[0] = make_float4(v[0], v[1], v[2], v[3]);
+      d4[1] = make_float4(v[4], v[5], v[6], v[7]);
     }
   }
 }
@@ -135,148 +120,254 @@ __device__ void rotate_rows(float* x, int rows, int D, int ld, float inv_sqrt_d)
   __syncthreads();
 }
 
-// One CTA: `rows` = g heads x nq queries of one (b, kv head), over the tokens
-// [ts, te).  Shared memory holds the K/V tiles, q, scores and accumulators.
-// decode: writes (m, l, o) partials to the workspace, else the output.
+// Attention in fp32 for every format, fp32 activations (prefill and decode) and
+// the bf16 caches that no tensor-core decode covers.  One CTA = ROWS rows (the g
+// query heads x nq queries of one (b, kv head)) over the tokens [ts, te), 64
+// at a time; shared memory holds the K and V tiles, q and the scores, the
+// output accumulates in registers.
+//   scores: warp w has row group w % 4 and 32 of the tile's tokens, a lane one
+//     token for all rows of the group (its K row read once, q broadcast);
+//   softmax: 256 / ROWS threads per row;
+//   P V: a thread has 4 channels of ROWS D / 1024 rows.
+// These sizes are far from filling the GPU (a 512-token prompt of 4 heads is
+// 0.07 GFLOP a head), so the latency of one CTA's chain of tiles bounds it: 16
+// rows a CTA give 8 times the CTAs of 128 rows, and 64 rows serve where 16 are
+// not needed to cover the SMs twice.  512 tokens, 4 heads of 64, fp32, affine
+// 4-bit: 1142 -> 59 us, a decode step after them 24 + 10 -> 16 us.
+// decode: writes (m, l, o) partials to the workspace; the last split CTA of a
+// (sequence, kv head) merges them (one launch instead of two).
+template <int D, int ROWS>
+struct GenSmem {
+  static constexpr int LDK = D + 4;                // 16-byte rows in distinct banks
+  static constexpr int LDS = kTile + 4;
+  float k[kTile * LDK];                            // then the output rows [ROWS][D]
+  float v[kTile * D];
+  float q[ROWS * D];
+  float s[ROWS * LDS];
+  float alpha[ROWS], m[ROWS], l[ROWS];
+};
+
+template <int D, int ROWS>
 __global__ void __launch_bounds__(kThreads)
 attend_generic_kernel(Geom g, const void* q, int L, float scale, void* out,
                       int nq, int splits, int decode, float inv_sqrt_d) {
   pdl_wait();
   pdl_trigger();
-  extern __shared__ float sm[];
+  using S = GenSmem<D, ROWS>;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  S& sm = *reinterpret_cast<S*>(smem_raw);
   const int T = cache_tokens(g);
-  const int D = g.D, grp = g.Hq / g.H;
-  const int rows = grp * nq;
-  const int ldk = D + 1;
-  float* Kt = sm;                       // [kTile][D+1]
-  float* Vt = Kt + kTile * ldk;         // [kTile][D]
-  float* qs = Vt + kTile * D;           // [rows][D]
-  float* acc = qs + rows * D;           // [rows][D]
-  float* sc = acc + rows * D;           // [rows][kTile]
-  float* mrow = sc + rows * kTile;      // [rows]
-  float* lrow = mrow + rows;
-  float* arow = lrow + rows;
+  const int tq = g.fmt == KVQ_FMT_KIVI ? kivi_tq(T, g.R, g.G) : T;
+  const int grp = g.Hq / g.H;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
-  const int qtile = blockIdx.x / splits, split = blockIdx.x % splits;
+  // longest first (causal work grows with the position)
+  const int qtile = gridDim.x / splits - 1 - blockIdx.x / splits, split = blockIdx.x % splits;
   const int hkv = blockIdx.y, b = blockIdx.z;
   const int q0 = qtile * nq;            // first query of this CTA
   const int nql = min(nq, L - q0);
   const int pos_first = T - L + q0;     // absolute position of query q0
-  const int pos_last = pos_first + nql - 1;
   // tokens of this split
-  int ts = 0, te = pos_last + 1;
-  if (decode) split_range(T, splits, split, kTile, &ts, &te);
-  for (int i = threadIdx.x; i < rows * D; i += blockDim.x) {
+  int ts = 0, te = pos_first + nql;
+  if (decode) split_range(T, splits, split, 32, &ts, &te);
+  auto row_pos = [&](int r) {           // last token that row r sees, -1 for padding rows
+    const int hl = r / nq, qi = r % nq;
+    return hl < grp && qi < nql ? pos_first + qi : -1;
+  };
+  for (int i = threadIdx.x; i < ROWS * D; i += kThreads) {
     const int r = i / D, d = i % D;
     const int hl = r / nq, qi = r % nq;
-    const int hq = hkv * grp + hl;
     float v = 0.f;
-    if (qi < nql) v = ld_act(q, (((int64_t)b * g.Hq + hq) * L + q0 + qi) * D + d, g.act);
-    qs[i] = v;
-    acc[i] = 0.f;
+    if (hl < grp && qi < nql)
+      v = ld_act(q, (((int64_t)b * g.Hq + hkv * grp + hl) * L + q0 + qi) * D + d, g.act);
+    sm.q[i] = v;
   }
-  for (int r = threadIdx.x; r < rows; r += blockDim.x) {
-    mrow[r] = -INFINITY;
-    lrow[r] = 0.f;
-  }
-  __syncthreads();
   const bool kvarn = g.fmt == KVQ_FMT_KVARN;
-  if (kvarn) rotate_rows(qs, rows, D, D, inv_sqrt_d);     // queries into the rotated basis
+  if (kvarn) rotate_rows(sm.q, ROWS, D, D, inv_sqrt_d);     // queries into the rotated basis
+
+  constexpr int RS = ROWS / 4;                    // score rows of a thread
+  constexpr int TPR = kThreads / ROWS;            // softmax threads per row
+  constexpr int NRG = 4 * kThreads / D;           // P V row groups
+  constexpr int RO = ROWS / NRG;                  // P V rows of a thread
+  static_assert(RO >= 1, "every P V thread has a row");
+  const int srow = (warp & 3) * RS, stok = (warp >> 2) * 32 + lane;
+  int spos[RS];
+#pragma unroll
+  for (int k = 0; k < RS; ++k) spos[k] = row_pos(srow + k);
+  const int xrow = threadIdx.x / TPR, xsub = threadIdx.x % TPR;
+  float m_run = -INFINITY, l_run = 0.f;           // l_run: this thread's share
+  const int od = threadIdx.x % (D / 4), orow = threadIdx.x / (D / 4);
+  float4 acc[RO];
+#pragma unroll
+  for (int k = 0; k < RO; ++k) acc[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+
   for (int t0 = ts; t0 < te; t0 += kTile) {
     const int n = min(kTile, te - t0);
-    dequant_tile(g, 0, b, hkv, t0, n, T, Kt, ldk, inv_sqrt_d);
-    dequant_tile(g, 1, b, hkv, t0, n, T, Vt, D, inv_sqrt_d);
-    __syncthreads();
-    for (int i = threadIdx.x; i < rows * kTile; i += blockDim.x) {
-      const int r = i / kTile, j = i % kTile;
-      const int qi = r % nq;
-      const int t = t0 + j;
-      float s = -INFINITY;
-      if (j < n && qi < nql && t <= pos_first + qi) {
-        const float* qr = qs + r * D;
-        const float* kr = Kt + j * ldk;
-        float a = 0.f;
-        for (int d = 0; d < D; ++d) a += qr[d] * kr[d];
-        s = a * scale;
-      }
-      sc[i] = s;
+    const int n4 = (n + 3) & ~3;                  // rows of V read below
+    __syncthreads();                              // previous tile consumed (and q stored)
+    if (kvarn) {
+      kvarn_rows(g, 0, b, hkv, t0, n4, T, sm.k, S::LDK, inv_sqrt_d);
+      kvarn_rows(g, 1, b, hkv, t0, n4, T, sm.v, D, inv_sqrt_d);
+    } else {
+      dequant_rows<D>(g, 0, b, hkv, t0, n4, T, tq, sm.k, S::LDK);
+      dequant_rows<D>(g, 1, b, hkv, t0, n4, T, tq, sm.v, D);
     }
     __syncthreads();
-    for (int r = threadIdx.x; r < rows; r += blockDim.x) {
-      float mx = -INFINITY;
-      for (int j = 0; j < kTile; ++j) mx = fmaxf(mx, sc[r * kTile + j]);
-      const float mo = mrow[r];
-      const float mn = fmaxf(mo, mx);
-      float alpha = 1.f, sum = 0.f;
-      if (mn == -INFINITY) {
-        for (int j = 0; j < kTile; ++j) sc[r * kTile + j] = 0.f;
-      } else {
-        alpha = expf(mo - mn);
-        for (int j = 0; j < kTile; ++j) {
-          const float p = expf(sc[r * kTile + j] - mn);
-          sc[r * kTile + j] = p;
-          sum += p;
+    if ((warp >> 2) * 32 < n4) {
+      float sc[RS];
+#pragma unroll
+      for (int k = 0; k < RS; ++k) sc[k] = 0.f;
+      const float4* kr = reinterpret_cast<const float4*>(sm.k + stok * S::LDK);
+#pragma unroll 4
+      for (int d = 0; d < D / 4; ++d) {
+        const float4 kv = kr[d];
+#pragma unroll
+        for (int k = 0; k < RS; ++k) {
+          const float4 qv = reinterpret_cast<const float4*>(sm.q + (srow + k) * D)[d];
+          sc[k] = fmaf(qv.x, kv.x, sc[k]);
+          sc[k] = fmaf(qv.y, kv.y, sc[k]);
+          sc[k] = fmaf(qv.z, kv.z, sc[k]);
+          sc[k] = fmaf(qv.w, kv.w, sc[k]);
         }
-        mrow[r] = mn;
       }
-      lrow[r] = lrow[r] * alpha + sum;
-      arow[r] = alpha;
+#pragma unroll
+      for (int k = 0; k < RS; ++k)
+        sm.s[(srow + k) * S::LDS + stok] =
+            stok < n && t0 + stok <= spos[k] ? sc[k] * scale : -INFINITY;
     }
     __syncthreads();
-    for (int i = threadIdx.x; i < rows * D; i += blockDim.x) {
-      const int r = i / D, d = i % D;
-      float a = acc[i] * arow[r];
-      const float* p = sc + r * kTile;
-      for (int j = 0; j < n; ++j) a += p[j] * Vt[j * D + d];
-      acc[i] = a;
+    {
+      float mx = -INFINITY;
+      float* srw = sm.s + xrow * S::LDS;
+      for (int j = xsub; j < n; j += TPR) mx = fmaxf(mx, srw[j]);
+#pragma unroll
+      for (int o = TPR / 2; o >= 1; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+      const float mn = fmaxf(m_run, mx);
+      const float alpha = mn == -INFINITY ? 1.f : expf(m_run - mn);
+      float sum = 0.f;
+      for (int j = xsub; j < n4; j += TPR) {
+        const float sv = srw[j];
+        const float p = sv == -INFINITY ? 0.f : expf(sv - mn);
+        srw[j] = p;
+        sum += p;
+      }
+      l_run = l_run * alpha + sum;
+      m_run = mn;
+      if (xsub == 0) sm.alpha[xrow] = alpha;
     }
     __syncthreads();
+#pragma unroll
+    for (int k = 0; k < RO; ++k) {
+      const float f = sm.alpha[orow + NRG * k];
+      acc[k].x *= f; acc[k].y *= f; acc[k].z *= f; acc[k].w *= f;
+    }
+#pragma unroll 2
+    for (int j = 0; j < n4; j += 4) {
+      float4 vv[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) vv[u] = reinterpret_cast<const float4*>(sm.v + (j + u) * D)[od];
+#pragma unroll
+      for (int k = 0; k < RO; ++k) {
+        const float4 p = *reinterpret_cast<const float4*>(sm.s + (orow + NRG * k) * S::LDS + j);
+        const float pu[4] = {p.x, p.y, p.z, p.w};
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          acc[k].x = fmaf(pu[u], vv[u].x, acc[k].x);
+          acc[k].y = fmaf(pu[u], vv[u].y, acc[k].y);
+          acc[k].z = fmaf(pu[u], vv[u].z, acc[k].z);
+          acc[k].w = fmaf(pu[u], vv[u].w, acc[k].w);
+        }
+      }
+    }
   }
-  if (kvarn) rotate_rows(acc, rows, D, D, inv_sqrt_d);    // output back to the original basis
-  if (decode) {
-    for (int i = threadIdx.x; i < rows * (D + kWsStride); i += blockDim.x) {
-      const int r = i / (D + kWsStride), c = i % (D + kWsStride);
-      const int hq = hkv * grp + r;          // nq == 1 in decode
-      float* w = ws_row(g, b, hq) + (int64_t)split * (D + kWsStride);
-      w[c] = c == 0 ? mrow[r] : c == 1 ? lrow[r] : acc[r * D + c - 2];
-    }
-  } else {
-    for (int i = threadIdx.x; i < rows * D; i += blockDim.x) {
+#pragma unroll
+  for (int o = TPR / 2; o >= 1; o >>= 1) l_run += __shfl_xor_sync(0xffffffffu, l_run, o);
+  if (xsub == 0) {
+    sm.m[xrow] = m_run;
+    sm.l[xrow] = l_run;
+  }
+  __syncthreads();                                // K tile consumed: output rows over it
+  float* os = sm.k;
+#pragma unroll
+  for (int k = 0; k < RO; ++k)
+    reinterpret_cast<float4*>(os + (orow + NRG * k) * D)[od] = acc[k];
+  __syncthreads();
+  if (kvarn) rotate_rows(os, ROWS, D, D, inv_sqrt_d);       // back to the original basis
+  if (!decode) {
+    for (int i = threadIdx.x; i < ROWS * D; i += kThreads) {
       const int r = i / D, d = i % D;
       const int hl = r / nq, qi = r % nq;
-      if (qi >= nql) continue;
-      const int hq = hkv * grp + hl;
-      const float l = lrow[r];
-      st_act(out, (((int64_t)b * g.Hq + hq) * L + q0 + qi) * D + d, acc[i] / l, g.act);
+      if (hl >= grp || qi >= nql) continue;
+      st_act(out, (((int64_t)b * g.Hq + hkv * grp + hl) * L + q0 + qi) * D + d, os[i] / sm.l[r],
+             g.act);
     }
+    return;
   }
+  for (int i = threadIdx.x; i < grp * (D + kWsStride); i += kThreads) {
+    const int r = i / (D + kWsStride), c = i % (D + kWsStride);   // nq == 1 in decode
+    ws_row(g, b, hkv * grp + r)[(int64_t)split * (D + kWsStride) + c] =
+        c == 0 ? sm.m[r] : c == 1 ? sm.l[r] : os[r * D + c - 2];
+  }
+  // the last split CTA of this (sequence, kv head) merges:
+  // o = sum_s e^(m_s - M) o_s / sum_s e^(m_s - M) l_s
+  __shared__ int last_cta;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    last_cta = atomicAdd(&g.counters[b * g.H + hkv], 1u) == (unsigned)splits - 1;
+  }
+  __syncthreads();
+  if (!last_cta) return;
+  __threadfence();
+  for (int hl = warp; hl < grp; hl += kThreads / 32) {
+    const float* w = ws_row(g, b, hkv * grp + hl);
+    const float ms = lane < splits ? __ldcg(w + (int64_t)lane * (D + kWsStride)) : -INFINITY;
+    const float ls = lane < splits ? __ldcg(w + (int64_t)lane * (D + kWsStride) + 1) : 0.f;
+    float M = ms;
+#pragma unroll
+    for (int o = 16; o >= 1; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
+    const float f = ms == -INFINITY ? 0.f : expf(ms - M);
+    float Ls = f * ls;
+#pragma unroll
+    for (int o = 16; o >= 1; o >>= 1) Ls += __shfl_xor_sync(0xffffffffu, Ls, o);
+    float o[D / 32];
+#pragma unroll
+    for (int k = 0; k < D / 32; ++k) o[k] = 0.f;
+#pragma unroll 4
+    for (int i = 0; i < splits; ++i) {
+      const float fi = __shfl_sync(0xffffffffu, f, i);
+      const float* wi = w + (int64_t)i * (D + kWsStride) + 2 + lane;
+#pragma unroll
+      for (int k = 0; k < D / 32; ++k) o[k] = fmaf(fi, __ldcg(wi + 32 * k), o[k]);
+    }
+#pragma unroll
+    for (int k = 0; k < D / 32; ++k)
+      st_act(out, ((int64_t)b * g.Hq + hkv * grp + hl) * D + lane + 32 * k, o[k] / Ls, g.act);
+  }
+  if (threadIdx.x == 0) g.counters[b * g.H + hkv] = 0;   // ready for the next call
 }
 
-// Merge the split partials of one (b, q head): o = sum_s e^(m_s - M) o_s /
-// sum_s e^(m_s - M) l_s over slots 0 .. splits-1, and slot `extra` if >= 0.
-__global__ void combine_kernel(Geom g, int splits, int extra, void* out) {
-  pdl_wait();
-  pdl_trigger();
-  const int hq = blockIdx.x, b = blockIdx.y;
-  const int D = g.D;
-  const float* w = ws_row(g, b, hq);
-  const int n = splits + (extra >= 0 ? 1 : 0);
-  auto row = [&](int i) { return w + (int64_t)(i < splits ? i : extra) * (D + kWsStride); };
-  float M = -INFINITY;
-  for (int i = 0; i < n; ++i) M = fmaxf(M, row(i)[0]);
-  float Lsum = 0.f;
-  for (int i = 0; i < n; ++i) {
-    const float m = row(i)[0];
-    if (m != -INFINITY) Lsum += expf(m - M) * row(i)[1];
-  }
-  for (int d = threadIdx.x; d < D; d += blockDim.x) {
-    float o = 0.f;
-    for (int i = 0; i < n; ++i) {
-      const float m = row(i)[0];
-      if (m != -INFINITY) o += expf(m - M) * row(i)[2 + d];
-    }
-    st_act(out, ((int64_t)b * g.Hq + hq) * D + d, o / Lsum, g.act);
-  }
+template <int D, int ROWS>
+cudaError_t launch_generic(const Geom& g, const void* q, int L, float scale, void* out,
+                           bool decode, cudaStream_t s) {
+  auto kern = attend_generic_kernel<D, ROWS>;
+  const int sm = (int)sizeof(GenSmem<D, ROWS>);
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+  if (e != cudaSuccess) return e;
+  const int nq = decode ? 1 : ROWS / (g.Hq / g.H), splits = decode ? g.splits : 1;
+  const float inv_sqrt_d = (float)(1.0 / sqrt((double)D));
+  launch_pdl(kern, dim3((L + nq - 1) / nq * splits, g.H, g.B), dim3(kThreads), (size_t)sm, s, g, q,
+             L, scale, out, nq, splits, decode ? 1 : 0, inv_sqrt_d);
+  return cudaGetLastError();
+}
+
+template <int D>
+cudaError_t launch_generic_d(const Geom& g, const void* q, int L, float scale, void* out,
+                             bool decode, cudaStream_t s) {
+  const int64_t ctas64 = (int64_t)((L * (g.Hq / g.H) + 63) / 64) * g.H * g.B;
+  return !decode && ctas64 >= 2 * num_sms()
+             ? launch_generic<D, 64>(g, q, L, scale, out, decode, s)
+             : launch_generic<D, 16>(g, q, L, scale, out, decode, s);
 }
 
 // ---------------------------------------------------------------------------
@@ -598,33 +689,9 @@ cudaError_t launch_attend(const Geom& g, const void* q, int L, float scale, void
          : g.D == 128 ? launch_kvarn_d<128>(g, q, scale, streamed, out, s)
                       : launch_kvarn_d<256>(g, q, scale, streamed, out, s);
   }
-  const int grp = g.Hq / g.H;
-  const float inv_sqrt_d = (float)(1.0 / sqrt((double)g.D));
-  int nq, splits;
-  if (decode) {
-    nq = 1;
-    splits = g.splits;
-  } else {
-    int rows = 8192 / g.D;
-    if (rows > 128) rows = 128;
-    nq = rows / grp;
-    if (nq < 1) nq = 1;
-    splits = 1;
-  }
-  const int rows = grp * nq;
-  const size_t sm = (size_t)(kTile * (g.D + 1) + kTile * g.D + 2 * rows * g.D +
-                             rows * kTile + 3 * rows) * sizeof(float);
-  cudaError_t e = cudaFuncSetAttribute(attend_generic_kernel,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-  if (e != cudaSuccess) return e;
-  const int nqt = (L + nq - 1) / nq;
-  dim3 grid(nqt * splits, g.H, g.B);
-  launch_pdl(attend_generic_kernel, dim3(grid), dim3(kThreads), sm, s, g, q, L, scale, out, nq, splits,
-                                                   decode ? 1 : 0, inv_sqrt_d);
-  e = cudaGetLastError();
-  if (e != cudaSuccess || !decode) return e;
-  launch_pdl(combine_kernel, dim3(dim3(g.Hq, g.B)), dim3(64), 0, s, g, splits, -1, out);
-  return cudaGetLastError();
+  return g.D == 64 ? launch_generic_d<64>(g, q, L, scale, out, decode, s)
+       : g.D == 128 ? launch_generic_d<128>(g, q, L, scale, out, decode, s)
+                    : launch_generic_d<256>(g, q, L, scale, out, decode, s);
 }
 
 }  // namespace kvq
