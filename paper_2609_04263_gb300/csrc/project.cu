@@ -16,116 +16,177 @@ namespace {
 using namespace pdec;
 
 constexpr int kMT = 32;     // rows per CTA
+constexpr int kNT = 64;     // output columns per CTA: 32 RoPE pairs of one head
 constexpr int kKC = 32;     // k chunk
-constexpr int kThreads = 256;
+constexpr int kThreads = 128;
 
-// One CTA: kMT rows of x times one head's D output columns.
-__global__ void __launch_bounds__(kThreads) project_simt_kernel(ProjArgs p) {
+// Elements k .. k + 3 of a row (zeros from K on).
+template <typename T>
+__device__ __forceinline__ float4 load4(const T* row, int k, int K, bool vec);
+template <>
+__device__ __forceinline__ float4 load4<float>(const float* row, int k, int K, bool vec) {
+  if (vec) return k < K ? *reinterpret_cast<const float4*>(row + k) : make_float4(0.f, 0.f, 0.f, 0.f);
+  float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (k < K) v.x = row[k];
+  if (k + 1 < K) v.y = row[k + 1];
+  if (k + 2 < K) v.z = row[k + 2];
+  if (k + 3 < K) v.w = row[k + 3];
+  return v;
+}
+template <>
+__device__ __forceinline__ float4 load4<__nv_bfloat16>(const __nv_bfloat16* row, int k, int K, bool) {
+  if (k >= K) return make_float4(0.f, 0.f, 0.f, 0.f);       // K is a multiple of 64
+  const uint2 u = *reinterpret_cast<const uint2*>(row + k);
+  const float2 a = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&u.x));
+  const float2 b = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&u.y));
+  return make_float4(a.x, a.y, b.x, b.y);
+}
+
+// More than 16 rows, fp32 (and the bf16 head shapes the tensor-core kernel does
+// not tile): one CTA = kMT rows of x times 32 channel pairs (c, c + D/2) of one
+// head, a thread 4 rows x 2 pairs in registers.  The rank-r product x A_p^T rides
+// along as up to 64 further columns, so x is read once per CTA; every output
+// is one fp32 chain over k in order, then over the ranks.
+// What bounds it at these sizes (512 rows x 768 outputs x 256 inputs: 0.2
+// GFLOP) is the chain of k chunks: small tiles keep 192 CTAs in flight and the
+// next chunk's loads go out before the current one is multiplied: 129 us with
+// one shared-memory read per multiplication, 29 us so.
+template <typename T>
+__global__ void __launch_bounds__(kThreads) project_tile_kernel(ProjArgs p) {
   pdl_wait();
   pdl_trigger();
-  extern __shared__ float sm[];
-  const int D = p.D, M = p.B * p.L;
-  const int hh = blockIdx.y;                 // stacked head index over q, k, v
+  __shared__ __align__(16) float Xs[2][kKC][kMT + 4];
+  __shared__ __align__(16) float Ws[2][kKC][kNT + 4];
+  __shared__ __align__(16) float As[2][kKC][64 + 4];        // then (alpha/r) x A^T [kMT][68]
+  const int D = p.D, M = p.B * p.L, K = p.d_in, half = D / 2;
+  const int tiles = D / kNT;                 // column tiles per head
+  const int hh = blockIdx.y / tiles;         // stacked head index over q, k, v
+  const int c0 = blockIdx.y % tiles * (kNT / 2);
   const int proj = hh < p.Hq ? 0 : hh < p.Hq + p.Hkv ? 1 : 2;
   const int head = proj == 0 ? hh : proj == 1 ? hh - p.Hq : hh - p.Hq - p.Hkv;
-  const int r = p.r[proj];
+  const int r = p.r[proj], ne = (r + 15) / 16;
   const int m0 = blockIdx.x * kMT;
-  float* Xs = sm;                            // [kMT][kKC+1]
-  float* Ws = Xs + kMT * (kKC + 1);          // [max(D, 64)][kKC+1]
-  float* U = Ws + 256 * (kKC + 1);           // [kMT][64]
-  float* Y = U + kMT * 64;                   // [kMT][D]
-  const int rg = kThreads / D > 0 ? kThreads / D : 1;   // row groups
-  const int col = threadIdx.x % D, rgi = threadIdx.x / D;
-  const int rows_per = kMT / rg;
-  float acc[32];
+  const bool vec = sizeof(T) == 2 || K % 4 == 0;
+  const T* x = reinterpret_cast<const T*>(p.x);
+  const T* w = reinterpret_cast<const T*>(p.w);
+  const T* am = reinterpret_cast<const T*>(p.a[proj]);
+  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+  // operand rows of this thread: x row tid % 32, W rows tid % 64, A rows tid % 64,
+  // at k chunks of 4 tid / 32 (x) or tid / 64 + 2 i (W, A)
+  const int xr = tid & 31, xk = (tid >> 5) * 4;
+  const int wr = tid & 63, wk = (tid >> 6) * 4;
+  const bool xin = m0 + xr < M, ain = wr < r;
+  const T* xrow = x + (int64_t)(xin ? m0 + xr : 0) * K;
+  const T* wrow = w + ((int64_t)hh * D + (wr < 32 ? c0 + wr : half + c0 + wr - 32)) * K;
+  const T* arow = am + (int64_t)(ain ? wr : 0) * K;
+  const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+  float4 xv[2], wv[4], av[4];
+  auto load = [&](int k0) {
 #pragma unroll
-  for (int i = 0; i < 32; ++i) acc[i] = 0.f;
-  float uacc[8];
+    for (int i = 0; i < 2; ++i) xv[i] = xin ? load4<T>(xrow, k0 + xk + 16 * i, K, vec) : zero;
 #pragma unroll
-  for (int i = 0; i < 8; ++i) uacc[i] = 0.f;
-
-  // x A^T (rank-r down projection), (m, j) pairs spread over the threads
-  if (r > 0) {
-    for (int k0 = 0; k0 < p.d_in; k0 += kKC) {
-      for (int i = threadIdx.x; i < kMT * kKC; i += kThreads) {
-        const int m = i / kKC, k = i % kKC;
-        const int gm = m0 + m;
-        Xs[m * (kKC + 1) + k] = (gm < M && k0 + k < p.d_in)
-            ? ld_act(p.x, (int64_t)gm * p.d_in + k0 + k, p.act) : 0.f;
-      }
-      for (int i = threadIdx.x; i < r * kKC; i += kThreads) {
-        const int j = i / kKC, k = i % kKC;
-        Ws[j * (kKC + 1) + k] = k0 + k < p.d_in
-            ? ld_act(p.a[proj], (int64_t)j * p.d_in + k0 + k, p.act) : 0.f;
-      }
-      __syncthreads();
+    for (int i = 0; i < 4; ++i) {
+      wv[i] = load4<T>(wrow, k0 + wk + 8 * i, K, vec);
+      av[i] = ain ? load4<T>(arow, k0 + wk + 8 * i, K, vec) : zero;
+    }
+  };
+  auto put = [](float (*s)[kNT + 4], int k, int row, const float4& v) {
+    s[k][row] = v.x;
+    s[k + 1][row] = v.y;
+    s[k + 2][row] = v.z;
+    s[k + 3][row] = v.w;
+  };
+  auto store = [&](int buf) {
 #pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const int idx = threadIdx.x + u * kThreads;
-        if (idx < kMT * r) {
-          const int m = idx / r, j = idx % r;
-          float a = uacc[u];
-          for (int k = 0; k < kKC; ++k) a += Xs[m * (kKC + 1) + k] * Ws[j * (kKC + 1) + k];
-          uacc[u] = a;
-        }
-      }
-      __syncthreads();
+    for (int i = 0; i < 2; ++i) {
+      const int k = xk + 16 * i;
+      Xs[buf][k][xr] = xv[i].x;
+      Xs[buf][k + 1][xr] = xv[i].y;
+      Xs[buf][k + 2][xr] = xv[i].z;
+      Xs[buf][k + 3][xr] = xv[i].w;
     }
 #pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      const int idx = threadIdx.x + u * kThreads;
-      if (idx < kMT * r) U[(idx / r) * 64 + idx % r] = uacc[u] * p.alpha_over_r;
+    for (int i = 0; i < 4; ++i) {
+      put(Ws[buf], wk + 8 * i, wr, wv[i]);
+      if (ne) put(As[buf], wk + 8 * i, wr, av[i]);
     }
-  }
-  // x W^T for this head's rows of W
-  for (int k0 = 0; k0 < p.d_in; k0 += kKC) {
-    for (int i = threadIdx.x; i < kMT * kKC; i += kThreads) {
-      const int m = i / kKC, k = i % kKC;
-      const int gm = m0 + m;
-      Xs[m * (kKC + 1) + k] = (gm < M && k0 + k < p.d_in)
-          ? ld_act(p.x, (int64_t)gm * p.d_in + k0 + k, p.act) : 0.f;
-    }
-    for (int i = threadIdx.x; i < D * kKC; i += kThreads) {
-      const int n = i / kKC, k = i % kKC;
-      Ws[n * (kKC + 1) + k] = k0 + k < p.d_in
-          ? ld_act(p.w, ((int64_t)hh * D + n) * p.d_in + k0 + k, p.act) : 0.f;
-    }
+  };
+  float acc[4][4] = {}, uacc[4][4] = {};     // [row][2 tx, 2 tx + 1, their partners], [row][16 e + tx]
+  const int chunks = (K + kKC - 1) / kKC;
+  load(0);
+  for (int c = 0; c < chunks; ++c) {
+    const int buf = c & 1;
+    store(buf);
     __syncthreads();
+    if (c + 1 < chunks) load((c + 1) * kKC);
+#pragma unroll 8
     for (int k = 0; k < kKC; ++k) {
-      const float wv = Ws[col * (kKC + 1) + k];
-      for (int i = 0; i < rows_per; ++i)
-        acc[i] += Xs[(rgi + i * rg) * (kKC + 1) + k] * wv;
+      const float4 xq = *reinterpret_cast<const float4*>(&Xs[buf][k][4 * ty]);
+      const float2 w0 = *reinterpret_cast<const float2*>(&Ws[buf][k][2 * tx]);
+      const float2 w1 = *reinterpret_cast<const float2*>(&Ws[buf][k][32 + 2 * tx]);
+      const float xm[4] = {xq.x, xq.y, xq.z, xq.w}, wn[4] = {w0.x, w0.y, w1.x, w1.y};
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(xm[i], wn[j], acc[i][j]);
+#pragma unroll
+      for (int e = 0; e < 4; ++e)
+        if (e < ne) {
+          const float ae = As[buf][k][16 * e + tx];
+#pragma unroll
+          for (int i = 0; i < 4; ++i) uacc[i][e] = fmaf(xm[i], ae, uacc[i][e]);
+        }
     }
-    __syncthreads();
+    // (the other buffer is free: every thread passed this chunk's barrier
+    // after it had finished the chunk before)
   }
   // + (alpha/r) (x A^T) B^T
   if (r > 0) {
-    const int64_t brow = (int64_t)head * D + col;
+    float (*U)[68] = reinterpret_cast<float (*)[68]>(&As[0][0][0]);
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) U[4 * ty + i][16 * e + tx] = uacc[i][e] * p.alpha_over_r;
+    __syncthreads();
+    const T* bm = reinterpret_cast<const T*>(p.bm[proj]);
+    const int ch[4] = {c0 + 2 * tx, c0 + 2 * tx + 1, half + c0 + 2 * tx, half + c0 + 2 * tx + 1};
     for (int j = 0; j < r; ++j) {
-      const float bv = ld_act(p.bm[proj], brow * r + j, p.act);
-      for (int i = 0; i < rows_per; ++i) acc[i] += U[(rgi + i * rg) * 64 + j] * bv;
+      float bv[4];
+#pragma unroll
+      for (int n = 0; n < 4; ++n) bv[n] = (float)bm[((int64_t)head * D + ch[n]) * r + j];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const float u = U[4 * ty + i][j];
+#pragma unroll
+        for (int n = 0; n < 4; ++n) acc[i][n] = fmaf(u, bv[n], acc[i][n]);
+      }
     }
   }
-  for (int i = 0; i < rows_per; ++i) Y[(rgi + i * rg) * D + col] = acc[i];
-  __syncthreads();
-  // RoPE (rotate-half) on q and k; angle in fp64 for accuracy
+  // RoPE (rotate-half) on q and k, head-major store
   const bool rope = proj < 2 && p.rope_base > 0.f;
   const int H = proj == 0 ? p.Hq : p.Hkv;
-  for (int i = threadIdx.x; i < kMT * D; i += kThreads) {
-    const int m = i / D, d = i % D;
-    const int gm = m0 + m;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int gm = m0 + 4 * ty + i;
     if (gm >= M) continue;
     const int b = gm / p.L, l = gm % p.L;
-    float v = Y[i];
-    if (rope) {
-      const int half = D / 2, fi = d % half;
-      float c, s;
-      rope_cos_sin(p.pos0 + pos_of(p.pos_dev, p.pos_stride, b) + l, p.theta_hi[fi],
-                   p.theta_lo[fi], &c, &s);
-      if (d < half) v = Y[m * D + d] * c - Y[m * D + d + half] * s;
-      else v = Y[m * D + d] * c + Y[m * D + d - half] * s;
+    const int64_t o = (((int64_t)b * H + head) * p.L + l) * D + c0 + 2 * tx;
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      float y1 = acc[i][j], y2 = acc[i][2 + j];
+      if (rope) {
+        float c, s;
+        const int fi = c0 + 2 * tx + j;
+        rope_cos_sin(p.pos0 + pos_of(p.pos_dev, p.pos_stride, b) + l, p.theta_hi[fi], p.theta_lo[fi],
+                     &c, &s);
+        const float r1 = y1 * c - y2 * s, r2 = y2 * c + y1 * s;
+        y1 = r1;
+        y2 = r2;
+      }
+      st_act(p.out[proj], o + j, y1, p.act);
+      st_act(p.out[proj], o + half + j, y2, p.act);
     }
-    st_act(p.out[proj], (((int64_t)b * H + head) * p.L + l) * D + d, v, p.act);
   }
 }
 
@@ -443,13 +504,9 @@ cudaError_t launch_project(const void* x, int B, int L, int d_in, const void* w,
     return launch_decode_mma(p, s);
   if (M <= kSkinnyMaxM && (size_t)M * d_in * 4 <= 120 * 1024 && d_in % 64 == 0)
     return act == KVQ_BF16 ? launch_skinny<__nv_bfloat16>(p, s) : launch_skinny<float>(p, s);
-  const size_t sm = (size_t)(kMT * (kKC + 1) + 256 * (kKC + 1) + kMT * 64 + kMT * D) *
-                    sizeof(float);
-  cudaError_t e = cudaFuncSetAttribute(project_simt_kernel,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-  if (e != cudaSuccess) return e;
-  dim3 grid((M + kMT - 1) / kMT, Hq + 2 * Hkv);
-  launch_pdl(project_simt_kernel, dim3(grid), dim3(kThreads), sm, s, p);
+  const dim3 grid((M + kMT - 1) / kMT, (Hq + 2 * Hkv) * (D / kNT));
+  if (act == KVQ_BF16) launch_pdl(project_tile_kernel<__nv_bfloat16>, grid, dim3(kThreads), 0, s, p);
+  else launch_pdl(project_tile_kernel<float>, grid, dim3(kThreads), 0, s, p);
   return cudaGetLastError();
 }
 
