@@ -1,0 +1,637 @@
+// Causal GQA prefill attention over a KVarN cache at head_dim 256 on the
+// 5th-generation tensor cores (tcgen05), Sections 3.1-3.3, in the
+// Hadamard-rotated basis: coded tokens are stored rotated (r_t c_j (s code + m)
+// with row scale r_t and per-block column scale c_j), the queries are rotated
+// once and the output is rotated back; sinks and staged tokens (stored in the
+// original basis) are rotated forward as their tiles are built.
+//
+// One CTA = 128 query rows of one (sequence, kv head): the g query heads of
+// the kv head x 128/g consecutive queries.  Keys and values stream in tiles of
+// 32 tokens.  Three roles:
+//   producers (warps 4-11): reconstruct each tile in fp32: K as a bf16 high
+//     part (the value truncated) plus the bf16 of the remainder, V rounded to
+//     fp16 and transposed (D rows, tokens along K), into three shared buffers.
+//     Warp w builds channels 32 w .. 32 w + 31, a lane one token; the packed
+//     words and scales of the next tile are loaded into registers before the
+//     current one is built, the tile's column scales go through a small
+//     shared array per warp;
+//   issuer (warp 12, one thread issues): S = Q_hi K_hi^T + Q_hi K_lo^T +
+//     Q_lo K_hi^T (a rotated query needs more than bf16's 8 bits too) into
+//     four TMEM tiles of 128 x 32 fp32, and O += P V into 128 x 256 fp32;
+//     S runs up to two tiles ahead of P V;
+//   softmax (warps 0-3): thread r owns row r (TMEM lane r): 32 scores, causal
+//     mask, running maximum and sum in log2 units, P as fp16 over its S tile; O
+//     is rescaled only when a row's maximum grows by more than 8.
+//
+// Space decides the layout: at D = 256 a 128-row query tile is 64 KB and has two
+// parts.  Q_hi stays in shared memory (the MMAs read it once per K step for
+// both K parts), Q_lo in 128 TMEM columns next to O's 256 and S's 4 x 32; that
+// leaves shared memory for three 48 KB K/V tiles of 32 tokens.
+// What bounds it: shared memory.  Per tile the MMAs read 64 KB of Q_hi, 48 KB of
+// K and 16 KB of V and the producers write 48 KB: about 1,400 cycles at 128
+// B/cycle, against 1,000 cycles of tensor pipe.
+// 8192 tokens, 16 query heads, 8 kv heads, one sequence: 7667 us on mma.sync (64
+// rows a CTA, 16-token tiles reconstructed by all its warps), 1526 us here (360
+// TFLOP/s of attention; the three Q K^T products make it 720 on the tensor cores).
+// Every wait is bounded and also gives up when another role has timed out;
+// the issuer drains its MMAs before TMEM is freed, and a timed-out CTA stores
+// nothing and sets the library's error word.
+#include <math.h>
+
+#include "tc_common.cuh"
+
+namespace kvq {
+namespace {
+using namespace tc;
+
+constexpr int kD = 256;
+constexpr int kM = 128;              // query rows per CTA (MMA M)
+constexpr int kTok = 32;             // tokens per KV tile
+constexpr int kG = 64;               // block length and group size
+constexpr int kProdWarps = 8;
+constexpr int kThreads = (4 + kProdWarps + 1) * 32;
+constexpr int kKvBufs = 3;
+constexpr int kSBufs = 4;
+constexpr float kRescale = 8.f;      // log2 growth of a row maximum that forces a rescale
+
+// Shared memory (bytes from a 1024-aligned base).
+constexpr int kQOff = 0;                               // Q_hi: 4 atoms of 128 rows x 128 B
+constexpr int kKvOff = kM * kD * 2;
+constexpr int kKH = 0;                                 // K hi: 4 atoms of 32 rows x 128 B
+constexpr int kKL = kTok * kD * 2;                     // K lo: the same
+constexpr int kVT = 2 * kTok * kD * 2;                 // V^T: 256 rows x 64 B, 64-byte swizzle
+constexpr int kKvB = 3 * kTok * kD * 2;
+constexpr int kColOff = kKvOff + kKvBufs * kKvB;       // per producer warp: 32 K, 32 V column scales
+constexpr int kTotal = kColOff + kProdWarps * 64 * 4;
+constexpr int kAlloc = kTotal + 1024;                  // alignment slack
+constexpr int kQlPitch = kD * 2 + 16;                  // Q_lo rows staged in the K/V area
+static_assert(kM * kQlPitch <= kKvBufs * kKvB, "Q_lo rows fit the K/V area");
+constexpr int kOPitch = kD + 1;                        // fp32 output rows over Q and K/V
+static_assert(kM * kOPitch * 4 <= kTotal, "output rows fit");
+static_assert(kAlloc <= 227 * 1024, "one CTA's shared memory");
+
+// TMEM columns: O, Q_lo (two bf16 per column), S tiles (P over them).
+constexpr int kTmO = 0, kTmQ = 256, kTmS = 384;
+
+// Descriptor of a K-major operand with 64-byte rows in the 64-byte swizzle
+// (8-row groups 512 bytes apart), and the byte offset of 16-byte chunk c of
+// row r in it.
+__device__ __forceinline__ uint64_t sw64_desc(const void* p) {
+  const uint64_t addr = smem_u32(p);
+  uint64_t d = 0;
+  d |= (addr >> 4) & 0x3FFFull;               // start address
+  d |= (uint64_t)1 << 16;                     // leading byte offset (unused)
+  d |= (uint64_t)(512 >> 4) << 32;            // stride byte offset: 8 rows x 64 B
+  d |= (uint64_t)1 << 46;                     // descriptor version (sm_100 family)
+  d |= (uint64_t)4 << 61;                     // layout: 64-byte swizzle
+  return d;
+}
+__device__ __forceinline__ int sw64(int r, int c) {
+  return r * 64 + ((c ^ ((r >> 1) & 3)) << 4);
+}
+
+// In-warp normalised Hadamard transform of a row held as x[i] = row[lane + 32 i].
+__device__ __forceinline__ void fwht256(float (&x)[8], int lane) {
+#pragma unroll
+  for (int h = 1; h < 32; h <<= 1)
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const float y = __shfl_xor_sync(0xffffffffu, x[i], h);
+      x[i] = (lane & h) ? y - x[i] : x[i] + y;
+    }
+#pragma unroll
+  for (int hs = 1; hs < 8; hs <<= 1)
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+      if (!(i & hs)) {
+        const float a = x[i], c = x[i + hs];
+        x[i] = a + c;
+        x[i + hs] = a - c;
+      }
+#pragma unroll
+  for (int i = 0; i < 8; ++i) x[i] *= 0.0625f;           // 1 / sqrt(256)
+}
+
+__device__ __forceinline__ uint64_t fmul2(uint64_t a, uint64_t b) {
+  uint64_t d;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+
+// Barrier of the producer warps (named barrier 1) that also returns whether
+// `ok` held in every producer thread, so all of them leave the loop together.
+__device__ __forceinline__ bool producers_all(bool ok) {
+  uint32_t r;
+  asm volatile(
+      "{\n .reg .pred p, q;\n setp.ne.u32 p, %1, 0;\n"
+      " bar.red.and.pred q, 1, 256, p;\n selp.u32 %0, 1, 0, q;\n}\n"
+      : "=r"(r) : "r"((uint32_t)ok) : "memory");
+  return r != 0;
+}
+
+// One thread's packed part of a coded tile: its token's codes of 32 channels
+// and scales, and two of the warp's column scales.
+template <int KB, int VB>
+struct Packed {
+  uint32_t kc[KB], vc[VB];           // 32 codes of KB (VB) bits
+  __half ks, kz, kr, vs, vz, vr;
+  __half2 col;
+};
+
+template <int N>
+__device__ __forceinline__ void load_words(uint32_t (&w)[N], const uint8_t* p) {
+  if constexpr (N == 4) {
+    const uint4 u = *reinterpret_cast<const uint4*>(p);
+    w[0] = u.x; w[1] = u.y; w[2] = u.z; w[3] = u.w;
+  } else {
+    const uint2 u = *reinterpret_cast<const uint2*>(p);
+    w[0] = u.x; w[1] = u.y;
+  }
+}
+
+// Where a head's coded rows start, at this thread's token of tile 0.
+struct Rows {
+  const uint8_t *kc, *vc;
+  const __half *ks, *kz, *kr, *kcol, *vs, *vz, *vr, *vcol;
+};
+
+// Tile at coded row q0 (a multiple of 32): pw the producer warp.
+template <int KB, int VB>
+__device__ __forceinline__ void load_packed(const Rows& r, int q0, int pw, int lane,
+                                            Packed<KB, VB>& p) {
+  const int64_t q = q0 + lane;
+  load_words<KB>(p.kc, r.kc + q * (kD * KB / 8) + pw * (32 * KB / 8));
+  load_words<VB>(p.vc, r.vc + q * (kD * VB / 8) + pw * (32 * VB / 8));
+  const int64_t m = q * (kD / kG) + pw / 2;
+  p.ks = r.ks[m];
+  p.kz = r.kz[m];
+  p.vs = r.vs[m];
+  p.vz = r.vz[m];
+  p.kr = r.kr[q];
+  p.vr = r.vr[q];
+  const int64_t c = (int64_t)(q0 / kG) * kD + pw * 32 + 2 * (lane & 15);
+  p.col = *reinterpret_cast<const __half2*>((lane < 16 ? r.kcol : r.vcol) + c);
+}
+
+// A coded tile into kv.  col: this warp's 64 floats of shared memory.
+template <int KB, int VB>
+__device__ __forceinline__ void build_coded(const Packed<KB, VB>& p, int pw, int lane, float* col,
+                                            unsigned char* kv) {
+  __syncwarp();                                  // the previous tile's scales are read
+  *reinterpret_cast<float2*>(col + 2 * lane) = __half22float2(p.col);   // K: 0..31, V: 32..63
+  __syncwarp();
+  const uint64_t bias2 = f2pack(-8388608.f, -8388608.f);
+  const float kr = __half2float(p.kr), vr = __half2float(p.vr);
+  const float ks = __half2float(p.ks) * kr, kz = __half2float(p.kz) * kr;
+  const float vs = __half2float(p.vs) * vr, vz = __half2float(p.vz) * vr;
+  const uint64_t ks2 = f2pack(ks, ks), kz2 = f2pack(kz, kz);
+  const uint64_t vs2 = f2pack(vs, vs), vz2 = f2pack(vz, vz);
+  // K: 4 chunks of 8 channels of token `lane`
+  unsigned char* kbase = kv + (pw >> 1) * (kTok * 128);
+#pragma unroll
+  for (int c = 0; c < 4; ++c) {
+    const uint32_t w = p.kc[c * KB / 4] >> (c * 8 * KB % 32);
+    const float4 c0 = *reinterpret_cast<const float4*>(col + 8 * c);
+    const float4 c1 = *reinterpret_cast<const float4*>(col + 8 * c + 4);
+    const uint64_t cc[4] = {f2pack(c0.x, c0.y), f2pack(c0.z, c0.w), f2pack(c1.x, c1.y),
+                            f2pack(c1.z, c1.w)};
+    uint32_t h[4], l[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const uint64_t code = fadd2(f2pack(code_biased<KB>(w, 2 * i), code_biased<KB>(w, 2 * i + 1)), bias2);
+      const uint64_t k2 = fmul2(ffma2(code, ks2, kz2), cc[i]);
+      float a, b;
+      f2unpack(k2, a, b);
+      const uint32_t ab = __float_as_uint(a) & 0xFFFF0000u, bb = __float_as_uint(b) & 0xFFFF0000u;
+      h[i] = __byte_perm(ab, bb, 0x7632);
+      float ra, rb;
+      f2unpack(fadd2(k2, f2pack(-__uint_as_float(ab), -__uint_as_float(bb))), ra, rb);
+      l[i] = pack_bf16(ra, rb);
+    }
+    const int off = sw128(lane, (pw & 1) * 4 + c);
+    *reinterpret_cast<uint4*>(kbase + kKH + off) = make_uint4(h[0], h[1], h[2], h[3]);
+    *reinterpret_cast<uint4*>(kbase + kKL + off) = make_uint4(l[0], l[1], l[2], l[3]);
+  }
+  // V^T: rows 32 pw + e, column `lane`
+  unsigned char* vbase = kv + kVT + pw * 32 * 64 + (lane & 7) * 2;
+#pragma unroll
+  for (int c = 0; c < 8; ++c) {
+    const uint32_t w = p.vc[c * VB / 8] >> (c * 4 * VB % 32);
+    const float4 c0 = *reinterpret_cast<const float4*>(col + 32 + 4 * c);
+    const uint64_t cc[2] = {f2pack(c0.x, c0.y), f2pack(c0.z, c0.w)};
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      const uint64_t code = fadd2(f2pack(code_biased<VB>(w, 2 * i), code_biased<VB>(w, 2 * i + 1)), bias2);
+      float a, b;
+      f2unpack(fmul2(ffma2(code, vs2, vz2), cc[i]), a, b);
+      const uint32_t v2 = pack_h2(a, b);
+      const int e = 4 * c + 2 * i;               // rows e, e + 1 share a swizzle phase
+      unsigned char* d = vbase + e * 64 + (((lane >> 3) ^ ((e >> 1) & 3)) << 4);
+      *reinterpret_cast<uint16_t*>(d) = (uint16_t)v2;
+      *reinterpret_cast<uint16_t*>(d + 64) = (uint16_t)(v2 >> 16);
+    }
+  }
+}
+
+// A tile with full-precision tokens (sinks, staged, or beyond T: zeros): a warp
+// per token, rotated forward in registers.  S and the coded tokens are
+// multiples of 32, so the tile holds no coded token.
+__device__ __noinline__ void build_full(const Geom& g, int b, int h, int t0, int T, int pw,
+                                        int lane, unsigned char* kv) {
+  for (int r = pw; r < kTok; r += kProdWarps) {
+    const int t = t0 + r;
+#pragma unroll
+    for (int which = 0; which < 2; ++which) {
+      float x[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) x[i] = 0.f;
+      if (t < T) {
+        const __nv_bfloat16* src =
+            t < g.S ? plane_ptr<__nv_bfloat16>(g, which ? KVQ_PLANE_V_FULL : KVQ_PLANE_K_FULL, b, h, t, 0)
+                    : plane_ptr<__nv_bfloat16>(g, which ? KVQ_PLANE_V_PEND : KVQ_PLANE_K_PEND, b, h,
+                                               (t - g.S) % kG, 0);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) x[i] = __bfloat162float(src[lane + 32 * i]);
+        fwht256(x, lane);
+      }
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const int j = lane + 32 * i;
+        if (which) {
+          *reinterpret_cast<__half*>(kv + kVT + sw64(j, r >> 3) + (r & 7) * 2) = __float2half_rn(x[i]);
+        } else {
+          unsigned char* d = kv + (j >> 6) * (kTok * 128) + sw128(r, (j & 63) >> 3) + (j & 7) * 2;
+          const float hi = __uint_as_float(__float_as_uint(x[i]) & 0xFFFF0000u);
+          *reinterpret_cast<__nv_bfloat16*>(d + kKH) = __float2bfloat16_rn(hi);
+          *reinterpret_cast<__nv_bfloat16*>(d + kKL) = __float2bfloat16_rn(x[i] - hi);
+        }
+      }
+    }
+  }
+}
+
+template <int KB, int VB>
+__global__ void __launch_bounds__(kThreads, 1)
+attend_prefill_kvarn_kernel(Geom g, const __nv_bfloat16* __restrict__ q, int L, float scale,
+                            __nv_bfloat16* __restrict__ out, int nq, int* err) {
+  pdl_wait();
+  pdl_trigger();
+  extern __shared__ unsigned char smem_raw[];
+  unsigned char* smem = reinterpret_cast<unsigned char*>(
+      (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  __shared__ uint64_t kv_full[kKvBufs], kv_free[kKvBufs], s_full[kSBufs], p_full[kSBufs],
+      s_free[kSBufs], done_bar;
+  __shared__ uint32_t tmem_base;
+  __shared__ int abort_flag;
+
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int qtile = gridDim.x - 1 - blockIdx.x;        // longest first
+  const int hkv = blockIdx.y, b = blockIdx.z;
+  const int grp = g.Hq / g.H;
+  const int T = cache_tokens(g);
+  const int q0 = qtile * nq;
+  const int nql = min(nq, L - q0);
+  const int pos_first = T - L + q0;
+  const int t_end = pos_first + nql;                   // keys [0, t_end)
+  const int ntiles = (t_end + kTok - 1) / kTok;
+  volatile int* abort = &abort_flag;
+
+  if (threadIdx.x == 0) {
+    for (int i = 0; i < kKvBufs; ++i) {
+      mbar_init(&kv_full[i], kProdWarps * 32);
+      mbar_init(&kv_free[i], 1);
+    }
+    for (int i = 0; i < kSBufs; ++i) {
+      mbar_init(&s_full[i], 1);
+      mbar_init(&p_full[i], kM);
+      mbar_init(&s_free[i], 1);
+    }
+    mbar_init(&done_bar, 1);
+    abort_flag = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 12) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;"
+                 ::"r"(smem_u32(&tmem_base)));
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+  }
+  // rotate the query rows: the high part into the swizzled Q tile, the bf16
+  // remainder into a staging row (then TMEM)
+  for (int r = warp; r < kM; r += kThreads / 32) {
+    const int hl = r / nq, qi = r % nq;
+    float x[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) x[i] = 0.f;
+    if (hl < grp && qi < nql) {
+      const __nv_bfloat16* src = q + (((int64_t)b * g.Hq + hkv * grp + hl) * L + q0 + qi) * kD;
+#pragma unroll
+      for (int i = 0; i < 8; ++i) x[i] = __bfloat162float(src[lane + 32 * i]);
+      fwht256(x, lane);
+    }
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int j = lane + 32 * i;
+      const __nv_bfloat16 hb = __float2bfloat16_rn(x[i]);
+      *reinterpret_cast<__nv_bfloat16*>(smem + kQOff + (j >> 6) * (kM * 128) +
+                                        sw128(r, (j & 63) >> 3) + (j & 7) * 2) = hb;
+      *reinterpret_cast<__nv_bfloat16*>(smem + kKvOff + r * kQlPitch + j * 2) =
+          __float2bfloat16_rn(x[i] - __bfloat162float(hb));
+    }
+  }
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = tmem_base;
+  const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
+  if (warp < 4) {
+    const unsigned char* src = smem + kKvOff + threadIdx.x * kQlPitch;
+#pragma unroll 2
+    for (int c = 0; c < 128; c += 16) {
+      uint32_t v[16];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const uint4 u = *reinterpret_cast<const uint4*>(src + 4 * c + 16 * i);
+        v[4 * i] = u.x; v[4 * i + 1] = u.y; v[4 * i + 2] = u.z; v[4 * i + 3] = u.w;
+      }
+      tmem_st16(tmem + lane_base + kTmQ + c, v);
+    }
+    tmem_wait_st();
+  }
+  tc_fence_before();
+  __syncthreads();                                     // Q_lo in TMEM, the K/V area is free
+  tc_fence_after();
+
+  float inv_l = 0.f;
+  if (warp >= 4 && warp < 12) {
+    // ---------------- producers: reconstruct K and V tiles ----------------
+    const int pw = warp - 4;
+    const int nbq = kvarn_nblocks(T, g.S, kG) * kG;
+    float* col = reinterpret_cast<float*>(smem + kColOff) + pw * 64;
+    Rows rows = {};
+    if (nbq > 0) {
+      rows.kc = plane_ptr<uint8_t>(g, KVQ_PLANE_K_CODES, b, hkv, 0);
+      rows.vc = plane_ptr<uint8_t>(g, KVQ_PLANE_V_CODES, b, hkv, 0);
+      rows.ks = plane_ptr<__half>(g, KVQ_PLANE_K_SCALE, b, hkv, 0);
+      rows.kz = plane_ptr<__half>(g, KVQ_PLANE_K_ZERO, b, hkv, 0);
+      rows.vs = plane_ptr<__half>(g, KVQ_PLANE_V_SCALE, b, hkv, 0);
+      rows.vz = plane_ptr<__half>(g, KVQ_PLANE_V_ZERO, b, hkv, 0);
+      rows.kr = plane_ptr<__half>(g, KVQ_PLANE_K_ROW, b, hkv, 0);
+      rows.vr = plane_ptr<__half>(g, KVQ_PLANE_V_ROW, b, hkv, 0);
+      rows.kcol = plane_ptr<__half>(g, KVQ_PLANE_K_COL, b, hkv, 0);
+      rows.vcol = plane_ptr<__half>(g, KVQ_PLANE_V_COL, b, hkv, 0);
+    }
+    auto coded = [&](int t0) { return t0 >= g.S && t0 < g.S + nbq; };
+    Packed<KB, VB> cur = {}, nxt = {};
+    if (coded(0)) load_packed<KB, VB>(rows, 0 - g.S, pw, lane, nxt);
+    for (int j = 0; j < ntiles; ++j) {
+      const int t0 = j * kTok, kb = j % kKvBufs;
+      cur = nxt;
+      if (j + 1 < ntiles && coded(t0 + kTok)) load_packed<KB, VB>(rows, t0 + kTok - g.S, pw, lane, nxt);
+      const bool ok = j < kKvBufs || mbar_wait_or_abort(&kv_free[kb], ((j - kKvBufs) / kKvBufs) & 1, abort);
+      if (!producers_all(ok)) break;
+      unsigned char* kv = smem + kKvOff + kb * kKvB;
+      if (coded(t0)) build_coded<KB, VB>(cur, pw, lane, col, kv);
+      else build_full(g, b, hkv, t0, T, pw, lane, kv);
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      mbar_arrive(&kv_full[kb]);
+    }
+  } else if (warp == 12) {
+    // ---------------- MMA issuer ----------------
+    // S of the next tile as soon as its K/V tile is built and its S buffer is
+    // free, P V of the next tile as soon as its P is written; the tensor pipe
+    // executes in issue order.  The whole warp runs the loop and one elected
+    // lane issues.  A K step of 16 elements advances a descriptor by 32 bytes.
+    constexpr uint32_t id_qk = idesc_bf16(kM, kTok);
+    constexpr uint32_t id_pv = idesc_f16(kM, kD);
+    const uint64_t qdesc0 = sw128_desc(smem + kQOff);
+    const uint64_t kdesc0 = sw128_desc(smem + kKvOff);
+    const uint64_t vdesc0 = sw64_desc(smem + kKvOff + kVT);
+    const bool leader = elect_one();
+    int nqk = 0, npv = 0;
+    long idle = 0;
+    uint64_t idle_since = 0;
+    while (npv < ntiles) {
+      bool progressed = false;
+      if (nqk < ntiles) {
+        const int kb = nqk % kKvBufs, sb = nqk % kSBufs;
+        bool ready = false;
+        if (lane == 0)
+          ready = mbar_test(&kv_full[kb], (nqk / kKvBufs) & 1) &&
+                  (nqk < kSBufs || mbar_test(&s_free[sb], ((nqk - kSBufs) / kSBufs) & 1));
+        if (__shfl_sync(0xffffffffu, ready, 0)) {
+          tc_fence_after();
+          if (leader) {
+            const uint32_t ts = tmem + kTmS + sb * kTok;
+#pragma unroll
+            for (int kk = 0; kk < kD / 16; ++kk) {
+              // Q atom: 128 rows x 128 B (1024 units); K atom: 32 rows x 128 B (256 units)
+              const uint64_t qd = qdesc0 + (uint64_t)((kk >> 2) * 1024 + (kk & 3) * 2);
+              const uint64_t kd = kdesc0 + (uint64_t)(kb * (kKvB >> 4) + (kk >> 2) * 256 + (kk & 3) * 2);
+              umma_a_fill(ts, qd, kd + (kKH >> 4), id_qk, kk > 0);     // Q_hi read once
+              umma_a_lastuse(ts, qd, kd + (kKL >> 4), id_qk, 1);       // for K hi and lo
+              umma_ts(ts, tmem + kTmQ + kk * 8, kd + (kKH >> 4), id_qk, 1);
+            }
+            umma_commit(&s_full[sb]);
+          }
+          __syncwarp();
+          ++nqk;
+          progressed = true;
+        }
+      }
+      if (npv < nqk) {
+        const int sb = npv % kSBufs, kb = npv % kKvBufs;
+        bool ready = false;
+        if (lane == 0) ready = mbar_test(&p_full[sb], (npv / kSBufs) & 1);
+        if (__shfl_sync(0xffffffffu, ready, 0)) {
+          tc_fence_after();
+          if (leader) {
+            const uint32_t tp = tmem + kTmS + sb * kTok;               // P (fp16 pairs) over S
+#pragma unroll
+            for (int kk = 0; kk < kTok / 16; ++kk)
+              umma_ts(tmem + kTmO, tp + kk * 8, vdesc0 + (uint64_t)(kb * (kKvB >> 4) + kk * 2), id_pv,
+                      (npv > 0 || kk > 0) ? 1u : 0u);
+            umma_commit(&s_free[sb]);            // S/P buffer free, and O holds tile npv
+            umma_commit(&kv_free[kb]);
+          }
+          __syncwarp();
+          ++npv;
+          progressed = true;
+        }
+      }
+      if (progressed) {
+        idle = 0;
+      } else {
+        if (idle == 0) idle_since = global_ns();
+        __nanosleep(20);
+        const bool stop = (++idle & 63) == 0 && (*abort || global_ns() - idle_since > kWaitNs);
+        if (__shfl_sync(0xffffffffu, stop, 0)) break;   // the whole warp leaves together
+      }
+    }
+    if (lane == 0 && npv < ntiles) *abort = 1;
+    if (leader) umma_commit(&done_bar);        // every MMA issued above has completed
+    if (lane == 0 && !mbar_wait(&done_bar, 0)) *abort = 1;
+    __syncwarp();
+  } else {
+    // ---------------- softmax: one row per thread ----------------
+    const int row = threadIdx.x;
+    const int hl = row / nq, qi = row % nq;
+    const int pos = hl < grp && qi < nql ? pos_first + qi : -1;
+    const uint32_t s_col = tmem + lane_base + kTmS, o_col = tmem + lane_base + kTmO;
+    const float c2 = scale * 1.4426950408889634f;   // scores in log2 units
+    const uint64_t c22 = f2pack(c2, c2);
+    float m = -INFINITY, l = 0.f;
+    bool ok = true;
+    for (int j = 0; j < ntiles; ++j) {
+      const int sb = j % kSBufs, t0 = j * kTok;
+      if (!warp_wait(&s_full[sb], (j / kSBufs) & 1, abort)) {
+        ok = false;
+        break;
+      }
+      tc_fence_after();
+      uint32_t sr[kTok];
+      tmem_ld16_nowait(s_col + sb * kTok, sr);
+      tmem_ld16_nowait(s_col + sb * kTok + 16, sr + 16);
+      tmem_wait_ld();
+      if (t0 + kTok - 1 > pos) {               // some key of the tile is in the row's future
+#pragma unroll
+        for (int i = 0; i < kTok; ++i)
+          if (t0 + i > pos) sr[i] = __float_as_uint(-INFINITY);
+      }
+      float mx4[4];
+#pragma unroll
+      for (int a = 0; a < 4; ++a) {
+        const uint32_t* v = sr + 8 * a;
+        float mv = fmax3(__uint_as_float(v[0]), __uint_as_float(v[1]), __uint_as_float(v[2]));
+        mv = fmax3(mv, __uint_as_float(v[3]), __uint_as_float(v[4]));
+        mv = fmax3(mv, __uint_as_float(v[5]), __uint_as_float(v[6]));
+        mx4[a] = fmaxf(mv, __uint_as_float(v[7]));
+      }
+      const float mx = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3]));
+      const float m_new = fmaxf(m, mx * c2);   // (c2 > 0: the maximum commutes)
+      if (j == 0) {
+        m = m_new;
+      } else if (__any_sync(0xffffffffu, m_new > m + kRescale)) {
+        // O is rewritten: the P V of tile j - 1 must have completed
+        if (!warp_wait(&s_free[(j - 1) % kSBufs], ((j - 1) / kSBufs) & 1, abort)) {
+          ok = false;
+          break;
+        }
+        tc_fence_after();
+        const float alpha = m_new > m ? ex2_approx(m - m_new) : 1.f;
+        if (m_new > m) {
+          l *= alpha;
+          m = m_new;
+        }
+#pragma unroll 1
+        for (int c = 0; c < kD; c += 16) {
+          uint32_t o[16];
+          tmem_ld16_nowait(o_col + c, o);
+          tmem_wait_ld();
+#pragma unroll
+          for (int i = 0; i < 16; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * alpha);
+          tmem_st16(o_col + c, o);
+        }
+      }
+      // P = 2^(s c2 - m) as fp16 pairs over the first 16 columns of this S
+      // buffer (a row without any visible key so far has m = -inf and P = 0)
+      const bool live = m != -INFINITY;
+      const uint64_t negm = f2pack(-m, -m);
+      uint64_t sum2 = f2pack(0.f, 0.f);
+      uint32_t pk[kTok / 2];
+#pragma unroll
+      for (int i = 0; i < kTok; i += 2) {
+        float a0, a1;
+        f2unpack(ffma2(f2pack(__uint_as_float(sr[i]), __uint_as_float(sr[i + 1])), c22, negm), a0, a1);
+        float p0 = ex2_approx(a0), p1 = ex2_approx(a1);
+        if (!live) p0 = p1 = 0.f;
+        sum2 = fadd2(sum2, f2pack(p0, p1));
+        pk[i / 2] = pack_h2(p0, p1);
+      }
+      tmem_st16(s_col + sb * kTok, pk);
+      float s0, s1;
+      f2unpack(sum2, s0, s1);
+      l += s0 + s1;
+      tmem_wait_st();
+      tc_fence_before();
+      mbar_arrive(&p_full[sb]);
+    }
+    if (ok && ntiles > 0 &&
+        !warp_wait(&s_free[(ntiles - 1) % kSBufs], ((ntiles - 1) / kSBufs) & 1, abort))
+      ok = false;
+    tc_fence_after();
+    inv_l = ok && l > 0.f ? 1.f / l : 0.f;
+  }
+  // ---------------- epilogue: normalise, rotate back, store ----------------
+  tc_fence_before();
+  __syncthreads();                                     // every MMA has completed
+  tc_fence_after();
+  const bool good = !*abort;
+  float* os = reinterpret_cast<float*>(smem);
+  if (warp < 4 && good) {
+    float* orow = os + threadIdx.x * kOPitch;
+#pragma unroll 1
+    for (int c = 0; c < kD; c += 16) {
+      uint32_t o[16];
+      tmem_ld16_nowait(tmem + lane_base + kTmO + c, o);
+      tmem_wait_ld();
+#pragma unroll
+      for (int i = 0; i < 16; ++i) orow[c + i] = __uint_as_float(o[i]) * inv_l;
+    }
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (good) {
+    for (int r = warp; r < kM; r += kThreads / 32) {
+      const int hl = r / nq, qi = r % nq;
+      if (hl >= grp || qi >= nql) continue;
+      float x[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) x[i] = os[r * kOPitch + lane + 32 * i];
+      fwht256(x, lane);
+      __nv_bfloat16* dst = out + (((int64_t)b * g.Hq + hkv * grp + hl) * L + q0 + qi) * kD;
+#pragma unroll
+      for (int i = 0; i < 8; ++i) dst[lane + 32 * i] = __float2bfloat16_rn(x[i]);
+    }
+  }
+  if (threadIdx.x == 0 && !good) atomicOr(err, 8);
+  if (warp == 12) {
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem));
+  }
+}
+
+template <int KB, int VB>
+cudaError_t launch(const Geom& g, const void* q, int L, float scale, void* out, int* err,
+                   cudaStream_t s) {
+  auto kern = attend_prefill_kvarn_kernel<KB, VB>;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kAlloc);
+  if (e != cudaSuccess) return e;
+  const int nq = kM / (g.Hq / g.H);
+  launch_pdl(kern, dim3((L + nq - 1) / nq, g.H, g.B), dim3(kThreads), (size_t)kAlloc, s, g,
+             reinterpret_cast<const __nv_bfloat16*>(q), L, scale,
+             reinterpret_cast<__nv_bfloat16*>(out), nq, err);
+  return cudaGetLastError();
+}
+
+}  // namespace
+
+// bf16 KVarN caches at head_dim 256 with 64-token blocks, 2- or 4-bit codes and a
+// number of sinks that ends on a 32-token tile (a tile is then either all
+// coded, inside one column-scale block, or all full precision).
+bool prefill_kvarn_supported(const Geom& g) {
+  return g.fmt == KVQ_FMT_KVARN && g.layout == KVQ_LAYOUT_UNIFORM && g.act == KVQ_BF16 &&
+         g.D == kD && g.G == kG && g.S % kTok == 0 && (g.kb == 2 || g.kb == 4) &&
+         (g.vb == 2 || g.vb == 4);
+}
+
+cudaError_t launch_prefill_kvarn(const Geom& g, const void* q, int L, float scale, void* out,
+                                 int* err, cudaStream_t s) {
+  if (g.kb == 4)
+    return g.vb == 4 ? launch<4, 4>(g, q, L, scale, out, err, s)
+                     : launch<4, 2>(g, q, L, scale, out, err, s);
+  return g.vb == 4 ? launch<2, 4>(g, q, L, scale, out, err, s)
+                   : launch<2, 2>(g, q, L, scale, out, err, s);
+}
+
+}  // namespace kvq

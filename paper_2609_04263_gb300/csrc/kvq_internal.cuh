@@ -219,6 +219,10 @@ bool decode_mma_supported(const Geom& g);
 bool prefill_m256_supported(const Geom& g);
 cudaError_t launch_prefill_m256(const Geom& g, const void* q, int L, float scale, void* out,
                                 int* err, cudaStream_t s);
+// tcgen05 causal prefill of KVarN caches at D = 256 (attend_prefill_kvarn.cu).
+bool prefill_kvarn_supported(const Geom& g);
+cudaError_t launch_prefill_kvarn(const Geom& g, const void* q, int L, float scale, void* out,
+                                 int* err, cudaStream_t s);
 // mma.sync causal prefill for the other formats and head dimensions
 // (attend_prefill_mma.cu).
 bool prefill_mma_supported(const Geom& g);
