@@ -644,7 +644,7 @@ __global__ void kvarn_block_kernel(Geom g, int L, TokSrc sk, TokSrc sv, float in
 // a value outside those bounds divides with __fdiv_rn.
 //
 // 4 sequences x 8 heads x 8000 tokens, D = 256, G = 64: 1990 us with the block
-// in shared memory, 792 us so.
+// in shared memory, 751 us so.
 __device__ __forceinline__ uint64_t pk2(float lo, float hi) {
   uint64_t r;
   asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
@@ -679,9 +679,16 @@ __device__ __forceinline__ uint64_t div2(uint64_t y, uint64_t ns, uint64_t v) {
   const uint64_t q = mul2(y, v);
   return fma2(fma2(q, ns, y), v, q);
 }
-__device__ __forceinline__ uint64_t div2_exact(uint64_t y, float s0, float s1) {
-  const float2 f = upk2(y);
-  return pk2(__fdiv_rn(f.x, s0), __fdiv_rn(f.y, s1));
+// The lane's elements (rows i, channels lane + 32 j of the warp's rows w in
+// shared memory) divided by IEEE division, row i by rs[i] or, if rs is NULL,
+// channel c by -cs[c].x.  Out of line and rolled: inlined at both places it
+// pushed the loop out of the instruction cache.
+template <int D, int NR>
+__device__ __noinline__ void divide_exact(float* w, int lane, const float* rs, const float2* cs) {
+#pragma unroll 1
+  for (int i = 0; i < NR; ++i)
+#pragma unroll 1
+    for (int c = lane; c < D; c += 32) w[i * D + c] = __fdiv_rn(w[i * D + c], rs ? rs[i] : -cs[c].x);
 }
 
 // Butterfly over the lanes in the order 16, 8, 4, 2, 1 of N = 4 .. 32 values
@@ -729,6 +736,7 @@ struct KvarnSmem {
   float rows[G * D];                 // Hadamard: channel order <-> lane order
   float part[8][D];                  // column sums of squares of each warp's rows
   float2 csig[D];                    // column divisors: -s, 1 / s
+  float rsig[8][8];                  // row divisors, when a warp divides exactly
   float4 grp[8][32];                 // coding: minimum, 1 / scale, scale
 };
 
@@ -853,18 +861,36 @@ kvarn_block_fast_kernel(Geom g, int L, TokSrc sk, TokSrc sv, float inv_sqrt_d, u
     const float inv = __frcp_rn(sg);
     rsc = __fmul_rn(rsc, sg);
     const bool fast = __all_sync(0xffffffffu, ymin >= kMinY && sg <= kMaxS);
+    auto exact = [&](const float* rs) {          // through this lane's part of the warp's rows
 #pragma unroll
-    for (int i = 0; i < NR; ++i) {
-      const float s = __shfl_sync(0xffffffffu, sg, i * (32 / NR));
-      const float v = __shfl_sync(0xffffffffu, inv, i * (32 / NR));
-      if (fast) {
+      for (int i = 0; i < NR; ++i)
+#pragma unroll
+        for (int p = 0; p < NP; ++p) {
+          const float2 f = upk2(y[i][p]);
+          wrows[i * D + lane + 64 * p] = f.x;
+          wrows[i * D + lane + 64 * p + 32] = f.y;
+        }
+      divide_exact<D, NR>(wrows, lane, rs, sm.csig);
+#pragma unroll
+      for (int i = 0; i < NR; ++i)
+#pragma unroll
+        for (int p = 0; p < NP; ++p)
+          y[i][p] = pk2(wrows[i * D + lane + 64 * p], wrows[i * D + lane + 64 * p + 32]);
+    };
+    if (fast) {
+#pragma unroll
+      for (int i = 0; i < NR; ++i) {
+        const float s = __shfl_sync(0xffffffffu, sg, i * (32 / NR));
+        const float v = __shfl_sync(0xffffffffu, inv, i * (32 / NR));
         const uint64_t ns2 = pk2(-s, -s), v2 = pk2(v, v);
 #pragma unroll
         for (int p = 0; p < NP; ++p) y[i][p] = div2(y[i][p], ns2, v2);
-      } else {
-#pragma unroll
-        for (int p = 0; p < NP; ++p) y[i][p] = div2_exact(y[i][p], s, s);
       }
+    } else {
+      if (lane % (32 / NR) == 0) sm.rsig[warp][lane / (32 / NR)] = sg;
+      __syncwarp();
+      exact(sm.rsig[warp]);
+      __syncwarp();
     }
     // ---- columns ----
 #pragma unroll
@@ -894,17 +920,22 @@ kvarn_block_fast_kernel(Geom g, int L, TokSrc sk, TokSrc sv, float inv_sqrt_d, u
       sm.csig[threadIdx.x] = make_float2(-cg, __frcp_rn(cg));
     }
     __syncthreads();
+    float2 cg[NS];
+    float cmax = 0.f;
 #pragma unroll
-    for (int p = 0; p < NP; ++p) {
-      const float2 c0 = sm.csig[lane + 64 * p], c1 = sm.csig[lane + 64 * p + 32];
-      if (__all_sync(0xffffffffu, fast && fmaxf(-c0.x, -c1.x) <= kMaxS)) {
-        const uint64_t ns2 = pk2(c0.x, c1.x), v2 = pk2(c0.y, c1.y);
+    for (int j = 0; j < NS; ++j) {
+      cg[j] = sm.csig[lane + 32 * j];
+      cmax = fmaxf(cmax, -cg[j].x);
+    }
+    if (__all_sync(0xffffffffu, fast && cmax <= kMaxS)) {
+#pragma unroll
+      for (int p = 0; p < NP; ++p) {
+        const uint64_t ns2 = pk2(cg[2 * p].x, cg[2 * p + 1].x), v2 = pk2(cg[2 * p].y, cg[2 * p + 1].y);
 #pragma unroll
         for (int i = 0; i < NR; ++i) y[i][p] = div2(y[i][p], ns2, v2);
-      } else {
-#pragma unroll
-        for (int i = 0; i < NR; ++i) y[i][p] = div2_exact(y[i][p], -c0.x, -c1.x);
       }
+    } else {
+      exact(nullptr);
     }
   }
 
