@@ -415,7 +415,7 @@ __device__ __forceinline__ uint32_t lane_codes(const uint8_t* row, int lane, int
 template <int D, int GM>
 __global__ void __launch_bounds__(256)
 attend_kvarn_decode_kernel(Geom g, const __nv_bfloat16* __restrict__ q, float scale,
-                           float inv_sqrt_d, int full_only, void* out) {
+                           float inv_sqrt_d, void* out) {
   pdl_wait();
   pdl_trigger();
   constexpr int NS = D / 32;
@@ -425,11 +425,8 @@ attend_kvarn_decode_kernel(Geom g, const __nv_bfloat16* __restrict__ q, float sc
   const int grp = g.Hq / g.H, G = g.G, S = g.S;
   const int T = cache_tokens(g);
   const int nbq = kvarn_nblocks(T, S, G) * G;
-  // full_only: the splits share the full-precision tokens alone (sinks, then
-  // staged), indexed f = 0 .. T - nbq - 1 and mapped to token f or f + nbq
   int ts, te;
-  if (full_only) split_range(T - nbq, g.splits, split, 1, &ts, &te);
-  else split_range(T, g.splits, split, G, &ts, &te);
+  split_range(T, g.splits, split, G, &ts, &te);
   const float c2 = scale * 1.4426950408889634f;   // scores in log2 units
   // rotated queries, pre-scaled
   float qr[GM][NS];
@@ -460,8 +457,7 @@ attend_kvarn_decode_kernel(Geom g, const __nv_bfloat16* __restrict__ q, float sc
   float qp[GM][NS], qs[GM];                         // q' = q_rot c_block and its lane sum
   float cv[NS];                                     // value column scales of the block
   int cur_blk = -1;
-  for (int f = w0; f < w1; ++f) {
-    const int t = full_only && f >= S ? f + nbq : f;
+  for (int t = w0; t < w1; ++t) {
     float kv[NS], vv[NS];
     const bool coded = t >= S && t - S < nbq;
     float dot[GM];
@@ -575,9 +571,7 @@ attend_kvarn_decode_kernel(Geom g, const __nv_bfloat16* __restrict__ q, float sc
 #pragma unroll
     for (int i = 0; i < NS; ++i) wsr[2 + NS * lane + i] = x[i];
   }
-  // ---- the last split CTA of this (sequence, kv head) merges the splits
-  // and, with full_only, the coded tokens' partial (slot kMaxSplits - 1,
-  // written by the streaming kernel that ran before this one) ----
+  // ---- the last split CTA of this (sequence, kv head) merges the splits ----
   __shared__ int last_cta;
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -587,10 +581,10 @@ attend_kvarn_decode_kernel(Geom g, const __nv_bfloat16* __restrict__ q, float sc
   __syncthreads();
   if (!last_cta) return;
   __threadfence();
-  const int n = g.splits + (full_only ? 1 : 0);
+  const int n = g.splits;
   for (int h = warp; h < grp; h += 8) {
     const float* w = ws_row(g, b, hkv * grp + h);
-    auto row = [&](int i) { return w + (int64_t)(i < g.splits ? i : kMaxSplits - 1) * (D + kWsStride); };
+    auto row = [&](int i) { return w + (int64_t)i * (D + kWsStride); };
     float M = -INFINITY;
     for (int i = lane; i < n; i += 32) M = fmaxf(M, __ldcg(row(i)));
 #pragma unroll
@@ -614,8 +608,7 @@ attend_kvarn_decode_kernel(Geom g, const __nv_bfloat16* __restrict__ q, float sc
 }
 
 template <int D>
-cudaError_t launch_kvarn_d(const Geom& g, const void* q, float scale, int full_only, void* out,
-                           cudaStream_t s) {
+cudaError_t launch_kvarn_d(const Geom& g, const void* q, float scale, void* out, cudaStream_t s) {
   const int grp = g.Hq / g.H;
   const float inv_sqrt_d = (float)(1.0 / sqrt((double)D));
   dim3 grid(g.splits, g.H, g.B);
@@ -624,7 +617,7 @@ cudaError_t launch_kvarn_d(const Geom& g, const void* q, float scale, int full_o
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
     launch_pdl(kern, dim3(grid), dim3(256), sm, s, g, reinterpret_cast<const __nv_bfloat16*>(q),
-               scale, inv_sqrt_d, full_only, out);
+               scale, inv_sqrt_d, out);
     return cudaGetLastError();
   };
   if (grp <= 2) return run(attend_kvarn_decode_kernel<D, 2>, 2);
@@ -645,7 +638,7 @@ int decode_splits(const Geom& g) {
   // every (sequence, kv head) runs in the first wave
   const int bh = g.B * g.H;
   int s = 2 * num_sms() / bh;
-  if (s > kMaxSplits - 1) s = kMaxSplits - 1;     // the last slot is reserved (KVarN)
+  if (s > kMaxSplits - 1) s = kMaxSplits - 1;
   return s < 1 ? 1 : s;
 }
 
@@ -678,21 +671,17 @@ cudaError_t launch_attend(const Geom& g, const void* q, int L, float scale, void
     return launch_decode_mma(g, q, scale, err, out, s);
   }
   if (decode && kvarn_decode_supported(g)) {
-    // long caches: the coded tokens on tensor cores (one partial per head in
-    // the reserved slot), the sinks and staged tokens in the split kernel
+    // long caches: the sinks and staged tokens leave partials, then the coded
+    // tokens go through the tensor cores and everything is merged
     const int64_t coded = (int64_t)g.B * g.H * (kvarn_nblocks(t_hint, g.S, g.G) * g.G / 32);
-    const bool streamed = decode_stream_kvarn_supported(g) &&
-                          coded >= 16 * (int64_t)decode_stream_ctas(g);
-    if (streamed) {
+    if (decode_stream_kvarn_supported(g) && coded >= 16 * (int64_t)decode_stream_ctas(g)) {
       int* err = device_error_word();
       if (!err) return cudaErrorInvalidDevice;
-      cudaError_t e = launch_decode_stream_kvarn(g, q, scale, err, s);
-      if (e != cudaSuccess) return e;
+      return launch_decode_stream_kvarn(g, q, scale, err, out, s);
     }
-    // the split kernel's last CTA per (sequence, kv head) merges everything
-    return g.D == 64 ? launch_kvarn_d<64>(g, q, scale, streamed, out, s)
-         : g.D == 128 ? launch_kvarn_d<128>(g, q, scale, streamed, out, s)
-                      : launch_kvarn_d<256>(g, q, scale, streamed, out, s);
+    return g.D == 64 ? launch_kvarn_d<64>(g, q, scale, out, s)
+         : g.D == 128 ? launch_kvarn_d<128>(g, q, scale, out, s)
+                      : launch_kvarn_d<256>(g, q, scale, out, s);
   }
   return g.D == 64 ? launch_generic_d<64>(g, q, L, scale, out, decode, s)
        : g.D == 128 ? launch_generic_d<128>(g, q, L, scale, out, decode, s)

@@ -19,10 +19,14 @@
 //   values  A = c_v,j * code (fp16), B = fp16(p) * (r_t s_tg); the offsets
 //     r_t m_tg enter through a small MMA (rows = groups) and are scaled by
 //     c_v,j when the block's contribution is added.
-// The sinks and the staged tokens (full precision, original basis) are left
-// to attend_kvarn_decode_kernel; this kernel leaves each head's result as one
-// more split partial (m, l, o rotated back) in workspace slot kFinalSlot,
-// which that kernel (launched next) merges with its own partials.
+// The sinks and the staged tokens (full precision, original basis: no rotation
+// is needed to attend them) go through kvarn_full_kernel, launched first: four
+// CTAs per head, a warp per token, partials in the top workspace slots.  The
+// streaming kernel starts while it runs (programmatic launch) and waits for it
+// only where it merges: the head's last CTA rotates the coded tokens' output back
+// and adds the four partials.  12B-class shape, batch 4, 8300 tokens: the split kernel
+// that used to take the full-precision tokens after the streaming kernel, rotating
+// each of them, added 17 us to its 52 (four layers: 274 -> 241 us).
 #include "decode_attn.cuh"
 #include "stream_common.cuh"
 
@@ -79,14 +83,175 @@ __device__ __forceinline__ void fwht_rows(float (&x)[D / 32], int lane, float in
   for (int i = 0; i < NS; ++i) x[i] *= inv_sqrt_d;
 }
 
+// Attention of every query head of one (sequence, kv head) over one of
+// kFullSplits shares of its full-precision tokens.  Lane l holds channels
+// NS l .. of the queries; a warp takes four tokens at a time, so that eight row
+// loads are in flight.  Partials (m in log2 units, l, o) go to workspace slots
+// kFullSlot ...
+constexpr int kFullWarps = 4;
+
+template <int D, int GM>
+__global__ void __launch_bounds__(kFullWarps * 32)
+kvarn_full_kernel(Geom g, const __nv_bfloat16* __restrict__ q, float scale) {
+  pdl_wait();
+  pdl_trigger();
+  constexpr int NS = D / 32, NB = 4;
+  __shared__ float red[kFullWarps][GM][D + 2];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int hkv = blockIdx.y, b = blockIdx.z, grp = g.Hq / g.H, S = g.S;
+  const int T = cache_tokens(g);
+  const int nbq = kvarn_nblocks(T, S, g.G) * g.G;
+  const int per = (T - nbq + kFullSplits - 1) / kFullSplits;
+  const int ts = blockIdx.x * per, te = min(T - nbq, ts + per);
+  const float c2 = scale * 1.4426950408889634f;   // scores in log2 units
+  struct __align__(NS * 2) Row { __nv_bfloat162 v[NS / 2]; };
+  float qf[GM][NS], o[GM][NS], m[GM], l[GM];
+#pragma unroll
+  for (int h = 0; h < GM; ++h) {
+    m[h] = -INFINITY;
+    l[h] = 0.f;
+    Row r = {};
+    if (h < grp)
+      r = *reinterpret_cast<const Row*>(q + ((int64_t)b * g.Hq + hkv * grp + h) * D + NS * lane);
+#pragma unroll
+    for (int i = 0; i < NS / 2; ++i) {
+      const float2 f = __bfloat1622float2(r.v[i]);
+      qf[h][2 * i] = f.x * c2;
+      qf[h][2 * i + 1] = f.y * c2;
+      o[h][2 * i] = o[h][2 * i + 1] = 0.f;
+    }
+  }
+  for (int f0 = ts + warp * NB; f0 < te; f0 += kFullWarps * NB) {
+    Row kr[NB], vr[NB];
+#pragma unroll
+    for (int u = 0; u < NB; ++u) {
+      const int f = min(f0 + u, te - 1);          // sinks, then staged tokens
+      const int slot = f < S ? f : (f + nbq - S) % g.G;
+      kr[u] = *reinterpret_cast<const Row*>(plane_ptr<__nv_bfloat16>(
+          g, f < S ? KVQ_PLANE_K_FULL : KVQ_PLANE_K_PEND, b, hkv, slot, NS * lane));
+      vr[u] = *reinterpret_cast<const Row*>(plane_ptr<__nv_bfloat16>(
+          g, f < S ? KVQ_PLANE_V_FULL : KVQ_PLANE_V_PEND, b, hkv, slot, NS * lane));
+    }
+    float sc[GM][NB];
+#pragma unroll
+    for (int u = 0; u < NB; ++u) {
+      float kf[NS];
+#pragma unroll
+      for (int i = 0; i < NS / 2; ++i) {
+        const float2 f = __bfloat1622float2(kr[u].v[i]);
+        kf[2 * i] = f.x;
+        kf[2 * i + 1] = f.y;
+      }
+#pragma unroll
+      for (int h = 0; h < GM; ++h) {
+        float d = 0.f;
+#pragma unroll
+        for (int i = 0; i < NS; ++i) d = fmaf(qf[h][i], kf[i], d);
+        sc[h][u] = d;
+      }
+    }
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1)
+#pragma unroll
+      for (int h = 0; h < GM; ++h)
+#pragma unroll
+        for (int u = 0; u < NB; ++u) sc[h][u] += __shfl_xor_sync(0xffffffffu, sc[h][u], off);
+#pragma unroll
+    for (int h = 0; h < GM; ++h) {
+      float mn = m[h];
+#pragma unroll
+      for (int u = 0; u < NB; ++u) {
+        if (f0 + u >= te) sc[h][u] = -INFINITY;
+        mn = fmaxf(mn, sc[h][u]);
+      }
+      const float alpha = exp2f(m[h] - mn);       // m = -inf at first: 0
+      m[h] = mn;
+      l[h] *= alpha;
+#pragma unroll
+      for (int i = 0; i < NS; ++i) o[h][i] *= alpha;
+#pragma unroll
+      for (int u = 0; u < NB; ++u) {
+        sc[h][u] = exp2f(sc[h][u] - mn);
+        l[h] += sc[h][u];
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < NB; ++u)
+#pragma unroll
+      for (int i = 0; i < NS / 2; ++i) {
+        const float2 f = __bfloat1622float2(vr[u].v[i]);
+#pragma unroll
+        for (int h = 0; h < GM; ++h) {
+          o[h][2 * i] = fmaf(sc[h][u], f.x, o[h][2 * i]);
+          o[h][2 * i + 1] = fmaf(sc[h][u], f.y, o[h][2 * i + 1]);
+        }
+      }
+  }
+#pragma unroll
+  for (int h = 0; h < GM; ++h) {
+    if (lane == 0) {
+      red[warp][h][0] = m[h];
+      red[warp][h][1] = l[h];
+    }
+#pragma unroll
+    for (int i = 0; i < NS; ++i) red[warp][h][2 + NS * lane + i] = o[h][i];
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < grp * (D + 2); i += kFullWarps * 32) {
+    const int h = i / (D + 2), c = i % (D + 2);
+    float M = -INFINITY;
+#pragma unroll
+    for (int w = 0; w < kFullWarps; ++w) M = fmaxf(M, red[w][h][0]);
+    float x = M;
+    if (c > 0) {
+      x = 0.f;
+#pragma unroll
+      for (int w = 0; w < kFullWarps; ++w)
+        if (red[w][h][0] != -INFINITY) x += exp2f(red[w][h][0] - M) * red[w][h][c];
+    }
+    reinterpret_cast<float*>(g.pl[KVQ_PLANE_WORKSPACE].p)[
+        (((int64_t)b * g.Hq + hkv * grp + h) * kMaxSplits + kFullSlot + blockIdx.x) * (D + kWsStride) + c] = x;
+  }
+}
+
+// One head's output: the coded tokens' rotated-back row x[i] = channel lane + 32 i
+// (m in log2 units and l; -inf and 0 if there are none) and the
+// full-precision tokens' partials wf (the head's workspace slot kFullSlot ...).
+template <int D>
+__device__ __forceinline__ void merge_full(const float* wf, float (&x)[D / 32], float m, float l,
+                                           int lane, __nv_bfloat16* out) {
+  constexpr int R = D + kWsStride;
+  float mf[kFullSplits], M = m;
+#pragma unroll
+  for (int s = 0; s < kFullSplits; ++s) {
+    mf[s] = __ldcg(wf + s * R);
+    M = fmaxf(M, mf[s]);
+  }
+  const float fx = m == -INFINITY ? 0.f : exp2f(m - M);
+  float L = fx * l;
+#pragma unroll
+  for (int i = 0; i < D / 32; ++i) x[i] = m == -INFINITY ? 0.f : x[i] * fx;
+#pragma unroll
+  for (int s = 0; s < kFullSplits; ++s) {
+    if (mf[s] == -INFINITY) continue;
+    const float f = exp2f(mf[s] - M);
+    L = fmaf(f, __ldcg(wf + s * R + 1), L);
+#pragma unroll
+    for (int i = 0; i < D / 32; ++i) x[i] = fmaf(f, __ldcg(wf + s * R + 2 + lane + 32 * i), x[i]);
+  }
+#pragma unroll
+  for (int i = 0; i < D / 32; ++i) out[lane + 32 * i] = __float2bfloat16_rn(x[i] / L);
+}
+
+// Launched after kvarn_full_kernel, whose start waited for everything before it:
+// only its partials have to be waited for (pdl_wait before the merges).
 template <int D, int KB, int VB, int G>
 __global__ void __launch_bounds__(kThreads, 1)
 decode_stream_kvarn_kernel(Geom g, const __nv_bfloat16* __restrict__ q, float scale,
-                           float inv_sqrt_d, int* err, int ns) {
+                           float inv_sqrt_d, int* err, __nv_bfloat16* __restrict__ out, int ns) {
   using C = KCfg<D, KB, VB, G>;
   constexpr int NG32 = C::NG32, NGG = C::NGG, MT = C::MT;
   extern __shared__ __align__(128) unsigned char smem[];
-  pdl_wait();
   pdl_trigger();
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -106,13 +271,13 @@ decode_stream_kvarn_kernel(Geom g, const __nv_bfloat16* __restrict__ q, float sc
   const int BH = g.B * g.H;
   const int nb = nbq / kBT;                          // blocks per head
   const int64_t N = (int64_t)BH * nb;
-  if (N == 0) {                                      // nothing coded: an empty partial
-    if (blockIdx.x == 0)
-      for (int i = threadIdx.x; i < g.B * g.Hq; i += blockDim.x) {
-        float* w = wsb + ((int64_t)i * kMaxSplits + kFinalSlot) * (D + kWsStride);
-        w[0] = -INFINITY;
-        w[1] = 0.f;
-      }
+  if (N == 0) {                                      // nothing coded
+    pdl_wait();
+    for (int i = blockIdx.x * (kThreads / 32) + warp; i < g.B * g.Hq; i += gridDim.x * (kThreads / 32)) {
+      float x[D / 32];
+      merge_full<D>(wsb + ((int64_t)i * kMaxSplits + kFullSlot) * (D + kWsStride), x, -INFINITY, 0.f,
+                    lane, out + (int64_t)i * D);
+    }
     return;
   }
   const int P = N < (int64_t)gridDim.x ? (int)N : (int)gridDim.x;
@@ -435,22 +600,19 @@ decode_stream_kvarn_kernel(Geom g, const __nv_bfloat16* __restrict__ q, float sc
     }
   };
 
-  // write the partial of head rows h < grp (m in log2 units, rotated o) from
-  // merged rows in qr: rotate back, natural-log m, to workspace slot kFinalSlot
-  auto final_partial = [&](int b, int hkv, const float* Mh, const float* Lh) {
+  // the output of head rows h < grp from merged rows in qr (m in log2 units,
+  // rotated o): rotate back, add the full-precision tokens' partials
+  auto finish = [&](int b, int hkv, const float* Mh, const float* Lh) {
     consumer_sync();
+    pdl_wait();
     if (warp < grp) {
       float x[D / 32];
 #pragma unroll
       for (int i = 0; i < D / 32; ++i) x[i] = qr[warp * D + lane + 32 * i];
       fwht_rows<D>(x, lane, inv_sqrt_d);
-      float* w = wsb + (((int64_t)b * g.Hq + hkv * grp + warp) * kMaxSplits + kFinalSlot) * (D + kWsStride);
-#pragma unroll
-      for (int i = 0; i < D / 32; ++i) w[2 + lane + 32 * i] = x[i];
-      if (lane == 0) {
-        w[0] = Mh[warp] == -INFINITY ? -INFINITY : Mh[warp] * 0.6931471805599453f;
-        w[1] = Lh[warp];
-      }
+      const int64_t row = (int64_t)b * g.Hq + hkv * grp + warp;
+      merge_full<D>(wsb + (row * kMaxSplits + kFullSlot) * (D + kWsStride), x, Mh[warp], Lh[warp], lane,
+                    out + row * D);
     }
     consumer_sync();
   };
@@ -539,7 +701,7 @@ decode_stream_kvarn_kernel(Geom g, const __nv_bfloat16* __restrict__ q, float sc
     consumer_sync();
     const int c0 = cta_of(hs, N, P), c1 = cta_of(hs + nb - 1, N, P);
     const int nct = c1 - c0 + 1;
-    if (nct > kMaxSplits - 1) {                      // the host sizes the grid so this cannot happen
+    if (nct > kFullSlot) {                           // the host sizes the grid so this cannot happen
       if (tc == 0) atomicOr(err, 4);
       continue;
     }
@@ -552,7 +714,7 @@ decode_stream_kvarn_kernel(Geom g, const __nv_bfloat16* __restrict__ q, float sc
       else wsb[((orow0 + h) * kMaxSplits + (blockIdx.x - c0)) * (D + kWsStride) + 2 + d] = acc;
     }
     if (nct == 1) {
-      final_partial(b, hkv, mg->M, mg->L);
+      finish(b, hkv, mg->M, mg->L);
       continue;
     }
     if (tc < grp) {
@@ -597,7 +759,7 @@ decode_stream_kvarn_kernel(Geom g, const __nv_bfloat16* __restrict__ q, float sc
       qr[h * D + d] = acc;
     }
     if (tc == 0) g.counters[hd] = 0;                 // ready for the next call
-    final_partial(b, hkv, mg->M, mg->L);
+    finish(b, hkv, mg->M, mg->L);
   }
 }
 
@@ -612,15 +774,20 @@ size_t stream_smem(int grp, int* ns) {
 }
 
 template <int D, int KB, int VB, int G>
-cudaError_t launch_t(const Geom& g, const void* q, float scale, int* err, cudaStream_t s) {
+cudaError_t launch_t(const Geom& g, const void* q, float scale, int* err, void* out,
+                     cudaStream_t s) {
   const int grp = g.Hq / g.H;
+  auto full = grp <= 2 ? kvarn_full_kernel<D, 2> : grp <= 4 ? kvarn_full_kernel<D, 4> : kvarn_full_kernel<D, 8>;
+  launch_pdl(full, dim3(kFullSplits, g.H, g.B), dim3(kFullWarps * 32), 0, s, g,
+             reinterpret_cast<const __nv_bfloat16*>(q), scale);
   int ns = 0;
   const size_t sm = stream_smem<D, KB, VB, G>(grp, &ns);
   auto kern = decode_stream_kvarn_kernel<D, KB, VB, G>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   if (e != cudaSuccess) return e;
   launch_pdl(kern, dim3(decode_stream_ctas(g)), dim3(kThreads), sm, s, g,
-             reinterpret_cast<const __nv_bfloat16*>(q), scale, (float)(1.0 / sqrt((double)D)), err, ns);
+             reinterpret_cast<const __nv_bfloat16*>(q), scale, (float)(1.0 / sqrt((double)D)), err,
+             reinterpret_cast<__nv_bfloat16*>(out), ns);
   return cudaGetLastError();
 }
 
@@ -633,9 +800,9 @@ bool decode_stream_kvarn_supported(const Geom& g) {
 }
 
 cudaError_t launch_decode_stream_kvarn(const Geom& g, const void* q, float scale, int* err,
-                                       cudaStream_t s) {
-  if (g.D == 256) return launch_t<256, 4, 2, 64>(g, q, scale, err, s);
-  return launch_t<64, 4, 2, 32>(g, q, scale, err, s);
+                                       void* out, cudaStream_t s) {
+  if (g.D == 256) return launch_t<256, 4, 2, 64>(g, q, scale, err, out, s);
+  return launch_t<64, 4, 2, 32>(g, q, scale, err, out, s);
 }
 
 }  // namespace kvq

@@ -15,9 +15,10 @@ constexpr int kNW = 11;            // consumer warps (12 warps: the register fil
 constexpr int kThreads = (kNW + 1) * 32;
 constexpr int kMaxStages = 64;
 constexpr int kSmemMax = 227 * 1024;
-// workspace slot where a KVarN head's coded-token partial waits for the
-// combine with the full-precision tokens' split partials (slots below it)
-constexpr int kFinalSlot = kMaxSplits - 1;
+// workspace slots of a KVarN head's full-precision tokens (sinks, staged): one
+// partial per CTA of their kernel, above the at most 17 of the coded tokens' CTAs
+constexpr int kFullSplits = 4;
+constexpr int kFullSlot = kMaxSplits - kFullSplits;
 
 // Transpose of an 8x8 tile of 16-bit values held as an mma fragment.
 __device__ __forceinline__ uint32_t movmatrix_t(uint32_t a) {
