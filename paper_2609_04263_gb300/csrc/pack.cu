@@ -638,13 +638,14 @@ __global__ void kvarn_block_kernel(Geom g, int L, TokSrc sk, TokSrc sv, float in
 // Division: y / s as q = RN(y v), RN(q + v (y - q s)) with v = RN(1 / s): the
 // correctly rounded quotient (P. Markstein, "Computation of elementary
 // functions on the IBM RISC System/6000 processor", 1990), given v correctly
-// rounded and y - q s exact.  s lies in [1e-8, 2^30] and every nonzero y is at
-// least 2^-50 in the row step, so at least 2^-80 in the column step: the
-// remainder is then representable and no quotient is subnormal.  A warp with
-// a value outside those bounds divides with __fdiv_rn.
+// rounded and y - q s exact.  That holds while s lies in [1e-8, 2^30] and no
+// nonzero y falls below 2^-90 (the remainder is then representable and no
+// quotient is subnormal).  y is its start over its row and column scales, so
+// one look at the start (nonzero values of at least 2^-50) and the scales kept
+// below 2^20 show it for every step; a warp that cannot divides with __fdiv_rn.
 //
 // 4 sequences x 8 heads x 8000 tokens, D = 256, G = 64: 1990 us with the block
-// in shared memory, 751 us so.
+// in shared memory, 718 us so.
 __device__ __forceinline__ uint64_t pk2(float lo, float hi) {
   uint64_t r;
   asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
@@ -737,6 +738,7 @@ struct KvarnSmem {
   float part[8][D];                  // column sums of squares of each warp's rows
   float2 csig[D];                    // column divisors: -s, 1 / s
   float rsig[8][8];                  // row divisors, when a warp divides exactly
+  int far;                           // a column's divisor or scale is out of bounds
   float4 grp[8][32];                 // coding: minimum, 1 / scale, scale
 };
 
@@ -832,23 +834,29 @@ kvarn_block_fast_kernel(Geom g, int L, TokSrc sk, TokSrc sv, float inv_sqrt_d, u
       y[i][p] = pk2(__fmul_rn(x[2 * p], inv_sqrt_d), __fmul_rn(x[2 * p + 1], inv_sqrt_d));
   }
 
-  constexpr float kMaxS = 0x1p30f;
+  constexpr float kMaxS = 0x1p30f, kMaxScale = 0x1p20f;
   constexpr uint32_t kMinY = (77u << 24) - 1;    // 2^-50, sign shifted out, less one
+  uint32_t ymin = 0xffffffffu;                   // smallest nonzero magnitude (0 wraps to the top)
+#pragma unroll
+  for (int i = 0; i < NR; ++i)
+#pragma unroll
+    for (int p = 0; p < NP; ++p) {
+      const float2 f = upk2(y[i][p]);
+      ymin = min(ymin, min((__float_as_uint(f.x) << 1) - 1, (__float_as_uint(f.y) << 1) - 1));
+    }
+  bool fast = __all_sync(0xffffffffu, ymin >= kMinY);   // this warp's divisions so far
+  if (threadIdx.x == 0) sm.far = 0;
+  __syncthreads();
   const float inv_d = 1.f / (float)D, inv_g = 1.f / (float)G;
   float rsc = 1.f, csc = 1.f;   // scale of row lane / (32 / NR), of column threadIdx.x
   for (int it = 0; it < g.iters; ++it) {
     // ---- rows ----
     float a[NR];
-    uint32_t ymin = 0xffffffffu;                 // smallest nonzero magnitude (0 wraps to the top)
 #pragma unroll
     for (int i = 0; i < NR; ++i) {
       uint64_t s[NP];
 #pragma unroll
-      for (int p = 0; p < NP; ++p) {
-        s[p] = square2(y[i][p], nz);
-        const float2 f = upk2(y[i][p]);
-        ymin = min(ymin, min((__float_as_uint(f.x) << 1) - 1, (__float_as_uint(f.y) << 1) - 1));
-      }
+      for (int p = 0; p < NP; ++p) s[p] = square2(y[i][p], nz);
 #pragma unroll
       for (int n = NP / 2; n >= 1; n >>= 1)
 #pragma unroll
@@ -860,7 +868,7 @@ kvarn_block_fast_kernel(Geom g, int L, TokSrc sk, TokSrc sv, float inv_sqrt_d, u
     const float sg = fmaxf(__fsqrt_rn(__fmul_rn(sum, inv_d)), 1e-8f);
     const float inv = __frcp_rn(sg);
     rsc = __fmul_rn(rsc, sg);
-    const bool fast = __all_sync(0xffffffffu, ymin >= kMinY && sg <= kMaxS);
+    fast = fast && __all_sync(0xffffffffu, sg <= kMaxS && rsc <= kMaxScale) && !sm.far;
     auto exact = [&](const float* rs) {          // through this lane's part of the warp's rows
 #pragma unroll
       for (int i = 0; i < NR; ++i)
@@ -918,19 +926,15 @@ kvarn_block_fast_kernel(Geom g, int L, TokSrc sk, TokSrc sv, float inv_sqrt_d, u
       const float cg = fmaxf(__fsqrt_rn(__fmul_rn(s[0], inv_g)), 1e-8f);
       csc = __fmul_rn(csc, cg);
       sm.csig[threadIdx.x] = make_float2(-cg, __frcp_rn(cg));
+      if (!(cg <= kMaxS && csc <= kMaxScale)) sm.far = 1;
     }
     __syncthreads();
-    float2 cg[NS];
-    float cmax = 0.f;
-#pragma unroll
-    for (int j = 0; j < NS; ++j) {
-      cg[j] = sm.csig[lane + 32 * j];
-      cmax = fmaxf(cmax, -cg[j].x);
-    }
-    if (__all_sync(0xffffffffu, fast && cmax <= kMaxS)) {
+    fast = fast && !sm.far;
+    if (fast) {
 #pragma unroll
       for (int p = 0; p < NP; ++p) {
-        const uint64_t ns2 = pk2(cg[2 * p].x, cg[2 * p + 1].x), v2 = pk2(cg[2 * p].y, cg[2 * p + 1].y);
+        const float2 c0 = sm.csig[lane + 64 * p], c1 = sm.csig[lane + 64 * p + 32];
+        const uint64_t ns2 = pk2(c0.x, c1.x), v2 = pk2(c0.y, c1.y);
 #pragma unroll
         for (int i = 0; i < NR; ++i) y[i][p] = div2(y[i][p], ns2, v2);
       }
