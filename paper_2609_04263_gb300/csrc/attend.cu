@@ -102,6 +102,54 @@ __device__ __forceinline__ void dequant_rows(const Geom& g, int which, int b, in
   }
 }
 
+// Affine and symmetric caches: this thread's part of a tile as stored, NI = D / 32
+// chunks of 8 channels (chunk threadIdx.x + 256 i, rows of D / 8 chunks), so that the
+// next tile's loads are in flight while a tile is multiplied.
+template <int D>
+struct PackedChunks {
+  static constexpr int NI = kTile * (D / 8) / kThreads;
+  uint64_t w[NI];
+  __half s[NI], z[NI];
+  __device__ __forceinline__ void load(const Geom& g, int which, int b, int h, int t0, int n, int T,
+                                       int lg) {
+    const int bits = which ? g.vb : g.kb;
+    const uint8_t* codes = plane_ptr<uint8_t>(g, which ? KVQ_PLANE_V_CODES : KVQ_PLANE_K_CODES, b, h, 0);
+    const __half* sp = plane_ptr<__half>(g, which ? KVQ_PLANE_V_SCALE : KVQ_PLANE_K_SCALE, b, h, 0);
+    const __half* zp = g.fmt == KVQ_FMT_SYMMETRIC
+                           ? nullptr : plane_ptr<__half>(g, which ? KVQ_PLANE_V_ZERO : KVQ_PLANE_K_ZERO, b, h, 0);
+#pragma unroll
+    for (int i = 0; i < NI; ++i) {
+      const int idx = threadIdx.x + kThreads * i, c = idx % (D / 8), t = t0 + idx / (D / 8);
+      w[i] = 0;
+      s[i] = z[i] = __half(0.f);
+      if (idx / (D / 8) >= n || t >= T) continue;
+      const uint8_t* p = codes + (int64_t)t * (D * bits / 8) + c * bits;
+      w[i] = bits == 4 ? *reinterpret_cast<const uint32_t*>(p)
+           : bits == 2 ? *reinterpret_cast<const uint16_t*>(p) : *reinterpret_cast<const uint64_t*>(p);
+      const int64_t m = (int64_t)t * (D >> lg) + ((8 * c) >> lg);
+      s[i] = sp[m];
+      if (zp) z[i] = zp[m];
+    }
+  }
+  __device__ __forceinline__ void expand(const Geom& g, int which, int n, float* dst, int ld) const {
+    const int bits = which ? g.vb : g.kb;
+    const unsigned mask = (1u << bits) - 1;
+#pragma unroll
+    for (int i = 0; i < NI; ++i) {
+      const int idx = threadIdx.x + kThreads * i, c = idx % (D / 8), r = idx / (D / 8);
+      if (r >= n) continue;
+      const float sc = __half2float(s[i]);
+      const float m = g.fmt == KVQ_FMT_SYMMETRIC ? -(float)(1 << (bits - 1)) * sc : __half2float(z[i]);
+      float v[8];
+#pragma unroll
+      for (int e = 0; e < 8; ++e) v[e] = (float)((unsigned)(w[i] >> (e * bits)) & mask) * sc + m;
+      float4* d = reinterpret_cast<float4*>(dst + r * ld + 8 * c);
+      d[0] = make_float4(v[0], v[1], v[2], v[3]);
+      d[1] = make_float4(v[4], v[5], v[6], v[7]);
+    }
+  }
+};
+
 // Normalised Hadamard transform of `rows` rows of D values at x [rows][ld]
 // (the whole CTA; H / sqrt(D) is its own inverse).
 __device__ void rotate_rows(float* x, int rows, int D, int ld, float inv_sqrt_d) {
@@ -133,7 +181,7 @@ __device__ void rotate_rows(float* x, int rows, int D, int ld, float inv_sqrt_d)
 // 0.07 GFLOP a head), so the latency of one CTA's chain of tiles bounds it: 16
 // rows a CTA give 8 times the CTAs of 128 rows, and 64 rows serve where 16 are
 // not needed to cover the SMs twice.  512 tokens, 4 heads of 64, fp32, affine
-// 4-bit: 1142 -> 59 us, a decode step after them 24 + 10 -> 16 us.
+// 4-bit: 1142 -> 34 us, a decode step after them 24 + 10 -> 14 us.
 // decode: writes (m, l, o) partials to the workspace; the last split CTA of a
 // (sequence, kv head) merges them (one launch instead of two).
 template <int D, int ROWS>
@@ -174,6 +222,14 @@ attend_generic_kernel(Geom g, const void* q, int L, float scale, void* out,
     const int hl = r / nq, qi = r % nq;
     return hl < grp && qi < nql ? pos_first + qi : -1;
   };
+  const bool kvarn = g.fmt == KVQ_FMT_KVARN;
+  const bool packed = g.fmt == KVQ_FMT_AFFINE || g.fmt == KVQ_FMT_SYMMETRIC;
+  const int lg = __ffs(g.G) - 1;                  // G is a power of two
+  PackedChunks<D> pk, pv;
+  if (packed && ts < te) {
+    pk.load(g, 0, b, hkv, ts, te - ts, T, lg);
+    pv.load(g, 1, b, hkv, ts, te - ts, T, lg);
+  }
   for (int i = threadIdx.x; i < ROWS * D; i += kThreads) {
     const int r = i / D, d = i % D;
     const int hl = r / nq, qi = r % nq;
@@ -182,7 +238,6 @@ attend_generic_kernel(Geom g, const void* q, int L, float scale, void* out,
       v = ld_act(q, (((int64_t)b * g.Hq + hkv * grp + hl) * L + q0 + qi) * D + d, g.act);
     sm.q[i] = v;
   }
-  const bool kvarn = g.fmt == KVQ_FMT_KVARN;
   if (kvarn) rotate_rows(sm.q, ROWS, D, D, inv_sqrt_d);     // queries into the rotated basis
 
   constexpr int RS = ROWS / 4;                    // score rows of a thread
@@ -205,7 +260,14 @@ attend_generic_kernel(Geom g, const void* q, int L, float scale, void* out,
     const int n = min(kTile, te - t0);
     const int n4 = (n + 3) & ~3;                  // rows of V read below
     __syncthreads();                              // previous tile consumed (and q stored)
-    if (kvarn) {
+    if (packed) {
+      pk.expand(g, 0, n4, sm.k, S::LDK);
+      pv.expand(g, 1, n4, sm.v, D);
+      if (t0 + kTile < te) {
+        pk.load(g, 0, b, hkv, t0 + kTile, te - t0 - kTile, T, lg);
+        pv.load(g, 1, b, hkv, t0 + kTile, te - t0 - kTile, T, lg);
+      }
+    } else if (kvarn) {
       kvarn_rows(g, 0, b, hkv, t0, n4, T, sm.k, S::LDK, inv_sqrt_d);
       kvarn_rows(g, 1, b, hkv, t0, n4, T, sm.v, D, inv_sqrt_d);
     } else {
