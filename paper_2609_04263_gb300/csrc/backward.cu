@@ -21,9 +21,12 @@
 //   dB_p = (alpha/r) g_p^T U_p      dA_p = (alpha/r) V_p^T x
 //   dx   = g W + sum_p (alpha/r) V_p A_p
 //
-// Every product runs on one fp32 SIMT GEMM kernel with strided operands,
-// batched over pairs and split over K where K is long and the output small.
+// Every product runs on one GEMM kernel with strided operands, batched over
+// pairs and split over K where K is long and the output small: fp32 operands as
+// three bf16 parts on the tensor cores (about 24 bits), bf16 operands as they are.
 #include <math.h>
+
+#include <type_traits>
 
 #include "kvq_internal.cuh"
 #include "proj_decode.cuh"
@@ -34,8 +37,22 @@ namespace {
 
 // ---------------------------------------------------------------------------
 // C[z] = alpha A[z] B[z] (+ C[z]) in fp32, A(m, k) and B(k, n) at strides.
+//
+// An fp32 operand x is split into three bf16 parts x = x0 + x1 + x2 (each the
+// rounding of what the parts before it leave: 24 significant bits) and the
+// products of parts i, j with i + j <= 2 run as mma.sync (6 of them for two
+// fp32 operands, 3 when the other is bf16, 1 when both are); the dropped ones
+// lie below 2^-24 of the product.  The tensor cores truncate as they
+// accumulate, so they sum 16 k at a time from zero (the products of the leading
+// parts last), added to the fp32 accumulator with a rounding addition: the error against
+// 64 bits is not above that of the fp32 chain this replaces.
+// What bounds it is the splitting and the fragment loads, not the MMAs (about 200
+// of 400 issue slots per warp and chunk at six products), which is why 64 x 64 tiles on
+// mma.sync, four CTAs per SM and no staging in tensor memory serve here.
+// All products of the attention backward of 1000 tokens, 32 / 8 heads of 128:
+// 1317 us in fp32 FMA, 548 us so.
 // ---------------------------------------------------------------------------
-constexpr int kBM = 64, kBN = 64, kBK = 16, kGemmThreads = 256;
+constexpr int kBM = 64, kBN = 64, kBK = 32, kGemmThreads = 128;
 
 enum MaskMode {
   kMaskNone = 0,
@@ -64,49 +81,117 @@ __device__ __forceinline__ int max_visible(int r0, int r1, int L, int T) {
   return T - L + last % L;
 }
 
-template <typename E>
-__device__ __forceinline__ float ldf(const E* p, int64_t i);
-template <>
-__device__ __forceinline__ float ldf<float>(const float* p, int64_t i) { return p[i]; }
-template <>
-__device__ __forceinline__ float ldf<__nv_bfloat16>(const __nv_bfloat16* p, int64_t i) {
-  return __bfloat162float(p[i]);
+__device__ __forceinline__ uint32_t smem_addr(const void* p) {
+  return static_cast<uint32_t>(__cvta_generic_to_shared(p));
+}
+__device__ __forceinline__ void ldsm4(uint32_t (&r)[4], const void* p) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(smem_addr(p)));
+}
+__device__ __forceinline__ void ldsm4_t(uint32_t (&r)[4], const void* p) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(smem_addr(p)));
+}
+__device__ __forceinline__ void mma_bf16(float (&c)[4], const uint32_t (&a)[4], uint32_t b0,
+                                         uint32_t b1) {
+  asm volatile(
+      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, "
+      "{%8,%9}, {%0,%1,%2,%3};\n"
+      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
-// Load one BK x 64 operand tile (rows r0.., k0..) into registers: 4 values per
-// thread, consecutive threads on consecutive addresses of the contiguous axis.
+// One operand tile (64 rows x 32 k) in shared memory, PARTS bf16 parts of it:
+// [row][k] when the operand is K-major in memory, else [k][row] (ldmatrix
+// transposes); rows of 80 or 144 bytes put 8 rows in distinct banks.
 template <typename E, bool KMAJOR>
-__device__ __forceinline__ void load_tile(const E* p, int64_t ld, int r0, int R, int k0, int K,
-                                          float v[4]) {
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int idx = threadIdx.x + kGemmThreads * i;
-    int r, k;
-    if (KMAJOR) { r = idx >> 4; k = idx & 15; } else { r = idx & 63; k = idx >> 6; }
-    r += r0;
-    k += k0;
-    v[i] = (r < R && k < K) ? ldf<E>(p, KMAJOR ? (int64_t)r * ld + k : (int64_t)k * ld + r) : 0.f;
-  }
-}
+struct Operand {
+  static constexpr int PARTS = sizeof(E) == 4 ? 3 : 1;
+  static constexpr int PITCH = KMAJOR ? kBK + 8 : kBM + 8;
+  static constexpr int PART = KMAJOR ? kBM * PITCH : kBK * PITCH;   // elements
+  using V4 = typename std::conditional<sizeof(E) == 4, float4, uint2>::type;   // 4 elements
 
-template <bool KMAJOR>
-__device__ __forceinline__ void store_tile(float (*s)[kBM + 4], const float v[4]) {
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
+  // Elements (r, k .. k + 3) or (r .. r + 3, k): four per thread and step,
+  // neighbouring threads on neighbouring addresses.
+  static __device__ __forceinline__ void where(int i, int* r, int* k) {
     const int idx = threadIdx.x + kGemmThreads * i;
-    int r, k;
-    if (KMAJOR) { r = idx >> 4; k = idx & 15; } else { r = idx & 63; k = idx >> 6; }
-    s[k][r] = v[i];
+    if (KMAJOR) { *r = idx >> 3; *k = (idx & 7) * 4; }
+    else { *r = (idx & 15) * 4; *k = idx >> 4; }
   }
-}
+  // vec: rows start on 4-element boundaries.
+  static __device__ __forceinline__ void load(const E* p, int64_t ld, int r0, int R, int k0, int K,
+                                              bool vec, V4 (&v)[4]) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      int r, k;
+      where(i, &r, &k);
+      r += r0;
+      k += k0;
+      const E* q = p + (KMAJOR ? (int64_t)r * ld + k : (int64_t)k * ld + r);
+      const int left = KMAJOR ? (r < R ? K - k : 0) : (k < K ? R - r : 0);   // elements from here on
+      if (vec && left >= 4) {
+        v[i] = *reinterpret_cast<const V4*>(q);
+      } else {
+        __align__(16) E e[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) e[j] = j < left ? q[j] : E(0.f);
+        v[i] = *reinterpret_cast<const V4*>(e);
+      }
+    }
+  }
+  static __device__ __forceinline__ void store(__nv_bfloat16* s, const V4 (&v)[4]) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      int r, k;
+      where(i, &r, &k);
+      __nv_bfloat16* d = s + (KMAJOR ? r * PITCH + k : k * PITCH + r);
+      if constexpr (PARTS == 1) {
+        *reinterpret_cast<uint2*>(d) = v[i];
+      } else {
+        float x[4] = {v[i].x, v[i].y, v[i].z, v[i].w};
+#pragma unroll
+        for (int part = 0; part < 3; ++part) {
+          uint2 u;
+          uint32_t* w = &u.x;
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            const __nv_bfloat162 t = __floats2bfloat162_rn(x[2 * h], x[2 * h + 1]);
+            w[h] = *reinterpret_cast<const uint32_t*>(&t);
+            const float2 f = __bfloat1622float2(t);
+            x[2 * h] -= f.x;
+            x[2 * h + 1] -= f.y;
+          }
+          *reinterpret_cast<uint2*>(d + part * PART) = u;
+        }
+      }
+    }
+  }
+  // The 16 x 16 A fragment at rows r, k-step k.
+  static __device__ __forceinline__ void frag_a(const __nv_bfloat16* s, int r, int k, int lane,
+                                                uint32_t (&f)[4]) {
+    if (KMAJOR) ldsm4(f, s + (r + (lane & 15)) * PITCH + k + (lane >> 4) * 8);
+    else ldsm4_t(f, s + (k + (lane >> 4) * 8 + (lane & 7)) * PITCH + r + ((lane >> 3) & 1) * 8);
+  }
+  // Two 16 x 8 B fragments (f[0..1], f[2..3]) at columns r, k-step k.
+  static __device__ __forceinline__ void frag_b(const __nv_bfloat16* s, int r, int k, int lane,
+                                                uint32_t (&f)[4]) {
+    const int j = lane >> 3, i = lane & 7;
+    if (KMAJOR) ldsm4(f, s + (r + (j >> 1) * 8 + i) * PITCH + k + (j & 1) * 8);
+    else ldsm4_t(f, s + (k + (j & 1) * 8 + i) * PITCH + r + (j >> 1) * 8);
+  }
+};
 
 // A_KMAJOR: A(m, k) = a[m lda + k], else a[k lda + m].
 // B_KMAJOR: B(k, n) = b[n ldb + k], else b[k ldb + n].
 template <typename TA, typename TB, bool A_KMAJOR, bool B_KMAJOR>
 __global__ void __launch_bounds__(kGemmThreads) bgemm_kernel(GemmArgs g) {
   pdl_wait();
-  __shared__ __align__(16) float As[2][kBK][kBM + 4];
-  __shared__ __align__(16) float Bs[2][kBK][kBN + 4];
+  pdl_trigger();
+  using OA = Operand<TA, A_KMAJOR>;
+  using OB = Operand<TB, B_KMAJOR>;
+  constexpr int PA = OA::PARTS, PB = OB::PARTS;
+  constexpr int kStage = PA * OA::PART + PB * OB::PART;
+  extern __shared__ __align__(16) __nv_bfloat16 tiles[];          // two stages of A, B parts
   const int z = blockIdx.z;
   const int bz = z / g.splits, sp = z % g.splits;
   const TA* A = reinterpret_cast<const TA*>(g.a) + (int64_t)bz * g.sa;
@@ -125,9 +210,13 @@ __global__ void __launch_bounds__(kGemmThreads) bgemm_kernel(GemmArgs g) {
   const int kt0 = sp * per, kt1 = min(ktiles, kt0 + per);
   if (kt0 >= kt1 && g.splits > 1) return;
 
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  float acc[4][4] = {};
-  float ra[4], rb[4];
+  const bool veca = ((reinterpret_cast<uintptr_t>(A) | (uintptr_t)(g.lda * sizeof(TA))) & (sizeof(typename OA::V4) - 1)) == 0;
+  const bool vecb = ((reinterpret_cast<uintptr_t>(Bp) | (uintptr_t)(g.ldb * sizeof(TB))) & (sizeof(typename OB::V4) - 1)) == 0;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int wm = (warp >> 1) * 32, wn = (warp & 1) * 32;          // this warp's 32 x 32 outputs
+  float acc[2][4][4] = {};
+  typename OA::V4 ra[4];
+  typename OB::V4 rb[4];
   auto skip = [&](int kt) {
     return g.mask == kMaskRowsKeysKQueries &&
            max_visible(kt * kBK, min(kt * kBK + kBK, g.K), g.L, g.T) < m0;
@@ -135,56 +224,85 @@ __global__ void __launch_bounds__(kGemmThreads) bgemm_kernel(GemmArgs g) {
   int kt = kt0;
   while (kt < kt1 && skip(kt)) ++kt;
   if (kt < kt1) {
-    load_tile<TA, A_KMAJOR>(A, g.lda, m0, g.M, kt * kBK, kend, ra);
-    load_tile<TB, B_KMAJOR>(Bp, g.ldb, n0, g.N, kt * kBK, kend, rb);
+    OA::load(A, g.lda, m0, g.M, kt * kBK, kend, veca, ra);
+    OB::load(Bp, g.ldb, n0, g.N, kt * kBK, kend, vecb, rb);
   }
   int buf = 0;
   while (kt < kt1) {
-    store_tile<A_KMAJOR>(As[buf], ra);
-    store_tile<B_KMAJOR>(Bs[buf], rb);
+    __nv_bfloat16* As = tiles + buf * kStage;
+    __nv_bfloat16* Bs = As + PA * OA::PART;
+    OA::store(As, ra);
+    OB::store(Bs, rb);
     __syncthreads();
     int nxt = kt + 1;
     while (nxt < kt1 && skip(nxt)) ++nxt;
     if (nxt < kt1) {                           // prefetch the next tile into registers
-      load_tile<TA, A_KMAJOR>(A, g.lda, m0, g.M, nxt * kBK, kend, ra);
-      load_tile<TB, B_KMAJOR>(Bp, g.ldb, n0, g.N, nxt * kBK, kend, rb);
+      OA::load(A, g.lda, m0, g.M, nxt * kBK, kend, veca, ra);
+      OB::load(Bp, g.ldb, n0, g.N, nxt * kBK, kend, vecb, rb);
     }
 #pragma unroll
-    for (int k = 0; k < kBK; ++k) {
-      const float4 av = *reinterpret_cast<const float4*>(&As[buf][k][ty * 4]);
-      const float4 bv = *reinterpret_cast<const float4*>(&Bs[buf][k][tx * 4]);
-      const float am[4] = {av.x, av.y, av.z, av.w};
-      const float bn[4] = {bv.x, bv.y, bv.z, bv.w};
+    for (int ks = 0; ks < kBK; ks += 16) {
+      float c[2][4][4] = {};                   // this step's sums
+      uint32_t fb[PB][2][4];
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
+      for (int p = 0; p < PB; ++p)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(am[i], bn[j], acc[i][j]);
+        for (int n = 0; n < 2; ++n) OB::frag_b(Bs + p * OB::PART, wn + 16 * n, ks, lane, fb[p][n]);
+#pragma unroll
+      for (int m = 0; m < 2; ++m)
+#pragma unroll
+        for (int pa = PA - 1; pa >= 0; --pa) { // small parts first
+          uint32_t fa[4];
+          OA::frag_a(As + pa * OA::PART, wm + 16 * m, ks, lane, fa);
+#pragma unroll
+          for (int pb = PB - 1; pb >= 0; --pb)
+            if (pa + pb <= 2)
+#pragma unroll
+              for (int n = 0; n < 4; ++n)
+                mma_bf16(c[m][n], fa, fb[pb][n >> 1][2 * (n & 1)], fb[pb][n >> 1][2 * (n & 1) + 1]);
+        }
+#pragma unroll
+      for (int m = 0; m < 2; ++m)
+#pragma unroll
+        for (int n = 0; n < 4; ++n)
+#pragma unroll
+          for (int i = 0; i < 4; ++i) acc[m][n][i] += c[m][n][i];
     }
     buf ^= 1;
     kt = nxt;
   }
   const bool atomic = g.splits > 1;
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int m = m0 + ty * 4 + i;
-    if (m >= g.M) continue;
+  for (int i = 0; i < 2; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int n = n0 + tx * 4 + j;
-      if (n >= g.N) continue;
-      float* dst = C + (int64_t)m * g.ldc + n;
-      const float v = g.alpha * acc[i][j];
-      if (atomic) atomicAdd(dst, v);
-      else *dst = g.accumulate ? *dst + v : v;
+    for (int hr = 0; hr < 2; ++hr) {
+      const int m = m0 + wm + 16 * i + 8 * hr + (lane >> 2);
+      if (m >= g.M) continue;
+#pragma unroll
+      for (int n = 0; n < 4; ++n)
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+          const int col = n0 + wn + 8 * n + 2 * (lane & 3) + e;
+          if (col >= g.N) continue;
+          float* dst = C + (int64_t)m * g.ldc + col;
+          const float v = g.alpha * acc[i][n][2 * hr + e];
+          if (atomic) atomicAdd(dst, v);
+          else *dst = g.accumulate ? *dst + v : v;
+        }
     }
-  }
 }
 
 template <typename TA, typename TB, bool AK, bool BK>
 cudaError_t run_gemm(const GemmArgs& g, cudaStream_t s) {
   if (g.M <= 0 || g.N <= 0 || g.batch <= 0) return cudaSuccess;
+  using OA = Operand<TA, AK>;
+  using OB = Operand<TB, BK>;
+  auto kern = bgemm_kernel<TA, TB, AK, BK>;
+  constexpr int sm = 2 * (OA::PARTS * OA::PART + OB::PARTS * OB::PART) * 2;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+  if (e != cudaSuccess) return e;
   dim3 grid((g.N + kBN - 1) / kBN, (g.M + kBM - 1) / kBM, g.batch * g.splits);
-  launch_pdl(bgemm_kernel<TA, TB, AK, BK>, grid, dim3(kGemmThreads), 0, s, g);
+  launch_pdl(kern, grid, dim3(kGemmThreads), (size_t)sm, s, g);
   return cudaGetLastError();
 }
 
@@ -194,7 +312,7 @@ int choose_splits(int M, int N, int K, int batch) {
   const int64_t want = 2LL * num_sms();
   if (tiles >= want) return 1;
   int s = (int)((want + tiles - 1) / tiles);
-  const int maxs = max(1, K / (8 * kBK));      // keep at least 8 K tiles per split
+  const int maxs = max(1, K / (4 * kBK));      // keep at least 4 K tiles per split
   return max(1, min(s, min(maxs, 64)));
 }
 
