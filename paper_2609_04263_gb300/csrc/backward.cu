@@ -61,14 +61,18 @@ enum MaskMode {
   kMaskRowsKeysKQueries = 3,      // m: keys, k: stacked query rows (dK, dV)
 };
 
-struct GemmArgs {
+struct GemmOp {
   const void* a;
   const void* b;
   float* c;
   int M, N, K;
   int64_t lda, ldb, ldc;      // A(m,k) = a[m lda + k] (K-major) or a[k lda + m]
+};
+struct GemmArgs {
+  GemmOp op[3];               // products of one launch, alike but for pointers and sizes
+  int ops;
   int64_t sa, sb, sc;         // batch strides in elements
-  int batch, splits;          // grid.z = batch x splits; splits > 1 adds atomically
+  int batch, splits;          // grid.z = ops x batch x splits; splits > 1 adds atomically
   float alpha;
   int accumulate;             // 1: C += alpha A B (splits > 1 implies it)
   int mask, L, T;             // causal structure of the attention products
@@ -184,7 +188,7 @@ struct Operand {
 // A_KMAJOR: A(m, k) = a[m lda + k], else a[k lda + m].
 // B_KMAJOR: B(k, n) = b[n ldb + k], else b[k ldb + n].
 template <typename TA, typename TB, bool A_KMAJOR, bool B_KMAJOR>
-__global__ void __launch_bounds__(kGemmThreads) bgemm_kernel(GemmArgs g) {
+__global__ void __launch_bounds__(kGemmThreads) bgemm_kernel(const __grid_constant__ GemmArgs g) {
   pdl_wait();
   pdl_trigger();
   using OA = Operand<TA, A_KMAJOR>;
@@ -192,26 +196,27 @@ __global__ void __launch_bounds__(kGemmThreads) bgemm_kernel(GemmArgs g) {
   constexpr int PA = OA::PARTS, PB = OB::PARTS;
   constexpr int kStage = PA * OA::PART + PB * OB::PART;
   extern __shared__ __align__(16) __nv_bfloat16 tiles[];          // two stages of A, B parts
-  const int z = blockIdx.z;
-  const int bz = z / g.splits, sp = z % g.splits;
-  const TA* A = reinterpret_cast<const TA*>(g.a) + (int64_t)bz * g.sa;
-  const TB* Bp = reinterpret_cast<const TB*>(g.b) + (int64_t)bz * g.sb;
-  float* C = g.c + (int64_t)bz * g.sc;
+  const int sp = blockIdx.z % g.splits, bz = blockIdx.z / g.splits % g.batch;
+  const GemmOp op = g.op[blockIdx.z / (g.splits * g.batch)];
+  const TA* A = reinterpret_cast<const TA*>(op.a) + (int64_t)bz * g.sa;
+  const TB* Bp = reinterpret_cast<const TB*>(op.b) + (int64_t)bz * g.sb;
+  float* C = op.c + (int64_t)bz * g.sc;
   const int m0 = blockIdx.y * kBM, n0 = blockIdx.x * kBN;
+  if (m0 >= op.M || n0 >= op.N) return;
 
   // K range of this split, clipped by the causal structure.
-  int kend = g.K;
+  int kend = op.K;
   if (g.mask == kMaskRowsQueriesColsKeys &&
-      n0 > max_visible(m0, min(m0 + kBM, g.M), g.L, g.T))
+      n0 > max_visible(m0, min(m0 + kBM, op.M), g.L, g.T))
     return;                                    // every score of the tile is masked
-  if (g.mask == kMaskRowsQueriesKKeys) kend = min(kend, max_visible(m0, min(m0 + kBM, g.M), g.L, g.T) + 1);
+  if (g.mask == kMaskRowsQueriesKKeys) kend = min(kend, max_visible(m0, min(m0 + kBM, op.M), g.L, g.T) + 1);
   const int ktiles = (kend + kBK - 1) / kBK;
   const int per = (ktiles + g.splits - 1) / g.splits;
   const int kt0 = sp * per, kt1 = min(ktiles, kt0 + per);
   if (kt0 >= kt1 && g.splits > 1) return;
 
-  const bool veca = ((reinterpret_cast<uintptr_t>(A) | (uintptr_t)(g.lda * sizeof(TA))) & (sizeof(typename OA::V4) - 1)) == 0;
-  const bool vecb = ((reinterpret_cast<uintptr_t>(Bp) | (uintptr_t)(g.ldb * sizeof(TB))) & (sizeof(typename OB::V4) - 1)) == 0;
+  const bool veca = ((reinterpret_cast<uintptr_t>(A) | (uintptr_t)(op.lda * sizeof(TA))) & (sizeof(typename OA::V4) - 1)) == 0;
+  const bool vecb = ((reinterpret_cast<uintptr_t>(Bp) | (uintptr_t)(op.ldb * sizeof(TB))) & (sizeof(typename OB::V4) - 1)) == 0;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int wm = (warp >> 1) * 32, wn = (warp & 1) * 32;          // this warp's 32 x 32 outputs
   float acc[2][4][4] = {};
@@ -219,13 +224,13 @@ __global__ void __launch_bounds__(kGemmThreads) bgemm_kernel(GemmArgs g) {
   typename OB::V4 rb[4];
   auto skip = [&](int kt) {
     return g.mask == kMaskRowsKeysKQueries &&
-           max_visible(kt * kBK, min(kt * kBK + kBK, g.K), g.L, g.T) < m0;
+           max_visible(kt * kBK, min(kt * kBK + kBK, op.K), g.L, g.T) < m0;
   };
   int kt = kt0;
   while (kt < kt1 && skip(kt)) ++kt;
   if (kt < kt1) {
-    OA::load(A, g.lda, m0, g.M, kt * kBK, kend, veca, ra);
-    OB::load(Bp, g.ldb, n0, g.N, kt * kBK, kend, vecb, rb);
+    OA::load(A, op.lda, m0, op.M, kt * kBK, kend, veca, ra);
+    OB::load(Bp, op.ldb, n0, op.N, kt * kBK, kend, vecb, rb);
   }
   int buf = 0;
   while (kt < kt1) {
@@ -237,8 +242,8 @@ __global__ void __launch_bounds__(kGemmThreads) bgemm_kernel(GemmArgs g) {
     int nxt = kt + 1;
     while (nxt < kt1 && skip(nxt)) ++nxt;
     if (nxt < kt1) {                           // prefetch the next tile into registers
-      OA::load(A, g.lda, m0, g.M, nxt * kBK, kend, veca, ra);
-      OB::load(Bp, g.ldb, n0, g.N, nxt * kBK, kend, vecb, rb);
+      OA::load(A, op.lda, m0, op.M, nxt * kBK, kend, veca, ra);
+      OB::load(Bp, op.ldb, n0, op.N, nxt * kBK, kend, vecb, rb);
     }
 #pragma unroll
     for (int ks = 0; ks < kBK; ks += 16) {
@@ -277,14 +282,14 @@ __global__ void __launch_bounds__(kGemmThreads) bgemm_kernel(GemmArgs g) {
 #pragma unroll
     for (int hr = 0; hr < 2; ++hr) {
       const int m = m0 + wm + 16 * i + 8 * hr + (lane >> 2);
-      if (m >= g.M) continue;
+      if (m >= op.M) continue;
 #pragma unroll
       for (int n = 0; n < 4; ++n)
 #pragma unroll
         for (int e = 0; e < 2; ++e) {
           const int col = n0 + wn + 8 * n + 2 * (lane & 3) + e;
-          if (col >= g.N) continue;
-          float* dst = C + (int64_t)m * g.ldc + col;
+          if (col >= op.N) continue;
+          float* dst = C + (int64_t)m * op.ldc + col;
           const float v = g.alpha * acc[i][n][2 * hr + e];
           if (atomic) atomicAdd(dst, v);
           else *dst = g.accumulate ? *dst + v : v;
@@ -294,14 +299,19 @@ __global__ void __launch_bounds__(kGemmThreads) bgemm_kernel(GemmArgs g) {
 
 template <typename TA, typename TB, bool AK, bool BK>
 cudaError_t run_gemm(const GemmArgs& g, cudaStream_t s) {
-  if (g.M <= 0 || g.N <= 0 || g.batch <= 0) return cudaSuccess;
+  int M = 0, N = 0;
+  for (int i = 0; i < g.ops; ++i) {
+    M = std::max(M, g.op[i].M);
+    N = std::max(N, g.op[i].N);
+  }
+  if (M <= 0 || N <= 0 || g.batch <= 0) return cudaSuccess;
   using OA = Operand<TA, AK>;
   using OB = Operand<TB, BK>;
   auto kern = bgemm_kernel<TA, TB, AK, BK>;
   constexpr int sm = 2 * (OA::PARTS * OA::PART + OB::PARTS * OB::PART) * 2;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
   if (e != cudaSuccess) return e;
-  dim3 grid((g.N + kBN - 1) / kBN, (g.M + kBM - 1) / kBM, g.batch * g.splits);
+  dim3 grid((N + kBN - 1) / kBN, (M + kBM - 1) / kBM, g.ops * g.batch * g.splits);
   launch_pdl(kern, grid, dim3(kGemmThreads), (size_t)sm, s, g);
   return cudaGetLastError();
 }
@@ -316,17 +326,38 @@ int choose_splits(int M, int N, int K, int batch) {
   return max(1, min(s, min(maxs, 64)));
 }
 
-GemmArgs gemm_args(const void* a, int64_t lda, int64_t sa, const void* b, int64_t ldb,
-                   int64_t sb, float* c, int64_t ldc, int64_t sc, int M, int N, int K,
-                   int batch, float alpha) {
+GemmArgs gemm_args(float alpha, int batch = 1, int64_t sa = 0, int64_t sb = 0, int64_t sc = 0) {
   GemmArgs g = {};
-  g.a = a; g.b = b; g.c = c;
-  g.M = M; g.N = N; g.K = K;
-  g.lda = lda; g.ldb = ldb; g.ldc = ldc;
   g.sa = sa; g.sb = sb; g.sc = sc;
   g.batch = batch; g.splits = 1;
   g.alpha = alpha;
   return g;
+}
+void add_op(GemmArgs& g, const void* a, int64_t lda, const void* b, int64_t ldb, float* c,
+            int64_t ldc, int M, int N, int K) {
+  g.op[g.ops++] = GemmOp{a, b, c, M, N, K, lda, ldb, ldc};
+}
+
+// fp32 ranges to zero (outputs that splits add to) and activation-typed ranges to
+// copy (the A_p, gathered below one another), in one launch.
+struct PrepArgs {
+  void* dst[16];
+  const void* src[16];          // NULL: zeros
+  int64_t n[16];
+  int act;
+};
+__global__ void __launch_bounds__(256) bwd_prepare_kernel(const __grid_constant__ PrepArgs a) {
+  pdl_wait();
+  pdl_trigger();
+  void* dst = a.dst[blockIdx.y];
+  const void* src = a.src[blockIdx.y];
+  const int64_t n = a.n[blockIdx.y];
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
+       i += (int64_t)gridDim.x * blockDim.x) {
+    if (!src) reinterpret_cast<float*>(dst)[i] = 0.f;
+    else if (a.act == KVQ_BF16) reinterpret_cast<uint16_t*>(dst)[i] = reinterpret_cast<const uint16_t*>(src)[i];
+    else reinterpret_cast<float*>(dst)[i] = reinterpret_cast<const float*>(src)[i];
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -615,11 +646,10 @@ cudaError_t launch_attend_backward(const Geom& g, int T, const void* q, const vo
                0, s, g, T, p0, np, kh, vh);
     e = cudaGetLastError();
     // S = Q K^T and dP = dO V^T (tiles above the causal edge skipped)
-    GemmArgs ga = gemm_args(qp, D, (int64_t)M * D, kh, D, (int64_t)T * D, S, ld, (int64_t)M * ld,
-                            M, T, D, np, 1.f);
+    GemmArgs ga = gemm_args(1.f, np, (int64_t)M * D, (int64_t)T * D, (int64_t)M * ld);
+    add_op(ga, qp, D, kh, D, S, ld, M, T, D);
+    add_op(ga, op, D, vh, D, dP, ld, M, T, D);
     ga.mask = kMaskRowsQueriesColsKeys; ga.L = L; ga.T = T;
-    if (e == cudaSuccess) e = gemm_act_a<true, true>(ga, act, s);
-    ga.a = op; ga.b = vh; ga.c = dP;
     if (e == cudaSuccess) e = gemm_act_a<true, true>(ga, act, s);
     if (e == cudaSuccess) {
       launch_pdl(bwd_softmax_ds_kernel, dim3((M + kRowWarps - 1) / kRowWarps, np),
@@ -627,16 +657,15 @@ cudaError_t launch_attend_backward(const Geom& g, int T, const void* q, const vo
       e = cudaGetLastError();
     }
     // dQ = dS K
-    GemmArgs gq = gemm_args(dP, ld, (int64_t)M * ld, kh, D, (int64_t)T * D,
-                            dq + (size_t)p0 * M * D, D, (int64_t)M * D, M, D, T, np, 1.f);
+    GemmArgs gq = gemm_args(1.f, np, (int64_t)M * ld, (int64_t)T * D, (int64_t)M * D);
+    add_op(gq, dP, ld, kh, D, dq + (size_t)p0 * M * D, D, M, D, T);
     gq.mask = kMaskRowsQueriesKKeys; gq.L = L; gq.T = T;
     if (e == cudaSuccess) e = run_gemm<float, float, true, false>(gq, s);
     // dK = dS^T Q and dV = P^T dO
-    GemmArgs gk = gemm_args(dP, ld, (int64_t)M * ld, qp, D, (int64_t)M * D,
-                            dk + (size_t)p0 * T * D, D, (int64_t)T * D, T, D, M, np, 1.f);
+    GemmArgs gk = gemm_args(1.f, np, (int64_t)M * ld, (int64_t)M * D, (int64_t)T * D);
+    add_op(gk, dP, ld, qp, D, dk + (size_t)p0 * T * D, D, T, D, M);
+    add_op(gk, S, ld, op, D, dv + (size_t)p0 * T * D, D, T, D, M);
     gk.mask = kMaskRowsKeysKQueries; gk.L = L; gk.T = T;
-    if (e == cudaSuccess) e = gemm_act_b<false, false>(gk, act, s);
-    gk.a = S; gk.b = op; gk.c = dv + (size_t)p0 * T * D;
     if (e == cudaSuccess) e = gemm_act_b<false, false>(gk, act, s);
   }
   return e;
@@ -646,6 +675,7 @@ size_t lora_backward_bytes(int B, int L, int d_in, int Hq, int Hkv, int D, const
   const size_t BL = (size_t)B * L;
   size_t n = a256(BL * (Hq + 2 * Hkv) * D * sizeof(float));
   for (int p = 0; p < 3; ++p) n += 2 * a256(BL * r[p] * sizeof(float));
+  n += a256((size_t)(r[0] + r[1] + r[2]) * d_in * sizeof(float));   // the A_p below one another
   n += a256((size_t)d_in * (Hq + 2 * Hkv) * D * 2);   // W^T in bf16 for the d_x product
   return n;
 }
@@ -670,12 +700,14 @@ cudaError_t launch_lora_backward(const void* x, int B, int L, int d_in, const vo
   char* wp = static_cast<char*>(ws);
   float* G = reinterpret_cast<float*>(wp);
   wp += a256((size_t)BL * ntot * sizeof(float));
+  const int R = r[0] + r[1] + r[2];
   float* U[3];
-  float* V[3];
+  float* V = reinterpret_cast<float*>(wp);               // [BL][R], one column block per projection
+  wp += a256((size_t)BL * R * sizeof(float));
+  char* Acat = wp;                                       // [R][d_in] in the activations' type
+  wp += a256((size_t)R * d_in * sizeof(float));
   for (int p = 0; p < 3; ++p) {
     U[p] = reinterpret_cast<float*>(wp);
-    wp += a256((size_t)BL * r[p] * sizeof(float));
-    V[p] = reinterpret_cast<float*>(wp);
     wp += a256((size_t)BL * r[p] * sizeof(float));
   }
   __nv_bfloat16* Wt = reinterpret_cast<__nv_bfloat16*>(wp);   // [d_in][ntot]
@@ -687,33 +719,50 @@ cudaError_t launch_lora_backward(const void* x, int B, int L, int d_in, const vo
   const int hblocks = std::max(1, std::min(Hq + 2 * Hkv, 8 * num_sms() / tblocks));   // cover the SMs
   launch_pdl(lora_gather_kernel, dim3(tblocks, hblocks), dim3(256), 0, s, ga);
   cudaError_t e = cudaGetLastError();
-  for (int p = 0; p < 3 && e == cudaSuccess; ++p) {
+  // per projection: U_p = x A_p^T and V_p = g_p B_p [BL][r] (narrow outputs over
+  // long K), dB_p = (alpha/r) g_p^T U_p [n_p][r], dA_p = (alpha/r) V_p^T x [r][d_in]
+  // (over the BL rows): split over K, added atomically into zeroed outputs
+  GemmArgs gu = gemm_args(1.f), gv = gemm_args(1.f), gb = gemm_args(alpha_over_r),
+           gA = gemm_args(alpha_over_r);
+  PrepArgs prep = {};
+  prep.act = act;
+  int np = 0, rmax = 0, nmax = 0, ro = 0;
+  const size_t esz = act == KVQ_BF16 ? 2 : 4;
+  for (int p = 0; p < 3; ++p) {
     if (r[p] == 0) continue;
-    // U_p = x A_p^T  [BL][r] and V_p = g_p B_p  [BL][r]: narrow outputs over
-    // long K, split over K (accumulated atomically into zeroed outputs)
-    GemmArgs gu = gemm_args(x, d_in, 0, a[p], d_in, 0, U[p], r[p], 0, BL, r[p], d_in, 1, 1.f);
-    gu.splits = choose_splits(BL, r[p], d_in, 1);
-    if (gu.splits > 1) e = cudaMemsetAsync(U[p], 0, (size_t)BL * r[p] * sizeof(float), s);
+    add_op(gu, x, d_in, a[p], d_in, U[p], r[p], BL, r[p], d_in);
+    add_op(gv, G + off[p], ntot, bm[p], r[p], V + ro, R, BL, r[p], nout[p]);
+    add_op(gb, G + off[p], ntot, U[p], r[p], db[p], r[p], nout[p], r[p], BL);
+    add_op(gA, V + ro, R, x, d_in, da[p], d_in, r[p], d_in, BL);
+    if (dx) {
+      prep.dst[np] = Acat + (size_t)ro * d_in * esz;
+      prep.src[np] = a[p];
+      prep.n[np++] = (int64_t)r[p] * d_in;
+    }
+    rmax = std::max(rmax, r[p]);
+    nmax = std::max(nmax, nout[p]);
+    ro += r[p];
+  }
+  if (R > 0 && e == cudaSuccess) {
+    gu.splits = choose_splits(BL, rmax, d_in, gu.ops);
+    gv.splits = choose_splits(BL, rmax, nmax, gv.ops);
+    gb.splits = choose_splits(nmax, rmax, BL, gb.ops);
+    gA.splits = choose_splits(rmax, d_in, BL, gA.ops);
+    auto zero = [&](float* d, int64_t n) {
+      prep.dst[np] = d;
+      prep.n[np++] = n;
+    };
+    if (gv.splits > 1) zero(V, (int64_t)BL * R);
+    for (const GemmArgs* gg : {&gu, &gb, &gA})
+      for (int i = 0; i < gg->ops && gg->splits > 1; ++i)
+        zero(gg->op[i].c, (int64_t)gg->op[i].M * gg->op[i].N);
+    if (np > 0) {
+      launch_pdl(bwd_prepare_kernel, dim3(32, np), dim3(256), 0, s, prep);
+      e = cudaGetLastError();
+    }
     if (e == cudaSuccess) e = gemm_act_ab<true, true>(gu, act, s);
-    GemmArgs gv = gemm_args(G + off[p], ntot, 0, bm[p], r[p], 0, V[p], r[p], 0, BL, r[p],
-                            nout[p], 1, 1.f);
-    gv.splits = choose_splits(BL, r[p], nout[p], 1);
-    if (e == cudaSuccess && gv.splits > 1)
-      e = cudaMemsetAsync(V[p], 0, (size_t)BL * r[p] * sizeof(float), s);
     if (e == cudaSuccess) e = gemm_act_b<true, false>(gv, act, s);
-    // dB_p = (alpha/r) g_p^T U_p  [n_p][r], split over the BL rows
-    GemmArgs gb = gemm_args(G + off[p], ntot, 0, U[p], r[p], 0, db[p], r[p], 0, nout[p], r[p],
-                            BL, 1, alpha_over_r);
-    gb.splits = choose_splits(nout[p], r[p], BL, 1);
-    if (e == cudaSuccess && gb.splits > 1)
-      e = cudaMemsetAsync(db[p], 0, (size_t)nout[p] * r[p] * sizeof(float), s);
     if (e == cudaSuccess) e = run_gemm<float, float, false, false>(gb, s);
-    // dA_p = (alpha/r) V_p^T x  [r][d_in]
-    GemmArgs gA = gemm_args(V[p], r[p], 0, x, d_in, 0, da[p], d_in, 0, r[p], d_in, BL, 1,
-                            alpha_over_r);
-    gA.splits = choose_splits(r[p], d_in, BL, 1);
-    if (e == cudaSuccess && gA.splits > 1)
-      e = cudaMemsetAsync(da[p], 0, (size_t)r[p] * d_in * sizeof(float), s);
     if (e == cudaSuccess) e = gemm_act_b<false, false>(gA, act, s);
   }
   if (dx && e == cudaSuccess) {
@@ -738,14 +787,15 @@ cudaError_t launch_lora_backward(const void* x, int B, int L, int d_in, const vo
       }
       if (e == cudaSuccess) e = launch_gemm_tc_bf16(G, BL, 2 * ntot, Wt, d_in, ntot, dx, err, s);
     } else {
-      GemmArgs gx = gemm_args(G, ntot, 0, w, d_in, 0, dx, d_in, 0, BL, d_in, ntot, 1, 1.f);
+      GemmArgs gx = gemm_args(1.f);
+      add_op(gx, G, ntot, w, d_in, dx, d_in, BL, d_in, ntot);
       e = gemm_act_b<true, false>(gx, act, s);
     }
-    for (int p = 0; p < 3 && e == cudaSuccess; ++p) {
-      if (r[p] == 0) continue;
-      GemmArgs gl = gemm_args(V[p], r[p], 0, a[p], d_in, 0, dx, d_in, 0, BL, d_in, r[p], 1,
-                              alpha_over_r);
+    // the adapters' part, [V_q | V_k | V_v] times the A_p, in one pass over dx
+    if (R > 0 && e == cudaSuccess) {
+      GemmArgs gl = gemm_args(alpha_over_r);
       gl.accumulate = 1;
+      add_op(gl, V, R, Acat, d_in, dx, d_in, BL, d_in, R);
       e = gemm_act_b<true, false>(gl, act, s);
     }
   }
