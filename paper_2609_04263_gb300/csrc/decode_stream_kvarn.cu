@@ -16,9 +16,10 @@
 //     quantization group; the 128 is removed with an MMA over a constant
 //     operand (which also gives sum_j q'_j, the offset's weight), then
 //       S = r_t sum_g [s_tg (acc_g - bias_g) + m_tg bias_g / 128].
-//   values  A = c_v,j * code (fp16), B = fp16(p) * (r_t s_tg); the offsets
-//     r_t m_tg enter through a small MMA (rows = groups) and are scaled by
-//     c_v,j when the block's contribution is added.
+//   values  A = codes read in place as exact subnormal fp16, B = fp16(p) *
+//     (r_t s_tg), one accumulator set per block and group; c_v,j is applied when the
+//     block's sums are added, with the offsets r_t m_tg from a small MMA (rows =
+//     groups).
 // The sinks and the staged tokens (full precision, original basis: no rotation
 // is needed to attend them) go through kvarn_full_kernel, launched first: four
 // CTAs per head, a warp per token, partials in the top workspace slots.  The
@@ -27,6 +28,8 @@
 // and adds the four partials.  12B-class shape, batch 4, 8300 tokens: the split kernel
 // that used to take the full-precision tokens after the streaming kernel, rotating
 // each of them, added 17 us to its 52 (four layers: 274 -> 241 us).
+#include <type_traits>
+
 #include "decode_attn.cuh"
 #include "stream_common.cuh"
 
@@ -57,6 +60,22 @@ struct KCfg {
   static_assert(G % kBT == 0 && G % 32 == 0, "blocks lie inside one column-scale block");
   static_assert(NGG <= 8, "offset MMA rows hold the groups");
 };
+
+// The MMAs without `volatile`: the compiler may move them among independent ones.
+__device__ __forceinline__ void mma_bf16(float (&c)[4], const uint32_t (&a)[4], uint32_t b0,
+                                         uint32_t b1) {
+  asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, "
+      "{%8,%9}, {%0,%1,%2,%3};\n"
+      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+__device__ __forceinline__ void mma_f16(float (&c)[4], const uint32_t (&a)[4], uint32_t b0,
+                                        uint32_t b1) {
+  asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, "
+      "{%8,%9}, {%0,%1,%2,%3};\n"
+      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
 
 // Normalised Hadamard transform of a row held as x[i] = row[lane + 32 i]
 // (butterflies over the lanes, then over the slots, then 1 / sqrt(D)).
@@ -245,12 +264,16 @@ __device__ __forceinline__ void merge_full(const float* wf, float (&x)[D / 32], 
 
 // Launched after kvarn_full_kernel, whose start waited for everything before it:
 // only its partials have to be waited for (pdl_wait before the merges).
-template <int D, int KB, int VB, int G>
+// PAIR: at most two query heads per kv head.
+template <int D, int KB, int VB, int G, bool PAIR>
 __global__ void __launch_bounds__(kThreads, 1)
 decode_stream_kvarn_kernel(Geom g, const __nv_bfloat16* __restrict__ q, float scale,
                            float inv_sqrt_d, int* err, __nv_bfloat16* __restrict__ out, int ns) {
+  static_assert(KB == 4 && VB == 2, "the code layouts below");
   using C = KCfg<D, KB, VB, G>;
   constexpr int NG32 = C::NG32, NGG = C::NGG, MT = C::MT;
+  constexpr int CPL = G / 8;                         // channels of a group per value row (gid)
+  constexpr int GT = CPL / 2;                        // P V m-tiles per group
   extern __shared__ __align__(128) unsigned char smem[];
   pdl_trigger();
 
@@ -382,10 +405,7 @@ decode_stream_kvarn_kernel(Geom g, const __nv_bfloat16* __restrict__ q, float sc
 
   // ------------------------------------------------------------------ consumers
   const float c2 = scale * 1.4426950408889634f;      // scores in log2 units
-  const uint32_t kmask = KB == 4 ? 0x000F000Fu : 0x00030003u;
-  const uint32_t vmask = VB == 4 ? 0x000F000Fu : 0x00030003u;
-  const __half h1024 = __float2half(1024.f);
-  const __half2 bias2 = __halves2half2(h1024, h1024);
+  constexpr uint32_t kmask = 0x000F000Fu;
   const uint32_t a128[4] = {kMagic, kMagic, kMagic, kMagic};
   const int tc = threadIdx.x;
 
@@ -406,25 +426,32 @@ decode_stream_kvarn_kernel(Geom g, const __nv_bfloat16* __restrict__ q, float sc
     const __half* vcol = reinterpret_cast<const __half*>(sp + C::VCOL + sub * D * 2);
 
     // ---------------------------------------------------------------- scores
-    float acc[NGG][2][4], bias[NGG][4];
+    // One group at a time: its G / 32 words per lane (8 codes each) of channels
+    // G gg + G / 4 tid + 8 w, then its share of the scores.
+    using GroupHalves = typename std::conditional<NGG == 4, uint2, uint32_t>::type;   // NGG fp16 of a token
+    static_assert(NGG * 2 == sizeof(GroupHalves), "a token's group metadata in one load");
+    GroupHalves ksv[4], kzv[4];
+    float S[2][4] = {};
 #pragma unroll
-    for (int gg = 0; gg < NGG; ++gg) {
-      bias[gg][0] = bias[gg][1] = bias[gg][2] = bias[gg][3] = 0.f;
-#pragma unroll
-      for (int mt = 0; mt < 2; ++mt) acc[gg][mt][0] = acc[gg][mt][1] = acc[gg][mt][2] = acc[gg][mt][3] = 0.f;
+    for (int i = 0; i < 4; ++i) {                    // tokens gid + 8 i
+      ksv[i] = *reinterpret_cast<const GroupHalves*>(ks + (gid + 8 * i) * NGG);
+      kzv[i] = *reinterpret_cast<const GroupHalves*>(kz + (gid + 8 * i) * NGG);
     }
-#pragma unroll
-    for (int gq = 0; gq < NG32; ++gq) {
-      const int gg = gq * 32 / G;
-      // q' = q_rot * c_k for head gid, channels 32 gq + 8 tid + e
-      const float4 qa = *reinterpret_cast<const float4*>(qr + gid * D + 32 * gq + 8 * tid);
-      const float4 qb4 = *reinterpret_cast<const float4*>(qr + gid * D + 32 * gq + 8 * tid + 4);
-      const uint4 cu = *reinterpret_cast<const uint4*>(kcol + 32 * gq + 8 * tid);
-      const __half* ch = reinterpret_cast<const __half*>(&cu);
+    uint32_t qh[4], ql[4];                           // q' of one word: [sb][half] high, low parts
+    auto fold = [&](int head, int unit, uint32_t (&h4)[4], uint32_t (&l4)[4]) {
+      // q' = q_rot * c_k of the word's 8 channels, as bf16 high and low parts
+      const int ch = unit * 32 / G * G + (G / 4) * tid + 8 * (unit % (G / 32));
+      const float4 qa = *reinterpret_cast<const float4*>(qr + head * D + ch);
+      const float4 qb4 = *reinterpret_cast<const float4*>(qr + head * D + ch + 4);
+      const uint4 cu = *reinterpret_cast<const uint4*>(kcol + ch);
+      const __half2* c2p = reinterpret_cast<const __half2*>(&cu);
       float x[8] = {qa.x, qa.y, qa.z, qa.w, qb4.x, qb4.y, qb4.z, qb4.w};
 #pragma unroll
-      for (int e = 0; e < 8; ++e) x[e] *= __half2float(ch[e]);
-      uint32_t qh[2][2], ql[2][2];
+      for (int e = 0; e < 4; ++e) {
+        const float2 cf = __half22float2(c2p[e]);
+        x[2 * e] *= cf.x;
+        x[2 * e + 1] *= cf.y;
+      }
 #pragma unroll
       for (int sb = 0; sb < 2; ++sb)
 #pragma unroll
@@ -432,57 +459,81 @@ decode_stream_kvarn_kernel(Geom g, const __nv_bfloat16* __restrict__ q, float sc
           const int e0 = qk_chan<KB>(sb, hf, 0), e1 = qk_chan<KB>(sb, hf, 1);
           const uint32_t hw = pack_bf16(x[e0], x[e1]);
           const float2 hv = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&hw));
-          qh[sb][hf] = hw;
-          ql[sb][hf] = pack_bf16(x[e0] - hv.x, x[e1] - hv.y);
+          h4[2 * sb + hf] = hw;
+          l4[2 * sb + hf] = pack_bf16(x[e0] - hv.x, x[e1] - hv.y);
         }
+    };
+    uint32_t sh[4], sl[4];                           // q' that this lane forms for the others
 #pragma unroll
-      for (int sb = 0; sb < 2; ++sb) {
-        mma16816(bias[gg], a128, qh[sb][0], qh[sb][1]);
-        mma16816(bias[gg], a128, ql[sb][0], ql[sb][1]);
+    for (int gg = 0; gg < NGG; ++gg) {
+      float acc[2][4] = {}, bias[4] = {};
+      uint32_t kw[4][G / 32];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {                  // rows gid + 8 i
+        const unsigned char* r = kc + (gid + 8 * i) * C::KCB + gg * (G / 2) + tid * (G / 8);
+        if constexpr (G == 64) {
+          const uint2 u = *reinterpret_cast<const uint2*>(r);
+          kw[i][0] = u.x;
+          kw[i][1] = u.y;
+        } else {
+          kw[i][0] = *reinterpret_cast<const uint32_t*>(r);
+        }
       }
 #pragma unroll
-      for (int mt = 0; mt < 2; ++mt) {
-        const unsigned char* r0 = kc + (16 * mt + gid) * C::KCB;
-        const unsigned char* r1 = r0 + 8 * C::KCB;
-        uint32_t w0, w1;
-        if (KB == 4) {
-          w0 = *reinterpret_cast<const uint32_t*>(r0 + 16 * gq + 4 * tid);
-          w1 = *reinterpret_cast<const uint32_t*>(r1 + 16 * gq + 4 * tid);
+      for (int w = 0; w < G / 32; ++w) {
+        const int unit = gg * (G / 32) + w;
+        if (PAIR) {
+          // two heads at most: the eight lanes that share a tid form two words
+          // of q' in turn (head gid % 2, word gid / 2) and pass them on; the
+          // columns beyond the group repeat the two heads and are not stored
+          constexpr int RND = NG32 < 4 ? NG32 : 4;
+          if (unit % RND == 0) fold(gid & 1, unit + (gid >> 1) % RND, sh, sl);
+          const int src = ((unit % RND) * 2 + (gid & 1)) * 4 + tid;
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            qh[i] = __shfl_sync(0xffffffffu, sh[i], src);
+            ql[i] = __shfl_sync(0xffffffffu, sl[i], src);
+          }
         } else {
-          const uint32_t v0 = *reinterpret_cast<const uint16_t*>(r0 + 8 * gq + 2 * tid);
-          const uint32_t v1 = *reinterpret_cast<const uint16_t*>(r1 + 8 * gq + 2 * tid);
-          w0 = v0 | (v0 << 14);
-          w1 = v1 | (v1 << 14);
+          fold(gid, unit, qh, ql);
         }
 #pragma unroll
         for (int sb = 0; sb < 2; ++sb) {
-          uint32_t a[4];
-          a[0] = magic2(w0 >> (8 * sb), kmask);
-          a[1] = magic2(w1 >> (8 * sb), kmask);
-          a[2] = magic2(w0 >> (8 * sb + 4), kmask);
-          a[3] = magic2(w1 >> (8 * sb + 4), kmask);
-          mma16816(acc[gg][mt], a, qh[sb][0], qh[sb][1]);
-          mma16816(acc[gg][mt], a, ql[sb][0], ql[sb][1]);
+          uint32_t a[2][4];
+#pragma unroll
+          for (int mt = 0; mt < 2; ++mt) {
+            const uint32_t w0 = kw[2 * mt][w], w1 = kw[2 * mt + 1][w];
+            a[mt][0] = magic2(w0 >> (8 * sb), kmask);
+            a[mt][1] = magic2(w1 >> (8 * sb), kmask);
+            a[mt][2] = magic2(w0 >> (8 * sb + 4), kmask);
+            a[mt][3] = magic2(w1 >> (8 * sb + 4), kmask);
+          }
+          // (in an order that keeps MMAs on one accumulator apart)
+          mma_bf16(bias, a128, qh[2 * sb], qh[2 * sb + 1]);
+          mma_bf16(acc[0], a[0], qh[2 * sb], qh[2 * sb + 1]);
+          mma_bf16(acc[1], a[1], qh[2 * sb], qh[2 * sb + 1]);
+          mma_bf16(bias, a128, ql[2 * sb], ql[2 * sb + 1]);
+          mma_bf16(acc[0], a[0], ql[2 * sb], ql[2 * sb + 1]);
+          mma_bf16(acc[1], a[1], ql[2 * sb], ql[2 * sb + 1]);
         }
+      }
+      const float bz0 = bias[0] * (1.f / 128.f), bz1 = bias[1] * (1.f / 128.f);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const float sc = __half2float(reinterpret_cast<const __half*>(&ksv[i])[gg]);
+        const float mz = __half2float(reinterpret_cast<const __half*>(&kzv[i])[gg]);
+        float* Si = &S[i >> 1][2 * (i & 1)];
+        const float* ai = &acc[i >> 1][2 * (i & 1)];
+        Si[0] += sc * (ai[0] - bias[0]) + mz * bz0;
+        Si[1] += sc * (ai[1] - bias[1]) + mz * bz1;
       }
     }
-    float S[2][4];
 #pragma unroll
-    for (int mt = 0; mt < 2; ++mt)
-#pragma unroll
-      for (int r = 0; r < 2; ++r) {
-        const int t = 16 * mt + gid + 8 * r;
-        float s0 = 0.f, s1 = 0.f;
-#pragma unroll
-        for (int gg = 0; gg < NGG; ++gg) {
-          const float sc = __half2float(ks[t * NGG + gg]), mz = __half2float(kz[t * NGG + gg]);
-          s0 += sc * (acc[gg][mt][2 * r] - bias[gg][0]) + mz * bias[gg][0] * (1.f / 128.f);
-          s1 += sc * (acc[gg][mt][2 * r + 1] - bias[gg][1]) + mz * bias[gg][1] * (1.f / 128.f);
-        }
-        const float rt = __half2float(kr[t]);
-        S[mt][2 * r] = rt * s0;
-        S[mt][2 * r + 1] = rt * s1;
-      }
+    for (int i = 0; i < 4; ++i) {
+      const float rt = __half2float(kr[gid + 8 * i]);
+      S[i >> 1][2 * (i & 1)] *= rt;
+      S[i >> 1][2 * (i & 1) + 1] *= rt;
+    }
 
     // --------------------------------------------------------------- softmax
     float mx[2];
@@ -522,80 +573,76 @@ decode_stream_kvarn_kernel(Geom g, const __nv_bfloat16* __restrict__ q, float sc
     }
 
     // ------------------------------------------------------------------- P V
+    // Value codes are read in place: bits 2 j, 2 j + 1 of a half word, masked,
+    // are the code times 2^(2 j) as a subnormal fp16 (times 2^-24), exact in the
+    // product; 2^(24 - 2 j) and the column scale are applied once per block in fp32.
     float offb[4] = {0.f, 0.f, 0.f, 0.f};            // sum_t p r_t m_tg, rows = groups
+    uint32_t bq[NGG][2][2];                          // B = P (r_t s_tg) per group
 #pragma unroll
     for (int mt = 0; mt < 2; ++mt) {
-      int tk[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) tk[i] = 16 * mt + 2 * tid + (i & 1) + 8 * (i >> 1);
-      const uint32_t vr01 = (uint32_t)vr[tk[0]] | ((uint32_t)vr[tk[1]] << 16);
-      const uint32_t vr89 = (uint32_t)vr[tk[2]] | ((uint32_t)vr[tk[3]] << 16);
+      const int t0 = 16 * mt + 2 * tid;              // tokens t0, t0 + 1 and t0 + 8, t0 + 9
+      const uint32_t vr01 = *reinterpret_cast<const uint32_t*>(vr + t0);
+      const uint32_t vr89 = *reinterpret_cast<const uint32_t*>(vr + t0 + 8);
       uint32_t a_off[4] = {0u, 0u, 0u, 0u};
       if (gid < NGG) {
-        const uint16_t* vzh = reinterpret_cast<const uint16_t*>(vz);
-        const uint32_t z01 = (uint32_t)vzh[tk[0] * NGG + gid] | ((uint32_t)vzh[tk[1] * NGG + gid] << 16);
-        const uint32_t z89 = (uint32_t)vzh[tk[2] * NGG + gid] | ((uint32_t)vzh[tk[3] * NGG + gid] << 16);
-        a_off[0] = hmul2u(vr01, z01);
-        a_off[2] = hmul2u(vr89, z89);
+        const uint16_t* vzh = reinterpret_cast<const uint16_t*>(vz) + t0 * NGG + gid;
+        a_off[0] = hmul2u(vr01, (uint32_t)vzh[0] | ((uint32_t)vzh[NGG] << 16));
+        a_off[2] = hmul2u(vr89, (uint32_t)vzh[8 * NGG] | ((uint32_t)vzh[9 * NGG] << 16));
       }
-      mma16816_f16(offb, a_off, pb[mt][0], pb[mt][1]);
-      uint32_t bq[NGG][2];                           // B = P (r_t s_tg) per group
+      mma_f16(offb, a_off, pb[mt][0], pb[mt][1]);
+      const uint16_t* vsh = reinterpret_cast<const uint16_t*>(vs) + t0 * NGG;
+      GroupHalves sv[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+        sv[i] = *reinterpret_cast<const GroupHalves*>(vsh + ((i & 1) + 8 * (i >> 1)) * NGG);
 #pragma unroll
       for (int gg = 0; gg < NGG; ++gg) {
-        const uint16_t* vsh = reinterpret_cast<const uint16_t*>(vs);
-        const uint32_t s01 = (uint32_t)vsh[tk[0] * NGG + gg] | ((uint32_t)vsh[tk[1] * NGG + gg] << 16);
-        const uint32_t s89 = (uint32_t)vsh[tk[2] * NGG + gg] | ((uint32_t)vsh[tk[3] * NGG + gg] << 16);
-        bq[gg][0] = hmul2u(pb[mt][0], hmul2u(vr01, s01));
-        bq[gg][1] = hmul2u(pb[mt][1], hmul2u(vr89, s89));
-      }
-#pragma unroll
-      for (int gq = 0; gq < NG32; ++gq) {
-        const int gg = gq * 32 / G;
-        uint32_t x01, x89;
-        if (VB == 4) {
-          x01 = (uint32_t)*reinterpret_cast<const uint16_t*>(vc + tk[0] * C::VCB + 16 * gq + 2 * gid) |
-                ((uint32_t)*reinterpret_cast<const uint16_t*>(vc + tk[1] * C::VCB + 16 * gq + 2 * gid) << 16);
-          x89 = (uint32_t)*reinterpret_cast<const uint16_t*>(vc + tk[2] * C::VCB + 16 * gq + 2 * gid) |
-                ((uint32_t)*reinterpret_cast<const uint16_t*>(vc + tk[3] * C::VCB + 16 * gq + 2 * gid) << 16);
-        } else {
-          x01 = (uint32_t)vc[tk[0] * C::VCB + 8 * gq + gid] | ((uint32_t)vc[tk[1] * C::VCB + 8 * gq + gid] << 16);
-          x89 = (uint32_t)vc[tk[2] * C::VCB + 8 * gq + gid] | ((uint32_t)vc[tk[3] * C::VCB + 8 * gq + gid] << 16);
-        }
-        // column scales of rows 32 gq + 4 gid + j, each as a (c, c) pair
-        const uint2 cw = *reinterpret_cast<const uint2*>(vcol + 32 * gq + 4 * gid);
-        const uint32_t cd[4] = {__byte_perm(cw.x, 0, 0x1010), __byte_perm(cw.x, 0, 0x3232),
-                                __byte_perm(cw.y, 0, 0x1010), __byte_perm(cw.y, 0, 0x3232)};
-        constexpr int SH = VB == 4 ? 4 : 2;
-#pragma unroll
-        for (int u = 0; u < 2; ++u) {
-          uint32_t a[4];
-#pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            const uint32_t xx = (k & 2) ? x89 : x01;
-            const uint32_t mg16 = magic2h(xx >> (2 * SH * u + (k & 1) * SH), vmask);
-            __half2 cv2 = __hsub2(*reinterpret_cast<const __half2*>(&mg16), bias2);   // exact codes
-            const uint32_t c = *reinterpret_cast<const uint32_t*>(&cv2);
-            a[k] = hmul2u(c, cd[2 * u + (k & 1)]);
-          }
-          mma16816_f16(o[2 * gq + u], a, bq[gg][0], bq[gg][1]);
-        }
+        const uint32_t sel = gg & 1 ? 0x7632 : 0x5410;
+        const uint32_t s01 = __byte_perm(reinterpret_cast<const uint32_t*>(&sv[0])[gg >> 1],
+                                         reinterpret_cast<const uint32_t*>(&sv[1])[gg >> 1], sel);
+        const uint32_t s89 = __byte_perm(reinterpret_cast<const uint32_t*>(&sv[2])[gg >> 1],
+                                         reinterpret_cast<const uint32_t*>(&sv[3])[gg >> 1], sel);
+        bq[gg][mt][0] = hmul2u(pb[mt][0], hmul2u(vr01, s01));
+        bq[gg][mt][1] = hmul2u(pb[mt][1], hmul2u(vr89, s89));
       }
     }
-    // the block's offsets, scaled by the column scale of each output channel
 #pragma unroll
-    for (int gq = 0; gq < NG32; ++gq) {
-      const int gg = gq * 32 / G;
+    for (int gg = 0; gg < NGG; ++gg) {
+      float blk[GT][4] = {};                         // tile i: channels G gg + CPL gid + 2 i, + 1
+#pragma unroll
+      for (int mt = 0; mt < 2; ++mt) {
+        // the lane's CPL channels of four tokens
+        const unsigned char* v0 = vc + (16 * mt + 2 * tid) * C::VCB + gg * (G / 4) + gid * (CPL / 4);
+        uint32_t x[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const unsigned char* vp = v0 + ((i & 1) + 8 * (i >> 1)) * C::VCB;
+          x[i] = CPL == 8 ? *reinterpret_cast<const uint16_t*>(vp) : *vp;
+        }
+        uint32_t x01 = x[0] | (x[1] << 16), x89 = x[2] | (x[3] << 16);
+#pragma unroll
+        for (int i = 0; i < GT; ++i) {
+          if (i == 2) {                              // the upper byte of each half word
+            x01 >>= 8;
+            x89 >>= 8;
+          }
+          const uint32_t m0 = 0x00030003u << (4 * (i & 1)), m1 = m0 << 2;
+          const uint32_t a[4] = {x01 & m0, x01 & m1, x89 & m0, x89 & m1};
+          mma_f16(blk[i], a, bq[gg][mt][0], bq[gg][mt][1]);
+        }
+      }
       const float f0 = __shfl_sync(0xffffffffu, offb[0], 4 * gg + tid);
       const float f1 = __shfl_sync(0xffffffffu, offb[1], 4 * gg + tid);
-      const uint2 cw = *reinterpret_cast<const uint2*>(vcol + 32 * gq + 4 * gid);
-      const __half* cc = reinterpret_cast<const __half*>(&cw);
+      const __half2* cc = reinterpret_cast<const __half2*>(vcol + G * gg + CPL * gid);
 #pragma unroll
-      for (int u = 0; u < 2; ++u) {
-        const float ca = __half2float(cc[2 * u]), cb = __half2float(cc[2 * u + 1]);
-        o[2 * gq + u][0] += ca * f0;
-        o[2 * gq + u][1] += ca * f1;
-        o[2 * gq + u][2] += cb * f0;
-        o[2 * gq + u][3] += cb * f1;
+      for (int i = 0; i < GT; ++i) {
+        const float2 c = __half22float2(cc[i]);
+        const float e0 = (float)(1 << (24 - 4 * (i & 1))), e1 = e0 * 0.25f;
+        float* oi = o[GT * gg + i];
+        oi[0] = fmaf(c.x, fmaf(blk[i][0], e0, f0), oi[0]);
+        oi[1] = fmaf(c.x, fmaf(blk[i][1], e0, f1), oi[1]);
+        oi[2] = fmaf(c.y, fmaf(blk[i][2], e1, f0), oi[2]);
+        oi[3] = fmaf(c.y, fmaf(blk[i][3], e1, f1), oi[3]);
       }
     }
   };
@@ -668,7 +715,7 @@ decode_stream_kvarn_kernel(Geom g, const __nv_bfloat16* __restrict__ q, float sc
       float* ws = slot + warp * PW;
 #pragma unroll
       for (int i = 0; i < MT; ++i) {
-        const int d0 = 32 * (i >> 1) + 4 * gid + 2 * (i & 1);
+        const int d0 = G * (i / GT) + CPL * gid + 2 * (i % GT);
 #pragma unroll
         for (int r = 0; r < 4; ++r) {
           const int h = 2 * tid + (r & 1);
@@ -782,7 +829,8 @@ cudaError_t launch_t(const Geom& g, const void* q, float scale, int* err, void* 
              reinterpret_cast<const __nv_bfloat16*>(q), scale);
   int ns = 0;
   const size_t sm = stream_smem<D, KB, VB, G>(grp, &ns);
-  auto kern = decode_stream_kvarn_kernel<D, KB, VB, G>;
+  auto kern = grp <= 2 ? decode_stream_kvarn_kernel<D, KB, VB, G, true>
+                       : decode_stream_kvarn_kernel<D, KB, VB, G, false>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   if (e != cudaSuccess) return e;
   launch_pdl(kern, dim3(decode_stream_ctas(g)), dim3(kThreads), sm, s, g,
