@@ -13,8 +13,8 @@
 //     tiles: K as a bf16 high part (the fp32 value truncated) plus the bf16
 //     of the remainder (about 16 significant bits: large logits need more
 //     than bf16's 8), V as fp16 computed in packed half2 arithmetic
-//     (code x scale + offset, one rounding), into double-buffered shared
-//     tiles in the 128-byte-swizzled K-major layout of the MMA descriptors
+//     (code x scale + offset, one rounding), into two to four shared
+//     tile buffers in the 128-byte-swizzled K-major layout of the MMA descriptors
 //     (V transposed: D rows, tokens along K);
 //   issuer (warp 12, one thread): per KV tile j, first O_X += P_X V of tile
 //     j - 1 into a TMEM accumulator (128 x D fp32) per query tile X = A, B
@@ -43,13 +43,19 @@ constexpr int kM = 128;              // rows per query tile (MMA M)
 constexpr int kTok = 64;             // tokens per KV tile
 constexpr int kRowsCta = 2 * kM;     // query rows per CTA
 constexpr int kThreads = 14 * 32;    // 8 softmax, 4 producer, 1 issuer, 1 loader warp
-constexpr int kKvBufs = 2;           // reconstructed K/V tile buffers
-constexpr int kRaw = 3;              // packed-tile stages (bulk copies run up to 3 tiles ahead)
 constexpr float kRescale = 8.f;      // log2 growth of a row maximum that forces a rescale
 
 // Shared memory (bytes from a 1024-aligned base).
 template <int D, int BITS>
 struct M256Layout {
+  // Reconstructed K/V tile buffers.  A buffer is held from the start of its build to
+  // the end of its P V, about three tile times of 2 x 128 rows: with two
+  // buffers the producers waited for half of the time (D = 64: 1,360 of 2,820
+  // cycles a tile) and the tensor pipe for them.  4 x 2029 tokens of 32 heads of
+  // 64, affine 4-bit: 229 us with two, 199 with four; 2 x 8192 tokens of 32 heads
+  // of 128, KIVI 2-bit: 2081 with two, 1745 with three (four do not fit, nor do
+  // three with 4-bit codes).
+  static constexpr int KVB = D == 64 ? 4 : BITS == 2 ? 3 : 2;
   static constexpr int QT = kM * D * 2;             // one query tile: D/64 atoms of 16 KB
   static constexpr int Q_OFF = 0;
   static constexpr int KV_OFF = 2 * QT;
@@ -66,9 +72,11 @@ struct M256Layout {
   static constexpr int RKS = 2 * kTok * CROW, RKZ = RKS + 4 * D, RVS = RKZ + 4 * D,
                        RVZ = RVS + 4 * D;
   static constexpr int RAW_B = RVZ + 4 * D;
-  static constexpr int RAW_OFF = KV_OFF + kKvBufs * KV_B;
-  static constexpr int TOTAL = RAW_OFF + kRaw * RAW_B;
+  static constexpr int RAW_OFF = KV_OFF + KVB * KV_B;
+  static constexpr int RAW = D == 128 && BITS == 2 ? 2 : 3;                 // packed-tile stages (copied ahead)
+  static constexpr int TOTAL = RAW_OFF + RAW * RAW_B;
   static constexpr int ALLOC = TOTAL + 1024;        // alignment slack
+  static_assert(ALLOC <= 226 * 1024, "one CTA's shared memory");
 };
 
 __device__ __forceinline__ void bulk_copy(void* dst, const void* src, uint32_t bytes,
@@ -328,7 +336,7 @@ attend_prefill_m256_kernel(Geom g, const __nv_bfloat16* __restrict__ q, int L, f
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem = reinterpret_cast<unsigned char*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  __shared__ uint64_t raw_full[kRaw], raw_free[kRaw], kv_full[kKvBufs], kv_free[kKvBufs],
+  __shared__ uint64_t raw_full[S::RAW], raw_free[S::RAW], kv_full[S::KVB], kv_free[S::KVB],
       s_full[2][2], p_full[2][2], s_free[2][2], done_bar;
   __shared__ uint32_t tmem_base;
   __shared__ int abort_flag;
@@ -351,11 +359,11 @@ attend_prefill_m256_kernel(Geom g, const __nv_bfloat16* __restrict__ q, int L, f
   volatile int* abort = &abort_flag;
 
   if (threadIdx.x == 0) {
-    for (int i = 0; i < kRaw; ++i) {
+    for (int i = 0; i < S::RAW; ++i) {
       mbar_init(&raw_full[i], 1);
       mbar_init(&raw_free[i], 128);
     }
-    for (int i = 0; i < kKvBufs; ++i) {
+    for (int i = 0; i < S::KVB; ++i) {
       mbar_init(&kv_full[i], 128);
       mbar_init(&kv_free[i], 1);
     }
@@ -402,8 +410,8 @@ attend_prefill_m256_kernel(Geom g, const __nv_bfloat16* __restrict__ q, int L, f
     if (lane == 0) {
       int issued = 0;
       for (int j = 0; j < ntiles; ++j) {
-        const int st = j % kRaw;
-        if (j >= kRaw && !mbar_wait_or_abort(&raw_free[st], ((j - kRaw) / kRaw) & 1, abort)) break;
+        const int st = j % S::RAW;
+        if (j >= S::RAW && !mbar_wait_or_abort(&raw_free[st], ((j - S::RAW) / S::RAW) & 1, abort)) break;
         load_raw<D, BITS, FMT>(g, b, hkv, j * kTok, smem + S::RAW_OFF + st * S::RAW_B,
                                &raw_full[st]);
         issued = j + 1;
@@ -411,17 +419,17 @@ attend_prefill_m256_kernel(Geom g, const __nv_bfloat16* __restrict__ q, int L, f
       // no copy may still be landing in shared memory when the CTA exits
       // (after a timeout the producers stop consuming): wait, bounded, for
       // the last tile issued on each stage
-      for (int t = issued > kRaw ? issued - kRaw : 0; t < issued; ++t)
-        if (!mbar_wait(&raw_full[t % kRaw], (t / kRaw) & 1)) *abort = 1;
+      for (int t = issued > S::RAW ? issued - S::RAW : 0; t < issued; ++t)
+        if (!mbar_wait(&raw_full[t % S::RAW], (t / S::RAW) & 1)) *abort = 1;
     }
   } else if (warp >= 8 && warp < 12) {
     // ---------------- producers: reconstruct K and V tiles ----------------
     const int tid = threadIdx.x - 256;
     for (int j = 0; j < ntiles; ++j) {
-      const int st = j % kRaw, kb = j % kKvBufs;
-      bool ok = mbar_wait_or_abort(&raw_full[st], (j / kRaw) & 1, abort);
-      ok = ok && (j < kKvBufs ||
-                  mbar_wait_or_abort(&kv_free[kb], ((j - kKvBufs) / kKvBufs) & 1, abort));
+      const int st = j % S::RAW, kb = j % S::KVB;
+      bool ok = mbar_wait_or_abort(&raw_full[st], (j / S::RAW) & 1, abort);
+      ok = ok && (j < S::KVB ||
+                  mbar_wait_or_abort(&kv_free[kb], ((j - S::KVB) / S::KVB) & 1, abort));
       if (!producers_all(ok)) break;
       unsigned char* kv = smem + S::KV_OFF + kb * S::KV_B;
       build_tile<D, BITS, FMT>(g, b, hkv, j * kTok, T, tq, tid, smem + S::RAW_OFF + st * S::RAW_B, kv);
@@ -450,11 +458,11 @@ attend_prefill_m256_kernel(Geom g, const __nv_bfloat16* __restrict__ q, int L, f
     while (npv[0] < ntiles || npv[1] < ntiles) {
       bool progressed = false;
       if (nqk < ntiles && nqk <= min(npv[0], npv[1]) + 1) {
-        const int kb = nqk % kKvBufs, bf = nqk & 1;
+        const int kb = nqk % S::KVB, bf = nqk & 1;
         const uint32_t fpar = (nqk >= 2) ? ((nqk - 2) >> 1) & 1 : 0;
         bool ready = false;
         if (lane == 0)
-          ready = mbar_test(&kv_full[kb], (nqk / kKvBufs) & 1) &&
+          ready = mbar_test(&kv_full[kb], (nqk / S::KVB) & 1) &&
                   (nqk < 2 || (mbar_test(&s_free[0][bf], fpar) && mbar_test(&s_free[1][bf], fpar)));
         if (__shfl_sync(0xffffffffu, ready, 0)) {
           tc_fence_after();
@@ -487,7 +495,7 @@ attend_prefill_m256_kernel(Geom g, const __nv_bfloat16* __restrict__ q, int L, f
         if (lane == 0) ready = mbar_test(&p_full[x][bf], (j >> 1) & 1);
         if (!__shfl_sync(0xffffffffu, ready, 0)) continue;
         tc_fence_after();
-        const int kb = j % kKvBufs;
+        const int kb = j % S::KVB;
         if (leader) {
           const uint32_t tp = tmem + x * 128 + bf * kTok;   // P (fp16 pairs) over S's columns
           const uint32_t to = tmem + 256 + x * D;
