@@ -3,23 +3,34 @@
 // adapter kept as an explicit rank-r branch (Section 3.4):
 //   y = x W_p^T + (alpha/r) (x A_p^T) B_p^T,   then RoPE on q and k.
 //
-// One CTA computes a 128 x BN tile of y inside one projection p (BN holds
-// whole heads).  Thread 0 streams K-slices of x, W and A_p with TMA
-// (128-byte swizzle) through a kStages-deep mbarrier ring; thread 32 issues
-// tcgen05.mma: x W^T accumulates in TMEM columns [0, BN), x A_p^T in columns
-// [BN, BN + RP).  Afterwards the 128 threads (one per row / TMEM lane) read
-// x A_p^T, scale it by alpha/r, round it to bf16 and write it to shared
-// memory as an MMA operand; one more MMA pass adds (alpha/r)(x A_p^T) B_p^T
+// A cluster of two CTAs computes a 256 x BN tile of y inside one projection p
+// (BN holds whole heads) as one pair (cta_group::2): each CTA keeps its own 128
+// rows of x, the accumulator rows that go with them and one half of the BN
+// rows of W.  One warp of each CTA streams its K-slices of x, W and A_p with
+// TMA (128-byte swizzle) through a kStages-deep ring whose full barriers sit in
+// the first CTA; one warp of that CTA issues tcgen05.mma for the pair: x W^T
+// accumulates in TMEM columns [0, BN), x A_p^T in columns [BN, BN + rank).
+// Afterwards the epilogue threads (one per row / TMEM lane, the columns in two
+// halves) read x A_p^T, scale it by alpha/r, round it to bf16 and write it to
+// shared memory as an MMA operand; one more MMA pass adds (alpha/r)(x A_p^T) B_p^T
 // into the main accumulator.  The epilogue reads the tile from TMEM, applies
-// rotate-half RoPE and stores head-major [B, H, L, D].  Every mbarrier wait is
-// bounded; a timeout sets the library's error word and the CTA still frees
-// its TMEM.
+// rotate-half RoPE and stores head-major [B, H, L, D].
+// What bounds it: for a 256 x 256 tile of K = 4096 the main loop took 31.8 us with
+// and without pairing while the issuing thread formed the shared-memory
+// descriptors of every MMA; 23.5 us with descriptors formed once and constants
+// added (19.2 without the x A_p^T MMAs of 16 columns, which cost the pipe as
+// much as wider ones).  Each tile then waits for its epilogue: 5.7 us, 3.9 with
+// the sines and cosines formed during the main loop.  8192 x 4096 -> 6144 with
+// rank 16: 439 us before, 359 here (1,160 TFLOP/s).
+// Every mbarrier wait is bounded; a timeout sets the library's error word and
+// the CTA still frees its TMEM.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 #include <math.h>
 #include <string.h>
 
 #include <mutex>
+#include <type_traits>
 
 #include "kvq_internal.cuh"
 #include "quant_common.cuh"
@@ -34,10 +45,70 @@ namespace {
 
 constexpr int BM = 128;
 constexpr int BK = 64;              // bf16 elements per 128-byte swizzle row
-constexpr int kStages = 3;
-constexpr int kThreads = 128;      // + 256 dequantising threads over an NF4 base
-constexpr int kDqWarps = 8;
+constexpr int kStages = 5;
+constexpr int kEpiWarps = 8;       // 2 threads per row of the epilogue
+// the warps that issue the loads and the MMAs: two more than the epilogue's, or
+// two of them where dequantising warps (from kDqWarp0 on, the epilogue's second
+// half among them) need the registers
+template <bool NF4> constexpr int kTmaWarp = NF4 ? 0 : kEpiWarps;
+template <bool NF4> constexpr int kMmaWarp = NF4 ? 1 : kEpiWarps + 1;
+constexpr int kDqWarp0 = 4;
 using namespace tc;
+
+// ---- the CTA pair (cluster of two) ----
+__device__ __forceinline__ uint32_t cluster_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+// Address in CTA `rank` of the cluster of this CTA's shared variable p.
+__device__ __forceinline__ uint32_t mapa(const void* p, uint32_t rank) {
+  uint32_t a;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(p)), "r"(rank));
+  return a;
+}
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release;\n barrier.cluster.wait.acquire;" ::: "memory");
+}
+// TMA load into this CTA that signals a barrier of either CTA of the pair.
+__device__ __forceinline__ void tma_load_2d_pair(void* dst, const CUtensorMap* map, int c0, int c1,
+                                                 uint32_t bar) {
+  asm volatile(
+      "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.cta_group::2"
+      " [%0], [%1, {%2, %3}], [%4];"
+      ::"r"(smem_u32(dst)), "l"(map), "r"(c0), "r"(c1), "r"(bar) : "memory");
+}
+__device__ __forceinline__ void umma_pair(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc,
+                                          uint32_t idesc, uint32_t accumulate) {
+  asm volatile(
+      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+      " tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n}\n"
+      ::"r"(tmem_d), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate));
+}
+// Arrival on the barrier at this offset in both CTAs once the pair's MMAs issued
+// so far have completed.
+__device__ __forceinline__ void umma_commit_pair(uint64_t* bar) {
+  asm volatile(
+      "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64"
+      " [%0], %1;"
+      ::"r"(smem_u32(bar)), "h"((uint16_t)3) : "memory");
+}
+__device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar) {
+  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+// mbar_wait that also acquires what the other CTA released by its arrivals.
+__device__ __forceinline__ bool mbar_wait_cluster(uint64_t* bar, uint32_t parity) {
+  const uint64_t t0 = global_ns();
+  for (long i = 0;; ++i) {
+    uint32_t ok;
+    asm volatile(
+        "{\n .reg .pred p;\n mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n"
+        " selp.u32 %0, 1, 0, p;\n}\n"
+        : "=r"(ok) : "r"(smem_u32(bar)), "r"(parity) : "memory");
+    if (ok) return true;
+    if ((i & 7) == 7 && global_ns() - t0 > kWaitNs) return false;
+  }
+}
 
 // The 16 NF4 levels, code 0 .. 15, as QLoRA publishes the data type.
 __constant__ float c_nf4_lv[16] = {
@@ -133,27 +204,31 @@ __device__ __forceinline__ void code_pair(const Geom& g, int which, int b, int h
 template <int BN>
 struct Smem {
   static constexpr int A_B = BM * BK * 2;            // 16 KB
-  static constexpr int B_B = BN * BK * 2;            // up to 32 KB
-  static constexpr int LA_B = 64 * BK * 2;           // LoRA A slice, up to 64 ranks (8 KB)
+  static constexpr int B_B = BN / 2 * BK * 2;        // this CTA's half of W's rows
+  static constexpr int LA_B = 32 * BK * 2;           // LoRA A slice, half of up to 64 ranks
   static constexpr int STAGE_B = A_B + B_B + LA_B;
   static constexpr int U_OFF = kStages * STAGE_B;    // (alpha/r) x A^T as bf16 operand
-  static constexpr int BP_OFF = U_OFF + BM * BK * 2; // B_p tile [BN][64 ranks]
-  static constexpr int TOTAL = BP_OFF + BN * BK * 2 + 1024;   // + alignment slack
+  static constexpr int BP_OFF = U_OFF + BM * BK * 2; // B_p tile [BN / 2][64 ranks]
+  static constexpr int TOTAL = BP_OFF + BN / 2 * BK * 2 + 1024;   // + alignment slack
 };
 
-// NF4: W arrives as 4-bit NormalFloat codes; warps 4-11 (256 threads: one
-// per tile row at BN = 256, two at BN = 128) turn each 64-input K slice into
-// the bf16 tile the TMA would have landed (level x absmax in fp32, rounded
-// once), 128-byte swizzled, and signal it on w_full; the x and A_p slices
-// still come by TMA.
+// NF4: W arrives as 4-bit NormalFloat codes; BN threads from warp 4 on (two
+// per row of this CTA's half of the tile) turn each 64-input K slice into the bf16
+// tile the TMA would have landed (level x absmax in fp32, rounded once),
+// 128-byte swizzled, and signal it on the first CTA's w_full; the x and A_p
+// slices still come by TMA.
 template <int BN, bool NF4>
-__global__ void __launch_bounds__(NF4 ? kThreads + 32 * kDqWarps : kThreads, 1)
+__host__ __device__ constexpr int tc_threads() {
+  return !NF4 ? (kEpiWarps + 2) * 32 : kDqWarp0 * 32 + BN > kEpiWarps * 32 ? kDqWarp0 * 32 + BN : kEpiWarps * 32;
+}
+template <int BN, bool NF4>
+__global__ void __launch_bounds__(tc_threads<BN, NF4>(), 1)
 project_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_w,
                   const __grid_constant__ CUtensorMap tm_a0, const __grid_constant__ CUtensorMap tm_a1,
                   const __grid_constant__ CUtensorMap tm_a2, const __grid_constant__ CUtensorMap tm_b0,
                   const __grid_constant__ CUtensorMap tm_b1, const __grid_constant__ CUtensorMap tm_b2,
                   const TcArgs args) {
-  static_assert(!NF4 || BN == 128 || BN == 256, "256 dequantising threads cover the tile's rows");
+  constexpr int kDqWarps = BN / 32;
   pdl_wait();
   pdl_trigger();
   using S = Smem<BN>;
@@ -164,14 +239,17 @@ project_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
   __shared__ uint64_t u_bar, bp_bar, acc_bar;
   __shared__ float nf4_lv[16];
   __shared__ uint32_t tmem_base;
-  __shared__ int fail;
+  __shared__ int fail, peer_fail;
 
   bool app_ok = true;                    // appending: the cache has room for the L tokens
   const int T0 = args.pack ? append_begin(args.g, args.L, &app_ok) : 0;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int n0 = blockIdx.x * BN, m0 = blockIdx.y * BM;
+  const uint32_t rank = cluster_rank();  // 0 issues the MMAs
+  const int pair = blockIdx.x >> 1, ntiles = args.n_off[3] / BN;   // column tiles first
+  const int n0 = pair % ntiles * BN, m0 = (pair / ntiles * 2 + (int)rank) * BM;
   const int proj = n0 < args.n_off[1] ? 0 : n0 < args.n_off[2] ? 1 : 2;
   const int r = args.r[proj], rp = args.rp[proj];
+  const int rp32 = (rp + 31) / 32 * 32;  // x A_p^T columns of the pair's MMA (zeros beyond the rank)
   const CUtensorMap* tm_a = proj == 0 ? &tm_a0 : proj == 1 ? &tm_a1 : &tm_a2;
   const CUtensorMap* tm_b = proj == 0 ? &tm_b0 : proj == 1 ? &tm_b1 : &tm_b2;
 
@@ -179,32 +257,35 @@ project_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
     for (int i = 0; i < kStages; ++i) {
       mbar_init(&full_bar[i], 1);
       mbar_init(&empty_bar[i], 1);
-      mbar_init(&w_full[i], kDqWarps);     // NF4: one arrival per dequantising warp
+      mbar_init(&w_full[i], 2 * kDqWarps); // NF4: one arrival per dequantising warp of the pair
     }
     mbar_init(&u_bar, 1);
     mbar_init(&bp_bar, 1);
     mbar_init(&acc_bar, 1);
-    fail = 0;
+    fail = peer_fail = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (NF4 && threadIdx.x < 16) nf4_lv[threadIdx.x] = c_nf4_lv[threadIdx.x];
-  if (warp == 1) {   // TMEM: 512 columns (main BN + LoRA <= 64)
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;"
+  if (warp == kMmaWarp<NF4>) {   // TMEM: 512 columns (main BN + LoRA <= 64)
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], 512;"
                  ::"r"(smem_u32(&tmem_base)));
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;");
   }
   tc_fence_before();
   __syncthreads();
+  cluster_sync();                        // both CTAs' barriers and TMEM exist
   tc_fence_after();
   const uint32_t tmem = tmem_base;
   const uint32_t tmem_u = tmem + BN;
   const int KB = args.k_blocks;
 
-  if (threadIdx.x == 0) {
+  if (threadIdx.x == kTmaWarp<NF4> * 32) {
     // ---------------- TMA producer ----------------
+    // (the first CTA's barriers expect both CTAs' bytes)
+    const int nh = n0 + (int)rank * (BN / 2);          // this CTA's rows of W and B_p
     if (r > 0) {
-      mbar_expect_tx(&bp_bar, BN * BK * 2);
-      tma_load_2d(smem + S::BP_OFF, tm_b, 0, n0 - args.n_off[proj], &bp_bar);
+      if (rank == 0) mbar_expect_tx(&bp_bar, 2 * (BN / 2) * BK * 2);
+      tma_load_2d_pair(smem + S::BP_OFF, tm_b, 0, nh - args.n_off[proj], mapa(&bp_bar, 0));
     }
     for (int kb = 0; kb < KB; ++kb) {
       const int s = kb % kStages;
@@ -213,52 +294,70 @@ project_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
         break;
       }
       unsigned char* st = smem + s * S::STAGE_B;
-      mbar_expect_tx(&full_bar[s], S::A_B + (NF4 ? 0 : S::B_B) + (r > 0 ? rp * BK * 2 : 0));
-      tma_load_2d(st, &tm_x, kb * BK, m0, &full_bar[s]);
+      if (rank == 0)
+        mbar_expect_tx(&full_bar[s], 2 * (S::A_B + (NF4 ? 0 : S::B_B)) + (r > 0 ? rp32 * BK * 2 : 0));
+      const uint32_t fb = mapa(&full_bar[s], 0);
+      tma_load_2d_pair(st, &tm_x, kb * BK, m0, fb);
       if (!NF4)
-        tma_load_2d(st + S::A_B, &tm_w, (args.kb_wrap ? kb % args.kb_wrap : kb) * BK, n0,
-                    &full_bar[s]);
-      if (r > 0) tma_load_2d(st + S::A_B + S::B_B, tm_a, kb * BK, 0, &full_bar[s]);
+        tma_load_2d_pair(st + S::A_B, &tm_w, (args.kb_wrap ? kb % args.kb_wrap : kb) * BK, nh, fb);
+      if (r > 0) tma_load_2d_pair(st + S::A_B + S::B_B, tm_a, kb * BK, (int)rank * (rp32 / 2), fb);
     }
-  } else if (threadIdx.x == 32) {
+  } else if (warp == kMmaWarp<NF4> && rank == 0) {
     // ---------------- MMA issuer ----------------
-    constexpr uint32_t id_main = idesc_bf16(BM, BN);
-    const uint32_t id_u = idesc_bf16(BM, rp > 0 ? rp : 16);
+    // The whole warp runs the loop (its values stay warp-uniform) and one elected
+    // lane issues.  Descriptors are formed once; a stage and a K step of 16
+    // elements (32 bytes) advance their start address, in 16-byte units.
+    constexpr uint32_t id_main = idesc_bf16(2 * BM, BN);
+    const uint32_t id_u = idesc_bf16(2 * BM, rp32 > 0 ? rp32 : 32);
+    const uint64_t desc0 = sw128_desc(smem);
+    const bool leader = elect_one();
     bool ok = true;
+    int s = 0, phase = 0;
     for (int kb = 0; kb < KB; ++kb) {
-      const int s = kb % kStages;
-      if (!mbar_wait(&full_bar[s], (kb / kStages) & 1) ||
-          (NF4 && !mbar_wait(&w_full[s], (kb / kStages) & 1))) {
+      bool ready = mbar_wait_cluster(&full_bar[s], phase);
+      if (NF4) ready = ready && mbar_wait_cluster(&w_full[s], phase);
+      if (!__all_sync(0xffffffffu, ready)) {
         ok = false;
         break;
       }
       tc_fence_after();
-      unsigned char* st = smem + s * S::STAGE_B;
+      if (leader) {
+        const uint64_t ad = desc0 + (uint64_t)(s * (S::STAGE_B >> 4));
 #pragma unroll
-      for (int kk = 0; kk < BK / 16; ++kk) {
-        const uint64_t ad = sw128_desc(st + kk * 32);
-        umma(tmem, ad, sw128_desc(st + S::A_B + kk * 32), id_main, (kb | kk) != 0);
-        if (r > 0) umma(tmem_u, ad, sw128_desc(st + S::A_B + S::B_B + kk * 32), id_u, (kb | kk) != 0);
+        for (int kk = 0; kk < BK / 16; ++kk)
+          umma_pair(tmem, ad + 2 * kk, ad + (S::A_B >> 4) + 2 * kk, id_main, (kb | kk) != 0);
+        if (r > 0)
+#pragma unroll
+          for (int kk = 0; kk < BK / 16; ++kk)
+            umma_pair(tmem_u, ad + 2 * kk, ad + ((S::A_B + S::B_B) >> 4) + 2 * kk, id_u, (kb | kk) != 0);
+        umma_commit_pair(&empty_bar[s]);   // frees the stage in both CTAs when these MMAs finish
       }
-      umma_commit(&empty_bar[s]);          // frees the stage when these MMAs finish
+      __syncwarp();
+      if (++s == kStages) {
+        s = 0;
+        phase ^= 1;
+      }
     }
-    if (!ok) atomicOr(&fail, 1);
-    umma_commit(&u_bar);                   // all main-loop MMAs done
-  } else if (NF4 && warp >= 4) {
-    // ---------- NF4 dequantisation: TPR threads per tile row ----------
-    constexpr int TPR = 32 * kDqWarps / BN;               // 1 (BN = 256) or 2 (BN = 128)
+    if (leader) {
+      if (!ok) atomicOr(&fail, 1);
+      umma_commit_pair(&u_bar);            // all main-loop MMAs done
+    }
+  } else if (NF4 && warp >= kDqWarp0 && warp < kDqWarp0 + kDqWarps) {
+    // ---------- NF4 dequantisation: two threads per row of this CTA's half ----------
+    constexpr int TPR = 2;
     constexpr int NQ = 2 / TPR;                           // 16-byte code words per thread and slice
-    const int dt = threadIdx.x - kThreads;                // 0 .. 255
+    const int dt = threadIdx.x - kDqWarp0 * 32;               // 0 .. BN - 1
     const int n = dt / TPR, h = dt % TPR;                 // row, part of the slice
-    const int nkb = args.k_blocks;
-    const uint8_t* crow = args.nf4_codes + (int64_t)(n0 + n) * (nkb * 32) + h * 16;
-    const float* arow = args.nf4_absmax + (int64_t)(n0 + n) * nkb;
-    // codes and absmax of this and the next two K slices in registers
-    // (rotated each slice, so no array is indexed at run time)
-    uint4 cq[3][NQ];
-    float am[3];
+    const int nkb = args.k_blocks, nrow = n0 + (int)rank * (BN / 2) + n;
+    const uint8_t* crow = args.nf4_codes + (int64_t)nrow * (nkb * 32) + h * 16;
+    const float* arow = args.nf4_absmax + (int64_t)nrow * nkb;
+    // codes and absmax of this and the next PF K slices in registers (rotated
+    // each slice, so no array is indexed at run time)
+    constexpr int PF = 2;
+    uint4 cq[PF + 1][NQ];
+    float am[PF + 1];
 #pragma unroll
-    for (int i = 0; i < 3; ++i) {
+    for (int i = 0; i <= PF; ++i) {
 #pragma unroll
       for (int q = 0; q < NQ; ++q) cq[i][q] = make_uint4(0, 0, 0, 0);
       am[i] = 0.f;
@@ -270,12 +369,12 @@ project_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
         xa = __ldg(arow + kb);
       }
     };
-    fetch(0, cq[0], am[0]);
-    fetch(1, cq[1], am[1]);
+#pragma unroll
+    for (int i = 0; i < PF; ++i) fetch(i, cq[i], am[i]);
     const int rsw = (n >> 3) * 1024 + (n & 7) * 128;      // the row in the swizzled tile
     for (int kb = 0; kb < KB; ++kb) {
       const int s = kb % kStages;
-      fetch(kb + 2, cq[2], am[2]);
+      fetch(kb + PF, cq[PF], am[PF]);
       if (kb >= kStages) {                                // lane 0 waits for the slot, then the warp
         bool ok = true;
         if (lane == 0) ok = mbar_wait(&empty_bar[s], ((kb / kStages) - 1) & 1);
@@ -293,12 +392,11 @@ project_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
       }
       const float a = am[0];
 #pragma unroll
-      for (int q = 0; q < NQ; ++q) {
-        cq[0][q] = cq[1][q];
-        cq[1][q] = cq[2][q];
+      for (int i = 0; i < PF; ++i) {
+#pragma unroll
+        for (int q = 0; q < NQ; ++q) cq[i][q] = cq[i + 1][q];
+        am[i] = am[i + 1];
       }
-      am[0] = am[1];
-      am[1] = am[2];
       uint64_t a2;
       asm("mov.b64 %0, {%1, %1};" : "=l"(a2) : "f"(a));
 #pragma unroll
@@ -327,17 +425,44 @@ project_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
       }
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // for the MMA's reads
       __syncwarp();
-      if (lane == 0) mbar_arrive(&w_full[s]);
+      if (lane == 0) mbar_arrive_cluster(mapa(&w_full[s], 0));
     }
   }
   // ---------------- (alpha/r) x A^T -> bf16 operand in shared memory ----------
-  const bool u_ok = __syncthreads_and(mbar_wait(&u_bar, 0)) != 0;   // uniform
+  const int row = (warp & 3) * 32 + lane;      // TMEM lane = tile row
+  const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
+  const int part = warp >> 2;                  // warps 0-3 and 4-7: every other column block
+  const int m = m0 + row;
+  const bool active = m < args.M;              // rows past M: load, do not store
+  const int mm = active ? m : 0;
+  const int b = mm / args.L, l = mm % args.L;
+  const int D = args.D, half = D / 2;
+  const bool rope = args.rope && proj < 2;
+  // A head's 32-frequency blocks go to the two parts in turn (at D = 64 its heads
+  // do); this thread's blocks: part, part + 2 (D = 256), part (D = 128), 0 (D = 64).
+  // Their sines and cosines are formed while the main loop runs (not over an NF4
+  // base, whose dequantising warps leave no registers for them).
+  auto tail = [&](auto nblocks) -> bool {
+  constexpr int NB = decltype(nblocks)::value;
+  constexpr int NC = NF4 ? 1 : NB;             // blocks whose sines and cosines are held
+  float cs[NC * 32], sn[NC * 32];
+  auto angles = [&](int k, float* c, float* s) {
+    const int pos = args.pos0 + pos_of(args.pos_dev, args.pos_stride, b) + l;
+    const int j0 = D == 64 ? 0 : 32 * (part + 2 * k);
+#pragma unroll
+    for (int i = 0; i < 32; ++i) rope_cs(pos, args.theta_hi[j0 + i], args.theta_lo[j0 + i], &c[i], &s[i]);
+  };
+  if (!NF4 && rope && part < 2) {
+#pragma unroll
+    for (int k = 0; k < NB; ++k) angles(k, cs + 32 * (k % NC), sn + 32 * (k % NC));
+  }
+  bool u_done = true;                          // one lane per warp polls: the issuer needs the slots
+  if (lane == 0) u_done = mbar_wait(&u_bar, 0);
+  const bool u_ok = __syncthreads_and(u_done) != 0;   // uniform
   tc_fence_after();
-  const int row = warp * 32 + lane;            // TMEM lane = tile row
-  const uint32_t lane_base = (uint32_t)(warp * 32) << 16;
-  if (r > 0 && u_ok && warp < 4) {
+  if (r > 0 && u_ok && part < 2) {
     unsigned char* us = smem + S::U_OFF;
-    for (int c0 = 0; c0 < rp; c0 += 16) {
+    for (int c0 = 16 * part; c0 < rp; c0 += 32) {
       float v[16];
       tmem_ld16(tmem_u + lane_base + c0, v);
       uint32_t w[8];
@@ -356,42 +481,40 @@ project_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
     // ranks rp .. 63 of the operand row are never read (the MMA uses K = rp)
   }
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  if (!u_ok && threadIdx.x == 0) atomicOr(&fail, 1);
   tc_fence_before();
   __syncthreads();
-  if (!u_ok && threadIdx.x == 0) atomicOr(&fail, 1);
-  if (threadIdx.x == 32) {
-    tc_fence_after();
-    if (r > 0 && u_ok && !fail) {
-      if (mbar_wait(&bp_bar, 0)) {
-        const uint32_t id_main = idesc_bf16(BM, BN);
+  if (threadIdx.x == 0 && *reinterpret_cast<volatile int*>(&fail))
+    asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(mapa(&peer_fail, rank ^ 1)), "r"(1) : "memory");
+  cluster_sync();                              // both operands of the up-projection are written
+  tc_fence_after();
+  const bool pair_ok = !*reinterpret_cast<volatile int*>(&fail) &&
+                       !*reinterpret_cast<volatile int*>(&peer_fail);
+  if (threadIdx.x == kMmaWarp<NF4> * 32 && rank == 0 && pair_ok) {
+    bool ok = true;
+    if (r > 0) {
+      ok = mbar_wait_cluster(&bp_bar, 0);
+      if (ok) {
+        constexpr uint32_t id_main = idesc_bf16(2 * BM, BN);
         for (int kk = 0; kk < rp / 16; ++kk)
-          umma(tmem, sw128_desc(smem + S::U_OFF + kk * 32),
-               sw128_desc(smem + S::BP_OFF + kk * 32), id_main, 1);
-      } else {
-        atomicOr(&fail, 1);
+          umma_pair(tmem, sw128_desc(smem + S::U_OFF + kk * 32),
+                    sw128_desc(smem + S::BP_OFF + kk * 32), id_main, 1);
       }
     }
-    umma_commit(&acc_bar);
+    if (ok) umma_commit_pair(&acc_bar);        // else both CTAs' waits below run out
   }
   // ---------------- epilogue: RoPE and head-major store ----------------
-  const bool acc_wait = mbar_wait(&acc_bar, 0);
-  const bool good = __syncthreads_and(acc_wait) && !*reinterpret_cast<volatile int*>(&fail);
+  const bool acc_wait = pair_ok && mbar_wait(&acc_bar, 0);
+  const bool good = __syncthreads_and(acc_wait) != 0;
   tc_fence_after();
-  const int m = m0 + row;
-  const bool active = m < args.M;                     // rows past M: load, do not store
-  if (good && warp < 4) {
-    const int D = args.D, half = D / 2;
-    const int mm = active ? m : 0;
-    const int b = mm / args.L, l = mm % args.L;
+  if (good && part < 2) {
     const int H = proj == 0 ? args.Hq : args.Hkv;
     const int col0 = n0 - args.n_off[proj];           // first column within projection
     __nv_bfloat16* out = reinterpret_cast<__nv_bfloat16*>(args.out[proj]);
-    const bool rope = args.rope && proj < 2;
-    const int pos = args.pos0 + pos_of(args.pos_dev, args.pos_stride, b) + l;
     if (args.plain_out) {
       // plain product: the accumulator row as fp32
       const int N = args.n_off[3];
-      for (int c = 0; c < BN; c += 16) {
+      for (int c = 16 * part; c < BN; c += 32) {
         float v[16];
         tmem_ld16(tmem + lane_base + c, v);
         if (!active) continue;
@@ -399,38 +522,40 @@ project_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
 #pragma unroll
         for (int i = 0; i < 4; ++i) d[i] = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
       }
-    } else if (args.pack && proj > 0) {
-      // append: k (after RoPE) and v rounded to bf16, then coded per token
-      // in groups of 32 channels straight into the cache planes
-      const Geom& gg = args.g;
-      const int bits = proj == 1 ? gg.kb : gg.vb;
-      const bool sym = gg.fmt == KVQ_FMT_SYMMETRIC;
-      const int t = T0 + l;
-      for (int hc = 0; hc < BN; hc += D) {
+      return good;
+    }
+#pragma unroll
+    for (int k = 0; k < NB; ++k) {
+      const int j = D == 64 ? 0 : 32 * (part + 2 * k);
+      if (NF4 && rope) angles(k, cs, sn);
+      for (int hc = D == 64 ? 64 * part : 0; hc < BN; hc += D == 64 ? 128 : D) {   // whole heads in the tile
         const int head = (col0 + hc) / D;
-        for (int j = 0; j < half; j += 32) {
-          float x1[32], x2[32];
+        float x1[32], x2[32];
+        uint32_t* u1 = reinterpret_cast<uint32_t*>(x1);
+        uint32_t* u2 = reinterpret_cast<uint32_t*>(x2);
+        tmem_ld16_nowait(tmem + lane_base + hc + j, u1);
+        tmem_ld16_nowait(tmem + lane_base + hc + j + 16, u1 + 16);
+        tmem_ld16_nowait(tmem + lane_base + hc + half + j, u2);
+        tmem_ld16_nowait(tmem + lane_base + hc + half + j + 16, u2 + 16);
+        tmem_wait_ld();
+        if (rope) {
 #pragma unroll
-          for (int u = 0; u < 32; u += 16) {
-            tmem_ld16(tmem + lane_base + hc + j + u, x1 + u);
-            tmem_ld16(tmem + lane_base + hc + half + j + u, x2 + u);
-            if (rope) {
-#pragma unroll
-              for (int i = 0; i < 16; ++i) {
-                float c, sn;
-                rope_cs(pos, args.theta_hi[j + u + i], args.theta_lo[j + u + i], &c, &sn);
-                rope_rot(x1[u + i], x2[u + i], c, sn);
-              }
-            }
-          }
-          if (!active || !app_ok) continue;
+          for (int i = 0; i < 32; ++i) rope_rot(x1[i], x2[i], cs[32 * (k % NC) + i], sn[32 * (k % NC) + i]);
+        }
+        if (!active) continue;
+        if (args.pack && proj > 0) {
+          // append: k (after RoPE) and v rounded to bf16, then coded per token
+          // in groups of 32 channels straight into the cache planes
+          if (!app_ok) continue;
 #pragma unroll
           for (int i = 0; i < 32; ++i) {
             x1[i] = __bfloat162float(__float2bfloat16_rn(x1[i]));
             x2[i] = __bfloat162float(__float2bfloat16_rn(x2[i]));
           }
+          const Geom& gg = args.g;
+          const int bits = proj == 1 ? gg.kb : gg.vb, t = T0 + l;
           const int g1 = j / 32, g2 = (half + j) / 32, which = proj - 1;
-          if (sym) {
+          if (gg.fmt == KVQ_FMT_SYMMETRIC) {
             if (bits == 2) code_pair<2, true>(gg, which, b, head, t, g1, g2, x1, x2);
             else if (bits == 4) code_pair<4, true>(gg, which, b, head, t, g1, g2, x1, x2);
             else code_pair<8, true>(gg, which, b, head, t, g1, g2, x1, x2);
@@ -439,48 +564,33 @@ project_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
             else if (bits == 4) code_pair<4, false>(gg, which, b, head, t, g1, g2, x1, x2);
             else code_pair<8, false>(gg, which, b, head, t, g1, g2, x1, x2);
           }
-        }
-      }
-    } else
-    for (int j = 0; j < half; j += 16) {              // 16 frequencies at a time
-      float cs[16], sn[16];
-      if (rope) {
+        } else {
+          __nv_bfloat16* orow = out + (((int64_t)b * H + head) * args.L + l) * D;
+          uint4* d1 = reinterpret_cast<uint4*>(orow + j);
+          uint4* d2 = reinterpret_cast<uint4*>(orow + half + j);
 #pragma unroll
-        for (int i = 0; i < 16; ++i)
-          rope_cs(pos, args.theta_hi[j + i], args.theta_lo[j + i], &cs[i], &sn[i]);
-      }
-      for (int hc = 0; hc < BN; hc += D) {            // whole heads in the tile
-        const int head = (col0 + hc) / D;
-        __nv_bfloat16* orow = out + (((int64_t)b * H + head) * args.L + l) * D;
-        float x1[16], x2[16];
-        tmem_ld16(tmem + lane_base + hc + j, x1);
-        tmem_ld16(tmem + lane_base + hc + half + j, x2);
-        if (rope) {
-#pragma unroll
-          for (int i = 0; i < 16; ++i) rope_rot(x1[i], x2[i], cs[i], sn[i]);
+          for (int i = 0; i < 4; ++i) {
+            d1[i] = make_uint4(pack_bf16(x1[8 * i], x1[8 * i + 1]), pack_bf16(x1[8 * i + 2], x1[8 * i + 3]),
+                               pack_bf16(x1[8 * i + 4], x1[8 * i + 5]), pack_bf16(x1[8 * i + 6], x1[8 * i + 7]));
+            d2[i] = make_uint4(pack_bf16(x2[8 * i], x2[8 * i + 1]), pack_bf16(x2[8 * i + 2], x2[8 * i + 3]),
+                               pack_bf16(x2[8 * i + 4], x2[8 * i + 5]), pack_bf16(x2[8 * i + 6], x2[8 * i + 7]));
+          }
         }
-        if (!active) continue;
-        uint32_t w1[8], w2[8];
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          w1[i] = pack_bf16(x1[2 * i], x1[2 * i + 1]);
-          w2[i] = pack_bf16(x2[2 * i], x2[2 * i + 1]);
-        }
-        uint4* d1 = reinterpret_cast<uint4*>(orow + j);
-        uint4* d2 = reinterpret_cast<uint4*>(orow + half + j);
-        d1[0] = make_uint4(w1[0], w1[1], w1[2], w1[3]);
-        d1[1] = make_uint4(w1[4], w1[5], w1[6], w1[7]);
-        d2[0] = make_uint4(w2[0], w2[1], w2[2], w2[3]);
-        d2[1] = make_uint4(w2[4], w2[5], w2[6], w2[7]);
       }
     }
   }
+  return good;
+  };
+  // (an NF4 base has heads of 64 or 128)
+  const bool good = !NF4 && D == 256 ? tail(std::integral_constant<int, NF4 ? 1 : 2>())
+                                     : tail(std::integral_constant<int, 1>());
   if (threadIdx.x == 0 && !good) atomicOr(args.err, 2);
   tc_fence_before();
   __syncthreads();
-  if (warp == 1) {
+  cluster_sync();                              // neither CTA's shared memory or TMEM is in use
+  if (warp == kMmaWarp<NF4>) {
     tc_fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem));
+    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, 512;" ::"r"(tmem));
   }
   // appending: the last CTA to arrive advances the cache's token count
   if (args.pack) quant::append_arrive_spread(args.g.state, T0, args.L, app_ok);
@@ -518,14 +628,37 @@ bool make_map(CUtensorMap* m, const void* base, uint64_t rows, uint64_t cols, ui
   return res == CUDA_SUCCESS;
 }
 
+// launch_pdl with clusters of two CTAs along x (a tcgen05 pair has to lie there).
+template <typename... KArgs, typename... Args>
+cudaError_t launch_pdl_pair(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem,
+                            cudaStream_t s, Args&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = 2;
+  attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 2;
+  return cudaLaunchKernelEx(&cfg, kern, std::forward<Args>(args)...);
+}
+
 template <int BN, bool NF4 = false>
 cudaError_t launch_bn(const CUtensorMap maps[8], const TcArgs& a, cudaStream_t s) {
   const int smem = Smem<BN>::TOTAL;
   auto kern = project_tc_kernel<BN, NF4>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
-  dim3 grid(a.n_off[3] / BN, (a.M + BM - 1) / BM);
-  launch_pdl(kern, dim3(grid), dim3(NF4 ? kThreads + 32 * kDqWarps : kThreads), smem, s, maps[0], maps[1], maps[2], maps[3], maps[4], maps[5],
+  const int64_t ctas = 2LL * (a.n_off[3] / BN) * ((a.M + 2 * BM - 1) / (2 * BM));
+  if (ctas > INT32_MAX) return cudaErrorInvalidConfiguration;
+  dim3 grid((unsigned)ctas);
+  launch_pdl_pair(kern, grid, dim3(tc_threads<BN, NF4>()), smem, s, maps[0], maps[1], maps[2], maps[3], maps[4], maps[5],
                                     maps[6], maps[7], a);
   return cudaGetLastError();
 }
@@ -576,12 +709,12 @@ static cudaError_t launch_tc(const void* x, int B, int L, int d_in, const void* 
   CUtensorMap maps[8];
   bool ok = make_map(&maps[0], x, M, d_in, BM);
   if (nf4) maps[1] = maps[0];                       // unused: any valid map
-  else ok = ok && make_map(&maps[1], w, (uint64_t)t.n_off[3], d_in, bn);
+  else ok = ok && make_map(&maps[1], w, (uint64_t)t.n_off[3], d_in, bn / 2);
   const int dout[3] = {Hq * D, Hkv * D, Hkv * D};
   for (int p = 0; p < 3 && ok; ++p) {
     if (r[p] > 0) {
-      ok = make_map(&maps[2 + p], a[p], r[p], d_in, t.rp[p]) &&
-           make_map(&maps[5 + p], bm[p], dout[p], r[p], bn);
+      ok = make_map(&maps[2 + p], a[p], r[p], d_in, (t.rp[p] + 31) / 32 * 16) &&
+           make_map(&maps[5 + p], bm[p], dout[p], r[p], bn / 2);
     } else {  // unused: any valid map
       maps[2 + p] = maps[0];
       maps[5 + p] = maps[0];
@@ -616,7 +749,7 @@ cudaError_t launch_gemm_tc_bf16(const void* a, int M, int K, const void* bt, int
   t.k_blocks = K / 64; t.kb_wrap = Kb / 64 == K / 64 ? 0 : Kb / 64; t.err = err;
   t.plain_out = c;
   CUtensorMap maps[8];
-  if (!make_map(&maps[0], a, M, K, BM) || !make_map(&maps[1], bt, N, Kb, bn))
+  if (!make_map(&maps[0], a, M, K, BM) || !make_map(&maps[1], bt, N, Kb, bn / 2))
     return cudaErrorInvalidValue;
   for (int i = 2; i < 8; ++i) maps[i] = maps[0];   // unused: no adapters
   return bn == 256 ? launch_bn<256>(maps, t, s) : launch_bn<128>(maps, t, s);
