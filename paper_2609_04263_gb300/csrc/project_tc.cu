@@ -55,61 +55,6 @@ template <bool NF4> constexpr int kMmaWarp = NF4 ? 1 : kEpiWarps + 1;
 constexpr int kDqWarp0 = 4;
 using namespace tc;
 
-// ---- the CTA pair (cluster of two) ----
-__device__ __forceinline__ uint32_t cluster_rank() {
-  uint32_t r;
-  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-  return r;
-}
-// Address in CTA `rank` of the cluster of this CTA's shared variable p.
-__device__ __forceinline__ uint32_t mapa(const void* p, uint32_t rank) {
-  uint32_t a;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(p)), "r"(rank));
-  return a;
-}
-__device__ __forceinline__ void cluster_sync() {
-  asm volatile("barrier.cluster.arrive.release;\n barrier.cluster.wait.acquire;" ::: "memory");
-}
-// TMA load into this CTA that signals a barrier of either CTA of the pair.
-__device__ __forceinline__ void tma_load_2d_pair(void* dst, const CUtensorMap* map, int c0, int c1,
-                                                 uint32_t bar) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.cta_group::2"
-      " [%0], [%1, {%2, %3}], [%4];"
-      ::"r"(smem_u32(dst)), "l"(map), "r"(c0), "r"(c1), "r"(bar) : "memory");
-}
-__device__ __forceinline__ void umma_pair(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc,
-                                          uint32_t idesc, uint32_t accumulate) {
-  asm volatile(
-      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-      " tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n}\n"
-      ::"r"(tmem_d), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate));
-}
-// Arrival on the barrier at this offset in both CTAs once the pair's MMAs issued
-// so far have completed.
-__device__ __forceinline__ void umma_commit_pair(uint64_t* bar) {
-  asm volatile(
-      "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64"
-      " [%0], %1;"
-      ::"r"(smem_u32(bar)), "h"((uint16_t)3) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar) {
-  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
-}
-// mbar_wait that also acquires what the other CTA released by its arrivals.
-__device__ __forceinline__ bool mbar_wait_cluster(uint64_t* bar, uint32_t parity) {
-  const uint64_t t0 = global_ns();
-  for (long i = 0;; ++i) {
-    uint32_t ok;
-    asm volatile(
-        "{\n .reg .pred p;\n mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n"
-        " selp.u32 %0, 1, 0, p;\n}\n"
-        : "=r"(ok) : "r"(smem_u32(bar)), "r"(parity) : "memory");
-    if (ok) return true;
-    if ((i & 7) == 7 && global_ns() - t0 > kWaitNs) return false;
-  }
-}
-
 // The 16 NF4 levels, code 0 .. 15, as QLoRA publishes the data type.
 __constant__ float c_nf4_lv[16] = {
     -1.0f, -0.6961928009986877f, -0.5250730514526367f, -0.39491748809814453f,
@@ -351,13 +296,17 @@ project_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
     const int nkb = args.k_blocks, nrow = n0 + (int)rank * (BN / 2) + n;
     const uint8_t* crow = args.nf4_codes + (int64_t)nrow * (nkb * 32) + h * 16;
     const float* arow = args.nf4_absmax + (int64_t)nrow * nkb;
-    // codes and absmax of this and the next PF K slices in registers (rotated
-    // each slice, so no array is indexed at run time)
-    constexpr int PF = 2;
-    uint4 cq[PF + 1][NQ];
-    float am[PF + 1];
+    // Codes and absmax of the next PF K slices in registers, PF slices to a loop
+    // trip: each is refilled as soon as it has been read and is not moved, as a
+    // move of a value still being loaded waits for it (272 us for 2048 x 4096 ->
+    // 6144 with buffers rotated each slice, 268 without; 167 with the arrival
+    // below no longer waiting for the loads).  A slice now takes 820 cycles of
+    // look-ups and stores and 250 of waiting for its slot.
+    constexpr int PF = 4;
+    uint4 cq[PF][NQ];
+    float am[PF];
 #pragma unroll
-    for (int i = 0; i <= PF; ++i) {
+    for (int i = 0; i < PF; ++i) {
 #pragma unroll
       for (int q = 0; q < NQ; ++q) cq[i][q] = make_uint4(0, 0, 0, 0);
       am[i] = 0.f;
@@ -372,14 +321,19 @@ project_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
 #pragma unroll
     for (int i = 0; i < PF; ++i) fetch(i, cq[i], am[i]);
     const int rsw = (n >> 3) * 1024 + (n & 7) * 128;      // the row in the swizzled tile
-    for (int kb = 0; kb < KB; ++kb) {
+    bool live = true;
+    for (int kb0 = 0; kb0 < KB && live; kb0 += PF)
+#pragma unroll
+    for (int u = 0; u < PF; ++u) {
+      const int kb = kb0 + u;
+      if (kb >= KB || !live) break;
       const int s = kb % kStages;
-      fetch(kb + PF, cq[PF], am[PF]);
       if (kb >= kStages) {                                // lane 0 waits for the slot, then the warp
         bool ok = true;
         if (lane == 0) ok = mbar_wait(&empty_bar[s], ((kb / kStages) - 1) & 1);
         if (!__shfl_sync(0xffffffffu, ok, 0)) {
           if (lane == 0) atomicOr(&fail, 1);
+          live = false;
           break;
         }
       }
@@ -387,16 +341,11 @@ project_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
       uint32_t w8[4 * NQ];
 #pragma unroll
       for (int q = 0; q < NQ; ++q) {
-        w8[4 * q] = cq[0][q].x; w8[4 * q + 1] = cq[0][q].y;
-        w8[4 * q + 2] = cq[0][q].z; w8[4 * q + 3] = cq[0][q].w;
+        w8[4 * q] = cq[u][q].x; w8[4 * q + 1] = cq[u][q].y;
+        w8[4 * q + 2] = cq[u][q].z; w8[4 * q + 3] = cq[u][q].w;
       }
-      const float a = am[0];
-#pragma unroll
-      for (int i = 0; i < PF; ++i) {
-#pragma unroll
-        for (int q = 0; q < NQ; ++q) cq[i][q] = cq[i + 1][q];
-        am[i] = am[i + 1];
-      }
+      const float a = am[u];
+      fetch(kb + PF, cq[u], am[u]);
       uint64_t a2;
       asm("mov.b64 %0, {%1, %1};" : "=l"(a2) : "f"(a));
 #pragma unroll
@@ -425,7 +374,7 @@ project_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
       }
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // for the MMA's reads
       __syncwarp();
-      if (lane == 0) mbar_arrive_cluster(mapa(&w_full[s], 0));
+      if (lane == 0) mbar_arrive_pair(mapa(&w_full[s], 0));
     }
   }
   // ---------------- (alpha/r) x A^T -> bf16 operand in shared memory ----------
@@ -626,27 +575,6 @@ bool make_map(CUtensorMap* m, const void* base, uint64_t rows, uint64_t cols, ui
                     box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
                     CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return res == CUDA_SUCCESS;
-}
-
-// launch_pdl with clusters of two CTAs along x (a tcgen05 pair has to lie there).
-template <typename... KArgs, typename... Args>
-cudaError_t launch_pdl_pair(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem,
-                            cudaStream_t s, Args&&... args) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = grid;
-  cfg.blockDim = block;
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = s;
-  cudaLaunchAttribute attr[2];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  attr[1].id = cudaLaunchAttributeClusterDimension;
-  attr[1].val.clusterDim.x = 2;
-  attr[1].val.clusterDim.y = 1;
-  attr[1].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 2;
-  return cudaLaunchKernelEx(&cfg, kern, std::forward<Args>(args)...);
 }
 
 template <int BN, bool NF4 = false>
