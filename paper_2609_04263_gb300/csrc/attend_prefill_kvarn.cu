@@ -5,34 +5,44 @@
 // once and the output is rotated back; sinks and staged tokens (stored in the
 // original basis) are rotated forward as their tiles are built.
 //
-// One CTA = 128 query rows of one (sequence, kv head): the g query heads of
-// the kv head x 128/g consecutive queries.  Keys and values stream in tiles of
-// 32 tokens.  Three roles:
-//   producers (warps 4-11): reconstruct each tile in fp32: K as a bf16 high
+// Two CTAs (a cluster, one MMA pair) hold 128 query rows each of one (sequence,
+// kv head): the g query heads of the kv head x 128/g consecutive queries, the
+// second CTA's following the first's.  Keys and values stream in tiles of 64
+// tokens that the two build together: of K each CTA 32 of the tokens, of V the
+// 64 tokens' half of the channels, which is how a pair of CTAs shares the second
+// operand of its MMAs.  Three roles:
+//   producers (warps 4-11): reconstruct their share in fp32: K as a bf16 high
 //     part (the value truncated) plus the bf16 of the remainder, V rounded to
-//     fp16 and transposed (D rows, tokens along K), into three shared buffers.
-//     Warp w builds channels 32 w .. 32 w + 31, a lane one token; the packed
-//     words and scales of the next tile are loaded into registers before the
-//     current one is built, the tile's column scales go through a small
-//     shared array per warp;
-//   issuer (warp 12, one thread issues): S = Q_hi K_hi^T + Q_hi K_lo^T +
-//     Q_lo K_hi^T (a rotated query needs more than bf16's 8 bits too) into
-//     four TMEM tiles of 128 x 32 fp32, and O += P V into 128 x 256 fp32;
-//     S runs up to two tiles ahead of P V;
-//   softmax (warps 0-3): thread r owns row r (TMEM lane r): 32 scores, causal
+//     fp16 and transposed (channels x tokens), into three shared buffers.  Of K
+//     warp w builds channels 32 w .. 32 w + 31, a lane one token; of V channels
+//     16 w .. 16 w + 15, a lane two neighbouring tokens (one 32-bit store each
+//     channel); the packed words and scales of the next tile are loaded into
+//     registers before the current one is built, the tile's column scales go
+//     through a small shared array per warp;
+//   issuer (warp 12 of the first CTA, one lane issues): S = Q_hi K_hi^T +
+//     Q_hi K_lo^T + Q_lo K_hi^T (a rotated query needs more than bf16's 8 bits
+//     too) into two TMEM tiles of 128 x 64 fp32 in each CTA, and O += P V into
+//     128 x 256 fp32; S runs up to two tiles ahead of P V;
+//   softmax (warps 0-3): thread r owns row r (TMEM lane r): 64 scores, causal
 //     mask, running maximum and sum in log2 units, P as fp16 over its S tile; O
 //     is rescaled only when a row's maximum grows by more than 8.
+// The barriers that wake the issuer (tiles built, P written) sit in the first
+// CTA and count one arrival per warp of both; the issuer's commits arrive on both
+// CTAs' barriers.
 //
 // Space decides the layout: at D = 256 a 128-row query tile is 64 KB and has two
 // parts.  Q_hi stays in shared memory (the MMAs read it once per K step for
-// both K parts), Q_lo in 128 TMEM columns next to O's 256 and S's 4 x 32; that
-// leaves shared memory for three 48 KB K/V tiles of 32 tokens.
-// What bounds it: shared memory.  Per tile the MMAs read 64 KB of Q_hi, 48 KB of
-// K and 16 KB of V and the producers write 48 KB: about 1,400 cycles at 128
-// B/cycle, against 1,000 cycles of tensor pipe.
-// 8192 tokens, 16 query heads, 8 kv heads, one sequence: 7667 us on mma.sync (64
-// rows a CTA, 16-token tiles reconstructed by all its warps), 1526 us here (360
-// TFLOP/s of attention; the three Q K^T products make it 720 on the tensor cores).
+// both K parts), Q_lo in 128 TMEM columns next to O's 256 and S's 2 x 64; that
+// leaves shared memory for three 48 KB shares of K/V tiles.
+// What bounds it: building the tiles, 2,700 of 3,980 cycles per 64 tokens (the
+// loads of the next packed tile 620); the MMAs and their waits take 2,800 without
+// it.  8192 tokens, 16 query heads, 8 kv heads, one sequence: 7667 us on mma.sync
+// (64 rows a CTA, 16-token tiles reconstructed by all its warps), 1526 with one
+// CTA building 32-token tiles of K and V for 128 rows, 1103 here.  Of that, 170 us
+// are the pair, 110 loads and arrivals that no longer wait (load_packed,
+// mbar_arrive_pair), and 150 the full-precision tiles, rotated queries and
+// output rows, whose loads and stores are wide and started together (a CTA spent
+// 45 us on its sinks and staged tokens, a row at a time).
 // Every wait is bounded and also gives up when another role has timed out;
 // the issuer drains its MMAs before TMEM is freed, and a timed-out CTA stores
 // nothing and sets the library's error word.
@@ -45,60 +55,37 @@ namespace {
 using namespace tc;
 
 constexpr int kD = 256;
-constexpr int kM = 128;              // query rows per CTA (MMA M)
-constexpr int kTok = 32;             // tokens per KV tile
+constexpr int kM = 128;              // query rows per CTA (half of the pair's MMA M)
+constexpr int kTok = 64;             // tokens per KV tile
+constexpr int kHalf = 32;            // tokens of K per CTA
 constexpr int kG = 64;               // block length and group size
 constexpr int kProdWarps = 8;
 constexpr int kThreads = (4 + kProdWarps + 1) * 32;
 constexpr int kKvBufs = 3;
-constexpr int kSBufs = 4;
+constexpr int kSBufs = 2;
 constexpr float kRescale = 8.f;      // log2 growth of a row maximum that forces a rescale
 
 // Shared memory (bytes from a 1024-aligned base).
 constexpr int kQOff = 0;                               // Q_hi: 4 atoms of 128 rows x 128 B
 constexpr int kKvOff = kM * kD * 2;
 constexpr int kKH = 0;                                 // K hi: 4 atoms of 32 rows x 128 B
-constexpr int kKL = kTok * kD * 2;                     // K lo: the same
-constexpr int kVT = 2 * kTok * kD * 2;                 // V^T: 256 rows x 64 B, 64-byte swizzle
-constexpr int kKvB = 3 * kTok * kD * 2;
-constexpr int kColOff = kKvOff + kKvBufs * kKvB;       // per producer warp: 32 K, 32 V column scales
+constexpr int kKL = kHalf * kD * 2;                    // K lo: the same
+constexpr int kVT = 2 * kHalf * kD * 2;                // V^T: 128 channels x 128 B
+constexpr int kKvB = kVT + kD / 2 * kTok * 2;
+constexpr int kColOff = kKvOff + kKvBufs * kKvB;       // per producer warp: 32 K, 2 x 16 V column scales
 constexpr int kTotal = kColOff + kProdWarps * 64 * 4;
 constexpr int kAlloc = kTotal + 1024;                  // alignment slack
 constexpr int kQlPitch = kD * 2 + 16;                  // Q_lo rows staged in the K/V area
 static_assert(kM * kQlPitch <= kKvBufs * kKvB, "Q_lo rows fit the K/V area");
-constexpr int kOPitch = kD + 1;                        // fp32 output rows over Q and K/V
+constexpr int kOPitch = kD + 4;                        // fp32 output rows over Q and K/V
 static_assert(kM * kOPitch * 4 <= kTotal, "output rows fit");
 static_assert(kAlloc <= 227 * 1024, "one CTA's shared memory");
 
 // TMEM columns: O, Q_lo (two bf16 per column), S tiles (P over them).
 constexpr int kTmO = 0, kTmQ = 256, kTmS = 384;
 
-// Descriptor of a K-major operand with 64-byte rows in the 64-byte swizzle
-// (8-row groups 512 bytes apart), and the byte offset of 16-byte chunk c of
-// row r in it.
-__device__ __forceinline__ uint64_t sw64_desc(const void* p) {
-  const uint64_t addr = smem_u32(p);
-  uint64_t d = 0;
-  d |= (addr >> 4) & 0x3FFFull;               // start address
-  d |= (uint64_t)1 << 16;                     // leading byte offset (unused)
-  d |= (uint64_t)(512 >> 4) << 32;            // stride byte offset: 8 rows x 64 B
-  d |= (uint64_t)1 << 46;                     // descriptor version (sm_100 family)
-  d |= (uint64_t)4 << 61;                     // layout: 64-byte swizzle
-  return d;
-}
-__device__ __forceinline__ int sw64(int r, int c) {
-  return r * 64 + ((c ^ ((r >> 1) & 3)) << 4);
-}
-
-// In-warp normalised Hadamard transform of a row held as x[i] = row[lane + 32 i].
+// In-warp normalised Hadamard transform of a row held as x[i] = row[8 lane + i].
 __device__ __forceinline__ void fwht256(float (&x)[8], int lane) {
-#pragma unroll
-  for (int h = 1; h < 32; h <<= 1)
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const float y = __shfl_xor_sync(0xffffffffu, x[i], h);
-      x[i] = (lane & h) ? y - x[i] : x[i] + y;
-    }
 #pragma unroll
   for (int hs = 1; hs < 8; hs <<= 1)
 #pragma unroll
@@ -109,7 +96,22 @@ __device__ __forceinline__ void fwht256(float (&x)[8], int lane) {
         x[i + hs] = a - c;
       }
 #pragma unroll
+  for (int h = 1; h < 32; h <<= 1)
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const float y = __shfl_xor_sync(0xffffffffu, x[i], h);
+      x[i] = (lane & h) ? y - x[i] : x[i] + y;
+    }
+#pragma unroll
   for (int i = 0; i < 8; ++i) x[i] *= 0.0625f;           // 1 / sqrt(256)
+}
+__device__ __forceinline__ void unpack8(const uint4& u, float (&x)[8]) {
+  const uint32_t w[4] = {u.x, u.y, u.z, u.w};
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    x[2 * i] = __uint_as_float(w[i] << 16);
+    x[2 * i + 1] = __uint_as_float(w[i] & 0xFFFF0000u);
+  }
 }
 
 __device__ __forceinline__ uint64_t fmul2(uint64_t a, uint64_t b) {
@@ -129,142 +131,192 @@ __device__ __forceinline__ bool producers_all(bool ok) {
   return r != 0;
 }
 
-// One thread's packed part of a coded tile: its token's codes of 32 channels
-// and scales, and two of the warp's column scales.
+// One thread's packed part of a tile: 32 channels' key codes of one token and 16
+// channels' value codes of two, their scales, and two of the warp's column scales.
 template <int KB, int VB>
 struct Packed {
-  uint32_t kc[KB], vc[VB];           // 32 codes of KB (VB) bits
-  __half ks, kz, kr, vs, vz, vr;
+  uint32_t kc[KB], vc[2][VB / 2];    // codes of KB (VB) bits
+  uint32_t ks, kz, kr, vs[2], vz[2], vr[2];   // fp16 bits
   __half2 col;
 };
+__device__ __forceinline__ float h2f(uint32_t bits) {
+  return __half2float(__ushort_as_half((unsigned short)bits));
+}
+// A 16-bit load into a register of its own: two that the compiler packs into one
+// register make the warp wait for them where they are issued.
+__device__ __forceinline__ uint32_t ld16(const __half* p) {
+  uint32_t v;
+  asm volatile("ld.global.u16 %0, [%1];" : "=r"(v) : "l"(p));
+  return v;
+}
 
 template <int N>
 __device__ __forceinline__ void load_words(uint32_t (&w)[N], const uint8_t* p) {
   if constexpr (N == 4) {
     const uint4 u = *reinterpret_cast<const uint4*>(p);
     w[0] = u.x; w[1] = u.y; w[2] = u.z; w[3] = u.w;
-  } else {
+  } else if constexpr (N == 2) {
     const uint2 u = *reinterpret_cast<const uint2*>(p);
     w[0] = u.x; w[1] = u.y;
+  } else {
+    w[0] = *reinterpret_cast<const uint32_t*>(p);
   }
 }
 
-// Where a head's coded rows start, at this thread's token of tile 0.
+// Where a head's coded rows start.
 struct Rows {
   const uint8_t *kc, *vc;
   const __half *ks, *kz, *kr, *kcol, *vs, *vz, *vr, *vcol;
 };
 
-// Tile at coded row q0 (a multiple of 32): pw the producer warp.
+// A tile whose first token is coded row q0 (-32: its second half is row 0), of
+// `rows` coded rows.  Lanes whose tokens are not coded load a row that is, which
+// is not used: loads under a branch that divides the warp were waited for at its
+// end (1,600 cycles a tile).
 template <int KB, int VB>
-__device__ __forceinline__ void load_packed(const Rows& r, int q0, int pw, int lane,
-                                            Packed<KB, VB>& p) {
-  const int64_t q = q0 + lane;
-  load_words<KB>(p.kc, r.kc + q * (kD * KB / 8) + pw * (32 * KB / 8));
-  load_words<VB>(p.vc, r.vc + q * (kD * VB / 8) + pw * (32 * VB / 8));
-  const int64_t m = q * (kD / kG) + pw / 2;
-  p.ks = r.ks[m];
-  p.kz = r.kz[m];
-  p.vs = r.vs[m];
-  p.vz = r.vz[m];
-  p.kr = r.kr[q];
-  p.vr = r.vr[q];
-  const int64_t c = (int64_t)(q0 / kG) * kD + pw * 32 + 2 * (lane & 15);
-  p.col = *reinterpret_cast<const __half2*>((lane < 16 ? r.kcol : r.vcol) + c);
+__device__ __forceinline__ void load_packed(const Rows& r, int q0, int rows, uint32_t rank, int pw,
+                                            int lane, Packed<KB, VB>& p) {
+  const int qk = min(max(q0 + (int)rank * kHalf + lane, 0), rows - 1);
+  load_words<KB>(p.kc, r.kc + (int64_t)qk * (kD * KB / 8) + pw * (32 * KB / 8));
+  const int64_t mk = (int64_t)qk * (kD / kG) + pw / 2;
+  p.ks = ld16(r.ks + mk);
+  p.kz = ld16(r.kz + mk);
+  p.kr = ld16(r.kr + qk);
+  const int ch = (int)rank * (kD / 2) + pw * 16;
+#pragma unroll
+  for (int u = 0; u < 2; ++u) {
+    const int qv = min(max(q0 + 2 * lane + u, 0), rows - 1);
+    load_words<VB / 2>(p.vc[u], r.vc + ((int64_t)qv * kD + ch) * VB / 8);
+    const int64_t m = (int64_t)qv * (kD / kG) + ch / kG;
+    p.vs[u] = ld16(r.vs + m);
+    p.vz[u] = ld16(r.vz + m);
+    p.vr[u] = ld16(r.vr + qv);
+  }
+  // two column scales: lanes 0-15 K's, 16-23 and 24-31 those of V's halves
+  const int qc = min(max(q0 + (lane < 16 ? (int)rank : lane < 24 ? 0 : 1) * kHalf, 0), rows - 1) / kG;
+  const __half* cp = (lane < 16 ? r.kcol : r.vcol) + (int64_t)qc * kD +
+                     (lane < 16 ? pw * 32 + 2 * lane : ch + 2 * (lane & 7));
+  p.col = *reinterpret_cast<const __half2*>(cp);
 }
 
-// A coded tile into kv.  col: this warp's 64 floats of shared memory.
+// The coded parts of a tile into kv.  col: this warp's 64 floats of shared memory.
 template <int KB, int VB>
-__device__ __forceinline__ void build_coded(const Packed<KB, VB>& p, int pw, int lane, float* col,
-                                            unsigned char* kv) {
+__device__ __forceinline__ void build_coded(const Packed<KB, VB>& p, bool kin, bool vin, int pw,
+                                            int lane, float* col, unsigned char* kv) {
   __syncwarp();                                  // the previous tile's scales are read
   *reinterpret_cast<float2*>(col + 2 * lane) = __half22float2(p.col);   // K: 0..31, V: 32..63
   __syncwarp();
   const uint64_t bias2 = f2pack(-8388608.f, -8388608.f);
-  const float kr = __half2float(p.kr), vr = __half2float(p.vr);
-  const float ks = __half2float(p.ks) * kr, kz = __half2float(p.kz) * kr;
-  const float vs = __half2float(p.vs) * vr, vz = __half2float(p.vz) * vr;
-  const uint64_t ks2 = f2pack(ks, ks), kz2 = f2pack(kz, kz);
-  const uint64_t vs2 = f2pack(vs, vs), vz2 = f2pack(vz, vz);
-  // K: 4 chunks of 8 channels of token `lane`
-  unsigned char* kbase = kv + (pw >> 1) * (kTok * 128);
+  if (kin) {
+    // K: 4 chunks of 8 channels of token `lane` of the half
+    const float kr = h2f(p.kr);
+    const float ks = h2f(p.ks) * kr, kz = h2f(p.kz) * kr;
+    const uint64_t ks2 = f2pack(ks, ks), kz2 = f2pack(kz, kz);
+    unsigned char* kbase = kv + (pw >> 1) * (kHalf * 128);
 #pragma unroll
-  for (int c = 0; c < 4; ++c) {
-    const uint32_t w = p.kc[c * KB / 4] >> (c * 8 * KB % 32);
-    const float4 c0 = *reinterpret_cast<const float4*>(col + 8 * c);
-    const float4 c1 = *reinterpret_cast<const float4*>(col + 8 * c + 4);
-    const uint64_t cc[4] = {f2pack(c0.x, c0.y), f2pack(c0.z, c0.w), f2pack(c1.x, c1.y),
-                            f2pack(c1.z, c1.w)};
-    uint32_t h[4], l[4];
+    for (int c = 0; c < 4; ++c) {
+      const uint32_t w = p.kc[c * KB / 4] >> (c * 8 * KB % 32);
+      const float4 c0 = *reinterpret_cast<const float4*>(col + 8 * c);
+      const float4 c1 = *reinterpret_cast<const float4*>(col + 8 * c + 4);
+      const uint64_t cc[4] = {f2pack(c0.x, c0.y), f2pack(c0.z, c0.w), f2pack(c1.x, c1.y),
+                              f2pack(c1.z, c1.w)};
+      uint32_t h[4], l[4];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const uint64_t code = fadd2(f2pack(code_biased<KB>(w, 2 * i), code_biased<KB>(w, 2 * i + 1)), bias2);
-      const uint64_t k2 = fmul2(ffma2(code, ks2, kz2), cc[i]);
-      float a, b;
-      f2unpack(k2, a, b);
-      const uint32_t ab = __float_as_uint(a) & 0xFFFF0000u, bb = __float_as_uint(b) & 0xFFFF0000u;
-      h[i] = __byte_perm(ab, bb, 0x7632);
-      float ra, rb;
-      f2unpack(fadd2(k2, f2pack(-__uint_as_float(ab), -__uint_as_float(bb))), ra, rb);
-      l[i] = pack_bf16(ra, rb);
+      for (int i = 0; i < 4; ++i) {
+        const uint64_t code = fadd2(f2pack(code_biased<KB>(w, 2 * i), code_biased<KB>(w, 2 * i + 1)), bias2);
+        const uint64_t k2 = fmul2(ffma2(code, ks2, kz2), cc[i]);
+        float a, b;
+        f2unpack(k2, a, b);
+        const uint32_t ab = __float_as_uint(a) & 0xFFFF0000u, bb = __float_as_uint(b) & 0xFFFF0000u;
+        h[i] = __byte_perm(ab, bb, 0x7632);
+        float ra, rb;
+        f2unpack(fadd2(k2, f2pack(-__uint_as_float(ab), -__uint_as_float(bb))), ra, rb);
+        l[i] = pack_bf16(ra, rb);
+      }
+      const int off = sw128(lane, (pw & 1) * 4 + c);
+      *reinterpret_cast<uint4*>(kbase + kKH + off) = make_uint4(h[0], h[1], h[2], h[3]);
+      *reinterpret_cast<uint4*>(kbase + kKL + off) = make_uint4(l[0], l[1], l[2], l[3]);
     }
-    const int off = sw128(lane, (pw & 1) * 4 + c);
-    *reinterpret_cast<uint4*>(kbase + kKH + off) = make_uint4(h[0], h[1], h[2], h[3]);
-    *reinterpret_cast<uint4*>(kbase + kKL + off) = make_uint4(l[0], l[1], l[2], l[3]);
   }
-  // V^T: rows 32 pw + e, column `lane`
-  unsigned char* vbase = kv + kVT + pw * 32 * 64 + (lane & 7) * 2;
+  if (vin) {
+    // V^T: rows 16 pw + e, tokens 2 lane and 2 lane + 1
+    float s[2], z[2];
 #pragma unroll
-  for (int c = 0; c < 8; ++c) {
-    const uint32_t w = p.vc[c * VB / 8] >> (c * 4 * VB % 32);
-    const float4 c0 = *reinterpret_cast<const float4*>(col + 32 + 4 * c);
-    const uint64_t cc[2] = {f2pack(c0.x, c0.y), f2pack(c0.z, c0.w)};
+    for (int u = 0; u < 2; ++u) {
+      const float vr = h2f(p.vr[u]);
+      s[u] = h2f(p.vs[u]) * vr;
+      z[u] = h2f(p.vz[u]) * vr;
+    }
+    const uint64_t vs2 = f2pack(s[0], s[1]), vz2 = f2pack(z[0], z[1]);
+    const float* vcol = col + 32 + (lane >> 4) * 16;
+    unsigned char* vbase = kv + kVT + pw * 16 * 128 + (lane & 3) * 4;
 #pragma unroll
-    for (int i = 0; i < 2; ++i) {
-      const uint64_t code = fadd2(f2pack(code_biased<VB>(w, 2 * i), code_biased<VB>(w, 2 * i + 1)), bias2);
-      float a, b;
-      f2unpack(fmul2(ffma2(code, vs2, vz2), cc[i]), a, b);
-      const uint32_t v2 = pack_h2(a, b);
-      const int e = 4 * c + 2 * i;               // rows e, e + 1 share a swizzle phase
-      unsigned char* d = vbase + e * 64 + (((lane >> 3) ^ ((e >> 1) & 3)) << 4);
-      *reinterpret_cast<uint16_t*>(d) = (uint16_t)v2;
-      *reinterpret_cast<uint16_t*>(d + 64) = (uint16_t)(v2 >> 16);
+    for (int c = 0; c < 4; ++c) {
+      const float4 c4 = *reinterpret_cast<const float4*>(vcol + 4 * c);
+      const float cc[4] = {c4.x, c4.y, c4.z, c4.w};
+      const uint32_t w0 = p.vc[0][c * VB / 8] >> (c * 4 * VB % 32);
+      const uint32_t w1 = p.vc[1][c * VB / 8] >> (c * 4 * VB % 32);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int e = 4 * c + i;
+        const uint64_t code = fadd2(f2pack(code_biased<VB>(w0, i), code_biased<VB>(w1, i)), bias2);
+        float a, b;
+        f2unpack(fmul2(ffma2(code, vs2, vz2), f2pack(cc[i], cc[i])), a, b);
+        *reinterpret_cast<uint32_t*>(vbase + e * 128 + (((lane >> 2) ^ (e & 7)) << 4)) = pack_h2(a, b);
+      }
     }
   }
 }
 
-// A tile with full-precision tokens (sinks, staged, or beyond T: zeros): a warp
-// per token, rotated forward in registers.  S and the coded tokens are
-// multiples of 32, so the tile holds no coded token.
-__device__ __noinline__ void build_full(const Geom& g, int b, int h, int t0, int T, int pw,
-                                        int lane, unsigned char* kv) {
-  for (int r = pw; r < kTok; r += kProdWarps) {
-    const int t = t0 + r;
+// The full-precision parts of the tile at t0 (sinks, staged tokens, zeros beyond
+// T): of K 32 tokens at t0 + 32 rank (kin false), of V the halves vin0, vin1 name
+// false.  A warp takes every eighth token; all its rows are loaded before the
+// first is rotated forward.
+__device__ __noinline__ void build_full(const Geom& g, int b, int h, int t0, int T, uint32_t rank,
+                                        bool kin, bool vin0, bool vin1, int pw, int lane,
+                                        unsigned char* kv) {
+  constexpr int NT = kHalf / kProdWarps;
+  uint4 raw[3][NT];
 #pragma unroll
-    for (int which = 0; which < 2; ++which) {
-      float x[8];
+  for (int s = 0; s < 3; ++s)                    // K, V half 0, V half 1
 #pragma unroll
-      for (int i = 0; i < 8; ++i) x[i] = 0.f;
-      if (t < T) {
+    for (int i = 0; i < NT; ++i) {
+      const int t = t0 + (s == 0 ? (int)rank : s - 1) * kHalf + pw + kProdWarps * i;
+      raw[s][i] = make_uint4(0, 0, 0, 0);
+      if (!(s == 0 ? kin : s == 1 ? vin0 : vin1) && t < T) {
         const __nv_bfloat16* src =
-            t < g.S ? plane_ptr<__nv_bfloat16>(g, which ? KVQ_PLANE_V_FULL : KVQ_PLANE_K_FULL, b, h, t, 0)
-                    : plane_ptr<__nv_bfloat16>(g, which ? KVQ_PLANE_V_PEND : KVQ_PLANE_K_PEND, b, h,
+            t < g.S ? plane_ptr<__nv_bfloat16>(g, s ? KVQ_PLANE_V_FULL : KVQ_PLANE_K_FULL, b, h, t, 0)
+                    : plane_ptr<__nv_bfloat16>(g, s ? KVQ_PLANE_V_PEND : KVQ_PLANE_K_PEND, b, h,
                                                (t - g.S) % kG, 0);
-#pragma unroll
-        for (int i = 0; i < 8; ++i) x[i] = __bfloat162float(src[lane + 32 * i]);
-        fwht256(x, lane);
+        raw[s][i] = *reinterpret_cast<const uint4*>(src + 8 * lane);
       }
+    }
 #pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const int j = lane + 32 * i;
-        if (which) {
-          *reinterpret_cast<__half*>(kv + kVT + sw64(j, r >> 3) + (r & 7) * 2) = __float2half_rn(x[i]);
-        } else {
-          unsigned char* d = kv + (j >> 6) * (kTok * 128) + sw128(r, (j & 63) >> 3) + (j & 7) * 2;
-          const float hi = __uint_as_float(__float_as_uint(x[i]) & 0xFFFF0000u);
-          *reinterpret_cast<__nv_bfloat16*>(d + kKH) = __float2bfloat16_rn(hi);
-          *reinterpret_cast<__nv_bfloat16*>(d + kKL) = __float2bfloat16_rn(x[i] - hi);
+  for (int s = 0; s < 3; ++s) {
+    if (s == 0 ? kin : s == 1 ? vin0 : vin1) continue;
+#pragma unroll
+    for (int i = 0; i < NT; ++i) {
+      const int r = pw + kProdWarps * i;
+      float x[8];
+      unpack8(raw[s][i], x);
+      fwht256(x, lane);
+      if (s == 0) {
+        uint32_t hw[4], lw[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const uint32_t a = __float_as_uint(x[2 * e]) & 0xFFFF0000u, c = __float_as_uint(x[2 * e + 1]) & 0xFFFF0000u;
+          hw[e] = __byte_perm(a, c, 0x7632);
+          lw[e] = pack_bf16(x[2 * e] - __uint_as_float(a), x[2 * e + 1] - __uint_as_float(c));
         }
+        unsigned char* d = kv + (lane >> 3) * (kHalf * 128) + sw128(r, lane & 7);
+        *reinterpret_cast<uint4*>(d + kKH) = make_uint4(hw[0], hw[1], hw[2], hw[3]);
+        *reinterpret_cast<uint4*>(d + kKL) = make_uint4(lw[0], lw[1], lw[2], lw[3]);
+      } else if ((uint32_t)(lane >> 4) == rank) {
+        const int tk = (s - 1) * kHalf + r;
+#pragma unroll
+        for (int e = 0; e < 8; ++e)
+          *reinterpret_cast<__half*>(kv + kVT + sw128(8 * (lane & 15) + e, tk >> 3) + (tk & 7) * 2) =
+              __float2half_rn(x[e]);
       }
     }
   }
@@ -285,25 +337,26 @@ attend_prefill_kvarn_kernel(Geom g, const __nv_bfloat16* __restrict__ q, int L, 
   __shared__ int abort_flag;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int qtile = gridDim.x - 1 - blockIdx.x;        // longest first
+  const uint32_t rank = cluster_rank();
+  const int qpair = (gridDim.x - 1 - blockIdx.x) / 2;  // longest first
   const int hkv = blockIdx.y, b = blockIdx.z;
   const int grp = g.Hq / g.H;
   const int T = cache_tokens(g);
-  const int q0 = qtile * nq;
-  const int nql = min(nq, L - q0);
+  const int q0 = (2 * qpair + (int)rank) * nq;
+  const int nql = min(nq, L - q0);                     // <= 0: no query here, only a share of K/V
   const int pos_first = T - L + q0;
-  const int t_end = pos_first + nql;                   // keys [0, t_end)
+  const int t_end = T - L + min((2 * qpair + 2) * nq, L);   // the pair's keys [0, t_end)
   const int ntiles = (t_end + kTok - 1) / kTok;
   volatile int* abort = &abort_flag;
 
   if (threadIdx.x == 0) {
     for (int i = 0; i < kKvBufs; ++i) {
-      mbar_init(&kv_full[i], kProdWarps * 32);
+      mbar_init(&kv_full[i], 2 * kProdWarps);
       mbar_init(&kv_free[i], 1);
     }
     for (int i = 0; i < kSBufs; ++i) {
       mbar_init(&s_full[i], 1);
-      mbar_init(&p_full[i], kM);
+      mbar_init(&p_full[i], 2 * (kM / 32));
       mbar_init(&s_free[i], 1);
     }
     mbar_init(&done_bar, 1);
@@ -311,31 +364,41 @@ attend_prefill_kvarn_kernel(Geom g, const __nv_bfloat16* __restrict__ q, int L, 
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 12) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;"
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], 512;"
                  ::"r"(smem_u32(&tmem_base)));
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;");
   }
   // rotate the query rows: the high part into the swizzled Q tile, the bf16
-  // remainder into a staging row (then TMEM)
-  for (int r = warp; r < kM; r += kThreads / 32) {
-    const int hl = r / nq, qi = r % nq;
-    float x[8];
+  // remainder into a staging row (then TMEM); a warp's rows are loaded five at a time
+  constexpr int kRows = 5;
+  for (int r0 = warp; r0 < kM; r0 += kRows * (kThreads / 32)) {
+    uint4 raw[kRows];
 #pragma unroll
-    for (int i = 0; i < 8; ++i) x[i] = 0.f;
-    if (hl < grp && qi < nql) {
-      const __nv_bfloat16* src = q + (((int64_t)b * g.Hq + hkv * grp + hl) * L + q0 + qi) * kD;
-#pragma unroll
-      for (int i = 0; i < 8; ++i) x[i] = __bfloat162float(src[lane + 32 * i]);
-      fwht256(x, lane);
+    for (int k = 0; k < kRows; ++k) {
+      const int r = r0 + k * (kThreads / 32), hl = r / nq, qi = r % nq;
+      raw[k] = make_uint4(0, 0, 0, 0);
+      if (r < kM && hl < grp && qi < nql)
+        raw[k] = *reinterpret_cast<const uint4*>(
+            q + (((int64_t)b * g.Hq + hkv * grp + hl) * L + q0 + qi) * kD + 8 * lane);
     }
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const int j = lane + 32 * i;
-      const __nv_bfloat16 hb = __float2bfloat16_rn(x[i]);
-      *reinterpret_cast<__nv_bfloat16*>(smem + kQOff + (j >> 6) * (kM * 128) +
-                                        sw128(r, (j & 63) >> 3) + (j & 7) * 2) = hb;
-      *reinterpret_cast<__nv_bfloat16*>(smem + kKvOff + r * kQlPitch + j * 2) =
-          __float2bfloat16_rn(x[i] - __bfloat162float(hb));
+    for (int k = 0; k < kRows; ++k) {
+      const int r = r0 + k * (kThreads / 32);
+      if (r >= kM) break;
+      float x[8];
+      unpack8(raw[k], x);
+      fwht256(x, lane);
+      uint32_t hw[4], lw[4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        hw[e] = pack_bf16(x[2 * e], x[2 * e + 1]);
+        lw[e] = pack_bf16(x[2 * e] - __uint_as_float(hw[e] << 16),
+                          x[2 * e + 1] - __uint_as_float(hw[e] & 0xFFFF0000u));
+      }
+      *reinterpret_cast<uint4*>(smem + kQOff + (lane >> 3) * (kM * 128) + sw128(r, lane & 7)) =
+          make_uint4(hw[0], hw[1], hw[2], hw[3]);
+      *reinterpret_cast<uint4*>(smem + kKvOff + r * kQlPitch + 16 * lane) =
+          make_uint4(lw[0], lw[1], lw[2], lw[3]);
     }
   }
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -360,6 +423,7 @@ attend_prefill_kvarn_kernel(Geom g, const __nv_bfloat16* __restrict__ q, int L, 
   }
   tc_fence_before();
   __syncthreads();                                     // Q_lo in TMEM, the K/V area is free
+  cluster_sync();                                      // in both CTAs, and their barriers are set up
   tc_fence_after();
 
   float inv_l = 0.f;
@@ -381,97 +445,106 @@ attend_prefill_kvarn_kernel(Geom g, const __nv_bfloat16* __restrict__ q, int L, 
       rows.kcol = plane_ptr<__half>(g, KVQ_PLANE_K_COL, b, hkv, 0);
       rows.vcol = plane_ptr<__half>(g, KVQ_PLANE_V_COL, b, hkv, 0);
     }
+    // S and the coded tokens are multiples of 32, so 32 tokens are either all
+    // coded, inside one block's column scales, or all full precision
     auto coded = [&](int t0) { return t0 >= g.S && t0 < g.S + nbq; };
     Packed<KB, VB> cur = {}, nxt = {};
-    if (coded(0)) load_packed<KB, VB>(rows, 0 - g.S, pw, lane, nxt);
+    if (coded(0) || coded(kHalf)) load_packed<KB, VB>(rows, 0 - g.S, nbq, rank, pw, lane, nxt);
     for (int j = 0; j < ntiles; ++j) {
-      const int t0 = j * kTok, kb = j % kKvBufs;
+      const int t0 = j * kTok, t1 = t0 + kTok, kb = j % kKvBufs;
       cur = nxt;
-      if (j + 1 < ntiles && coded(t0 + kTok)) load_packed<KB, VB>(rows, t0 + kTok - g.S, pw, lane, nxt);
+      if (j + 1 < ntiles && (coded(t1) || coded(t1 + kHalf)))
+        load_packed<KB, VB>(rows, t1 - g.S, nbq, rank, pw, lane, nxt);
       const bool ok = j < kKvBufs || mbar_wait_or_abort(&kv_free[kb], ((j - kKvBufs) / kKvBufs) & 1, abort);
       if (!producers_all(ok)) break;
       unsigned char* kv = smem + kKvOff + kb * kKvB;
-      if (coded(t0)) build_coded<KB, VB>(cur, pw, lane, col, kv);
-      else build_full(g, b, hkv, t0, T, pw, lane, kv);
-      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-      mbar_arrive(&kv_full[kb]);
+      const bool kin = coded(t0 + (int)rank * kHalf), vin0 = coded(t0), vin1 = coded(t0 + kHalf);
+      if (kin || vin0 || vin1)
+        build_coded<KB, VB>(cur, kin, lane < 16 ? vin0 : vin1, pw, lane, col, kv);
+      if (!kin || !vin0 || !vin1)
+        build_full(g, b, hkv, t0, T, rank, kin, vin0, vin1, pw, lane, kv);
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // for the MMAs' reads
+      __syncwarp();
+      if (lane == 0) mbar_arrive_pair(mapa(&kv_full[kb], 0));
     }
   } else if (warp == 12) {
-    // ---------------- MMA issuer ----------------
-    // S of the next tile as soon as its K/V tile is built and its S buffer is
-    // free, P V of the next tile as soon as its P is written; the tensor pipe
-    // executes in issue order.  The whole warp runs the loop and one elected
-    // lane issues.  A K step of 16 elements advances a descriptor by 32 bytes.
-    constexpr uint32_t id_qk = idesc_bf16(kM, kTok);
-    constexpr uint32_t id_pv = idesc_f16(kM, kD);
-    const uint64_t qdesc0 = sw128_desc(smem + kQOff);
-    const uint64_t kdesc0 = sw128_desc(smem + kKvOff);
-    const uint64_t vdesc0 = sw64_desc(smem + kKvOff + kVT);
-    const bool leader = elect_one();
-    int nqk = 0, npv = 0;
-    long idle = 0;
-    uint64_t idle_since = 0;
-    while (npv < ntiles) {
-      bool progressed = false;
-      if (nqk < ntiles) {
-        const int kb = nqk % kKvBufs, sb = nqk % kSBufs;
-        bool ready = false;
-        if (lane == 0)
-          ready = mbar_test(&kv_full[kb], (nqk / kKvBufs) & 1) &&
-                  (nqk < kSBufs || mbar_test(&s_free[sb], ((nqk - kSBufs) / kSBufs) & 1));
-        if (__shfl_sync(0xffffffffu, ready, 0)) {
-          tc_fence_after();
-          if (leader) {
-            const uint32_t ts = tmem + kTmS + sb * kTok;
+    if (rank == 0) {
+      // ---------------- MMA issuer ----------------
+      // S of the next tile as soon as its K/V tile is built and its S buffer is
+      // free, P V of the next tile as soon as its P is written; the tensor pipe
+      // executes in issue order.  The whole warp runs the loop and one elected
+      // lane issues.  A K step of 16 elements advances a descriptor by 32 bytes.
+      constexpr uint32_t id_qk = idesc_bf16(2 * kM, kTok);
+      constexpr uint32_t id_pv = idesc_f16(2 * kM, kD);
+      const uint64_t qdesc0 = sw128_desc(smem + kQOff);
+      const uint64_t kdesc0 = sw128_desc(smem + kKvOff);
+      const uint64_t vdesc0 = sw128_desc(smem + kKvOff + kVT);
+      const bool leader = elect_one();
+      int nqk = 0, npv = 0;
+      long idle = 0;
+      uint64_t idle_since = 0;
+      while (npv < ntiles) {
+        bool progressed = false;
+        if (nqk < ntiles) {
+          const int kb = nqk % kKvBufs, sb = nqk % kSBufs;
+          bool ready = false;
+          if (lane == 0)
+            ready = mbar_test_cluster(&kv_full[kb], (nqk / kKvBufs) & 1) &&
+                    (nqk < kSBufs || mbar_test(&s_free[sb], ((nqk - kSBufs) / kSBufs) & 1));
+          if (__shfl_sync(0xffffffffu, ready, 0)) {
+            tc_fence_after();
+            if (leader) {
+              const uint32_t ts = tmem + kTmS + sb * kTok;
 #pragma unroll
-            for (int kk = 0; kk < kD / 16; ++kk) {
-              // Q atom: 128 rows x 128 B (1024 units); K atom: 32 rows x 128 B (256 units)
-              const uint64_t qd = qdesc0 + (uint64_t)((kk >> 2) * 1024 + (kk & 3) * 2);
-              const uint64_t kd = kdesc0 + (uint64_t)(kb * (kKvB >> 4) + (kk >> 2) * 256 + (kk & 3) * 2);
-              umma_a_fill(ts, qd, kd + (kKH >> 4), id_qk, kk > 0);     // Q_hi read once
-              umma_a_lastuse(ts, qd, kd + (kKL >> 4), id_qk, 1);       // for K hi and lo
-              umma_ts(ts, tmem + kTmQ + kk * 8, kd + (kKH >> 4), id_qk, 1);
+              for (int kk = 0; kk < kD / 16; ++kk) {
+                // Q atom: 128 rows x 128 B (1024 units); K atom: 32 rows x 128 B (256 units)
+                const uint64_t qd = qdesc0 + (uint64_t)((kk >> 2) * 1024 + (kk & 3) * 2);
+                const uint64_t kd = kdesc0 + (uint64_t)(kb * (kKvB >> 4) + (kk >> 2) * 256 + (kk & 3) * 2);
+                umma_pair_a_fill(ts, qd, kd + (kKH >> 4), id_qk, kk > 0);     // Q_hi read once
+                umma_pair_a_lastuse(ts, qd, kd + (kKL >> 4), id_qk, 1);       // for K hi and lo
+                umma_pair_ts(ts, tmem + kTmQ + kk * 8, kd + (kKH >> 4), id_qk, 1);
+              }
+              umma_commit_pair(&s_full[sb]);
             }
-            umma_commit(&s_full[sb]);
+            __syncwarp();
+            ++nqk;
+            progressed = true;
           }
-          __syncwarp();
-          ++nqk;
-          progressed = true;
         }
-      }
-      if (npv < nqk) {
-        const int sb = npv % kSBufs, kb = npv % kKvBufs;
-        bool ready = false;
-        if (lane == 0) ready = mbar_test(&p_full[sb], (npv / kSBufs) & 1);
-        if (__shfl_sync(0xffffffffu, ready, 0)) {
-          tc_fence_after();
-          if (leader) {
-            const uint32_t tp = tmem + kTmS + sb * kTok;               // P (fp16 pairs) over S
+        if (npv < nqk) {
+          const int sb = npv % kSBufs, kb = npv % kKvBufs;
+          bool ready = false;
+          if (lane == 0) ready = mbar_test_cluster(&p_full[sb], (npv / kSBufs) & 1);
+          if (__shfl_sync(0xffffffffu, ready, 0)) {
+            tc_fence_after();
+            if (leader) {
+              const uint32_t tp = tmem + kTmS + sb * kTok;               // P (fp16 pairs) over S
 #pragma unroll
-            for (int kk = 0; kk < kTok / 16; ++kk)
-              umma_ts(tmem + kTmO, tp + kk * 8, vdesc0 + (uint64_t)(kb * (kKvB >> 4) + kk * 2), id_pv,
-                      (npv > 0 || kk > 0) ? 1u : 0u);
-            umma_commit(&s_free[sb]);            // S/P buffer free, and O holds tile npv
-            umma_commit(&kv_free[kb]);
+              for (int kk = 0; kk < kTok / 16; ++kk)
+                umma_pair_ts(tmem + kTmO, tp + kk * 8, vdesc0 + (uint64_t)(kb * (kKvB >> 4) + kk * 2), id_pv,
+                        (npv > 0 || kk > 0) ? 1u : 0u);
+              umma_commit_pair(&s_free[sb]);            // S/P buffer free, and O holds tile npv
+              umma_commit_pair(&kv_free[kb]);
+            }
+            __syncwarp();
+            ++npv;
+            progressed = true;
           }
-          __syncwarp();
-          ++npv;
-          progressed = true;
+        }
+        if (progressed) {
+          idle = 0;
+        } else {
+          if (idle == 0) idle_since = global_ns();
+          __nanosleep(20);
+          const bool stop = (++idle & 63) == 0 && (*abort || global_ns() - idle_since > kWaitNs);
+          if (__shfl_sync(0xffffffffu, stop, 0)) break;   // the whole warp leaves together
         }
       }
-      if (progressed) {
-        idle = 0;
-      } else {
-        if (idle == 0) idle_since = global_ns();
-        __nanosleep(20);
-        const bool stop = (++idle & 63) == 0 && (*abort || global_ns() - idle_since > kWaitNs);
-        if (__shfl_sync(0xffffffffu, stop, 0)) break;   // the whole warp leaves together
-      }
+      if (lane == 0 && npv < ntiles) *abort = 1;
+      if (leader) umma_commit_pair(&done_bar);        // every MMA issued above has completed
+      if (lane == 0 && !mbar_wait(&done_bar, 0)) *abort = 1;
+      __syncwarp();
     }
-    if (lane == 0 && npv < ntiles) *abort = 1;
-    if (leader) umma_commit(&done_bar);        // every MMA issued above has completed
-    if (lane == 0 && !mbar_wait(&done_bar, 0)) *abort = 1;
-    __syncwarp();
   } else {
     // ---------------- softmax: one row per thread ----------------
     const int row = threadIdx.x;
@@ -490,8 +563,8 @@ attend_prefill_kvarn_kernel(Geom g, const __nv_bfloat16* __restrict__ q, int L, 
       }
       tc_fence_after();
       uint32_t sr[kTok];
-      tmem_ld16_nowait(s_col + sb * kTok, sr);
-      tmem_ld16_nowait(s_col + sb * kTok + 16, sr + 16);
+#pragma unroll
+      for (int c = 0; c < kTok; c += 16) tmem_ld16_nowait(s_col + sb * kTok + c, sr + c);
       tmem_wait_ld();
       if (t0 + kTok - 1 > pos) {               // some key of the tile is in the row's future
 #pragma unroll
@@ -501,11 +574,11 @@ attend_prefill_kvarn_kernel(Geom g, const __nv_bfloat16* __restrict__ q, int L, 
       float mx4[4];
 #pragma unroll
       for (int a = 0; a < 4; ++a) {
-        const uint32_t* v = sr + 8 * a;
+        const uint32_t* v = sr + 16 * a;
         float mv = fmax3(__uint_as_float(v[0]), __uint_as_float(v[1]), __uint_as_float(v[2]));
-        mv = fmax3(mv, __uint_as_float(v[3]), __uint_as_float(v[4]));
-        mv = fmax3(mv, __uint_as_float(v[5]), __uint_as_float(v[6]));
-        mx4[a] = fmaxf(mv, __uint_as_float(v[7]));
+#pragma unroll
+        for (int k = 3; k < 15; k += 2) mv = fmax3(mv, __uint_as_float(v[k]), __uint_as_float(v[k + 1]));
+        mx4[a] = fmaxf(mv, __uint_as_float(v[15]));
       }
       const float mx = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3]));
       const float m_new = fmaxf(m, mx * c2);   // (c2 > 0: the maximum commutes)
@@ -533,7 +606,7 @@ attend_prefill_kvarn_kernel(Geom g, const __nv_bfloat16* __restrict__ q, int L, 
           tmem_st16(o_col + c, o);
         }
       }
-      // P = 2^(s c2 - m) as fp16 pairs over the first 16 columns of this S
+      // P = 2^(s c2 - m) as fp16 pairs over the first 32 columns of this S
       // buffer (a row without any visible key so far has m = -inf and P = 0)
       const bool live = m != -INFINITY;
       const uint64_t negm = f2pack(-m, -m);
@@ -549,12 +622,14 @@ attend_prefill_kvarn_kernel(Geom g, const __nv_bfloat16* __restrict__ q, int L, 
         pk[i / 2] = pack_h2(p0, p1);
       }
       tmem_st16(s_col + sb * kTok, pk);
+      tmem_st16(s_col + sb * kTok + 16, pk + 16);
       float s0, s1;
       f2unpack(sum2, s0, s1);
       l += s0 + s1;
       tmem_wait_st();
       tc_fence_before();
-      mbar_arrive(&p_full[sb]);
+      __syncwarp();
+      if (lane == 0) mbar_arrive_pair(mapa(&p_full[sb], 0));
     }
     if (ok && ntiles > 0 &&
         !warp_wait(&s_free[(ntiles - 1) % kSBufs], ((ntiles - 1) / kSBufs) & 1, abort))
@@ -576,7 +651,10 @@ attend_prefill_kvarn_kernel(Geom g, const __nv_bfloat16* __restrict__ q, int L, 
       tmem_ld16_nowait(tmem + lane_base + kTmO + c, o);
       tmem_wait_ld();
 #pragma unroll
-      for (int i = 0; i < 16; ++i) orow[c + i] = __uint_as_float(o[i]) * inv_l;
+      for (int i = 0; i < 16; i += 4)
+        *reinterpret_cast<float4*>(orow + c + i) =
+            make_float4(__uint_as_float(o[i]) * inv_l, __uint_as_float(o[i + 1]) * inv_l,
+                        __uint_as_float(o[i + 2]) * inv_l, __uint_as_float(o[i + 3]) * inv_l);
     }
   }
   tc_fence_before();
@@ -585,19 +663,23 @@ attend_prefill_kvarn_kernel(Geom g, const __nv_bfloat16* __restrict__ q, int L, 
     for (int r = warp; r < kM; r += kThreads / 32) {
       const int hl = r / nq, qi = r % nq;
       if (hl >= grp || qi >= nql) continue;
-      float x[8];
-#pragma unroll
-      for (int i = 0; i < 8; ++i) x[i] = os[r * kOPitch + lane + 32 * i];
+      const float4 u = *reinterpret_cast<const float4*>(os + r * kOPitch + 8 * lane);
+      const float4 v = *reinterpret_cast<const float4*>(os + r * kOPitch + 8 * lane + 4);
+      float x[8] = {u.x, u.y, u.z, u.w, v.x, v.y, v.z, v.w};
       fwht256(x, lane);
       __nv_bfloat16* dst = out + (((int64_t)b * g.Hq + hkv * grp + hl) * L + q0 + qi) * kD;
-#pragma unroll
-      for (int i = 0; i < 8; ++i) dst[lane + 32 * i] = __float2bfloat16_rn(x[i]);
+      *reinterpret_cast<uint4*>(dst + 8 * lane) = make_uint4(pack_bf16(x[0], x[1]), pack_bf16(x[2], x[3]),
+                                                             pack_bf16(x[4], x[5]), pack_bf16(x[6], x[7]));
     }
   }
   if (threadIdx.x == 0 && !good) atomicOr(err, 8);
+  // the issuer's last arrival on this CTA's barriers has landed
+  if (warp == 12 && lane == 0 && rank == 1 && !mbar_wait(&done_bar, 0)) atomicOr(err, 8);
+  tc_fence_before();
+  cluster_sync();                                      // neither CTA's TMEM or shared memory is in use
   if (warp == 12) {
     tc_fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem));
+    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, 512;" ::"r"(tmem));
   }
 }
 
@@ -608,7 +690,7 @@ cudaError_t launch(const Geom& g, const void* q, int L, float scale, void* out, 
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kAlloc);
   if (e != cudaSuccess) return e;
   const int nq = kM / (g.Hq / g.H);
-  launch_pdl(kern, dim3((L + nq - 1) / nq, g.H, g.B), dim3(kThreads), (size_t)kAlloc, s, g,
+  launch_pdl_pair(kern, dim3((L + 2 * nq - 1) / (2 * nq) * 2, g.H, g.B), dim3(kThreads), (size_t)kAlloc, s, g,
              reinterpret_cast<const __nv_bfloat16*>(q), L, scale,
              reinterpret_cast<__nv_bfloat16*>(out), nq, err);
   return cudaGetLastError();
@@ -617,11 +699,11 @@ cudaError_t launch(const Geom& g, const void* q, int L, float scale, void* out, 
 }  // namespace
 
 // bf16 KVarN caches at head_dim 256 with 64-token blocks, 2- or 4-bit codes and a
-// number of sinks that ends on a 32-token tile (a tile is then either all
+// number of sinks that is a multiple of 32 (32 tokens of a tile are then either all
 // coded, inside one column-scale block, or all full precision).
 bool prefill_kvarn_supported(const Geom& g) {
   return g.fmt == KVQ_FMT_KVARN && g.layout == KVQ_LAYOUT_UNIFORM && g.act == KVQ_BF16 &&
-         g.D == kD && g.G == kG && g.S % kTok == 0 && (g.kb == 2 || g.kb == 4) &&
+         g.D == kD && g.G == kG && g.S % kHalf == 0 && (g.kb == 2 || g.kb == 4) &&
          (g.vb == 2 || g.vb == 4);
 }
 

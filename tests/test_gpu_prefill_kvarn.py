@@ -1,7 +1,9 @@
 """The tcgen05 prefill attention of KVarN caches (head_dim 256, 64-token blocks)
-at the edges of its 32-token tiles and 128-row CTAs: sinks only, the first
-coded block, staged tokens, a chunk of queries at the end of a longer cache,
-GQA groups that do not divide the rows, 2- and 4-bit codes.  Tolerance: the
+at the edges of its 64-token tiles, their 32-token halves and the pairs of
+128-row CTAs: sinks only, sinks that end inside a tile, the first coded block,
+staged tokens, a chunk of queries at the end of a longer cache, queries in the
+first CTA only and one in the second, GQA groups that do not divide the rows,
+2- and 4-bit codes.  Tolerance: the
 parity bound of the other bf16 attention tests."""
 import numpy as np
 import pytest
@@ -33,6 +35,9 @@ CASES = [   # kb, vb, sinks, B, H, Hq, tokens, queries
     (4, 4, 0, 1, 1, 2, 200, 200),
     (2, 2, 32, 1, 2, 4, 500, 77),
     (2, 4, 64, 1, 1, 2, 130, 130),
+    (4, 2, 96, 2, 1, 1, 300, 129),
+    (2, 2, 64, 1, 1, 1, 257, 257),
+    (4, 4, 32, 1, 2, 2, 1025, 128),
     (4, 2, 40, 1, 1, 2, 200, 200),      # sinks off the tile: the other kernel
 ]
 
