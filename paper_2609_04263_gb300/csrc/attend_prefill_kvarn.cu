@@ -11,14 +11,14 @@
 // tokens that the two build together: of K each CTA 32 of the tokens, of V the
 // 64 tokens' half of the channels, which is how a pair of CTAs shares the second
 // operand of its MMAs.  Three roles:
-//   producers (warps 4-11): reconstruct their share in fp32: K as a bf16 high
-//     part (the value truncated) plus the bf16 of the remainder, V rounded to
-//     fp16 and transposed (channels x tokens), into three shared buffers.  Of K
-//     warp w builds channels 32 w .. 32 w + 31, a lane one token; of V channels
-//     16 w .. 16 w + 15, a lane two neighbouring tokens (one 32-bit store each
-//     channel); the packed words and scales of the next tile are loaded into
-//     registers before the current one is built, the tile's column scales go
-//     through a small shared array per warp;
+//   producers: reconstruct their share in fp32 into three shared buffers, K
+//     (warps 4-7) as a bf16 high part (the value truncated) plus the bf16 of the
+//     remainder, V (warps 8-11) rounded to fp16 and transposed (channels x
+//     tokens).  A key warp builds 64 channels, a lane one token; a value warp 32
+//     channels, a lane two neighbouring tokens (one 32-bit store each channel).
+//     The packed words and scales of the next tile are loaded into registers
+//     before the current one is built, the tile's column scales go through a
+//     small shared array per warp;
 //   issuer (warp 12 of the first CTA, one lane issues): S = Q_hi K_hi^T +
 //     Q_hi K_lo^T + Q_lo K_hi^T (a rotated query needs more than bf16's 8 bits
 //     too) into two TMEM tiles of 128 x 64 fp32 in each CTA, and O += P V into
@@ -34,15 +34,18 @@
 // parts.  Q_hi stays in shared memory (the MMAs read it once per K step for
 // both K parts), Q_lo in 128 TMEM columns next to O's 256 and S's 2 x 64; that
 // leaves shared memory for three 48 KB shares of K/V tiles.
-// What bounds it: building the tiles, 2,700 of 3,980 cycles per 64 tokens (the
-// loads of the next packed tile 620); the MMAs and their waits take 2,800 without
-// it.  8192 tokens, 16 query heads, 8 kv heads, one sequence: 7667 us on mma.sync
-// (64 rows a CTA, 16-token tiles reconstructed by all its warps), 1526 with one
-// CTA building 32-token tiles of K and V for 128 rows, 1103 here.  Of that, 170 us
-// are the pair, 110 loads and arrivals that no longer wait (load_packed,
-// mbar_arrive_pair), and 150 the full-precision tiles, rotated queries and
-// output rows, whose loads and stores are wide and started together (a CTA spent
-// 45 us on its sinks and staged tokens, a row at a time).
+// What bounds it: a 64-token tile takes about 3,000 cycles, the MMAs 2,050 of them;
+// with two score buffers Q K^T of a tile starts when P V of the tile two before it
+// has completed, so the pipe idles while that is signalled, and building the tiles
+// (1,850 cycles of each producer warp) slows the chain (2,700 cycles without it).
+// A CTA's start and end (rotating queries, sinks and output rows) take 50,000
+// cycles.  8192 tokens, 16 query heads, 8 kv heads, one sequence: 7667 us on
+// mma.sync (64 rows a CTA, 16-token tiles reconstructed by all its warps), 1526
+// with one CTA building 32-token tiles of K and V for 128 rows, 898 here: 1,480 as
+// a pair, 1,380 with arrivals that do not wait (mbar_arrive_pair), 1,100 with the
+// packed tile loaded without a branch that divides the warp (load_packed) and
+// rows of sinks, queries and outputs loaded together, 994 with K and V built by
+// warps of their own (no spills), 898 with four rows to a warp in the rotation.
 // Every wait is bounded and also gives up when another role has timed out;
 // the issuer drains its MMAs before TMEM is freed, and a timed-out CTA stores
 // nothing and sets the library's error word.
@@ -72,7 +75,7 @@ constexpr int kKH = 0;                                 // K hi: 4 atoms of 32 ro
 constexpr int kKL = kHalf * kD * 2;                    // K lo: the same
 constexpr int kVT = 2 * kHalf * kD * 2;                // V^T: 128 channels x 128 B
 constexpr int kKvB = kVT + kD / 2 * kTok * 2;
-constexpr int kColOff = kKvOff + kKvBufs * kKvB;       // per producer warp: 32 K, 2 x 16 V column scales
+constexpr int kColOff = kKvOff + kKvBufs * kKvB;       // per producer warp: 64 column scales
 constexpr int kTotal = kColOff + kProdWarps * 64 * 4;
 constexpr int kAlloc = kTotal + 1024;                  // alignment slack
 constexpr int kQlPitch = kD * 2 + 16;                  // Q_lo rows staged in the K/V area
@@ -84,33 +87,54 @@ static_assert(kAlloc <= 227 * 1024, "one CTA's shared memory");
 // TMEM columns: O, Q_lo (two bf16 per column), S tiles (P over them).
 constexpr int kTmO = 0, kTmQ = 256, kTmS = 384;
 
-// In-warp normalised Hadamard transform of a row held as x[i] = row[8 lane + i].
-__device__ __forceinline__ void fwht256(float (&x)[8], int lane) {
+// Four rows of 256 per warp: eight lanes hold row lane / 8, lane sub = lane % 8 the
+// 16-byte bf16 chunks sub + 8 k of it, x[8 k + e] = row[8 (sub + 8 k) + e].  Three of
+// the eight stages of a normalised Hadamard transform cross lanes (five with a row
+// to a warp), and a chunk is a whole 16-byte swizzle unit.  N = 16: the remaining
+// seven stages of one half of the channels, after the stage across the halves.
+template <int N>
+__device__ __forceinline__ void fwht256(float (&x)[N], int sub) {
+  auto in_regs = [&](int h) {
 #pragma unroll
-  for (int hs = 1; hs < 8; hs <<= 1)
-#pragma unroll
-    for (int i = 0; i < 8; ++i)
-      if (!(i & hs)) {
-        const float a = x[i], c = x[i + hs];
+    for (int i = 0; i < N; ++i)
+      if (!(i & h)) {
+        const float a = x[i], c = x[i + h];
         x[i] = a + c;
-        x[i + hs] = a - c;
+        x[i + h] = a - c;
       }
+  };
+  in_regs(1);
+  in_regs(2);
+  in_regs(4);
 #pragma unroll
-  for (int h = 1; h < 32; h <<= 1)
+  for (int h = 1; h < 8; h <<= 1) {
+    const float sg = (sub & h) ? -1.f : 1.f;             // a product with +-1 is exact
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
+    for (int i = 0; i < N; ++i) {
       const float y = __shfl_xor_sync(0xffffffffu, x[i], h);
-      x[i] = (lane & h) ? y - x[i] : x[i] + y;
+      x[i] = fmaf(sg, x[i], y);
     }
+  }
+  in_regs(8);
+  if constexpr (N == 32) in_regs(16);
 #pragma unroll
-  for (int i = 0; i < 8; ++i) x[i] *= 0.0625f;           // 1 / sqrt(256)
+  for (int i = 0; i < N; ++i) x[i] *= 0.0625f;           // 1 / sqrt(256)
 }
-__device__ __forceinline__ void unpack8(const uint4& u, float (&x)[8]) {
-  const uint32_t w[4] = {u.x, u.y, u.z, u.w};
+// The four chunks of this lane of a bf16 row (zeros without one).
+__device__ __forceinline__ void load_chunks(const __nv_bfloat16* row, int sub, uint4 (&u)[4]) {
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    x[2 * i] = __uint_as_float(w[i] << 16);
-    x[2 * i + 1] = __uint_as_float(w[i] & 0xFFFF0000u);
+  for (int k = 0; k < 4; ++k)
+    u[k] = row ? *reinterpret_cast<const uint4*>(row + 8 * (sub + 8 * k)) : make_uint4(0, 0, 0, 0);
+}
+__device__ __forceinline__ void unpack_chunks(const uint4 (&u)[4], float (&x)[32]) {
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const uint32_t w[4] = {u[k].x, u[k].y, u[k].z, u[k].w};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      x[8 * k + 2 * i] = __uint_as_float(w[i] << 16);
+      x[8 * k + 2 * i + 1] = __uint_as_float(w[i] & 0xFFFF0000u);
+    }
   }
 }
 
@@ -120,23 +144,13 @@ __device__ __forceinline__ uint64_t fmul2(uint64_t a, uint64_t b) {
   return d;
 }
 
-// Barrier of the producer warps (named barrier 1) that also returns whether
-// `ok` held in every producer thread, so all of them leave the loop together.
-__device__ __forceinline__ bool producers_all(bool ok) {
-  uint32_t r;
-  asm volatile(
-      "{\n .reg .pred p, q;\n setp.ne.u32 p, %1, 0;\n"
-      " bar.red.and.pred q, 1, 256, p;\n selp.u32 %0, 1, 0, q;\n}\n"
-      : "=r"(r) : "r"((uint32_t)ok) : "memory");
-  return r != 0;
-}
-
-// One thread's packed part of a tile: 32 channels' key codes of one token and 16
-// channels' value codes of two, their scales, and two of the warp's column scales.
-template <int KB, int VB>
+// One producer thread's packed part of a tile and two of its warp's column scales.
+// Keys: 64 channels of one token; values: 32 channels of two tokens.
+template <int BITS, bool V>
 struct Packed {
-  uint32_t kc[KB], vc[2][VB / 2];    // codes of KB (VB) bits
-  uint32_t ks, kz, kr, vs[2], vz[2], vr[2];   // fp16 bits
+  static constexpr int NT = V ? 2 : 1, NW = V ? BITS : 2 * BITS;
+  uint32_t c[NT][NW];                // codes
+  uint32_t s[NT], z[NT], r[NT];      // scale, offset and row scale: fp16 bits
   __half2 col;
 };
 __device__ __forceinline__ float h2f(uint32_t bits) {
@@ -152,70 +166,68 @@ __device__ __forceinline__ uint32_t ld16(const __half* p) {
 
 template <int N>
 __device__ __forceinline__ void load_words(uint32_t (&w)[N], const uint8_t* p) {
-  if constexpr (N == 4) {
-    const uint4 u = *reinterpret_cast<const uint4*>(p);
-    w[0] = u.x; w[1] = u.y; w[2] = u.z; w[3] = u.w;
-  } else if constexpr (N == 2) {
+  if constexpr (N >= 4) {
+#pragma unroll
+    for (int i = 0; i < N; i += 4) {
+      const uint4 u = *reinterpret_cast<const uint4*>(p + 4 * i);
+      w[i] = u.x; w[i + 1] = u.y; w[i + 2] = u.z; w[i + 3] = u.w;
+    }
+  } else {
     const uint2 u = *reinterpret_cast<const uint2*>(p);
     w[0] = u.x; w[1] = u.y;
-  } else {
-    w[0] = *reinterpret_cast<const uint32_t*>(p);
   }
 }
 
-// Where a head's coded rows start.
+// Where a head's coded keys or values start.
 struct Rows {
-  const uint8_t *kc, *vc;
-  const __half *ks, *kz, *kr, *kcol, *vs, *vz, *vr, *vcol;
+  const uint8_t* c;
+  const __half *s, *z, *r, *col;
 };
 
-// A tile whose first token is coded row q0 (-32: its second half is row 0), of
-// `rows` coded rows.  Lanes whose tokens are not coded load a row that is, which
-// is not used: loads under a branch that divides the warp were waited for at its
-// end (1,600 cycles a tile).
-template <int KB, int VB>
-__device__ __forceinline__ void load_packed(const Rows& r, int q0, int rows, uint32_t rank, int pw,
-                                            int lane, Packed<KB, VB>& p) {
-  const int qk = min(max(q0 + (int)rank * kHalf + lane, 0), rows - 1);
-  load_words<KB>(p.kc, r.kc + (int64_t)qk * (kD * KB / 8) + pw * (32 * KB / 8));
-  const int64_t mk = (int64_t)qk * (kD / kG) + pw / 2;
-  p.ks = ld16(r.ks + mk);
-  p.kz = ld16(r.kz + mk);
-  p.kr = ld16(r.kr + qk);
-  const int ch = (int)rank * (kD / 2) + pw * 16;
+// The keys (this CTA's 32) or values (its half of the channels) of the tile whose
+// first token is coded row q0 (-32: its second half is row 0), of `rows` coded rows.
+// Lanes whose tokens are not coded load a row that is, which is not used: loads
+// under a branch that divides the warp were waited for at its end (1,600 cycles a
+// tile).
+template <int BITS, bool V>
+__device__ __forceinline__ void load_packed(const Rows& r, int q0, int rows, uint32_t rank, int w,
+                                            int lane, Packed<BITS, V>& p) {
+  const int ch = V ? (int)rank * (kD / 2) + w * 32 : w * 64;
 #pragma unroll
-  for (int u = 0; u < 2; ++u) {
-    const int qv = min(max(q0 + 2 * lane + u, 0), rows - 1);
-    load_words<VB / 2>(p.vc[u], r.vc + ((int64_t)qv * kD + ch) * VB / 8);
-    const int64_t m = (int64_t)qv * (kD / kG) + ch / kG;
-    p.vs[u] = ld16(r.vs + m);
-    p.vz[u] = ld16(r.vz + m);
-    p.vr[u] = ld16(r.vr + qv);
+  for (int u = 0; u < p.NT; ++u) {
+    const int t = V ? 2 * lane + u : (int)rank * kHalf + lane;
+    const int q = min(max(q0 + t, 0), rows - 1);
+    load_words<p.NW>(p.c[u], r.c + ((int64_t)q * kD + ch) * BITS / 8);
+    const int64_t m = (int64_t)q * (kD / kG) + ch / kG;
+    p.s[u] = ld16(r.s + m);
+    p.z[u] = ld16(r.z + m);
+    p.r[u] = ld16(r.r + q);
   }
-  // two column scales: lanes 0-15 K's, 16-23 and 24-31 those of V's halves
-  const int qc = min(max(q0 + (lane < 16 ? (int)rank : lane < 24 ? 0 : 1) * kHalf, 0), rows - 1) / kG;
-  const __half* cp = (lane < 16 ? r.kcol : r.vcol) + (int64_t)qc * kD +
-                     (lane < 16 ? pw * 32 + 2 * lane : ch + 2 * (lane & 7));
-  p.col = *reinterpret_cast<const __half2*>(cp);
+  // keys: 64 channels' column scales; values: 32 channels', for each half of the tile
+  const int t = V ? (lane >> 4) * kHalf : (int)rank * kHalf;
+  const int qc = min(max(q0 + t, 0), rows - 1) / kG;
+  p.col = *reinterpret_cast<const __half2*>(r.col + (int64_t)qc * kD + ch + 2 * (V ? lane & 15 : lane));
 }
 
-// The coded parts of a tile into kv.  col: this warp's 64 floats of shared memory.
-template <int KB, int VB>
-__device__ __forceinline__ void build_coded(const Packed<KB, VB>& p, bool kin, bool vin, int pw,
-                                            int lane, float* col, unsigned char* kv) {
+// The coded keys or values of a tile into kv, for lanes whose tokens are coded
+// (`in`).  col: this warp's 64 floats of shared memory.
+template <int BITS, bool V>
+__device__ __forceinline__ void build_coded(const Packed<BITS, V>& p, bool in, int w, int lane,
+                                            float* col, unsigned char* kv) {
   __syncwarp();                                  // the previous tile's scales are read
-  *reinterpret_cast<float2*>(col + 2 * lane) = __half22float2(p.col);   // K: 0..31, V: 32..63
+  *reinterpret_cast<float2*>(col + 2 * lane) = __half22float2(p.col);
   __syncwarp();
+  if (!in) return;
   const uint64_t bias2 = f2pack(-8388608.f, -8388608.f);
-  if (kin) {
-    // K: 4 chunks of 8 channels of token `lane` of the half
-    const float kr = h2f(p.kr);
-    const float ks = h2f(p.ks) * kr, kz = h2f(p.kz) * kr;
+  if constexpr (!V) {
+    // K: 8 chunks of 8 channels of token `lane` of the half
+    const float kr = h2f(p.r[0]);
+    const float ks = h2f(p.s[0]) * kr, kz = h2f(p.z[0]) * kr;
     const uint64_t ks2 = f2pack(ks, ks), kz2 = f2pack(kz, kz);
-    unsigned char* kbase = kv + (pw >> 1) * (kHalf * 128);
+    unsigned char* kbase = kv + w * (kHalf * 128);
 #pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      const uint32_t w = p.kc[c * KB / 4] >> (c * 8 * KB % 32);
+    for (int c = 0; c < 8; ++c) {
+      const uint32_t cw = p.c[0][c * BITS / 4] >> (c * 8 * BITS % 32);
       const float4 c0 = *reinterpret_cast<const float4*>(col + 8 * c);
       const float4 c1 = *reinterpret_cast<const float4*>(col + 8 * c + 4);
       const uint64_t cc[4] = {f2pack(c0.x, c0.y), f2pack(c0.z, c0.w), f2pack(c1.x, c1.y),
@@ -223,7 +235,7 @@ __device__ __forceinline__ void build_coded(const Packed<KB, VB>& p, bool kin, b
       uint32_t h[4], l[4];
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
-        const uint64_t code = fadd2(f2pack(code_biased<KB>(w, 2 * i), code_biased<KB>(w, 2 * i + 1)), bias2);
+        const uint64_t code = fadd2(f2pack(code_biased<BITS>(cw, 2 * i), code_biased<BITS>(cw, 2 * i + 1)), bias2);
         const uint64_t k2 = fmul2(ffma2(code, ks2, kz2), cc[i]);
         float a, b;
         f2unpack(k2, a, b);
@@ -233,33 +245,32 @@ __device__ __forceinline__ void build_coded(const Packed<KB, VB>& p, bool kin, b
         f2unpack(fadd2(k2, f2pack(-__uint_as_float(ab), -__uint_as_float(bb))), ra, rb);
         l[i] = pack_bf16(ra, rb);
       }
-      const int off = sw128(lane, (pw & 1) * 4 + c);
+      const int off = sw128(lane, c);
       *reinterpret_cast<uint4*>(kbase + kKH + off) = make_uint4(h[0], h[1], h[2], h[3]);
       *reinterpret_cast<uint4*>(kbase + kKL + off) = make_uint4(l[0], l[1], l[2], l[3]);
     }
-  }
-  if (vin) {
-    // V^T: rows 16 pw + e, tokens 2 lane and 2 lane + 1
+  } else {
+    // V^T: rows 32 w + e, tokens 2 lane and 2 lane + 1
     float s[2], z[2];
 #pragma unroll
     for (int u = 0; u < 2; ++u) {
-      const float vr = h2f(p.vr[u]);
-      s[u] = h2f(p.vs[u]) * vr;
-      z[u] = h2f(p.vz[u]) * vr;
+      const float vr = h2f(p.r[u]);
+      s[u] = h2f(p.s[u]) * vr;
+      z[u] = h2f(p.z[u]) * vr;
     }
     const uint64_t vs2 = f2pack(s[0], s[1]), vz2 = f2pack(z[0], z[1]);
-    const float* vcol = col + 32 + (lane >> 4) * 16;
-    unsigned char* vbase = kv + kVT + pw * 16 * 128 + (lane & 3) * 4;
+    const float* vcol = col + (lane >> 4) * 32;
+    unsigned char* vbase = kv + kVT + w * 32 * 128 + (lane & 3) * 4;
 #pragma unroll
-    for (int c = 0; c < 4; ++c) {
+    for (int c = 0; c < 8; ++c) {
       const float4 c4 = *reinterpret_cast<const float4*>(vcol + 4 * c);
       const float cc[4] = {c4.x, c4.y, c4.z, c4.w};
-      const uint32_t w0 = p.vc[0][c * VB / 8] >> (c * 4 * VB % 32);
-      const uint32_t w1 = p.vc[1][c * VB / 8] >> (c * 4 * VB % 32);
+      const uint32_t w0 = p.c[0][c * BITS / 8] >> (c * 4 * BITS % 32);
+      const uint32_t w1 = p.c[1][c * BITS / 8] >> (c * 4 * BITS % 32);
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
         const int e = 4 * c + i;
-        const uint64_t code = fadd2(f2pack(code_biased<VB>(w0, i), code_biased<VB>(w1, i)), bias2);
+        const uint64_t code = fadd2(f2pack(code_biased<BITS>(w0, i), code_biased<BITS>(w1, i)), bias2);
         float a, b;
         f2unpack(fmul2(ffma2(code, vs2, vz2), f2pack(cc[i], cc[i])), a, b);
         *reinterpret_cast<uint32_t*>(vbase + e * 128 + (((lane >> 2) ^ (e & 7)) << 4)) = pack_h2(a, b);
@@ -268,57 +279,100 @@ __device__ __forceinline__ void build_coded(const Packed<KB, VB>& p, bool kin, b
   }
 }
 
-// The full-precision parts of the tile at t0 (sinks, staged tokens, zeros beyond
-// T): of K 32 tokens at t0 + 32 rank (kin false), of V the halves vin0, vin1 name
-// false.  A warp takes every eighth token; all its rows are loaded before the
-// first is rotated forward.
+// The full-precision tokens (sinks, staged tokens, zeros beyond T) of a tile.  Keys:
+// the 32 at t0, into rows 0 .. 31 of the share.  Values: this CTA's half of the
+// channels of the halves of the tile at t0 that in0, in1 do not name as coded.
+// A warp takes four tokens at a time; all its rows are loaded before the first
+// is rotated forward.
+template <bool V>
 __device__ __noinline__ void build_full(const Geom& g, int b, int h, int t0, int T, uint32_t rank,
-                                        bool kin, bool vin0, bool vin1, int pw, int lane,
-                                        unsigned char* kv) {
-  constexpr int NT = kHalf / kProdWarps;
-  uint4 raw[3][NT];
+                                        bool in0, bool in1, int w, int lane, unsigned char* kv) {
+  constexpr int NW = kProdWarps / 2, NT = (V ? kTok : kHalf) / (4 * NW);
+  const int sub = lane & 7;
+  uint4 raw[NT][4];
 #pragma unroll
-  for (int s = 0; s < 3; ++s)                    // K, V half 0, V half 1
-#pragma unroll
-    for (int i = 0; i < NT; ++i) {
-      const int t = t0 + (s == 0 ? (int)rank : s - 1) * kHalf + pw + kProdWarps * i;
-      raw[s][i] = make_uint4(0, 0, 0, 0);
-      if (!(s == 0 ? kin : s == 1 ? vin0 : vin1) && t < T) {
-        const __nv_bfloat16* src =
-            t < g.S ? plane_ptr<__nv_bfloat16>(g, s ? KVQ_PLANE_V_FULL : KVQ_PLANE_K_FULL, b, h, t, 0)
-                    : plane_ptr<__nv_bfloat16>(g, s ? KVQ_PLANE_V_PEND : KVQ_PLANE_K_PEND, b, h,
+  for (int i = 0; i < NT; ++i) {
+    const int t = t0 + 4 * (w + NW * i) + (lane >> 3);
+    const __nv_bfloat16* src = nullptr;
+    if (t < T && !(i < NT / 2 || !V ? in0 : in1))
+      src = t < g.S ? plane_ptr<__nv_bfloat16>(g, V ? KVQ_PLANE_V_FULL : KVQ_PLANE_K_FULL, b, h, t, 0)
+                    : plane_ptr<__nv_bfloat16>(g, V ? KVQ_PLANE_V_PEND : KVQ_PLANE_K_PEND, b, h,
                                                (t - g.S) % kG, 0);
-        raw[s][i] = *reinterpret_cast<const uint4*>(src + 8 * lane);
-      }
-    }
+    load_chunks(src, sub, raw[i]);
+  }
 #pragma unroll
-  for (int s = 0; s < 3; ++s) {
-    if (s == 0 ? kin : s == 1 ? vin0 : vin1) continue;
+  for (int i = 0; i < NT; ++i) {
+    if (i < NT / 2 || !V ? in0 : in1) continue;
+    const int r = 4 * (w + NW * i) + (lane >> 3);
+    float x[32];
+    unpack_chunks(raw[i], x);
+    if constexpr (!V) {
+      fwht256(x, sub);
 #pragma unroll
-    for (int i = 0; i < NT; ++i) {
-      const int r = pw + kProdWarps * i;
-      float x[8];
-      unpack8(raw[s][i], x);
-      fwht256(x, lane);
-      if (s == 0) {
+      for (int k = 0; k < 4; ++k) {
         uint32_t hw[4], lw[4];
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
-          const uint32_t a = __float_as_uint(x[2 * e]) & 0xFFFF0000u, c = __float_as_uint(x[2 * e + 1]) & 0xFFFF0000u;
+          const float x0 = x[8 * k + 2 * e], x1 = x[8 * k + 2 * e + 1];
+          const uint32_t a = __float_as_uint(x0) & 0xFFFF0000u, c = __float_as_uint(x1) & 0xFFFF0000u;
           hw[e] = __byte_perm(a, c, 0x7632);
-          lw[e] = pack_bf16(x[2 * e] - __uint_as_float(a), x[2 * e + 1] - __uint_as_float(c));
+          lw[e] = pack_bf16(x0 - __uint_as_float(a), x1 - __uint_as_float(c));
         }
-        unsigned char* d = kv + (lane >> 3) * (kHalf * 128) + sw128(r, lane & 7);
+        unsigned char* d = kv + k * (kHalf * 128) + sw128(r, sub);
         *reinterpret_cast<uint4*>(d + kKH) = make_uint4(hw[0], hw[1], hw[2], hw[3]);
         *reinterpret_cast<uint4*>(d + kKL) = make_uint4(lw[0], lw[1], lw[2], lw[3]);
-      } else if ((uint32_t)(lane >> 4) == rank) {
-        const int tk = (s - 1) * kHalf + r;
+      }
+    } else {
+      // the stage across the channel halves, then the half that is this CTA's
+      const float sg = rank ? -1.f : 1.f;
+      float y[16];
+#pragma unroll
+      for (int e = 0; e < 16; ++e) y[e] = fmaf(sg, x[16 + e], x[e]);
+      fwht256(y, sub);
+#pragma unroll
+      for (int k = 0; k < 2; ++k)
 #pragma unroll
         for (int e = 0; e < 8; ++e)
-          *reinterpret_cast<__half*>(kv + kVT + sw128(8 * (lane & 15) + e, tk >> 3) + (tk & 7) * 2) =
-              __float2half_rn(x[e]);
-      }
+          *reinterpret_cast<__half*>(kv + kVT + sw128(8 * (sub + 8 * k) + e, r >> 3) + (r & 7) * 2) =
+              __float2half_rn(y[8 * k + e]);
     }
+  }
+}
+
+// The tile loop of the warps that build keys (V false) or values.
+template <int BITS, bool V>
+__device__ __forceinline__ void produce(const Geom& g, int b, int h, int T, int ntiles, uint32_t rank,
+                                        int w, int lane, float* col, unsigned char* kv_base,
+                                        uint64_t* kv_full, uint64_t* kv_free, volatile int* abort) {
+  // S and the coded tokens are multiples of 32, so 32 tokens are either all
+  // coded, inside one block's column scales, or all full precision
+  const int nbq = kvarn_nblocks(T, g.S, kG) * kG;
+  auto coded = [&](int t0) { return t0 >= g.S && t0 < g.S + nbq; };
+  Rows rows = {};
+  if (nbq > 0) {
+    rows.c = plane_ptr<uint8_t>(g, V ? KVQ_PLANE_V_CODES : KVQ_PLANE_K_CODES, b, h, 0);
+    rows.s = plane_ptr<__half>(g, V ? KVQ_PLANE_V_SCALE : KVQ_PLANE_K_SCALE, b, h, 0);
+    rows.z = plane_ptr<__half>(g, V ? KVQ_PLANE_V_ZERO : KVQ_PLANE_K_ZERO, b, h, 0);
+    rows.r = plane_ptr<__half>(g, V ? KVQ_PLANE_V_ROW : KVQ_PLANE_K_ROW, b, h, 0);
+    rows.col = plane_ptr<__half>(g, V ? KVQ_PLANE_V_COL : KVQ_PLANE_K_COL, b, h, 0);
+  }
+  Packed<BITS, V> cur = {}, nxt = {};
+  if (coded(0) || coded(kHalf)) load_packed<BITS, V>(rows, 0 - g.S, nbq, rank, w, lane, nxt);
+  for (int j = 0; j < ntiles; ++j) {
+    const int t0 = j * kTok, t1 = t0 + kTok, kb = j % kKvBufs;
+    cur = nxt;
+    if (j + 1 < ntiles && (coded(t1) || coded(t1 + kHalf)))
+      load_packed<BITS, V>(rows, t1 - g.S, nbq, rank, w, lane, nxt);
+    const bool ok = j < kKvBufs || mbar_wait_or_abort(&kv_free[kb], ((j - kKvBufs) / kKvBufs) & 1, abort);
+    if (!__all_sync(0xffffffffu, ok)) break;
+    unsigned char* kv = kv_base + kb * kKvB;
+    const bool in0 = coded(V ? t0 : t0 + (int)rank * kHalf), in1 = V ? coded(t0 + kHalf) : in0;
+    if (in0 || in1) build_coded<BITS, V>(cur, V && lane >= 16 ? in1 : in0, w, lane, col, kv);
+    if (!in0 || !in1)
+      build_full<V>(g, b, h, V ? t0 : t0 + (int)rank * kHalf, T, rank, in0, in1, w, lane, kv);
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // for the MMAs' reads
+    __syncwarp();
+    if (lane == 0) mbar_arrive_pair(mapa(&kv_full[kb], 0));
   }
 }
 
@@ -368,37 +422,41 @@ attend_prefill_kvarn_kernel(Geom g, const __nv_bfloat16* __restrict__ q, int L, 
                  ::"r"(smem_u32(&tmem_base)));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;");
   }
-  // rotate the query rows: the high part into the swizzled Q tile, the bf16
-  // remainder into a staging row (then TMEM); a warp's rows are loaded five at a time
-  constexpr int kRows = 5;
-  for (int r0 = warp; r0 < kM; r0 += kRows * (kThreads / 32)) {
-    uint4 raw[kRows];
+  // rotate the query rows, four to a warp: the high part into the swizzled Q tile,
+  // the bf16 remainder into a staging row (then TMEM)
+  const int sub = lane & 7;
+  constexpr int kPasses = (kM / 4 + kThreads / 32 - 1) / (kThreads / 32);
+  {
+    uint4 raw[kPasses][4];
 #pragma unroll
-    for (int k = 0; k < kRows; ++k) {
-      const int r = r0 + k * (kThreads / 32), hl = r / nq, qi = r % nq;
-      raw[k] = make_uint4(0, 0, 0, 0);
-      if (r < kM && hl < grp && qi < nql)
-        raw[k] = *reinterpret_cast<const uint4*>(
-            q + (((int64_t)b * g.Hq + hkv * grp + hl) * L + q0 + qi) * kD + 8 * lane);
+    for (int i = 0; i < kPasses; ++i) {
+      const int r = 4 * (warp + i * (kThreads / 32)) + (lane >> 3), hl = r / nq, qi = r % nq;
+      load_chunks(r < kM && hl < grp && qi < nql
+                      ? q + (((int64_t)b * g.Hq + hkv * grp + hl) * L + q0 + qi) * kD
+                      : nullptr,
+                  sub, raw[i]);
     }
 #pragma unroll
-    for (int k = 0; k < kRows; ++k) {
-      const int r = r0 + k * (kThreads / 32);
-      if (r >= kM) break;
-      float x[8];
-      unpack8(raw[k], x);
-      fwht256(x, lane);
-      uint32_t hw[4], lw[4];
+    for (int i = 0; i < kPasses; ++i) {
+      const int r = 4 * (warp + i * (kThreads / 32)) + (lane >> 3);
+      if (r >= kM) break;                              // the whole warp: kM is a multiple of 4
+      float x[32];
+      unpack_chunks(raw[i], x);
+      fwht256(x, sub);
 #pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        hw[e] = pack_bf16(x[2 * e], x[2 * e + 1]);
-        lw[e] = pack_bf16(x[2 * e] - __uint_as_float(hw[e] << 16),
-                          x[2 * e + 1] - __uint_as_float(hw[e] & 0xFFFF0000u));
+      for (int k = 0; k < 4; ++k) {
+        uint32_t hw[4], lw[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const float x0 = x[8 * k + 2 * e], x1 = x[8 * k + 2 * e + 1];
+          hw[e] = pack_bf16(x0, x1);
+          lw[e] = pack_bf16(x0 - __uint_as_float(hw[e] << 16), x1 - __uint_as_float(hw[e] & 0xFFFF0000u));
+        }
+        *reinterpret_cast<uint4*>(smem + kQOff + k * (kM * 128) + sw128(r, sub)) =
+            make_uint4(hw[0], hw[1], hw[2], hw[3]);
+        *reinterpret_cast<uint4*>(smem + kKvOff + r * kQlPitch + 16 * (sub + 8 * k)) =
+            make_uint4(lw[0], lw[1], lw[2], lw[3]);
       }
-      *reinterpret_cast<uint4*>(smem + kQOff + (lane >> 3) * (kM * 128) + sw128(r, lane & 7)) =
-          make_uint4(hw[0], hw[1], hw[2], hw[3]);
-      *reinterpret_cast<uint4*>(smem + kKvOff + r * kQlPitch + 16 * lane) =
-          make_uint4(lw[0], lw[1], lw[2], lw[3]);
     }
   }
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -430,43 +488,12 @@ attend_prefill_kvarn_kernel(Geom g, const __nv_bfloat16* __restrict__ q, int L, 
   if (warp >= 4 && warp < 12) {
     // ---------------- producers: reconstruct K and V tiles ----------------
     const int pw = warp - 4;
-    const int nbq = kvarn_nblocks(T, g.S, kG) * kG;
     float* col = reinterpret_cast<float*>(smem + kColOff) + pw * 64;
-    Rows rows = {};
-    if (nbq > 0) {
-      rows.kc = plane_ptr<uint8_t>(g, KVQ_PLANE_K_CODES, b, hkv, 0);
-      rows.vc = plane_ptr<uint8_t>(g, KVQ_PLANE_V_CODES, b, hkv, 0);
-      rows.ks = plane_ptr<__half>(g, KVQ_PLANE_K_SCALE, b, hkv, 0);
-      rows.kz = plane_ptr<__half>(g, KVQ_PLANE_K_ZERO, b, hkv, 0);
-      rows.vs = plane_ptr<__half>(g, KVQ_PLANE_V_SCALE, b, hkv, 0);
-      rows.vz = plane_ptr<__half>(g, KVQ_PLANE_V_ZERO, b, hkv, 0);
-      rows.kr = plane_ptr<__half>(g, KVQ_PLANE_K_ROW, b, hkv, 0);
-      rows.vr = plane_ptr<__half>(g, KVQ_PLANE_V_ROW, b, hkv, 0);
-      rows.kcol = plane_ptr<__half>(g, KVQ_PLANE_K_COL, b, hkv, 0);
-      rows.vcol = plane_ptr<__half>(g, KVQ_PLANE_V_COL, b, hkv, 0);
-    }
-    // S and the coded tokens are multiples of 32, so 32 tokens are either all
-    // coded, inside one block's column scales, or all full precision
-    auto coded = [&](int t0) { return t0 >= g.S && t0 < g.S + nbq; };
-    Packed<KB, VB> cur = {}, nxt = {};
-    if (coded(0) || coded(kHalf)) load_packed<KB, VB>(rows, 0 - g.S, nbq, rank, pw, lane, nxt);
-    for (int j = 0; j < ntiles; ++j) {
-      const int t0 = j * kTok, t1 = t0 + kTok, kb = j % kKvBufs;
-      cur = nxt;
-      if (j + 1 < ntiles && (coded(t1) || coded(t1 + kHalf)))
-        load_packed<KB, VB>(rows, t1 - g.S, nbq, rank, pw, lane, nxt);
-      const bool ok = j < kKvBufs || mbar_wait_or_abort(&kv_free[kb], ((j - kKvBufs) / kKvBufs) & 1, abort);
-      if (!producers_all(ok)) break;
-      unsigned char* kv = smem + kKvOff + kb * kKvB;
-      const bool kin = coded(t0 + (int)rank * kHalf), vin0 = coded(t0), vin1 = coded(t0 + kHalf);
-      if (kin || vin0 || vin1)
-        build_coded<KB, VB>(cur, kin, lane < 16 ? vin0 : vin1, pw, lane, col, kv);
-      if (!kin || !vin0 || !vin1)
-        build_full(g, b, hkv, t0, T, rank, kin, vin0, vin1, pw, lane, kv);
-      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // for the MMAs' reads
-      __syncwarp();
-      if (lane == 0) mbar_arrive_pair(mapa(&kv_full[kb], 0));
-    }
+    if (pw < kProdWarps / 2)
+      produce<KB, false>(g, b, hkv, T, ntiles, rank, pw, lane, col, smem + kKvOff, kv_full, kv_free, abort);
+    else
+      produce<VB, true>(g, b, hkv, T, ntiles, rank, pw - kProdWarps / 2, lane, col, smem + kKvOff, kv_full,
+                        kv_free, abort);
   } else if (warp == 12) {
     if (rank == 0) {
       // ---------------- MMA issuer ----------------
@@ -660,16 +687,24 @@ attend_prefill_kvarn_kernel(Geom g, const __nv_bfloat16* __restrict__ q, int L, 
   tc_fence_before();
   __syncthreads();
   if (good) {
-    for (int r = warp; r < kM; r += kThreads / 32) {
+    for (int r = 4 * warp + (lane >> 3); r < kM; r += 4 * (kThreads / 32)) {
       const int hl = r / nq, qi = r % nq;
+      float x[32];
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+#pragma unroll
+        for (int e = 0; e < 8; e += 4) {
+          const float4 u = *reinterpret_cast<const float4*>(os + r * kOPitch + 8 * (sub + 8 * k) + e);
+          x[8 * k + e] = u.x; x[8 * k + e + 1] = u.y; x[8 * k + e + 2] = u.z; x[8 * k + e + 3] = u.w;
+        }
+      fwht256(x, sub);
       if (hl >= grp || qi >= nql) continue;
-      const float4 u = *reinterpret_cast<const float4*>(os + r * kOPitch + 8 * lane);
-      const float4 v = *reinterpret_cast<const float4*>(os + r * kOPitch + 8 * lane + 4);
-      float x[8] = {u.x, u.y, u.z, u.w, v.x, v.y, v.z, v.w};
-      fwht256(x, lane);
       __nv_bfloat16* dst = out + (((int64_t)b * g.Hq + hkv * grp + hl) * L + q0 + qi) * kD;
-      *reinterpret_cast<uint4*>(dst + 8 * lane) = make_uint4(pack_bf16(x[0], x[1]), pack_bf16(x[2], x[3]),
-                                                             pack_bf16(x[4], x[5]), pack_bf16(x[6], x[7]));
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        *reinterpret_cast<uint4*>(dst + 8 * (sub + 8 * k)) =
+            make_uint4(pack_bf16(x[8 * k], x[8 * k + 1]), pack_bf16(x[8 * k + 2], x[8 * k + 3]),
+                       pack_bf16(x[8 * k + 4], x[8 * k + 5]), pack_bf16(x[8 * k + 6], x[8 * k + 7]));
     }
   }
   if (threadIdx.x == 0 && !good) atomicOr(err, 8);
