@@ -34,18 +34,19 @@
 // parts.  Q_hi stays in shared memory (the MMAs read it once per K step for
 // both K parts), Q_lo in 128 TMEM columns next to O's 256 and S's 2 x 64; that
 // leaves shared memory for three 48 KB shares of K/V tiles.
-// What bounds it: a 64-token tile takes about 3,000 cycles, the MMAs 2,050 of them;
+// What bounds it: a 64-token tile takes about 2,800 cycles, the MMAs 2,050 of them;
 // with two score buffers Q K^T of a tile starts when P V of the tile two before it
 // has completed, so the pipe idles while that is signalled, and building the tiles
 // (1,850 cycles of each producer warp) slows the chain (2,700 cycles without it).
 // A CTA's start and end (rotating queries, sinks and output rows) take 50,000
 // cycles.  8192 tokens, 16 query heads, 8 kv heads, one sequence: 7667 us on
 // mma.sync (64 rows a CTA, 16-token tiles reconstructed by all its warps), 1526
-// with one CTA building 32-token tiles of K and V for 128 rows, 898 here: 1,480 as
+// with one CTA building 32-token tiles of K and V for 128 rows, 824 here: 1,480 as
 // a pair, 1,380 with arrivals that do not wait (mbar_arrive_pair), 1,100 with the
 // packed tile loaded without a branch that divides the warp (load_packed) and
 // rows of sinks, queries and outputs loaded together, 994 with K and V built by
-// warps of their own (no spills), 898 with four rows to a warp in the rotation.
+// warps of their own (no spills), 898 with four rows to a warp in the rotation,
+// 824 with the issuer blocking instead of polling.
 // Every wait is bounded and also gives up when another role has timed out;
 // the issuer drains its MMAs before TMEM is freed, and a timed-out CTA stores
 // nothing and sets the library's error word.
@@ -497,78 +498,58 @@ attend_prefill_kvarn_kernel(Geom g, const __nv_bfloat16* __restrict__ q, int L, 
   } else if (warp == 12) {
     if (rank == 0) {
       // ---------------- MMA issuer ----------------
-      // S of the next tile as soon as its K/V tile is built and its S buffer is
-      // free, P V of the next tile as soon as its P is written; the tensor pipe
-      // executes in issue order.  The whole warp runs the loop and one elected
-      // lane issues.  A K step of 16 elements advances a descriptor by 32 bytes.
+      // Q K^T of tile j + 1, then P V of tile j, each blocking on what it needs (a
+      // loop that polled for whichever came first answered later: 898 us for 8192
+      // tokens, 855 with a warp for each product, 824 so).  The whole warp runs
+      // the loop and one elected lane issues.  A K step of 16 elements advances a
+      // descriptor by 32 bytes.
       constexpr uint32_t id_qk = idesc_bf16(2 * kM, kTok);
       constexpr uint32_t id_pv = idesc_f16(2 * kM, kD);
       const uint64_t qdesc0 = sw128_desc(smem + kQOff);
       const uint64_t kdesc0 = sw128_desc(smem + kKvOff);
       const uint64_t vdesc0 = sw128_desc(smem + kKvOff + kVT);
       const bool leader = elect_one();
-      int nqk = 0, npv = 0;
-      long idle = 0;
-      uint64_t idle_since = 0;
-      while (npv < ntiles) {
-        bool progressed = false;
-        if (nqk < ntiles) {
-          const int kb = nqk % kKvBufs, sb = nqk % kSBufs;
-          bool ready = false;
-          if (lane == 0)
-            ready = mbar_test_cluster(&kv_full[kb], (nqk / kKvBufs) & 1) &&
-                    (nqk < kSBufs || mbar_test(&s_free[sb], ((nqk - kSBufs) / kSBufs) & 1));
-          if (__shfl_sync(0xffffffffu, ready, 0)) {
-            tc_fence_after();
-            if (leader) {
-              const uint32_t ts = tmem + kTmS + sb * kTok;
+      bool ok = true;
+      for (int i = 0; i <= ntiles; ++i) {
+        if (i < ntiles) {
+          const int j = i, kb = j % kKvBufs, sb = j % kSBufs;
+          ok = warp_wait_cluster(&kv_full[kb], (j / kKvBufs) & 1, abort) &&
+               (j < kSBufs || warp_wait(&s_free[sb], ((j - kSBufs) / kSBufs) & 1, abort));
+          if (!ok) break;
+          tc_fence_after();
+          if (leader) {
+            const uint32_t ts = tmem + kTmS + sb * kTok;
 #pragma unroll
-              for (int kk = 0; kk < kD / 16; ++kk) {
-                // Q atom: 128 rows x 128 B (1024 units); K atom: 32 rows x 128 B (256 units)
-                const uint64_t qd = qdesc0 + (uint64_t)((kk >> 2) * 1024 + (kk & 3) * 2);
-                const uint64_t kd = kdesc0 + (uint64_t)(kb * (kKvB >> 4) + (kk >> 2) * 256 + (kk & 3) * 2);
-                umma_pair_a_fill(ts, qd, kd + (kKH >> 4), id_qk, kk > 0);     // Q_hi read once
-                umma_pair_a_lastuse(ts, qd, kd + (kKL >> 4), id_qk, 1);       // for K hi and lo
-                umma_pair_ts(ts, tmem + kTmQ + kk * 8, kd + (kKH >> 4), id_qk, 1);
-              }
-              umma_commit_pair(&s_full[sb]);
+            for (int kk = 0; kk < kD / 16; ++kk) {
+              // Q atom: 128 rows x 128 B (1024 units); K atom: 32 rows x 128 B (256 units)
+              const uint64_t qd = qdesc0 + (uint64_t)((kk >> 2) * 1024 + (kk & 3) * 2);
+              const uint64_t kd = kdesc0 + (uint64_t)(kb * (kKvB >> 4) + (kk >> 2) * 256 + (kk & 3) * 2);
+              umma_pair_a_fill(ts, qd, kd + (kKH >> 4), id_qk, kk > 0);     // Q_hi read once
+              umma_pair_a_lastuse(ts, qd, kd + (kKL >> 4), id_qk, 1);       // for K hi and lo
+              umma_pair_ts(ts, tmem + kTmQ + kk * 8, kd + (kKH >> 4), id_qk, 1);
             }
-            __syncwarp();
-            ++nqk;
-            progressed = true;
+            umma_commit_pair(&s_full[sb]);
           }
+          __syncwarp();
         }
-        if (npv < nqk) {
-          const int sb = npv % kSBufs, kb = npv % kKvBufs;
-          bool ready = false;
-          if (lane == 0) ready = mbar_test_cluster(&p_full[sb], (npv / kSBufs) & 1);
-          if (__shfl_sync(0xffffffffu, ready, 0)) {
-            tc_fence_after();
-            if (leader) {
-              const uint32_t tp = tmem + kTmS + sb * kTok;               // P (fp16 pairs) over S
+        if (i > 0) {
+          const int j = i - 1, kb = j % kKvBufs, sb = j % kSBufs;
+          ok = warp_wait_cluster(&p_full[sb], (j / kSBufs) & 1, abort);
+          if (!ok) break;
+          tc_fence_after();
+          if (leader) {
+            const uint32_t tp = tmem + kTmS + sb * kTok;               // P (fp16 pairs) over S
 #pragma unroll
-              for (int kk = 0; kk < kTok / 16; ++kk)
-                umma_pair_ts(tmem + kTmO, tp + kk * 8, vdesc0 + (uint64_t)(kb * (kKvB >> 4) + kk * 2), id_pv,
-                        (npv > 0 || kk > 0) ? 1u : 0u);
-              umma_commit_pair(&s_free[sb]);            // S/P buffer free, and O holds tile npv
-              umma_commit_pair(&kv_free[kb]);
-            }
-            __syncwarp();
-            ++npv;
-            progressed = true;
+            for (int kk = 0; kk < kTok / 16; ++kk)
+              umma_pair_ts(tmem + kTmO, tp + kk * 8, vdesc0 + (uint64_t)(kb * (kKvB >> 4) + kk * 2), id_pv,
+                           (j > 0 || kk > 0) ? 1u : 0u);
+            umma_commit_pair(&s_free[sb]);            // S/P buffer free, and O holds tile j
+            umma_commit_pair(&kv_free[kb]);
           }
-        }
-        if (progressed) {
-          idle = 0;
-        } else {
-          if (idle == 0) idle_since = global_ns();
-          __nanosleep(20);
-          const bool stop = (++idle & 63) == 0 && (*abort || global_ns() - idle_since > kWaitNs);
-          if (__shfl_sync(0xffffffffu, stop, 0)) break;   // the whole warp leaves together
+          __syncwarp();
         }
       }
-      if (lane == 0 && npv < ntiles) *abort = 1;
-      if (leader) umma_commit_pair(&done_bar);        // every MMA issued above has completed
+      if (leader) umma_commit_pair(&done_bar);   // every MMA issued above has completed
       if (lane == 0 && !mbar_wait(&done_bar, 0)) *abort = 1;
       __syncwarp();
     }
