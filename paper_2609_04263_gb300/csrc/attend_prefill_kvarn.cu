@@ -513,7 +513,7 @@ attend_prefill_kvarn_kernel(Geom g, const __nv_bfloat16* __restrict__ q, int L, 
       for (int i = 0; i <= ntiles; ++i) {
         if (i < ntiles) {
           const int j = i, kb = j % kKvBufs, sb = j % kSBufs;
-          ok = warp_wait_cluster(&kv_full[kb], (j / kKvBufs) & 1, abort) &&
+          ok = warp_wait(&kv_full[kb], (j / kKvBufs) & 1, abort) &&
                (j < kSBufs || warp_wait(&s_free[sb], ((j - kSBufs) / kSBufs) & 1, abort));
           if (!ok) break;
           tc_fence_after();
@@ -534,7 +534,7 @@ attend_prefill_kvarn_kernel(Geom g, const __nv_bfloat16* __restrict__ q, int L, 
         }
         if (i > 0) {
           const int j = i - 1, kb = j % kKvBufs, sb = j % kSBufs;
-          ok = warp_wait_cluster(&p_full[sb], (j / kSBufs) & 1, abort);
+          ok = warp_wait(&p_full[sb], (j / kSBufs) & 1, abort);
           if (!ok) break;
           tc_fence_after();
           if (leader) {

@@ -4,30 +4,44 @@
 // value is the cache's reconstruction (codes x scale + offset, or the
 // full-precision residual window of a KIVI cache).
 //
-// One CTA = 256 query rows of one (sequence, kv head): the g query heads of
-// the kv head x 256/g consecutive queries, head-major, split into two
-// 128-row query tiles A (rows 0..127) and B (rows 128..255) that share every
-// reconstructed key/value tile.  Keys and values stream in tiles of 64
-// tokens.  Four roles:
-//   producers (warps 8-11): reconstruct each K/V tile once for both query
-//     tiles: K as a bf16 high part (the fp32 value truncated) plus the bf16
-//     of the remainder (about 16 significant bits: large logits need more
-//     than bf16's 8), V as fp16 computed in packed half2 arithmetic
-//     (code x scale + offset, one rounding), into two to four shared
-//     tile buffers in the 128-byte-swizzled K-major layout of the MMA descriptors
-//     (V transposed: D rows, tokens along K);
-//   issuer (warp 12, one thread): per KV tile j, first O_X += P_X V of tile
-//     j - 1 into a TMEM accumulator (128 x D fp32) per query tile X = A, B
-//     (this frees tile j - 1's K/V buffer, so the producers run a tile
-//     ahead), then S_X = Q_X K_hi^T + Q_X K_lo^T of tile j into
-//     double-buffered TMEM tiles (128 x 64 fp32); completions are signalled
-//     by tcgen05.commit on mbarriers;
+// A CTA holds 256 query rows of one (sequence, kv head): the g query heads of the
+// kv head x 256/g consecutive queries, head-major, as two 128-row query tiles A
+// and B that share every reconstructed key/value tile of 64 tokens.  At head_dim
+// 128 two CTAs (a cluster, one MMA pair) share it too: the second's queries follow
+// the first's, the MMAs take tile A (or B) of both, and of K each CTA builds 32 of
+// the tokens, of V the 64 tokens' half of the channels, which is how a pair shares
+// the second operand of its MMAs.  Four roles:
+//   loader (warp 13): the packed rows of a tile, a bulk copy per plane;
+//   producers (warps 8-11): reconstruct the tile, or the CTA's share of it: K as a
+//     bf16 high part (the fp32 value truncated) plus the bf16 of the remainder
+//     (about 16 significant bits: large logits need more than bf16's 8), V as fp16
+//     computed in packed half2 arithmetic (code x scale + offset, one rounding),
+//     into four shared tile buffers in the 128-byte-swizzled K-major layout of the
+//     MMA descriptors (V transposed: channels x tokens);
+//   issuer (warp 12, of a pair the first CTA's; one lane issues): S_X = Q_X K_hi^T
+//     + Q_X K_lo^T into double-buffered TMEM tiles (128 x 64 fp32 in each CTA) and
+//     O_X += P_X V into 128 x D fp32 for X = A, B; completions are signalled by
+//     tcgen05.commit on mbarriers (of both CTAs);
 //   softmax A (warps 0-3) and B (warps 4-7): thread r owns row r of its
 //     query tile (TMEM lane r): reads the 64 scores, masks causally, keeps
-//     the running maximum m and sum l in log2 units, writes P as fp16 into
-//     its query tile's P buffer.  O is rescaled (in TMEM) only when a row's
-//     maximum grows by more than 8 (so P stays <= 2^8 in fp16); the final
-//     O / l is stored as bf16.
+//     the running maximum m and sum l in log2 units, writes P as fp16 over
+//     its S tile.  O is rescaled (in TMEM) only when a row's maximum grows by
+//     more than 8 (so P stays <= 2^8 in fp16); the final O / l is stored as
+//     bf16.
+// The barriers that wake the issuer (tiles built, P written) sit in the first
+// CTA and count one arrival per warp.
+// What bounds it, per 64-token tile: D = 128, building K, 2,200 of 2,800 cycles
+// (2,300 without building: the MMAs, 1,540, and the waits between them and the
+// softmax warps); D = 64, the chain from scores over softmax to P V and the buffers
+// it frees, about 2,000 cycles, 1,060 of them softmax.
+//   2 x 8192 tokens, 32 / 8 heads of 128, KIVI 2-bit: 2081 us with two tile
+// buffers, 1745 with three, 1400 here.  With every loop unrolled the roles' code did
+// not fit the instruction cache (1.5 of 10 cycles an instruction went to fetching
+// it): 1,800 us as a pair, 1,480 with one copy of each product in the issuer, 1,420
+// with the build loops rolled up.
+//   4 x 2029 tokens, 32 / 4 heads of 64, affine 4-bit: 229 us with two tile buffers,
+// 199 with four, 179 here.  As a pair 192: less to build, which did not bound it,
+// and longer waits.
 // Every wait is bounded and also gives up when another role has timed out;
 // the issuer drains its MMAs before TMEM is freed, and a timed-out CTA
 // stores nothing and sets the library's error word.
@@ -42,27 +56,36 @@ using namespace tc;
 constexpr int kM = 128;              // rows per query tile (MMA M)
 constexpr int kTok = 64;             // tokens per KV tile
 constexpr int kRowsCta = 2 * kM;     // query rows per CTA
+constexpr int kProdWarps = 4;        // two build K, two V
 constexpr int kThreads = 14 * 32;    // 8 softmax, 4 producer, 1 issuer, 1 loader warp
 constexpr float kRescale = 8.f;      // log2 growth of a row maximum that forces a rescale
 
 // Shared memory (bytes from a 1024-aligned base).
 template <int D, int BITS>
 struct M256Layout {
+  // Two CTAs share each K/V tile where building it bounds the kernel: D = 128 takes
+  // 1745 us alone and 1400 paired, D = 64 179 alone and 192 paired (shapes above).
+  static constexpr bool PAIR = D == 128;
+  static constexpr int KT = PAIR ? kTok / 2 : kTok; // tokens of K per CTA
+  static constexpr int VC = PAIR ? D / 2 : D;       // channels of V per CTA
+  // A pair's CTA builds K with half of its producer threads and V with the others;
+  // a CTA alone with all of them K, then V.
+  static constexpr int NP = PAIR ? 64 : 128;
+  static constexpr int KC = KT * D / NP;            // channels of K per thread
+  static constexpr int UNROLL = PAIR ? 1 : 2;       // trips of the build loops unrolled
+  static constexpr int CV = VC * 8 / NP;            // channels of V per thread
+  // score tiles (TMEM) per query tile: what O (2 D columns) leaves of 512
+  static constexpr int SB = 2;
   // Reconstructed K/V tile buffers.  A buffer is held from the start of its build to
-  // the end of its P V, about three tile times of 2 x 128 rows: with two
-  // buffers the producers waited for half of the time (D = 64: 1,360 of 2,820
-  // cycles a tile) and the tensor pipe for them.  4 x 2029 tokens of 32 heads of
-  // 64, affine 4-bit: 229 us with two, 199 with four; 2 x 8192 tokens of 32 heads
-  // of 128, KIVI 2-bit: 2081 with two, 1745 with three (four do not fit, nor do
-  // three with 4-bit codes).
-  static constexpr int KVB = D == 64 ? 4 : BITS == 2 ? 3 : 2;
+  // the end of its P V, about three tile times.
+  static constexpr int KVB = 4;
   static constexpr int QT = kM * D * 2;             // one query tile: D/64 atoms of 16 KB
   static constexpr int Q_OFF = 0;
   static constexpr int KV_OFF = 2 * QT;
-  static constexpr int KH = 0;                      // K hi: D/64 atoms of 64 rows x 128 B
-  static constexpr int KL = kTok * D * 2;           // K lo: the same
-  static constexpr int VT = 2 * kTok * D * 2;       // V^T: D rows x 128 B (64 tokens)
-  static constexpr int KV_B = VT + D * 128;
+  static constexpr int KH = 0;                      // K hi: D/64 atoms of KT rows x 128 B
+  static constexpr int KL = KT * D * 2;             // K lo: the same
+  static constexpr int VT = 2 * KT * D * 2;         // V^T: VC rows x 128 B (64 tokens)
+  static constexpr int KV_B = VT + VC * 128;
   // packed tile as stored in the cache planes: 64 code rows of K and of V,
   // then four metadata pieces of 4 D bytes each (per-token group scales and
   // offsets of 64 tokens, or KIVI's per-channel scales and offsets of the
@@ -73,29 +96,60 @@ struct M256Layout {
                        RVZ = RVS + 4 * D;
   static constexpr int RAW_B = RVZ + 4 * D;
   static constexpr int RAW_OFF = KV_OFF + KVB * KV_B;
-  static constexpr int RAW = D == 128 && BITS == 2 ? 2 : 3;                 // packed-tile stages (copied ahead)
-  static constexpr int TOTAL = RAW_OFF + RAW * RAW_B;
+  static constexpr int RAW = 3;                     // packed-tile stages (copied ahead)
+  static constexpr int KS_OFF = RAW_OFF + RAW * RAW_B;   // KIVI: a key warp's fp32 scales and offsets
+  static constexpr int TOTAL = KS_OFF + NP / 32 * 2 * KC * 4;
   static constexpr int ALLOC = TOTAL + 1024;        // alignment slack
   static_assert(ALLOC <= 226 * 1024, "one CTA's shared memory");
 };
+
+// The instructions of one CTA or of a pair.
+template <bool PAIR>
+__device__ __forceinline__ void mma_a_fill(uint32_t d, uint64_t a, uint64_t b, uint32_t id, uint32_t acc) {
+  if (PAIR) umma_pair_a_fill(d, a, b, id, acc);
+  else umma_a_fill(d, a, b, id, acc);
+}
+template <bool PAIR>
+__device__ __forceinline__ void mma_a_lastuse(uint32_t d, uint64_t a, uint64_t b, uint32_t id, uint32_t acc) {
+  if (PAIR) umma_pair_a_lastuse(d, a, b, id, acc);
+  else umma_a_lastuse(d, a, b, id, acc);
+}
+template <bool PAIR>
+__device__ __forceinline__ void mma_ts(uint32_t d, uint32_t a, uint64_t b, uint32_t id, uint32_t acc) {
+  if (PAIR) umma_pair_ts(d, a, b, id, acc);
+  else umma_ts(d, a, b, id, acc);
+}
+template <bool PAIR>
+__device__ __forceinline__ void mma_commit(uint64_t* bar) {
+  if (PAIR) umma_commit_pair(bar);
+  else umma_commit(bar);
+}
+template <bool PAIR>
+__device__ __forceinline__ void arrive_first(uint64_t* bar) {   // on the first CTA's barrier
+  if (PAIR) mbar_arrive_pair(mapa(bar, 0));
+  else mbar_arrive(bar);
+}
+template <bool PAIR>
+__device__ __forceinline__ void tmem_alloc512(uint32_t* base) {
+  if (PAIR) {
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(smem_u32(base)));
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;");
+  } else {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(smem_u32(base)));
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+  }
+}
+template <bool PAIR>
+__device__ __forceinline__ void tmem_free512(uint32_t tmem) {
+  if (PAIR) asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, 512;" ::"r"(tmem));
+  else asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem));
+}
 
 __device__ __forceinline__ void bulk_copy(void* dst, const void* src, uint32_t bytes,
                                           uint64_t* bar) {
   asm volatile(
       "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
       ::"r"(smem_u32(dst)), "l"(src), "r"(bytes), "r"(smem_u32(bar)) : "memory");
-}
-
-// Barrier of the four producer warps (named barrier 1) that also returns
-// whether `ok` held in every producer thread, so all of them leave the tile
-// loop together.
-__device__ __forceinline__ bool producers_all(bool ok) {
-  uint32_t r;
-  asm volatile(
-      "{\n .reg .pred p, q;\n setp.ne.u32 p, %1, 0;\n"
-      " bar.red.and.pred q, 1, 128, p;\n selp.u32 %0, 1, 0, q;\n}\n"
-      : "=r"(r) : "r"((uint32_t)ok) : "memory");
-  return r != 0;
 }
 
 // Bytes of one packed tile the loader copies (codes of K and V, metadata).
@@ -151,28 +205,48 @@ __device__ __forceinline__ void split_store(const uint64_t (&k2)[4], unsigned ch
   *reinterpret_cast<uint4*>(lo_dst) = make_uint4(l[0], l[1], l[2], l[3]);
 }
 
-// Producers: reconstruct the K and V operand tiles of KV tile t0 from the
-// packed tile in `raw` (tokens below tq), the KIVI residual ring (tq <= t <
-// T) or zeros (t >= T).
-//   K: thread (tk = tid % 64, hf = tid / 64): token tk, channels of half hf.
-//   V: thread (tb = tid % 8, vq = tid / 8): tokens 8 tb .. 8 tb + 7 and
-//      channels CV vq .. CV vq + CV - 1 (CV = D / 16), in half2 arithmetic,
-//      stored as D rows of the transposed tile (one 16-byte chunk per row).
+// Producers: reconstruct this CTA's share of the K and V operand tiles of KV tile
+// t0 from the packed tile in `raw` (tokens below tq), the KIVI residual ring
+// (tq <= t < T) or zeros (t >= T).  tid 0..127:
+//   K: thread (tk = tid % KT, hf = tid / KT): token KT rank + tk, channels
+//      KC hf .. KC hf + KC - 1.
+//   V: thread (tb = tid % 8, vq = tid % NP / 8): tokens 8 tb .. 8 tb + 7 and
+//      channels CV vq .. CV vq + CV - 1 of this CTA's, in half2 arithmetic, stored
+//      as rows of the transposed tile (half a 16-byte chunk per row and trip).
 template <int D, int BITS, int FMT>
 __device__ __forceinline__ void build_tile(const Geom& g, int b, int h, int t0, int T, int tq,
-                                           int tid, const unsigned char* raw, unsigned char* kv) {
+                                           int tid, int rank, const unsigned char* raw, float* ksz,
+                                           unsigned char* kv) {
   using S = M256Layout<D, BITS>;
   constexpr bool KIVI = FMT == KVQ_FMT_KIVI;
   constexpr bool SYM = FMT == KVQ_FMT_SYMMETRIC;
-  constexpr int CV = D / 16;
-  constexpr int NCH = D / 16;                     // K chunks of 8 channels per thread
-  constexpr int NKW = D / 2 * BITS / 32;          // K code words per thread
-  const int tk = tid & 63, hf = tid >> 6;
-  const int t = t0 + tk;
+  constexpr int CV = S::CV;
+  constexpr int NCH = S::KC / 8;                  // K chunks of 8 channels per thread
+  constexpr int NKW = S::KC * BITS / 32;          // K code words per thread
+  if (!S::PAIR || tid < S::NP) {
   // ---- K tile ----
+  const int tk = tid % S::KT, hf = tid / S::KT, tt = rank * S::KT + tk;
+  const int t = t0 + tt;
+  // KIVI: the warp's tokens are one block; its scales and offsets of the warp's
+  // channels are converted once (a lane one or two channels) and read back as fp32.
+  // Converted by every lane for its own token, 128 conversions a tile kept the unit
+  // that also serves the softmax warps' exponentials busy (2,282 us against
+  // 1,796, shape above, before the loops were rolled up).
+  float* kf = ksz + (tid >> 5) * (2 * S::KC);
+  if constexpr (KIVI) {
+    __syncwarp();                                  // the previous tile's are read
+#pragma unroll
+    for (int i = 0; i < S::KC / 32; ++i) {
+      const int e = 32 * i + (tid & 31);
+      const __half* sp = reinterpret_cast<const __half*>(raw + S::RKS) + (tt >> 5) * D + hf * S::KC + e;
+      kf[e] = __half2float(sp[0]);
+      kf[S::KC + e] = __half2float(sp[(S::RKZ - S::RKS) / 2]);
+    }
+    __syncwarp();
+  }
   if (t < tq) {
     uint32_t kw[NKW];
-    const unsigned char* cp = raw + S::RKC + tk * S::CROW + hf * (S::CROW / 2);
+    const unsigned char* cp = raw + S::RKC + tt * S::CROW + hf * (S::KC * BITS / 8);
     if constexpr (NKW >= 4) {
 #pragma unroll
       for (int i = 0; i < NKW / 4; ++i) {
@@ -183,10 +257,10 @@ __device__ __forceinline__ void build_tile(const Geom& g, int b, int h, int t0, 
       const uint2 u = *reinterpret_cast<const uint2*>(cp);
       kw[0] = u.x; kw[1] = u.y;
     }
-    uint32_t ks = 0, kz = 0;                      // affine/symmetric: the half's group metadata
+    uint32_t ks = 0, kz = 0;                      // affine/symmetric: the groups' metadata
     if constexpr (!KIVI) {
-      const unsigned char* sp = raw + S::RKS + tk * (D / 16) + hf * (D / 32);
-      if constexpr (D == 128) {
+      const unsigned char* sp = raw + S::RKS + tt * (D / 16) + hf * (S::KC / 16);
+      if constexpr (S::KC == 64) {
         ks = *reinterpret_cast<const uint32_t*>(sp);
         if (!SYM) kz = *reinterpret_cast<const uint32_t*>(sp + (S::RKZ - S::RKS));
       } else {
@@ -195,26 +269,34 @@ __device__ __forceinline__ void build_tile(const Geom& g, int b, int h, int t0, 
       }
     }
     const uint64_t bias2 = f2pack(-8388608.f, -8388608.f);
+    // Two chunks to a trip: the roles' loops share the instruction cache, and with
+    // every loop unrolled fetching bound the tile (figures above).
+    constexpr int WT = BITS / 2;                  // code words per trip
+#pragma unroll S::UNROLL
+    for (int c0 = 0; c0 < NCH; c0 += 2) {
+      uint32_t cw[WT];
 #pragma unroll
-    for (int c = 0; c < NCH; ++c) {
-      const int cc = hf * NCH + c;                // chunk along D
-      constexpr int CB = 8 * BITS;                // code bits per chunk
-      const uint32_t w = kw[(c * CB) / 32] >> ((c * CB) % 32);
+      for (int i = 0; i < WT; ++i) cw[i] = kw[i];
+#pragma unroll
+      for (int i = 0; i + WT < NKW; ++i) kw[i] = kw[i + WT];
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      const int c = c0 + u, cc = hf * NCH + c;    // chunk along D
+      const uint32_t w = BITS == 4 ? cw[u * (WT - 1)] : cw[0] >> (16 * u);
       uint64_t k2[4];
       if constexpr (KIVI) {
-        const unsigned char* st = raw + S::RKS + (tk >> 5) * (2 * D) + cc * 16;
-        const uint4 su = *reinterpret_cast<const uint4*>(st);
-        const uint4 zu = *reinterpret_cast<const uint4*>(st + (S::RKZ - S::RKS));
-        const __half2* s2 = reinterpret_cast<const __half2*>(&su);
-        const __half2* z2 = reinterpret_cast<const __half2*>(&zu);
+        const float4* sp = reinterpret_cast<const float4*>(kf + 8 * c);
+        const float4* zp = reinterpret_cast<const float4*>(kf + S::KC + 8 * c);
+        const float4 sv[2] = {sp[0], sp[1]}, zv[2] = {zp[0], zp[1]};
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-          const float2 sf = __half22float2(s2[i]), zf = __half22float2(z2[i]);
+          const float4 sq = sv[i / 2], zq = zv[i / 2];
           const uint64_t c2 = fadd2(f2pack(code_biased<BITS>(w, 2 * i), code_biased<BITS>(w, 2 * i + 1)), bias2);
-          k2[i] = ffma2(c2, f2pack(sf.x, sf.y), f2pack(zf.x, zf.y));
+          k2[i] = i & 1 ? ffma2(c2, f2pack(sq.z, sq.w), f2pack(zq.z, zq.w))
+                        : ffma2(c2, f2pack(sq.x, sq.y), f2pack(zq.x, zq.y));
         }
       } else {
-        const int gi = (c * 8) / 32;              // group within the half
+        const int gi = (c * 8) / 32;              // group of the thread's
         const __half2 s2 = *reinterpret_cast<const __half2*>(&ks);
         const __half2 z2 = *reinterpret_cast<const __half2*>(&kz);
         const float s = gi ? __high2float(s2) : __low2float(s2);
@@ -226,35 +308,41 @@ __device__ __forceinline__ void build_tile(const Geom& g, int b, int h, int t0, 
           k2[i] = ffma2(c2, ss, mm);
         }
       }
-      unsigned char* base = kv + (cc >> 3) * (kTok * 128);
+      unsigned char* base = kv + (cc >> 3) * (S::KT * 128);
       split_store(k2, base + S::KH + sw128(tk, cc & 7), base + S::KL + sw128(tk, cc & 7));
+    }
     }
   } else {
     // KIVI residual window (full precision) or beyond the cache (zeros)
-#pragma unroll
+#pragma unroll 1
     for (int c = 0; c < NCH; ++c) {
       const int cc = hf * NCH + c;
       uint4 u = make_uint4(0, 0, 0, 0);
       if (KIVI && t < T)
         u = *reinterpret_cast<const uint4*>(
             plane_ptr<__nv_bfloat16>(g, KVQ_PLANE_K_FULL, b, h, t % g.ring, 8 * cc));
-      unsigned char* base = kv + (cc >> 3) * (kTok * 128);
+      unsigned char* base = kv + (cc >> 3) * (S::KT * 128);
       *reinterpret_cast<uint4*>(base + S::KH + sw128(tk, cc & 7)) = u;
       *reinterpret_cast<uint4*>(base + S::KL + sw128(tk, cc & 7)) = make_uint4(0, 0, 0, 0);
     }
   }
-  // ---- V^T tile: rows d = CV vq + e, 16-byte chunk tb (tokens 8 tb ..) ----
-  const int tb = tid & 7, vq = tid >> 3;
-  const int grp_v = vq * CV / 32;
-  uint32_t out[CV][4];
+  if (S::PAIR) return;
+  }
+  // ---- V^T tile: rows CV vq + e, 16-byte chunk tb (tokens 8 tb ..) ----
+  const int tb = tid & 7, vq = tid % S::NP >> 3;
+  const int ch = rank * S::VC + vq * CV, grp_v = ch / 32;
   const __half2 bias = __float2half2_rn(1024.f);
+#pragma unroll S::UNROLL
+  for (int p0 = 0; p0 < 4; p0 += 2) {             // tokens 2 p0 .. 2 p0 + 3
+  uint32_t out[CV][2];
 #pragma unroll
-  for (int p = 0; p < 4; ++p) {                   // token pair (2p, 2p + 1)
+  for (int pp = 0; pp < 2; ++pp) {                // token pair (2p, 2p + 1)
+    const int p = p0 + pp;
     uint32_t w2[2], s2u, z2u;
 #pragma unroll
     for (int u = 0; u < 2; ++u) {
       const int tv = 8 * tb + 2 * p + u;          // token within the tile
-      const unsigned char* cp = raw + S::RVC + tv * S::CROW + vq * (CV * BITS / 8);
+      const unsigned char* cp = raw + S::RVC + tv * S::CROW + ch * BITS / 8;
       if constexpr (CV * BITS == 32) w2[u] = *reinterpret_cast<const uint32_t*>(cp);
       else if constexpr (CV * BITS == 16) w2[u] = *reinterpret_cast<const unsigned short*>(cp);
       else w2[u] = *cp;
@@ -288,19 +376,19 @@ __device__ __forceinline__ void build_tile(const Geom& g, int b, int h, int t0, 
       const uint32_t x = ((pw[(e * BITS) / 16] >> ((e * BITS) % 16)) & m2) | 0x64006400u;
       const __half2 c2 = __hsub2(*reinterpret_cast<const __half2*>(&x), bias);
       const __half2 v2 = __hfma2(s2, c2, z2);
-      out[e][p] = *reinterpret_cast<const uint32_t*>(&v2);
+      out[e][pp] = *reinterpret_cast<const uint32_t*>(&v2);
     }
   }
   // tokens of the KIVI residual window, or beyond the cache, replace theirs
-  const int tv0 = t0 + 8 * tb;
-  if (tv0 + 7 >= tq) {
+  const int tv0 = t0 + 8 * tb + 2 * p0;
+  if (tv0 + 3 >= tq) {
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
+    for (int i = 0; i < 4; ++i) {
       const int tv = tv0 + i;
       if (tv < tq) continue;
       __nv_bfloat16 vals[CV];
       if (KIVI && tv < T) {
-        const __nv_bfloat16* src = plane_ptr<__nv_bfloat16>(g, KVQ_PLANE_V_FULL, b, h, tv % g.ring, vq * CV);
+        const __nv_bfloat16* src = plane_ptr<__nv_bfloat16>(g, KVQ_PLANE_V_FULL, b, h, tv % g.ring, ch);
         if constexpr (CV == 8) {
           const uint4 u = *reinterpret_cast<const uint4*>(src);
           memcpy(vals, &u, sizeof(vals));
@@ -322,8 +410,8 @@ __device__ __forceinline__ void build_tile(const Geom& g, int b, int h, int t0, 
   }
 #pragma unroll
   for (int e = 0; e < CV; ++e)
-    *reinterpret_cast<uint4*>(kv + S::VT + sw128(CV * vq + e, tb)) =
-        make_uint4(out[e][0], out[e][1], out[e][2], out[e][3]);
+    *reinterpret_cast<uint2*>(kv + S::VT + sw128(CV * vq + e, tb) + 4 * p0) = make_uint2(out[e][0], out[e][1]);
+  }
 }
 
 template <int D, int BITS, int FMT>
@@ -337,40 +425,41 @@ attend_prefill_m256_kernel(Geom g, const __nv_bfloat16* __restrict__ q, int L, f
   unsigned char* smem = reinterpret_cast<unsigned char*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   __shared__ uint64_t raw_full[S::RAW], raw_free[S::RAW], kv_full[S::KVB], kv_free[S::KVB],
-      s_full[2][2], p_full[2][2], s_free[2][2], done_bar;
+      s_full[2][S::SB], p_full[2][S::SB], s_free[2][S::SB], done_bar;
   __shared__ uint32_t tmem_base;
   __shared__ int abort_flag;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int nqt = gridDim.x;
-  const int qtile = nqt - 1 - blockIdx.x;              // longest first
+  constexpr int NC = S::PAIR ? 2 : 1;                  // CTAs that share a K/V tile
+  const uint32_t rank = S::PAIR ? cluster_rank() : 0;
+  const int qset = (gridDim.x - 1 - blockIdx.x) / NC;  // longest first
   const int hkv = blockIdx.y, b = blockIdx.z;
   const int grp = g.Hq / g.H;
   const int T = seq_tokens(g, b);
   const int tq = FMT == KVQ_FMT_KIVI ? kivi_tq(T, g.R, g.G) : T;
   // a ragged cache's sequence b attends the rows of its last append
   const int Lb = g.layout == KVQ_LAYOUT_UNIFORM ? L : g.seq_new[b];
-  const int q0 = qtile * nq;
-  if (q0 >= Lb) return;                                // no query of this sequence here
-  const int nql = min(nq, Lb - q0);
+  if (NC * qset * nq >= Lb) return;                    // no query of this sequence here
+  const int q0 = (NC * qset + (int)rank) * nq;
+  const int nql = min(nq, Lb - q0);                    // <= 0: no query here, only a share of K/V
   const int pos_first = T - Lb + q0;
-  const int t_end = pos_first + nql;                   // keys [0, t_end)
+  const int t_end = T - Lb + min(NC * (qset + 1) * nq, Lb);   // keys [0, t_end), the pair's
   const int ntiles = (t_end + kTok - 1) / kTok;
   volatile int* abort = &abort_flag;
 
   if (threadIdx.x == 0) {
     for (int i = 0; i < S::RAW; ++i) {
       mbar_init(&raw_full[i], 1);
-      mbar_init(&raw_free[i], 128);
+      mbar_init(&raw_free[i], kProdWarps);
     }
     for (int i = 0; i < S::KVB; ++i) {
-      mbar_init(&kv_full[i], 128);
+      mbar_init(&kv_full[i], NC * kProdWarps);
       mbar_init(&kv_free[i], 1);
     }
     for (int x = 0; x < 2; ++x)
-      for (int i = 0; i < 2; ++i) {
+      for (int i = 0; i < S::SB; ++i) {
         mbar_init(&s_full[x][i], 1);
-        mbar_init(&p_full[x][i], 128);
+        mbar_init(&p_full[x][i], NC * (kM / 32));
         mbar_init(&s_free[x][i], 1);
       }
     mbar_init(&done_bar, 1);
@@ -378,9 +467,7 @@ attend_prefill_m256_kernel(Geom g, const __nv_bfloat16* __restrict__ q, int L, f
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 12) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;"
-                 ::"r"(smem_u32(&tmem_base)));
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+    tmem_alloc512<S::PAIR>(&tmem_base);
   }
   // queries -> the swizzled Q tiles (softmax threads, one row each)
   const int row = threadIdx.x;                          // 0..255 for the softmax roles
@@ -401,7 +488,8 @@ attend_prefill_m256_kernel(Geom g, const __nv_bfloat16* __restrict__ q, int L, f
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
   tc_fence_before();
-  __syncthreads();
+  if (S::PAIR) cluster_sync();                         // both CTAs' barriers are set up
+  else __syncthreads();
   tc_fence_after();
   const uint32_t tmem = tmem_base;
 
@@ -430,112 +518,117 @@ attend_prefill_m256_kernel(Geom g, const __nv_bfloat16* __restrict__ q, int L, f
       bool ok = mbar_wait_or_abort(&raw_full[st], (j / S::RAW) & 1, abort);
       ok = ok && (j < S::KVB ||
                   mbar_wait_or_abort(&kv_free[kb], ((j - S::KVB) / S::KVB) & 1, abort));
-      if (!producers_all(ok)) break;
+      if (!__all_sync(0xffffffffu, ok)) break;
       unsigned char* kv = smem + S::KV_OFF + kb * S::KV_B;
-      build_tile<D, BITS, FMT>(g, b, hkv, j * kTok, T, tq, tid, smem + S::RAW_OFF + st * S::RAW_B, kv);
-      mbar_arrive(&raw_free[st]);
-      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-      mbar_arrive(&kv_full[kb]);
+      build_tile<D, BITS, FMT>(g, b, hkv, j * kTok, T, tq, tid, (int)rank,
+                               smem + S::RAW_OFF + st * S::RAW_B,
+                               reinterpret_cast<float*>(smem + S::KS_OFF), kv);
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // for the MMAs' reads
+      __syncwarp();
+      if (lane == 0) {
+        mbar_arrive(&raw_free[st]);
+        arrive_first<S::PAIR>(&kv_full[kb]);
+      }
     }
   } else if (warp == 12) {
-    // ---------------- MMA issuer ----------------
-    // Issues, as soon as each is ready: Q K^T of the next tile for both
-    // query tiles (its K/V tile built, the S buffer's previous P V done),
-    // and P V of each query tile's next tile (its P written).  S runs one
-    // tile ahead of the softmax threads; the tensor pipe executes in issue
-    // order.  The whole warp runs the loop (its values stay warp-uniform)
-    // and one elected lane issues the MMAs and their commits.  Descriptors
-    // are formed once: a K step of 16 elements advances the start address by
-    // 32 bytes (2 in the descriptor's 16-byte units).
-    constexpr uint32_t id_qk = idesc_bf16(kM, kTok);
-    constexpr uint32_t id_pv = idesc_f16(kM, D);
-    const uint64_t qdesc0 = sw128_desc(smem + S::Q_OFF);
-    const uint64_t kvdesc0 = sw128_desc(smem + S::KV_OFF);   // K/V buffer b: + b KV_B / 16
-    const bool leader = elect_one();
-    int nqk = 0, npv[2] = {0, 0};
-    long idle = 0;
-    uint64_t idle_since = 0;
-    while (npv[0] < ntiles || npv[1] < ntiles) {
-      bool progressed = false;
-      if (nqk < ntiles && nqk <= min(npv[0], npv[1]) + 1) {
-        const int kb = nqk % S::KVB, bf = nqk & 1;
-        const uint32_t fpar = (nqk >= 2) ? ((nqk - 2) >> 1) & 1 : 0;
-        bool ready = false;
-        if (lane == 0)
-          ready = mbar_test(&kv_full[kb], (nqk / S::KVB) & 1) &&
-                  (nqk < 2 || (mbar_test(&s_free[0][bf], fpar) && mbar_test(&s_free[1][bf], fpar)));
-        if (__shfl_sync(0xffffffffu, ready, 0)) {
-          tc_fence_after();
-          if (leader) {
-#pragma unroll
-            for (int x = 0; x < 2; ++x) {
-              const uint32_t ts = tmem + x * 128 + bf * kTok;
-#pragma unroll
-              for (int kk = 0; kk < D / 16; ++kk) {
-                // Q atom: 128 rows x 128 B (1024 units); K atom: 64 rows x 128 B (512 units)
-                const uint64_t qd = qdesc0 + (uint64_t)(x * (S::QT >> 4) + (kk >> 2) * 1024 + (kk & 3) * 2);
-                const uint64_t kd = kvdesc0 + (uint64_t)(kb * (S::KV_B >> 4) + (kk >> 2) * 512 + (kk & 3) * 2);
-                umma_a_fill(ts, qd, kd + (S::KH >> 4), id_qk, kk > 0);   // Q read once
-                umma_a_lastuse(ts, qd, kd + (S::KL >> 4), id_qk, 1);     // for K hi and lo
-              }
-              umma_commit(&s_full[x][bf]);
-            }
-          }
-          __syncwarp();
-          ++nqk;
-          progressed = true;
-        }
-      }
-#pragma unroll
-      for (int x = 0; x < 2; ++x) {
-        const int j = npv[x];
-        if (j >= nqk) continue;
-        const int bf = j & 1;
-        bool ready = false;
-        if (lane == 0) ready = mbar_test(&p_full[x][bf], (j >> 1) & 1);
-        if (!__shfl_sync(0xffffffffu, ready, 0)) continue;
+    if (rank == 0) {
+      // ---------------- MMA issuer ----------------
+      // For each query tile X in turn Q_X K^T of a later tile, then P_X V of tile
+      // j, each blocking on the barrier it needs: what Q_X K^T waits for, P_X V of
+      // an earlier tile, is two steps of the other query tile back, so the tensor
+      // pipe has work meanwhile.  While that later tile is not built yet, P V
+      // goes first (D = 128).  An issuer that polled for whichever came first answered
+      // several hundred cycles late, twice in the chain of every tile (D = 64: 199 us,
+      // 179 so).  The whole warp runs the loop (its values stay
+      // warp-uniform) and one elected lane issues the MMAs and their commits.
+      // Descriptors are formed once: a K step of 16 elements advances the start
+      // address by 32 bytes (2 in the descriptor's 16-byte units).
+      constexpr uint32_t id_qk = idesc_bf16(NC * kM, kTok);
+      constexpr uint32_t id_pv = idesc_f16(NC * kM, D);
+      const uint64_t qdesc0 = sw128_desc(smem + S::Q_OFF);
+      const uint64_t kvdesc0 = sw128_desc(smem + S::KV_OFF);   // K/V buffer b: + b KV_B / 16
+      const bool leader = elect_one();
+      auto qk = [&](int x, int j) -> bool {
+        const int kb = j % S::KVB, bf = j % S::SB;
+        if ((x == 0 && !warp_wait(&kv_full[kb], (j / S::KVB) & 1, abort)) ||
+            (j >= S::SB && !warp_wait(&s_free[x][bf], ((j - S::SB) / S::SB) & 1, abort)))
+          return false;
         tc_fence_after();
-        const int kb = j % S::KVB;
         if (leader) {
-          const uint32_t tp = tmem + x * 128 + bf * kTok;   // P (fp16 pairs) over S's columns
-          const uint32_t to = tmem + 256 + x * D;
+          const uint32_t ts = tmem + (x * S::SB + bf) * kTok;
 #pragma unroll
-          for (int kk = 0; kk < kTok / 16; ++kk)
-            umma_ts(to, tp + kk * 8, kvdesc0 + (uint64_t)(kb * (S::KV_B >> 4) + (S::VT >> 4) + kk * 2),
-                    id_pv, (j > 0 || kk > 0) ? 1u : 0u);
-          umma_commit(&s_free[x][bf]);           // S/P buffer free, and O holds tile j
-          if (npv[x ^ 1] > j) umma_commit(&kv_free[kb]);   // both query tiles done with it
+          for (int kk = 0; kk < D / 16; ++kk) {
+            // Q atom: 128 rows x 128 B (1024 units); K atom: KT rows x 128 B (8 KT units)
+            const uint64_t qd = qdesc0 + (uint64_t)(x * (S::QT >> 4) + (kk >> 2) * 1024 + (kk & 3) * 2);
+            const uint64_t kd = kvdesc0 + (uint64_t)(kb * (S::KV_B >> 4) + (kk >> 2) * (8 * S::KT) + (kk & 3) * 2);
+            mma_a_fill<S::PAIR>(ts, qd, kd + (S::KH >> 4), id_qk, kk > 0);   // Q read once
+            mma_a_lastuse<S::PAIR>(ts, qd, kd + (S::KL >> 4), id_qk, 1);     // for K hi and lo
+          }
+          mma_commit<S::PAIR>(&s_full[x][bf]);
         }
         __syncwarp();
-        ++npv[x];
-        progressed = true;
+        return true;
+      };
+      auto pv = [&](int x, int j) -> bool {
+        const int kb = j % S::KVB, bf = j % S::SB;
+        if (!warp_wait(&p_full[x][bf], (j / S::SB) & 1, abort)) return false;
+        tc_fence_after();
+        if (leader) {
+          const uint32_t tp = tmem + (x * S::SB + bf) * kTok;   // P (fp16 pairs) over S's columns
+          const uint32_t to = tmem + 2 * S::SB * kTok + x * D;
+#pragma unroll
+          for (int kk = 0; kk < kTok / 16; ++kk)
+            mma_ts<S::PAIR>(to, tp + kk * 8, kvdesc0 + (uint64_t)(kb * (S::KV_B >> 4) + (S::VT >> 4) + kk * 2),
+                         id_pv, (j > 0 || kk > 0) ? 1u : 0u);
+          mma_commit<S::PAIR>(&s_free[x][bf]);           // S/P buffer free, and O holds tile j
+          if (x == 1) mma_commit<S::PAIR>(&kv_free[kb]); // both query tiles done with it
+        }
+        __syncwarp();
+        return true;
+      };
+      bool ok = true;
+#pragma unroll 1
+      for (int j = -1; j < ntiles && ok; ++j) {
+        const int n = j + 1;
+        if constexpr (!S::PAIR) {
+#pragma unroll
+          for (int x = 0; x < 2; ++x) {
+            if (ok && n < ntiles) ok = qk(x, n);
+            if (ok && j >= 0) ok = pv(x, j);
+          }
+        } else {
+          bool first = n < ntiles;             // Q K^T of tile n before P V of tile j
+          if (first && j >= 0) {
+            if (lane == 0) first = mbar_test(&kv_full[n % S::KVB], (n / S::KVB) & 1);
+            first = __shfl_sync(0xffffffffu, first, 0);
+          }
+          // four steps: Q K^T and P V of A, then of B; or both P V, then both Q K^T
+#pragma unroll 1                               // one copy of each in the instruction cache
+          for (int i = 0; i < 4 && ok; ++i) {
+            const bool is_qk = first ? (i & 1) == 0 : i >= 2;
+            const int x = first ? i >> 1 : i & 1;
+            if (is_qk) ok = n >= ntiles || qk(x, n);
+            else ok = j < 0 || pv(x, j);
+          }
+        }
       }
-      if (progressed) {
-        idle = 0;
-      } else {
-        if (idle == 0) idle_since = global_ns();
-        __nanosleep(20);
-        const bool stop = (++idle & 63) == 0 && (*abort || global_ns() - idle_since > kWaitNs);
-        if (__shfl_sync(0xffffffffu, stop, 0)) break;   // the whole warp leaves together
-      }
+      if (leader) mma_commit<S::PAIR>(&done_bar);   // every MMA issued above has completed
+      if (lane == 0 && !mbar_wait(&done_bar, 0)) *abort = 1;
+      __syncwarp();
     }
-    if (lane == 0 && (npv[0] < ntiles || npv[1] < ntiles)) *abort = 1;
-    if (leader) umma_commit(&done_bar);        // every MMA issued above has completed
-    if (lane == 0 && !mbar_wait(&done_bar, 0)) *abort = 1;
-    __syncwarp();
   } else if (warp < 8) {
     // ---------------- softmax: one row per thread ----------------
     const int x = warp >> 2;                   // query tile
     const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
-    const uint32_t s_col = tmem + lane_base + x * 128;
-    const uint32_t o_col = tmem + lane_base + 256 + x * D;
+    const uint32_t s_col = tmem + lane_base + x * S::SB * kTok;
+    const uint32_t o_col = tmem + lane_base + 2 * S::SB * kTok + x * D;
     const float c2 = scale * 1.4426950408889634f;   // scores in log2 units
     const uint64_t c22 = f2pack(c2, c2);
     float m = -INFINITY, l = 0.f;
     bool ok = true;
     for (int j = 0; j < ntiles; ++j) {
-      const int bf = j & 1, t0 = j * kTok;
-      if (!warp_wait(&s_full[x][bf], (j >> 1) & 1, abort)) {
+      const int bf = j % S::SB, t0 = j * kTok;
+      if (!warp_wait(&s_full[x][bf], (j / S::SB) & 1, abort)) {
         ok = false;
         break;
       }
@@ -568,7 +661,7 @@ attend_prefill_m256_kernel(Geom g, const __nv_bfloat16* __restrict__ q, int L, f
         m = m_new;
       } else if (__any_sync(0xffffffffu, m_new > m + kRescale)) {
         // O is rewritten: the P V of tile j - 1 must have completed
-        if (!warp_wait(&s_free[x][(j - 1) & 1], ((j - 1) >> 1) & 1, abort)) {
+        if (!warp_wait(&s_free[x][(j - 1) % S::SB], ((j - 1) / S::SB) & 1, abort)) {
           ok = false;
           break;
         }
@@ -611,11 +704,12 @@ attend_prefill_m256_kernel(Geom g, const __nv_bfloat16* __restrict__ q, int L, f
       l += s0 + s1;
       tmem_wait_st();
       tc_fence_before();
-      mbar_arrive(&p_full[x][bf]);
+      __syncwarp();
+      if (lane == 0) arrive_first<S::PAIR>(&p_full[x][bf]);
     }
     // ---------------- epilogue ----------------
     if (ok && ntiles > 0 &&
-        !warp_wait(&s_free[x][(ntiles - 1) & 1], ((ntiles - 1) >> 1) & 1, abort))
+        !warp_wait(&s_free[x][(ntiles - 1) % S::SB], ((ntiles - 1) / S::SB) & 1, abort))
       ok = false;
     if (__all_sync(0xffffffffu, ok && !*abort)) {
       tc_fence_after();
@@ -638,12 +732,15 @@ attend_prefill_m256_kernel(Geom g, const __nv_bfloat16* __restrict__ q, int L, f
       }
     }
   }
+  // the issuer's last arrival on the second CTA's barriers has landed
+  if (warp == 12 && lane == 0 && rank == 1 && !mbar_wait(&done_bar, 0)) *abort = 1;
   tc_fence_before();
-  __syncthreads();
+  if (S::PAIR) cluster_sync();                         // neither CTA's TMEM or shared memory is in use
+  else __syncthreads();
   if (threadIdx.x == 0 && *abort) atomicOr(err, 8);
   if (warp == 12) {
     tc_fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem));
+    tmem_free512<S::PAIR>(tmem);
   }
 }
 
@@ -655,10 +752,15 @@ cudaError_t launch_m256(const Geom& g, const void* q, int L, float scale, void* 
                                        M256Layout<D, BITS>::ALLOC);
   if (e != cudaSuccess) return e;
   const int nq = kRowsCta / (g.Hq / g.H);
-  dim3 grid((L + nq - 1) / nq, g.H, g.B);
-  launch_pdl(kern, dim3(grid), dim3(kThreads), (size_t)M256Layout<D, BITS>::ALLOC, s, g,
-             reinterpret_cast<const __nv_bfloat16*>(q), L, scale,
-             reinterpret_cast<__nv_bfloat16*>(out), nq, err);
+  constexpr int NC = M256Layout<D, BITS>::PAIR ? 2 : 1;
+  const dim3 grid((L + NC * nq - 1) / (NC * nq) * NC, g.H, g.B);
+  const auto start = [&](auto launcher) {
+    return launcher(kern, grid, dim3(kThreads), (size_t)M256Layout<D, BITS>::ALLOC, s, g,
+                    reinterpret_cast<const __nv_bfloat16*>(q), L, scale,
+                    reinterpret_cast<__nv_bfloat16*>(out), nq, err);
+  };
+  if (NC == 2) start([](auto... a) { return launch_pdl_pair(a...); });
+  else start([](auto... a) { return launch_pdl(a...); });
   return cudaGetLastError();
 }
 

@@ -259,8 +259,8 @@ project_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
     bool ok = true;
     int s = 0, phase = 0;
     for (int kb = 0; kb < KB; ++kb) {
-      bool ready = mbar_wait_cluster(&full_bar[s], phase);
-      if (NF4) ready = ready && mbar_wait_cluster(&w_full[s], phase);
+      bool ready = mbar_wait(&full_bar[s], phase);
+      if (NF4) ready = ready && mbar_wait(&w_full[s], phase);
       if (!__all_sync(0xffffffffu, ready)) {
         ok = false;
         break;
@@ -442,7 +442,7 @@ project_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
   if (threadIdx.x == kMmaWarp<NF4> * 32 && rank == 0 && pair_ok) {
     bool ok = true;
     if (r > 0) {
-      ok = mbar_wait_cluster(&bp_bar, 0);
+      ok = mbar_wait(&bp_bar, 0);
       if (ok) {
         constexpr uint32_t id_main = idesc_bf16(2 * BM, BN);
         for (int kk = 0; kk < rp / 16; ++kk)

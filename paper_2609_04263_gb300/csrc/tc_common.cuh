@@ -295,32 +295,13 @@ __device__ __forceinline__ void umma_commit_pair(uint64_t* bar) {
 // Arrival on a barrier of either CTA of the pair for what this CTA's warp wrote to
 // its own shared memory (after fence.proxy.async) or TMEM (after
 // tcgen05.fence::before_thread_sync), where its own SM's tensor core reads it.
-// Nothing is handed to the other CTA's threads, so the arrival does not release at
-// cluster scope: that made it wait for the thread's global loads in flight, 1,200
-// of a dequantising warp's 2,100 cycles per slice (NF4 base, 2048 x 4096 -> 6144:
-// 268 us with it, 225 passed on by a thread without loads, 167 without).
+// Nothing is handed to the other CTA's threads, so neither the arrival releases nor
+// the issuer's wait acquires at cluster scope.  A release that wide made the arrival
+// wait for the thread's global loads in flight, 1,200 of a dequantising warp's 2,100
+// cycles per slice (NF4 base, 2048 x 4096 -> 6144: 268 us with it, 225 passed on by
+// a thread without loads, 167 without).
 __device__ __forceinline__ void mbar_arrive_pair(uint32_t bar) {
   asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
-}
-// mbar_wait that also acquires what the other CTA released by its arrivals.
-__device__ __forceinline__ bool mbar_wait_cluster(uint64_t* bar, uint32_t parity) {
-  const uint64_t t0 = global_ns();
-  for (long i = 0;; ++i) {
-    uint32_t ok;
-    asm volatile(
-        "{\n .reg .pred p;\n mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n"
-        " selp.u32 %0, 1, 0, p;\n}\n"
-        : "=r"(ok) : "r"(smem_u32(bar)), "r"(parity) : "memory");
-    if (ok) return true;
-    if ((i & 7) == 7 && global_ns() - t0 > kWaitNs) return false;
-  }
-}
-
-// warp_wait that also acquires what the other CTA released by its arrivals.
-__device__ __forceinline__ bool warp_wait_cluster(uint64_t* bar, uint32_t parity, volatile int* abort) {
-  bool ok = mbar_wait_or_abort(bar, parity, abort);
-  ok = ok && mbar_wait_cluster(bar, parity);
-  return __all_sync(0xffffffffu, ok);
 }
 __device__ __forceinline__ void umma_pair_a_fill(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc,
                                                  uint32_t idesc, uint32_t accumulate) {
