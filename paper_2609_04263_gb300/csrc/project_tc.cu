@@ -56,11 +56,20 @@ constexpr int kDqWarp0 = 4;
 using namespace tc;
 
 // The 16 NF4 levels, code 0 .. 15, as QLoRA publishes the data type.
-__constant__ float c_nf4_lv[16] = {
-    -1.0f, -0.6961928009986877f, -0.5250730514526367f, -0.39491748809814453f,
-    -0.28444138169288635f, -0.18477343022823334f, -0.09105003625154495f, 0.0f,
-    0.07958029955625534f, 0.16093020141124725f, 0.24611230194568634f, 0.33791524171829224f,
-    0.44070982933044434f, 0.5626170039176941f, 0.7229568362236023f, 1.0f};
+__device__ __forceinline__ constexpr float nf4_level(int code) {
+  constexpr float lv[16] = {
+      -1.0f, -0.6961928009986877f, -0.5250730514526367f, -0.39491748809814453f,
+      -0.28444138169288635f, -0.18477343022823334f, -0.09105003625154495f, 0.0f,
+      0.07958029955625534f, 0.16093020141124725f, 0.24611230194568634f, 0.33791524171829224f,
+      0.44070982933044434f, 0.5626170039176941f, 0.7229568362236023f, 1.0f};
+  return lv[code];
+}
+// Byte permute; a selector nibble 8 + k gives the sign of byte k in every bit.
+__device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel) {
+  uint32_t d;
+  asm("prmt.b32 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(sel));
+  return d;
+}
 
 struct TcArgs {
   void* out[3];
@@ -182,7 +191,6 @@ project_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   __shared__ uint64_t full_bar[kStages], empty_bar[kStages], w_full[kStages];
   __shared__ uint64_t u_bar, bp_bar, acc_bar;
-  __shared__ float nf4_lv[16];
   __shared__ uint32_t tmem_base;
   __shared__ int fail, peer_fail;
 
@@ -210,7 +218,6 @@ project_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
     fail = peer_fail = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  if (NF4 && threadIdx.x < 16) nf4_lv[threadIdx.x] = c_nf4_lv[threadIdx.x];
   if (warp == kMmaWarp<NF4>) {   // TMEM: 512 columns (main BN + LoRA <= 64)
     asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], 512;"
                  ::"r"(smem_u32(&tmem_base)));
@@ -300,8 +307,7 @@ project_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
     // trip: each is refilled as soon as it has been read and is not moved, as a
     // move of a value still being loaded waits for it (272 us for 2048 x 4096 ->
     // 6144 with buffers rotated each slice, 268 without; 167 with the arrival
-    // below no longer waiting for the loads).  A slice now takes 820 cycles of
-    // look-ups and stores and 250 of waiting for its slot.
+    // below no longer waiting for the loads).
     constexpr int PF = 4;
     uint4 cq[PF][NQ];
     float am[PF];
@@ -346,29 +352,32 @@ project_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
       }
       const float a = am[u];
       fetch(kb + PF, cq[u], am[u]);
-      uint64_t a2;
-      asm("mov.b64 %0, {%1, %1};" : "=l"(a2) : "f"(a));
+      // The 16 levels times absmax (fp32 products, rounded to bf16 once) as bytes in
+      // registers, 4 codes to a byte permute: with the levels looked up in shared
+      // memory and multiplied code by code a slice took 820 cycles (166 us for 2048 x 4096
+      // -> 6144; 134 so).
+      uint32_t tl[4], th[4];                              // low, high bytes of entries 4 k ..
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const uint32_t p0 = pack_bf16(nf4_level(4 * k) * a, nf4_level(4 * k + 1) * a);
+        const uint32_t p1 = pack_bf16(nf4_level(4 * k + 2) * a, nf4_level(4 * k + 3) * a);
+        tl[k] = prmt(p0, p1, 0x6420u);
+        th[k] = prmt(p0, p1, 0x7531u);
+      }
 #pragma unroll
       for (int j = 0; j < 4 * NQ; ++j) {                  // chunk c: inputs 8c .. 8c + 7
         const int c = 4 * NQ * h + j;
+        const uint32_t w = w8[j], sel = w & 0x77777777u, y = w << 4;
         uint32_t o[4];
-        // byte offsets into the level table (4 x code) of the word's low and
-        // high nibbles, four at a time
-        const uint32_t lo4 = (w8[j] << 2) & 0x3C3C3C3Cu, hi4 = (w8[j] >> 2) & 0x3C3C3C3Cu;
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {                     // byte i of word j: inputs 8c + 2i, + 1
-          // the two levels times absmax as one packed fp32 multiply (each
-          // product rounded as a scalar one would be), then one bf16 pair
-          const char* lvb = reinterpret_cast<const char*>(nf4_lv);
-          const uint32_t sel = 0x4440u | (uint32_t)i;     // byte i into byte 0, zeros above
-          const float l0 = *reinterpret_cast<const float*>(lvb + __byte_perm(lo4, 0u, sel));
-          const float l1 = *reinterpret_cast<const float*>(lvb + __byte_perm(hi4, 0u, sel));
-          uint64_t p2, l2;
-          asm("mov.b64 %0, {%1, %2};" : "=l"(l2) : "f"(l0), "f"(l1));
-          asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(p2) : "l"(l2), "l"(a2));
-          float q0, q1;
-          asm("mov.b64 {%0, %1}, %2;" : "=f"(q0), "=f"(q1) : "l"(p2));
-          o[i] = pack_bf16(q0, q1);
+        for (int u = 0; u < 2; ++u) {                     // inputs 4u .. 4u + 3 of the chunk
+          const uint32_t s4 = u ? sel >> 16 : sel;        // entry within its half of the table
+          // bytes of ones where bit 3 of the code is set: the upper half
+          const uint32_t m = prmt(y, w, u ? 0xFBEAu : 0xD9C8u);
+          const uint32_t lo = (prmt(tl[0], tl[1], s4) & ~m) | (prmt(tl[2], tl[3], s4) & m);
+          const uint32_t hi = (prmt(th[0], th[1], s4) & ~m) | (prmt(th[2], th[3], s4) & m);
+          o[2 * u] = prmt(lo, hi, 0x5140u);
+          o[2 * u + 1] = prmt(lo, hi, 0x7362u);
         }
         *reinterpret_cast<uint4*>(wt + rsw + ((c ^ (n & 7)) << 4)) = make_uint4(o[0], o[1], o[2], o[3]);
       }
