@@ -30,15 +30,16 @@
 //     bf16.
 // The barriers that wake the issuer (tiles built, P written) sit in the first
 // CTA and count one arrival per warp.
-// What bounds it, per 64-token tile: D = 128, building K, 2,200 of 2,800 cycles
-// (2,300 without building: the MMAs, 1,540, and the waits between them and the
-// softmax warps); D = 64, the chain from scores over softmax to P V and the buffers
+// What bounds it, per 64-token tile: D = 128, building the tiles, most of 2,700
+// cycles (2,300 without building: the MMAs, 1,540, and the waits between them and
+// the softmax warps); D = 64, the chain from scores over softmax to P V and the buffers
 // it frees, about 2,000 cycles, 1,060 of them softmax.
 //   2 x 8192 tokens, 32 / 8 heads of 128, KIVI 2-bit: 2081 us with two tile
-// buffers, 1745 with three, 1400 here.  With every loop unrolled the roles' code did
-// not fit the instruction cache (1.5 of 10 cycles an instruction went to fetching
-// it): 1,800 us as a pair, 1,480 with one copy of each product in the issuer, 1,420
-// with the build loops rolled up.
+// buffers, 1745 with three, 1335 here.  A thread's share of a tile is kept small
+// and the issuer holds one copy of each product: with 64 channels of K or V to a
+// thread unrolled and five copies the roles' code did not fit the instruction
+// cache (1.5 of 10 cycles an instruction went to fetching it), 1,800 us as a pair
+// (1,480 with one copy, 1,400 with the build loops rolled up as well).
 //   4 x 2029 tokens, 32 / 4 heads of 64, affine 4-bit: 229 us with two tile buffers,
 // 199 with four, 179 here.  As a pair 192: less to build, which did not bound it,
 // and longer waits.
@@ -56,7 +57,7 @@ using namespace tc;
 constexpr int kM = 128;              // rows per query tile (MMA M)
 constexpr int kTok = 64;             // tokens per KV tile
 constexpr int kRowsCta = 2 * kM;     // query rows per CTA
-constexpr int kProdWarps = 4;        // two build K, two V
+constexpr int kProdWarps = 4;
 constexpr int kThreads = 14 * 32;    // 8 softmax, 4 producer, 1 issuer, 1 loader warp
 constexpr float kRescale = 8.f;      // log2 growth of a row maximum that forces a rescale
 
@@ -64,15 +65,12 @@ constexpr float kRescale = 8.f;      // log2 growth of a row maximum that forces
 template <int D, int BITS>
 struct M256Layout {
   // Two CTAs share each K/V tile where building it bounds the kernel: D = 128 takes
-  // 1745 us alone and 1400 paired, D = 64 179 alone and 192 paired (shapes above).
+  // 1745 us alone and 1335 paired, D = 64 179 alone and 192 paired (shapes above).
   static constexpr bool PAIR = D == 128;
   static constexpr int KT = PAIR ? kTok / 2 : kTok; // tokens of K per CTA
   static constexpr int VC = PAIR ? D / 2 : D;       // channels of V per CTA
-  // A pair's CTA builds K with half of its producer threads and V with the others;
-  // a CTA alone with all of them K, then V.
-  static constexpr int NP = PAIR ? 64 : 128;
+  static constexpr int NP = 32 * kProdWarps;        // producer threads
   static constexpr int KC = KT * D / NP;            // channels of K per thread
-  static constexpr int UNROLL = PAIR ? 1 : 2;       // trips of the build loops unrolled
   static constexpr int CV = VC * 8 / NP;            // channels of V per thread
   // score tiles (TMEM) per query tile: what O (2 D columns) leaves of 512
   static constexpr int SB = 2;
@@ -223,7 +221,7 @@ __device__ __forceinline__ void build_tile(const Geom& g, int b, int h, int t0, 
   constexpr int CV = S::CV;
   constexpr int NCH = S::KC / 8;                  // K chunks of 8 channels per thread
   constexpr int NKW = S::KC * BITS / 32;          // K code words per thread
-  if (!S::PAIR || tid < S::NP) {
+  {
   // ---- K tile ----
   const int tk = tid % S::KT, hf = tid / S::KT, tt = rank * S::KT + tk;
   const int t = t0 + tt;
@@ -231,7 +229,7 @@ __device__ __forceinline__ void build_tile(const Geom& g, int b, int h, int t0, 
   // channels are converted once (a lane one or two channels) and read back as fp32.
   // Converted by every lane for its own token, 128 conversions a tile kept the unit
   // that also serves the softmax warps' exponentials busy (2,282 us against
-  // 1,796, shape above, before the loops were rolled up).
+  // 1,796, shape above, in the version with 64 channels to a thread).
   float* kf = ksz + (tid >> 5) * (2 * S::KC);
   if constexpr (KIVI) {
     __syncwarp();                                  // the previous tile's are read
@@ -269,10 +267,8 @@ __device__ __forceinline__ void build_tile(const Geom& g, int b, int h, int t0, 
       }
     }
     const uint64_t bias2 = f2pack(-8388608.f, -8388608.f);
-    // Two chunks to a trip: the roles' loops share the instruction cache, and with
-    // every loop unrolled fetching bound the tile (figures above).
     constexpr int WT = BITS / 2;                  // code words per trip
-#pragma unroll S::UNROLL
+#pragma unroll
     for (int c0 = 0; c0 < NCH; c0 += 2) {
       uint32_t cw[WT];
 #pragma unroll
@@ -326,13 +322,12 @@ __device__ __forceinline__ void build_tile(const Geom& g, int b, int h, int t0, 
       *reinterpret_cast<uint4*>(base + S::KL + sw128(tk, cc & 7)) = make_uint4(0, 0, 0, 0);
     }
   }
-  if (S::PAIR) return;
   }
   // ---- V^T tile: rows CV vq + e, 16-byte chunk tb (tokens 8 tb ..) ----
   const int tb = tid & 7, vq = tid % S::NP >> 3;
   const int ch = rank * S::VC + vq * CV, grp_v = ch / 32;
   const __half2 bias = __float2half2_rn(1024.f);
-#pragma unroll S::UNROLL
+#pragma unroll
   for (int p0 = 0; p0 < 4; p0 += 2) {             // tokens 2 p0 .. 2 p0 + 3
   uint32_t out[CV][2];
 #pragma unroll
