@@ -262,6 +262,11 @@ __device__ __forceinline__ void merge_full(const float* wf, float (&x)[D / 32], 
   for (int i = 0; i < D / 32; ++i) out[lane + 32 * i] = __float2bfloat16_rn(x[i] / L);
 }
 
+// Floats of the warps' partials of `pw` floats each, up to the next 16 bytes: the
+// queries behind them are read four at a time, and pw is not a multiple of four
+// where the group is odd.
+__host__ __device__ constexpr int slot_floats(int pw) { return (kNW * pw + 3) / 4 * 4; }
+
 // Launched after kvarn_full_kernel, whose start waited for everything before it:
 // only its partials have to be waited for (pdl_wait before the merges).
 // PAIR: at most two query heads per kv head.
@@ -282,7 +287,7 @@ decode_stream_kvarn_kernel(Geom g, const __nv_bfloat16* __restrict__ q, float sc
   const int grp = g.Hq / g.H;
   const int PW = grp * (D + 2);
   float* slot = reinterpret_cast<float*>(smem + (size_t)ns * C::STAGE);   // [kNW][PW]
-  float* qr = slot + kNW * PW;                       // [8][D] rotated queries, then merged rows
+  float* qr = slot + slot_floats(PW);                // [8][D] rotated queries, then merged rows
   Merge* mg = reinterpret_cast<Merge*>(qr + 8 * D);
   uint64_t* full = reinterpret_cast<uint64_t*>(mg + 1);
   uint64_t* empty = full + ns;
@@ -813,7 +818,7 @@ decode_stream_kvarn_kernel(Geom g, const __nv_bfloat16* __restrict__ q, float sc
 template <int D, int KB, int VB, int G>
 size_t stream_smem(int grp, int* ns) {
   using C = KCfg<D, KB, VB, G>;
-  const size_t fixed = (size_t)kNW * grp * (D + 2) * 4 + (size_t)8 * D * 4 + sizeof(Merge);
+  const size_t fixed = (size_t)slot_floats(grp * (D + 2)) * 4 + (size_t)8 * D * 4 + sizeof(Merge);
   int n = (int)((kSmemMax - fixed) / (C::STAGE + 16));
   if (n > kMaxStages) n = kMaxStages;
   *ns = n;
