@@ -846,10 +846,18 @@ cudaError_t launch_t(const Geom& g, const void* q, float scale, int* err, void* 
 
 }  // namespace
 
+// At least two ring stages: a warp's next block can lie two stages on, and in a ring
+// of one it would take the phase before last for the one it waits for (eight heads of
+// 256, whose partials leave room for one; the split kernel takes those).
 bool decode_stream_kvarn_supported(const Geom& g) {
   const bool shape = (g.D == 256 && g.G == 64) || (g.D == 64 && g.G == 32);
-  return g.fmt == KVQ_FMT_KVARN && g.act == KVQ_BF16 && shape && g.kb == 4 && g.vb == 2 &&
-         g.Hq / g.H <= 8;
+  if (!(g.fmt == KVQ_FMT_KVARN && g.act == KVQ_BF16 && shape && g.kb == 4 && g.vb == 2 &&
+        g.Hq / g.H <= 8))
+    return false;
+  int ns = 0;
+  if (g.D == 256) stream_smem<256, 4, 2, 64>(g.Hq / g.H, &ns);
+  else stream_smem<64, 4, 2, 32>(g.Hq / g.H, &ns);
+  return ns >= 2;
 }
 
 cudaError_t launch_decode_stream_kvarn(const Geom& g, const void* q, float scale, int* err,
