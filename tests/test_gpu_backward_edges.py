@@ -1,0 +1,38 @@
+"""The straight-through backward's products at the edges of their 128-wide tiles and
+of its softmax's key ranges: one query, stacked rows a row short of and past a
+tile, key counts that no vector load divides, head_dim 64 to 256, adapters of
+unlike ranks (whose products share a launch) and rows short of a tile.  The
+checks and tolerances are those of the other backward tests."""
+import pytest
+
+from tests import test_gpu_backward as TB
+from tests.gpu_common import require_gpu
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _gpu():
+    require_gpu()
+
+
+@pytest.mark.parametrize("fmt,act,B,Hkv,Hq,D,T0,L", [
+    ("affine4", "bf16", 1, 1, 1, 64, 0, 1),
+    ("affine4", "f32", 1, 1, 1, 64, 3, 127),
+    ("sym2", "bf16", 1, 1, 3, 128, 2, 43),       # 129 stacked rows, 45 keys
+    ("kivi2", "bf16", 1, 2, 2, 64, 126, 3),
+    ("affine2", "f32", 2, 1, 2, 128, 0, 65),     # 130 stacked rows
+    ("affine4", "bf16", 1, 1, 2, 256, 1, 130),
+])
+def test_attend_backward_tiles(fmt, act, B, Hkv, Hq, D, T0, L):
+    TB.test_attend_backward_parity(fmt, act, B, Hkv, Hq, D, T0, L)
+
+
+@pytest.mark.parametrize("act,B,L,d_in,Hq,Hkv,D,ranks,extra,pos0,base", [
+    ("bf16", 1, 1, 256, 2, 2, 64, (8, 64, 16), 0, 7, 10000.0),
+    ("bf16", 1, 129, 320, 4, 1, 64, (64, 0, 8), 3, 0, 10000.0),
+    ("f32", 1, 127, 192, 2, 2, 128, (0, 40, 8), 0, 1, 500000.0),
+    ("bf16", 1, 257, 640, 2, 2, 128, (0, 0, 16), 0, 0, 0.0),
+])
+def test_lora_backward_tiles(act, B, L, d_in, Hq, Hkv, D, ranks, extra, pos0, base):
+    TB.test_lora_backward_parity(act, B, L, d_in, Hq, Hkv, D, ranks, extra, pos0, base)
