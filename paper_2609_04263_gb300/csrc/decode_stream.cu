@@ -46,6 +46,9 @@ using namespace stream;
 // bookkeeping of 8-block stages; 77.9 -> 73.4 us on the 8B-shaped KIVI cache),
 // where KVarN's larger blocks keep stream_common's 8
 constexpr int kSBD = 16;
+// Every consumer warp has a block of every whole stage, so none skips one (a barrier
+// is waited for by parity, which tells a phase only from its neighbours).
+static_assert(kSBD >= kNW, "no warp skips a ring stage");
 
 template <int D, int KB, int VB, int FMT>
 struct SCfg {

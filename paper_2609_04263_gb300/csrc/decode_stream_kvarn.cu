@@ -8,7 +8,7 @@
 // CTAs stream equal shares of the flattened (sequence, kv head, 32-token
 // block) space of coded blocks; a producer warp copies runs of blocks (codes,
 // group metadata, row scales) and each block's column-scale rows into ring
-// stages; eight consumer warps take the blocks in turn, tokens as the MMA rows
+// stages; eleven consumer warps take the blocks in turn, tokens as the MMA rows
 // and the GQA heads as its columns.
 //   scores  q_rot = H q / sqrt(D) (times the softmax scale in log2 units) is
 //     formed once per head; per block B = q_rot * c_k as bf16 high + low parts
@@ -31,6 +31,7 @@
 #include <type_traits>
 
 #include "decode_attn.cuh"
+#include "ring_pass.h"
 #include "stream_common.cuh"
 
 namespace kvq {
@@ -316,7 +317,7 @@ decode_stream_kvarn_kernel(Geom g, const __nv_bfloat16* __restrict__ q, float sc
   if (threadIdx.x == 0) {
     for (int i = 0; i < ns; ++i) {
       mbar_init(&full[i], 1);
-      mbar_init(&empty[i], kSB);                     // one arrival per block
+      mbar_init(&empty[i], kNW);                     // every consumer warp leaves every stage
     }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -417,6 +418,10 @@ decode_stream_kvarn_kernel(Geom g, const __nv_bfloat16* __restrict__ q, float sc
   float m_run[2], l_run[2];
   float o[MT][4];
   bool bad = false;
+  static_assert(kSB <= kNW, "a warp has one block of a stage at most");
+  int next = 0;                                      // first stage this warp (lane 0) has not left
+  auto wait_stage = [&](int s) { return mbar_wait(&full[s % ns], (s / ns) & 1); };
+  auto leave_stage = [&](int s) { mbar_arrive1(&empty[s % ns]); };
 
   auto process = [&](const unsigned char* sp, int sub) {
     const unsigned char* kc = sp + C::KC + sub * kBT * C::KCB;
@@ -696,7 +701,7 @@ decode_stream_kvarn_kernel(Geom g, const __nv_bfloat16* __restrict__ q, float sc
     for (int j = jst; j < e && !bad; j += kNW) {
       const int sj = j / kSB, st = sj % ns;
       bool ok = true;
-      if (lane == 0) ok = mbar_wait(&full[st], (sj / ns) & 1);
+      if (lane == 0) ok = ring_pass(next, sj, wait_stage, leave_stage) && wait_stage(sj);
       if (!__shfl_sync(0xffffffffu, ok, 0)) {
         if (lane == 0) atomicOr(err, 1);
         bad = true;
@@ -704,8 +709,15 @@ decode_stream_kvarn_kernel(Geom g, const __nv_bfloat16* __restrict__ q, float sc
       }
       process(smem + (size_t)st * C::STAGE, j % kSB);
       __syncwarp();
-      if (lane == 0) mbar_arrive1(&empty[st]);
+      if (lane == 0) leave_stage(next++);
     }
+    // the other warps may still be waiting for stages of this head: leave all that
+    // come before its last one (which can hold a block of the next head for this warp)
+    if (lane == 0 && !bad && !ring_pass(next, (e - 1) / kSB, wait_stage, leave_stage)) {
+      atomicOr(err, 1);
+      bad = true;
+    }
+    bad = __shfl_sync(0xffffffffu, bad, 0);
     if (mine) {
 #pragma unroll
       for (int jh = 0; jh < 2; ++jh) {
@@ -846,9 +858,8 @@ cudaError_t launch_t(const Geom& g, const void* q, float scale, int* err, void* 
 
 }  // namespace
 
-// At least two ring stages: a warp's next block can lie two stages on, and in a ring
-// of one it would take the phase before last for the one it waits for (eight heads of
-// 256, whose partials leave room for one; the split kernel takes those).
+// At least two ring stages: with one (eight heads of 256, whose partials leave room for
+// one) nothing is copied while a stage is worked on; the split kernel takes those.
 bool decode_stream_kvarn_supported(const Geom& g) {
   const bool shape = (g.D == 256 && g.G == 64) || (g.D == 64 && g.G == 32);
   if (!(g.fmt == KVQ_FMT_KVARN && g.act == KVQ_BF16 && shape && g.kb == 4 && g.vb == 2 &&
