@@ -187,7 +187,9 @@ struct Operand {
 
 // A_KMAJOR: A(m, k) = a[m lda + k], else a[k lda + m].
 // B_KMAJOR: B(k, n) = b[n ldb + k], else b[k ldb + n].
-template <typename TA, typename TB, bool A_KMAJOR, bool B_KMAJOR>
+// CHAIN: the ops are one product, their K ranges behind one another (one batch entry,
+// no splits, no mask).
+template <typename TA, typename TB, bool A_KMAJOR, bool B_KMAJOR, bool CHAIN>
 __global__ void __launch_bounds__(kGemmThreads) bgemm_kernel(const __grid_constant__ GemmArgs g) {
   pdl_wait();
   pdl_trigger();
@@ -197,7 +199,7 @@ __global__ void __launch_bounds__(kGemmThreads) bgemm_kernel(const __grid_consta
   constexpr int kStage = PA * OA::PART + PB * OB::PART;
   extern __shared__ __align__(16) __nv_bfloat16 tiles[];          // two stages of A, B parts
   const int sp = blockIdx.z % g.splits, bz = blockIdx.z / g.splits % g.batch;
-  const GemmOp op = g.op[blockIdx.z / (g.splits * g.batch)];
+  const GemmOp op = g.op[CHAIN ? 0 : blockIdx.z / (g.splits * g.batch)];
   const TA* A = reinterpret_cast<const TA*>(op.a) + (int64_t)bz * g.sa;
   const TB* Bp = reinterpret_cast<const TB*>(op.b) + (int64_t)bz * g.sb;
   float* C = op.c + (int64_t)bz * g.sc;
@@ -210,13 +212,18 @@ __global__ void __launch_bounds__(kGemmThreads) bgemm_kernel(const __grid_consta
       n0 > max_visible(m0, min(m0 + kBM, op.M), g.L, g.T))
     return;                                    // every score of the tile is masked
   if (g.mask == kMaskRowsQueriesKKeys) kend = min(kend, max_visible(m0, min(m0 + kBM, op.M), g.L, g.T) + 1);
-  const int ktiles = (kend + kBK - 1) / kBK;
+  int ktiles = (kend + kBK - 1) / kBK;
+  if (CHAIN)
+    for (int i = 1; i < g.ops; ++i) ktiles += (g.op[i].K + kBK - 1) / kBK;
   const int per = (ktiles + g.splits - 1) / g.splits;
   const int kt0 = sp * per, kt1 = min(ktiles, kt0 + per);
   if (kt0 >= kt1 && g.splits > 1) return;
 
-  const bool veca = ((reinterpret_cast<uintptr_t>(A) | (uintptr_t)(op.lda * sizeof(TA))) & (sizeof(typename OA::V4) - 1)) == 0;
-  const bool vecb = ((reinterpret_cast<uintptr_t>(Bp) | (uintptr_t)(op.ldb * sizeof(TB))) & (sizeof(typename OB::V4) - 1)) == 0;
+  auto aligned = [](const void* p, int64_t ld, int elem, int n) {   // rows start on n-byte boundaries
+    return ((reinterpret_cast<uintptr_t>(p) | (uintptr_t)(ld * elem)) & (n - 1)) == 0;
+  };
+  const bool veca = aligned(A, op.lda, sizeof(TA), sizeof(typename OA::V4));
+  const bool vecb = aligned(Bp, op.ldb, sizeof(TB), sizeof(typename OB::V4));
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int wm = (warp >> 1) * 32, wn = (warp & 1) * 32;          // this warp's 32 x 32 outputs
   float acc[2][4][4] = {};
@@ -226,12 +233,23 @@ __global__ void __launch_bounds__(kGemmThreads) bgemm_kernel(const __grid_consta
     return g.mask == kMaskRowsKeysKQueries &&
            max_visible(kt * kBK, min(kt * kBK + kBK, op.K), g.L, g.T) < m0;
   };
+  auto load = [&](int kt) {
+    if constexpr (CHAIN) {
+      int i = 0;
+      for (int n; kt >= (n = (g.op[i].K + kBK - 1) / kBK); ++i) kt -= n;
+      const GemmOp& o = g.op[i];
+      OA::load(reinterpret_cast<const TA*>(o.a), o.lda, m0, op.M, kt * kBK, o.K,
+               aligned(o.a, o.lda, sizeof(TA), sizeof(typename OA::V4)), ra);
+      OB::load(reinterpret_cast<const TB*>(o.b), o.ldb, n0, op.N, kt * kBK, o.K,
+               aligned(o.b, o.ldb, sizeof(TB), sizeof(typename OB::V4)), rb);
+    } else {
+      OA::load(A, op.lda, m0, op.M, kt * kBK, kend, veca, ra);
+      OB::load(Bp, op.ldb, n0, op.N, kt * kBK, kend, vecb, rb);
+    }
+  };
   int kt = kt0;
   while (kt < kt1 && skip(kt)) ++kt;
-  if (kt < kt1) {
-    OA::load(A, op.lda, m0, op.M, kt * kBK, kend, veca, ra);
-    OB::load(Bp, op.ldb, n0, op.N, kt * kBK, kend, vecb, rb);
-  }
+  if (kt < kt1) load(kt);
   int buf = 0;
   while (kt < kt1) {
     __nv_bfloat16* As = tiles + buf * kStage;
@@ -241,10 +259,7 @@ __global__ void __launch_bounds__(kGemmThreads) bgemm_kernel(const __grid_consta
     __syncthreads();
     int nxt = kt + 1;
     while (nxt < kt1 && skip(nxt)) ++nxt;
-    if (nxt < kt1) {                           // prefetch the next tile into registers
-      OA::load(A, op.lda, m0, op.M, nxt * kBK, kend, veca, ra);
-      OB::load(Bp, op.ldb, n0, op.N, nxt * kBK, kend, vecb, rb);
-    }
+    if (nxt < kt1) load(nxt);                  // prefetch the next tile into registers
 #pragma unroll
     for (int ks = 0; ks < kBK; ks += 16) {
       float c[2][4][4] = {};                   // this step's sums
@@ -297,7 +312,7 @@ __global__ void __launch_bounds__(kGemmThreads) bgemm_kernel(const __grid_consta
     }
 }
 
-template <typename TA, typename TB, bool AK, bool BK>
+template <typename TA, typename TB, bool AK, bool BK, bool CHAIN = false>
 cudaError_t run_gemm(const GemmArgs& g, cudaStream_t s) {
   int M = 0, N = 0;
   for (int i = 0; i < g.ops; ++i) {
@@ -307,11 +322,12 @@ cudaError_t run_gemm(const GemmArgs& g, cudaStream_t s) {
   if (M <= 0 || N <= 0 || g.batch <= 0) return cudaSuccess;
   using OA = Operand<TA, AK>;
   using OB = Operand<TB, BK>;
-  auto kern = bgemm_kernel<TA, TB, AK, BK>;
+  auto kern = bgemm_kernel<TA, TB, AK, BK, CHAIN>;
   constexpr int sm = 2 * (OA::PARTS * OA::PART + OB::PARTS * OB::PART) * 2;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
   if (e != cudaSuccess) return e;
-  dim3 grid((N + kBN - 1) / kBN, (M + kBM - 1) / kBM, g.ops * g.batch * g.splits);
+  dim3 grid((N + kBN - 1) / kBN, (M + kBM - 1) / kBM,
+                  (CHAIN ? 1 : g.ops) * g.batch * g.splits);
   launch_pdl(kern, grid, dim3(kGemmThreads), (size_t)sm, s, g);
   return cudaGetLastError();
 }
@@ -338,26 +354,19 @@ void add_op(GemmArgs& g, const void* a, int64_t lda, const void* b, int64_t ldb,
   g.op[g.ops++] = GemmOp{a, b, c, M, N, K, lda, ldb, ldc};
 }
 
-// fp32 ranges to zero (outputs that splits add to) and activation-typed ranges to
-// copy (the A_p, gathered below one another), in one launch.
-struct PrepArgs {
-  void* dst[16];
-  const void* src[16];          // NULL: zeros
-  int64_t n[16];
-  int act;
+// The fp32 outputs that splits add to, zeroed in one launch.
+struct ZeroArgs {
+  float* dst[12];
+  int64_t n[12];
 };
-__global__ void __launch_bounds__(256) bwd_prepare_kernel(const __grid_constant__ PrepArgs a) {
+__global__ void __launch_bounds__(256) bwd_zero_kernel(const __grid_constant__ ZeroArgs a) {
   pdl_wait();
   pdl_trigger();
-  void* dst = a.dst[blockIdx.y];
-  const void* src = a.src[blockIdx.y];
+  float* dst = a.dst[blockIdx.y];
   const int64_t n = a.n[blockIdx.y];
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    if (!src) reinterpret_cast<float*>(dst)[i] = 0.f;
-    else if (a.act == KVQ_BF16) reinterpret_cast<uint16_t*>(dst)[i] = reinterpret_cast<const uint16_t*>(src)[i];
-    else reinterpret_cast<float*>(dst)[i] = reinterpret_cast<const float*>(src)[i];
-  }
+       i += (int64_t)gridDim.x * blockDim.x)
+    dst[i] = 0.f;
 }
 
 // ---------------------------------------------------------------------------
@@ -597,10 +606,10 @@ int grid_for(int64_t n, int threads) {
 namespace {
 
 // run_gemm with the activation-typed operand(s) chosen by `act`.
-template <bool AK, bool BK>
+template <bool AK, bool BK, bool CHAIN = false>
 cudaError_t gemm_act_b(const GemmArgs& g, int act, cudaStream_t s) {   // B in act dtype
-  return act == KVQ_BF16 ? run_gemm<float, __nv_bfloat16, AK, BK>(g, s)
-                         : run_gemm<float, float, AK, BK>(g, s);
+  return act == KVQ_BF16 ? run_gemm<float, __nv_bfloat16, AK, BK, CHAIN>(g, s)
+                         : run_gemm<float, float, AK, BK, CHAIN>(g, s);
 }
 template <bool AK, bool BK>
 cudaError_t gemm_act_a(const GemmArgs& g, int act, cudaStream_t s) {   // A in act dtype
@@ -675,7 +684,6 @@ size_t lora_backward_bytes(int B, int L, int d_in, int Hq, int Hkv, int D, const
   const size_t BL = (size_t)B * L;
   size_t n = a256(BL * (Hq + 2 * Hkv) * D * sizeof(float));
   for (int p = 0; p < 3; ++p) n += 2 * a256(BL * r[p] * sizeof(float));
-  n += a256((size_t)(r[0] + r[1] + r[2]) * d_in * sizeof(float));   // the A_p below one another
   n += a256((size_t)d_in * (Hq + 2 * Hkv) * D * 2);   // W^T in bf16 for the d_x product
   return n;
 }
@@ -700,14 +708,12 @@ cudaError_t launch_lora_backward(const void* x, int B, int L, int d_in, const vo
   char* wp = static_cast<char*>(ws);
   float* G = reinterpret_cast<float*>(wp);
   wp += a256((size_t)BL * ntot * sizeof(float));
-  const int R = r[0] + r[1] + r[2];
   float* U[3];
-  float* V = reinterpret_cast<float*>(wp);               // [BL][R], one column block per projection
-  wp += a256((size_t)BL * R * sizeof(float));
-  char* Acat = wp;                                       // [R][d_in] in the activations' type
-  wp += a256((size_t)R * d_in * sizeof(float));
+  float* V[3];
   for (int p = 0; p < 3; ++p) {
     U[p] = reinterpret_cast<float*>(wp);
+    wp += a256((size_t)BL * r[p] * sizeof(float));
+    V[p] = reinterpret_cast<float*>(wp);
     wp += a256((size_t)BL * r[p] * sizeof(float));
   }
   __nv_bfloat16* Wt = reinterpret_cast<__nv_bfloat16*>(wp);   // [d_in][ntot]
@@ -723,41 +729,32 @@ cudaError_t launch_lora_backward(const void* x, int B, int L, int d_in, const vo
   // long K), dB_p = (alpha/r) g_p^T U_p [n_p][r], dA_p = (alpha/r) V_p^T x [r][d_in]
   // (over the BL rows): split over K, added atomically into zeroed outputs
   GemmArgs gu = gemm_args(1.f), gv = gemm_args(1.f), gb = gemm_args(alpha_over_r),
-           gA = gemm_args(alpha_over_r);
-  PrepArgs prep = {};
-  prep.act = act;
-  int np = 0, rmax = 0, nmax = 0, ro = 0;
-  const size_t esz = act == KVQ_BF16 ? 2 : 4;
+           gA = gemm_args(alpha_over_r), gl = gemm_args(alpha_over_r);
+  int rmax = 0, nmax = 0;
   for (int p = 0; p < 3; ++p) {
     if (r[p] == 0) continue;
     add_op(gu, x, d_in, a[p], d_in, U[p], r[p], BL, r[p], d_in);
-    add_op(gv, G + off[p], ntot, bm[p], r[p], V + ro, R, BL, r[p], nout[p]);
+    add_op(gv, G + off[p], ntot, bm[p], r[p], V[p], r[p], BL, r[p], nout[p]);
     add_op(gb, G + off[p], ntot, U[p], r[p], db[p], r[p], nout[p], r[p], BL);
-    add_op(gA, V + ro, R, x, d_in, da[p], d_in, r[p], d_in, BL);
-    if (dx) {
-      prep.dst[np] = Acat + (size_t)ro * d_in * esz;
-      prep.src[np] = a[p];
-      prep.n[np++] = (int64_t)r[p] * d_in;
-    }
+    add_op(gA, V[p], r[p], x, d_in, da[p], d_in, r[p], d_in, BL);
+    add_op(gl, V[p], r[p], a[p], d_in, dx, d_in, BL, d_in, r[p]);
     rmax = std::max(rmax, r[p]);
     nmax = std::max(nmax, nout[p]);
-    ro += r[p];
   }
-  if (R > 0 && e == cudaSuccess) {
+  if (gu.ops > 0 && e == cudaSuccess) {
     gu.splits = choose_splits(BL, rmax, d_in, gu.ops);
     gv.splits = choose_splits(BL, rmax, nmax, gv.ops);
     gb.splits = choose_splits(nmax, rmax, BL, gb.ops);
     gA.splits = choose_splits(rmax, d_in, BL, gA.ops);
-    auto zero = [&](float* d, int64_t n) {
-      prep.dst[np] = d;
-      prep.n[np++] = n;
-    };
-    if (gv.splits > 1) zero(V, (int64_t)BL * R);
-    for (const GemmArgs* gg : {&gu, &gb, &gA})
-      for (int i = 0; i < gg->ops && gg->splits > 1; ++i)
-        zero(gg->op[i].c, (int64_t)gg->op[i].M * gg->op[i].N);
-    if (np > 0) {
-      launch_pdl(bwd_prepare_kernel, dim3(32, np), dim3(256), 0, s, prep);
+    ZeroArgs z = {};
+    int nz = 0;
+    for (const GemmArgs* gg : {&gu, &gv, &gb, &gA})
+      for (int i = 0; i < gg->ops && gg->splits > 1; ++i) {
+        z.dst[nz] = gg->op[i].c;
+        z.n[nz++] = (int64_t)gg->op[i].M * gg->op[i].N;
+      }
+    if (nz > 0) {
+      launch_pdl(bwd_zero_kernel, dim3(32, nz), dim3(256), 0, s, z);
       e = cudaGetLastError();
     }
     if (e == cudaSuccess) e = gemm_act_ab<true, true>(gu, act, s);
@@ -791,12 +788,10 @@ cudaError_t launch_lora_backward(const void* x, int B, int L, int d_in, const vo
       add_op(gx, G, ntot, w, d_in, dx, d_in, BL, d_in, ntot);
       e = gemm_act_b<true, false>(gx, act, s);
     }
-    // the adapters' part, [V_q | V_k | V_v] times the A_p, in one pass over dx
-    if (R > 0 && e == cudaSuccess) {
-      GemmArgs gl = gemm_args(alpha_over_r);
+    // the adapters' part, sum_p V_p A_p, in one pass over dx
+    if (gl.ops > 0 && e == cudaSuccess) {
       gl.accumulate = 1;
-      add_op(gl, V, R, Acat, d_in, dx, d_in, BL, d_in, R);
-      e = gemm_act_b<true, false>(gl, act, s);
+      e = gemm_act_b<true, false, true>(gl, act, s);
     }
   }
   return e;

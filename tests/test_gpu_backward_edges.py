@@ -33,6 +33,7 @@ def test_attend_backward_tiles(fmt, act, B, Hkv, Hq, D, T0, L):
     ("bf16", 1, 129, 320, 4, 1, 64, (64, 0, 8), 3, 0, 10000.0),
     ("f32", 1, 127, 192, 2, 2, 128, (0, 40, 8), 0, 1, 500000.0),
     ("bf16", 1, 257, 640, 2, 2, 128, (0, 0, 16), 0, 0, 0.0),
+    ("f32", 1, 66, 192, 2, 1, 64, (5, 33, 64), 0, 0, 10000.0),    # d_x over ranks no K tile divides
 ])
 def test_lora_backward_tiles(act, B, L, d_in, Hq, Hkv, D, ranks, extra, pos0, base):
     TB.test_lora_backward_parity(act, B, L, d_in, Hq, Hkv, D, ranks, extra, pos0, base)
