@@ -410,34 +410,41 @@ __global__ void bwd_reconstruct_kernel(Geom g, int T, int p0, int npairs, float*
 // dS = P o (dP - sum_n P dP) scale over dP; masked entries become 0 as far as
 // the products read them (the 64-row tile's last visible key, rounded up to a
 // 64-key tile).  A warp per row: one pass for the running maximum, sum and
-// sum of P dP, one that rewrites the row, 16 bytes a lane.
+// sum of P dP, one that rewrites the row, 16 bytes a lane where the row length allows.
 // Bound by HBM: S and dP are read twice (once from L2) and written once, the
 // visible half only: 32000 rows of 1000 keys in 62 us (137 us with a CTA per row).
+// Rows follow one another without padding, which would enlarge the workspace; where
+// T is no multiple of 4 this kernel and the products take them element by element:
+// the whole backward of 1000, 1001 tokens (32 / 8 heads of 128) takes 860, 942 us.
 // ---------------------------------------------------------------------------
 constexpr int kRowWarps = 8;
 
+// W: elements per access, 4 where rows start on 16-byte boundaries (T a multiple of 4).
+template <int W>
 __global__ void __launch_bounds__(kRowWarps * 32)
-bwd_softmax_ds_kernel(float* S, float* dP, int M, int T, int ld, int L, float scale) {
+bwd_softmax_ds_kernel(float* S, float* dP, int M, int T, int L, float scale) {
   pdl_wait();
   pdl_trigger();
   const int m = blockIdx.x * kRowWarps + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (m >= M) return;
-  const int64_t row = ((int64_t)blockIdx.y * M + m) * ld;
-  float4* s4 = reinterpret_cast<float4*>(S + row);
-  float4* d4 = reinterpret_cast<float4*>(dP + row);
+  struct __align__(4 * W) Vec { float x[W]; };
+  const int64_t row = ((int64_t)blockIdx.y * M + m) * T;
+  Vec* sv = reinterpret_cast<Vec*>(S + row);
+  Vec* dv = reinterpret_cast<Vec*>(dP + row);
   const int nvis = T - L + m % L + 1;        // keys 0 .. T - L + l are visible
   const int tile = m / kBM * kBM;
   const int nend = min(T, (max_visible(tile, min(tile + kBM, M), L, T) / kBN + 1) * kBN);
   float mx = -INFINITY, sum = 0.f, dot = 0.f;
 #pragma unroll 4
-  for (int n = 4 * lane; n < nvis; n += 128) {
-    const float4 a = s4[n / 4], b = d4[n / 4];
-    const float d[4] = {b.x, b.y, b.z, b.w};
-    float s[4] = {a.x, a.y, a.z, a.w};
+  for (int n = W * lane; n < nvis; n += 32 * W) {
+    Vec s = sv[n / W];
+    const Vec d = dv[n / W];
+    float top = -INFINITY;
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
-      if (n + i >= nvis) s[i] = -INFINITY;
-    const float top = fmaxf(fmaxf(s[0], s[1]), fmaxf(s[2], s[3]));
+    for (int i = 0; i < W; ++i) {
+      if (n + i >= nvis) s.x[i] = -INFINITY;
+      top = fmaxf(top, s.x[i]);
+    }
     if (top > mx) {
       const float f = expf(scale * (mx - top));
       sum *= f;
@@ -445,11 +452,11 @@ bwd_softmax_ds_kernel(float* S, float* dP, int M, int T, int ld, int L, float sc
       mx = top;
     }
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+    for (int i = 0; i < W; ++i)
       if (n + i < nvis) {
-        const float e = expf(scale * (s[i] - mx));
+        const float e = expf(scale * (s.x[i] - mx));
         sum += e;
-        dot = fmaf(e, d[i], dot);
+        dot = fmaf(e, d.x[i], dot);
       }
   }
   float top = mx;
@@ -466,20 +473,19 @@ bwd_softmax_ds_kernel(float* S, float* dP, int M, int T, int ld, int L, float sc
   const float inv = 1.f / sum;
   const float delta = dot * inv;             // sum_n P dP
 #pragma unroll 4
-  for (int n = 4 * lane; n < nend; n += 128) {
-    const float4 a = s4[n / 4], b = d4[n / 4];
-    const float s[4] = {a.x, a.y, a.z, a.w}, d[4] = {b.x, b.y, b.z, b.w};
-    float p[4], ds[4];
+  for (int n = W * lane; n < nend; n += 32 * W) {
+    const Vec s = sv[n / W], d = dv[n / W];
+    Vec p, ds;
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      p[i] = ds[i] = 0.f;
+    for (int i = 0; i < W; ++i) {
+      p.x[i] = ds.x[i] = 0.f;
       if (n + i < nvis) {
-        p[i] = expf(scale * (s[i] - top)) * inv;
-        ds[i] = p[i] * (d[i] - delta) * scale;
+        p.x[i] = expf(scale * (s.x[i] - top)) * inv;
+        ds.x[i] = p.x[i] * (d.x[i] - delta) * scale;
       }
     }
-    s4[n / 4] = make_float4(p[0], p[1], p[2], p[3]);
-    d4[n / 4] = make_float4(ds[0], ds[1], ds[2], ds[3]);
+    sv[n / W] = p;
+    dv[n / W] = ds;
   }
 }
 
@@ -626,12 +632,9 @@ size_t a256(size_t x) { return (x + 255) & ~size_t(255); }
 
 }  // namespace
 
-// Rows of S and dP in the workspace start on 16-byte boundaries.
-static int score_pitch(int T) { return (T + 3) & ~3; }
-
 size_t attend_backward_pair_bytes(const Geom& g, int T, int L) {
   const size_t gl = (size_t)(g.Hq / g.H) * L;
-  return a256((2 * (size_t)T * g.D + 2 * gl * score_pitch(T)) * sizeof(float));
+  return a256((2 * (size_t)T * g.D + 2 * gl * T) * sizeof(float));
 }
 
 cudaError_t launch_attend_backward(const Geom& g, int T, const void* q, const void* d_out,
@@ -639,7 +642,7 @@ cudaError_t launch_attend_backward(const Geom& g, int T, const void* q, const vo
                                    void* ws, size_t ws_bytes, cudaStream_t s) {
   const int pairs = g.B * g.H, grp = g.Hq / g.H, D = g.D;
   const int M = grp * L;
-  const int act = g.act, ld = score_pitch(T);
+  const int act = g.act;
   const size_t esz = act == KVQ_BF16 ? 2 : 4;
   const int chunk = (int)std::min<size_t>(pairs, ws_bytes / attend_backward_pair_bytes(g, T, L));
   cudaError_t e = cudaSuccess;
@@ -648,32 +651,33 @@ cudaError_t launch_attend_backward(const Geom& g, int T, const void* q, const vo
     float* kh = static_cast<float*>(ws);
     float* vh = kh + (size_t)np * T * D;
     float* S = vh + (size_t)np * T * D;
-    float* dP = S + (size_t)np * M * ld;
+    float* dP = S + (size_t)np * M * T;
     const char* qp = static_cast<const char*>(q) + (size_t)p0 * M * D * esz;
     const char* op = static_cast<const char*>(d_out) + (size_t)p0 * M * D * esz;
     launch_pdl(bwd_reconstruct_kernel, dim3(grid_for((int64_t)np * T * D / 8, 256)), dim3(256),
                0, s, g, T, p0, np, kh, vh);
     e = cudaGetLastError();
     // S = Q K^T and dP = dO V^T (tiles above the causal edge skipped)
-    GemmArgs ga = gemm_args(1.f, np, (int64_t)M * D, (int64_t)T * D, (int64_t)M * ld);
-    add_op(ga, qp, D, kh, D, S, ld, M, T, D);
-    add_op(ga, op, D, vh, D, dP, ld, M, T, D);
+    GemmArgs ga = gemm_args(1.f, np, (int64_t)M * D, (int64_t)T * D, (int64_t)M * T);
+    add_op(ga, qp, D, kh, D, S, T, M, T, D);
+    add_op(ga, op, D, vh, D, dP, T, M, T, D);
     ga.mask = kMaskRowsQueriesColsKeys; ga.L = L; ga.T = T;
     if (e == cudaSuccess) e = gemm_act_a<true, true>(ga, act, s);
     if (e == cudaSuccess) {
-      launch_pdl(bwd_softmax_ds_kernel, dim3((M + kRowWarps - 1) / kRowWarps, np),
-                 dim3(kRowWarps * 32), 0, s, S, dP, M, T, ld, L, scale);
+      launch_pdl(T % 4 == 0 ? bwd_softmax_ds_kernel<4> : bwd_softmax_ds_kernel<1>,
+                 dim3((M + kRowWarps - 1) / kRowWarps, np), dim3(kRowWarps * 32), 0, s, S, dP, M, T,
+                 L, scale);
       e = cudaGetLastError();
     }
     // dQ = dS K
-    GemmArgs gq = gemm_args(1.f, np, (int64_t)M * ld, (int64_t)T * D, (int64_t)M * D);
-    add_op(gq, dP, ld, kh, D, dq + (size_t)p0 * M * D, D, M, D, T);
+    GemmArgs gq = gemm_args(1.f, np, (int64_t)M * T, (int64_t)T * D, (int64_t)M * D);
+    add_op(gq, dP, T, kh, D, dq + (size_t)p0 * M * D, D, M, D, T);
     gq.mask = kMaskRowsQueriesKKeys; gq.L = L; gq.T = T;
     if (e == cudaSuccess) e = run_gemm<float, float, true, false>(gq, s);
     // dK = dS^T Q and dV = P^T dO
-    GemmArgs gk = gemm_args(1.f, np, (int64_t)M * ld, (int64_t)M * D, (int64_t)T * D);
-    add_op(gk, dP, ld, qp, D, dk + (size_t)p0 * T * D, D, T, D, M);
-    add_op(gk, S, ld, op, D, dv + (size_t)p0 * T * D, D, T, D, M);
+    GemmArgs gk = gemm_args(1.f, np, (int64_t)M * T, (int64_t)M * D, (int64_t)T * D);
+    add_op(gk, dP, T, qp, D, dk + (size_t)p0 * T * D, D, T, D, M);
+    add_op(gk, S, T, op, D, dv + (size_t)p0 * T * D, D, T, D, M);
     gk.mask = kMaskRowsKeysKQueries; gk.L = L; gk.T = T;
     if (e == cudaSuccess) e = gemm_act_b<false, false>(gk, act, s);
   }

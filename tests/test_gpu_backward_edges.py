@@ -37,3 +37,16 @@ def test_attend_backward_tiles(fmt, act, B, Hkv, Hq, D, T0, L):
 ])
 def test_lora_backward_tiles(act, B, L, d_in, Hq, Hkv, D, ranks, extra, pos0, base):
     TB.test_lora_backward_parity(act, B, L, d_in, Hq, Hkv, D, ranks, extra, pos0, base)
+
+
+@pytest.mark.parametrize("L", [44, 45, 46, 47])
+def test_attend_backward_workspace(L):
+    """One pair's workspace is its K, V reconstruction and its S and dP, nothing more,
+    whatever the number of keys is a multiple of."""
+    from paper_2609_04263_gb300 import kvq
+    B, Hkv, Hq, D, T0 = 1, 1, 3, 64, 20
+    gc, _ = TB._filled(TB.FORMATS["affine4"], "bf16", B, Hkv, Hq, D, T0, L, seed=L)
+    T = T0 + L
+    want = (2 * T * D + 2 * (Hq // Hkv) * L * T) * 4
+    assert kvq.kvq_attend_backward_workspace(gc.handle, L, Hq) == (want + 255) // 256 * 256
+    TB.test_attend_backward_parity("affine4", "bf16", B, Hkv, Hq, D, T0, L)
