@@ -644,7 +644,9 @@ cudaError_t launch_attend_backward(const Geom& g, int T, const void* q, const vo
   const int M = grp * L;
   const int act = g.act;
   const size_t esz = act == KVQ_BF16 ? 2 : 4;
-  const int chunk = (int)std::min<size_t>(pairs, ws_bytes / attend_backward_pair_bytes(g, T, L));
+  // (two products of every pair share a launch: grid.z is at most 65,535)
+  const int chunk = (int)std::min<size_t>(std::min(pairs, 65535 / 2),
+                                          ws_bytes / attend_backward_pair_bytes(g, T, L));
   cudaError_t e = cudaSuccess;
   for (int p0 = 0; p0 < pairs && e == cudaSuccess; p0 += chunk) {
     const int np = std::min(chunk, pairs - p0);

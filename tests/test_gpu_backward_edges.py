@@ -4,6 +4,7 @@ tile, key counts that no vector load divides, head_dim 64 to 256, adapters of
 unlike ranks (whose products share a launch) and rows short of a tile.  The
 checks and tolerances are those of the other backward tests."""
 import pytest
+import torch
 
 from tests import test_gpu_backward as TB
 from tests.gpu_common import require_gpu
@@ -50,3 +51,20 @@ def test_attend_backward_workspace(L):
     want = (2 * T * D + 2 * (Hq // Hkv) * L * T) * 4
     assert kvq.kvq_attend_backward_workspace(gc.handle, L, Hq) == (want + 255) // 256 * 256
     TB.test_attend_backward_parity("affine4", "bf16", B, Hkv, Hq, D, T0, L)
+
+
+def test_attend_backward_many_pairs():
+    """More (sequence, kv head) pairs than one launch of paired products has grid
+    slices for (32,767), against fp64 autograd."""
+    B, H, L, D, scale = 33000, 1, 3, 64, 0.125
+    gc = TB.gpu_cache(TB.FORMATS["float"], B, H, H, D, L, "f32")
+    gen = torch.Generator("cuda").manual_seed(4)
+    q, k, v, do = (torch.randn(B, H, L, D, generator=gen, device="cuda") for _ in range(4))
+    gc.append(k, v)
+    got = gc.attend_backward(q, do, scale=scale)
+    ref = [t.double().requires_grad_() for t in (q, k, v)]
+    s = ref[0] @ ref[1].transpose(-1, -2) * scale
+    s = s.masked_fill(torch.ones(L, L, dtype=torch.bool, device="cuda").triu(1), float("-inf"))
+    (s.softmax(-1) @ ref[2]).backward(do.double())
+    for g, r, what in zip(got, ref, ("dq", "dk", "dv")):
+        TB._close(g.cpu().numpy(), r.grad.cpu().numpy(), what)
