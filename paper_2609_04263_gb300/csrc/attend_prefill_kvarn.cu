@@ -12,8 +12,8 @@
 // 64 tokens' half of the channels, which is how a pair of CTAs shares the second
 // operand of its MMAs.  Three roles:
 //   producers: reconstruct their share in fp32 into three shared buffers, K
-//     (warps 4-7) as a bf16 high part (the value truncated) plus the bf16 of the
-//     remainder, V (warps 8-11) rounded to fp16 and transposed (channels x
+//     (warps 4-7) as a bf16 high part (the value rounded: a truncated one would leave
+//     a remainder of one bit more) plus the bf16 of the remainder, V (warps 8-11) rounded to fp16 and transposed (channels x
 //     tokens).  A key warp builds 64 channels, a lane one token; a value warp 32
 //     channels, a lane two neighbouring tokens (one 32-bit store each channel).
 //     The packed words and scales of the next tile are loaded into registers
@@ -240,10 +240,10 @@ __device__ __forceinline__ void build_coded(const Packed<BITS, V>& p, bool in, i
         const uint64_t k2 = fmul2(ffma2(code, ks2, kz2), cc[i]);
         float a, b;
         f2unpack(k2, a, b);
-        const uint32_t ab = __float_as_uint(a) & 0xFFFF0000u, bb = __float_as_uint(b) & 0xFFFF0000u;
-        h[i] = __byte_perm(ab, bb, 0x7632);
+        h[i] = pack_bf16(a, b);
+        const float ah = __uint_as_float(h[i] << 16), bh = __uint_as_float(h[i] & 0xFFFF0000u);
         float ra, rb;
-        f2unpack(fadd2(k2, f2pack(-__uint_as_float(ab), -__uint_as_float(bb))), ra, rb);
+        f2unpack(fadd2(k2, f2pack(-ah, -bh)), ra, rb);
         l[i] = pack_bf16(ra, rb);
       }
       const int off = sw128(lane, c);
@@ -315,9 +315,8 @@ __device__ __noinline__ void build_full(const Geom& g, int b, int h, int t0, int
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
           const float x0 = x[8 * k + 2 * e], x1 = x[8 * k + 2 * e + 1];
-          const uint32_t a = __float_as_uint(x0) & 0xFFFF0000u, c = __float_as_uint(x1) & 0xFFFF0000u;
-          hw[e] = __byte_perm(a, c, 0x7632);
-          lw[e] = pack_bf16(x0 - __uint_as_float(a), x1 - __uint_as_float(c));
+          hw[e] = pack_bf16(x0, x1);
+          lw[e] = pack_bf16(x0 - __uint_as_float(hw[e] << 16), x1 - __uint_as_float(hw[e] & 0xFFFF0000u));
         }
         unsigned char* d = kv + k * (kHalf * 128) + sw128(r, sub);
         *reinterpret_cast<uint4*>(d + kKH) = make_uint4(hw[0], hw[1], hw[2], hw[3]);

@@ -55,3 +55,52 @@ def test_prefill_parity(kb, vb, S, B, H, Hq, T, L):
     assert kvq.kvq_device_status(torch.cuda.current_stream().cuda_stream) == 0
     err = np.abs(got - O.attend(oc, q.float().numpy())).max()
     assert err <= 2e-2, f"max-abs {err}"
+
+
+def _one_query(gc, Q):
+    """The newest token's query Q e_1 (rotated: Q / 16 with alternating signs), at scale 1:
+    the output's channel 0 over 16."""
+    q = torch.zeros(1, 1, 1, D)
+    q[..., 1] = Q
+    return gc.attend_prefill(q.bfloat16().cuda(), scale=1.0).float().cpu().numpy()[0, 0, 0, 0] / 16
+
+
+def test_full_precision_key_bits():
+    """A sink's key keeps 16 bits and more beside a bf16 high part that is rounded: its
+    rotated channels are (1 +- b +- g) / 16 with b = 255 2^-15 and g = 2^-16, and a
+    query that sees g alone has the score 2^16 g = 1 against the zero key's 0.
+    After a truncated high part the remainder b +- g needs nine bits, and the
+    score comes out as 1.5.  The bound is bf16's of the output."""
+    gc = gpu_cache(dict(fmt=O.FMT_KVARN, key_bits=4, value_bits=2, group_size=64, sink_tokens=128,
+                        norm_iters=8), 1, 1, 1, D, 8, "bf16")
+    k, v = torch.zeros(1, 1, 2, D), torch.zeros(1, 1, 2, D)
+    k[0, 0, 1, 0], k[0, 0, 1, 2], k[0, 0, 1, 1] = 1.0, 255 * 2.0 ** -15, 2.0 ** -16
+    v[0, 0, 1, 0] = 16.0
+    gc.append(k.bfloat16().cuda(), v.bfloat16().cuda())
+    want = 1 / (1 + np.exp(-1.0))
+    assert abs(_one_query(gc, 2.0 ** 16) - want) <= 2 ** -8 * want
+
+
+def test_coded_key_bits():
+    """The same of coded keys: two tokens of one block with equal scores, 543.  One key is
+    r c_j with factors whose product a truncated high part and a bf16 remainder hold
+    2^-16 off (score 1 off), a rounded one exactly; the other's group
+    offsets (52, 60, 64, 72 / 1024 above 1, mean 62) are exact either way.  The
+    block's other keys are zero."""
+    gc = gpu_cache(dict(fmt=O.FMT_KVARN, key_bits=4, value_bits=2, group_size=64, sink_tokens=0,
+                        norm_iters=8), 1, 1, 1, D, 64, "bf16")
+    kt, vt, _, _ = kv_pair(1, 1, 64, D, "bf16", seed=1)
+    gc.append(kt, vt)
+    pl = gc.planes()
+    for n in ("k_codes", "k_scale", "k_row", "v_codes", "v_scale", "v_row"):
+        pl[n].zero_()
+    for n in ("k_zero", "v_zero", "v_col"):
+        pl[n].fill_(1.0)
+    pl["k_col"][..., 0::2] = 1 + 24 / 1024
+    pl["k_col"][..., 1::2] = 1 + 8 / 1024
+    rows = pl["k_row"].view(-1)
+    rows[0] = 1 + 62 / 1024
+    rows[1] = 1.0
+    pl["k_zero"][0, 0, 1] = 1 + torch.tensor([52.0, 60.0, 64.0, 72.0]) / 1024
+    pl["v_row"].view(-1)[0] = 1.0
+    assert abs(_one_query(gc, 2.0 ** 12) - 0.5) <= 2 ** -8 * 0.5
