@@ -134,15 +134,17 @@ struct PackedChunks {
   __device__ __forceinline__ void expand(const Geom& g, int which, int n, float* dst, int ld) const {
     const int bits = which ? g.vb : g.kb;
     const unsigned mask = (1u << bits) - 1;
+    // symmetric: (code - zero) x scale, which is infinite, not NaN, where the scale is
+    const int zero = g.fmt == KVQ_FMT_SYMMETRIC ? 1 << (bits - 1) : 0;
 #pragma unroll
     for (int i = 0; i < NI; ++i) {
       const int idx = threadIdx.x + kThreads * i, c = idx % (D / 8), r = idx / (D / 8);
       if (r >= n) continue;
-      const float sc = __half2float(s[i]);
-      const float m = g.fmt == KVQ_FMT_SYMMETRIC ? -(float)(1 << (bits - 1)) * sc : __half2float(z[i]);
+      const float sc = __half2float(s[i]), m = __half2float(z[i]);
       float v[8];
 #pragma unroll
-      for (int e = 0; e < 8; ++e) v[e] = (float)((unsigned)(w[i] >> (e * bits)) & mask) * sc + m;
+      for (int e = 0; e < 8; ++e)
+        v[e] = (float)((int)((unsigned)(w[i] >> (e * bits)) & mask) - zero) * sc + m;
       float4* d = reinterpret_cast<float4*>(dst + r * ld + 8 * c);
       d[0] = make_float4(v[0], v[1], v[2], v[3]);
       d[1] = make_float4(v[4], v[5], v[6], v[7]);

@@ -60,3 +60,19 @@ def test_prefill_64_row_ctas():
 def test_decode(name, act, D, B, H, Hq, T):
     gc, oc = _caches(name, act, B, H, Hq, D, T)
     _check(gc, oc, B, Hq, 1, D, act, True)
+
+
+@pytest.mark.parametrize("decode", [False, True])
+def test_infinite_scale(decode):
+    """A symmetric group whose scale is beyond fp16 stores an infinite scale, and its
+    value is an infinity of the code's sign (the channels' codes here are all
+    below zero): so is the output, and the other channels are what they were."""
+    D, T = 64, 5
+    gc = gpu_cache(FORMATS["sym4"], 1, 1, 1, D, T, "f32")
+    kt, vt, _, _ = kv_pair(1, 1, T, D, "f32", seed=3)
+    vt[..., 32:] = -1e6
+    gc.append(kt, vt)
+    assert torch.isinf(gc.planes()["v_scale"][0, 0, :T, 1]).all()
+    q = torch.from_numpy(synth.queries((1, 1, 1, D), seed=2)).cuda()
+    got = (gc.attend_decode if decode else gc.attend_prefill)(q)[0, 0, 0]
+    assert torch.isneginf(got[32:]).all() and torch.isfinite(got[:32]).all()
