@@ -26,8 +26,8 @@ __device__ __forceinline__ unsigned code_at(const uint8_t* row, int d, int bits)
 // KVarN: tokens [t0, t0 + n) of one (b, h) in the rotated basis into dst
 // [n][ld] (fp32): the coded rows are stored rotated, the full-precision rows
 // (sinks, staged) are rotated forward.  which = 0 keys, 1 values; T = tokens
-// stored; tokens from T on are zero.
-__device__ void kvarn_rows(const Geom& g, int which, int b, int h, int t0, int n, int T,
+// stored; tokens from `end` on are zero.
+__device__ void kvarn_rows(const Geom& g, int which, int b, int h, int t0, int n, int end, int T,
                            float* dst, int ld, float inv_sqrt_d) {
   const int D = g.D, G = g.G;
   const int bits = which ? g.vb : g.kb;
@@ -42,7 +42,7 @@ __device__ void kvarn_rows(const Geom& g, int which, int b, int h, int t0, int n
   for (int i = threadIdx.x; i < n * D; i += blockDim.x) {
     const int r = i / D, d = i % D, t = t0 + r;
     float val = 0.f;
-    if (t < T) {
+    if (t < end) {
       if (t < g.S) {
         val = ld_act(g.pl[P_FULL].p, plane_index(g.pl[P_FULL], b, h, g.H, t, d), g.act);
       } else if (t - g.S < nbq) {
@@ -79,23 +79,24 @@ __device__ void kvarn_rows(const Geom& g, int which, int b, int h, int t0, int n
   }
 }
 
-// The other formats: 8 channels of a token per thread and step.
+// The other formats: 8 channels of a token per thread and step; tokens from `end` on
+// are zero.
 template <int D>
 __device__ __forceinline__ void dequant_rows(const Geom& g, int which, int b, int h, int t0, int n,
-                                             int T, int tq, float* dst, int ld) {
+                                             int end, int tq, float* dst, int ld) {
   const bool f32 = g.act == KVQ_F32;
   const int P_FULL = which ? KVQ_PLANE_V_FULL : KVQ_PLANE_K_FULL;
   for (int i = threadIdx.x; i < n * (D / 8); i += kThreads) {
     const int r = i / (D / 8), c = i % (D / 8), t = t0 + r;
     float4* d4 = reinterpret_cast<float4*>(dst + r * ld + 8 * c);
-    if (f32 && t < T && (g.fmt == KVQ_FMT_FLOAT || (g.fmt == KVQ_FMT_KIVI && t >= tq))) {
+    if (f32 && t < end && (g.fmt == KVQ_FMT_FLOAT || (g.fmt == KVQ_FMT_KIVI && t >= tq))) {
       const float4* src = reinterpret_cast<const float4*>(
           plane_ptr<float>(g, P_FULL, b, h, g.fmt == KVQ_FMT_KIVI ? t % g.ring : t, 8 * c));
       d4[0] = src[0];
       d4[1] = src[1];
     } else {
       float v[8];
-      deq8(g, which, b, h, t, c, T, tq, v);
+      deq8(g, which, b, h, t, c, end, tq, v);
       d4[0] = make_float4(v[0], v[1], v[2], v[3]);
       d4[1] = make_float4(v[4], v[5], v[6], v[7]);
     }
@@ -260,7 +261,9 @@ attend_generic_kernel(Geom g, const void* q, int L, float scale, void* out,
 
   for (int t0 = ts; t0 < te; t0 += kTile) {
     const int n = min(kTile, te - t0);
-    const int n4 = (n + 3) & ~3;                  // rows of V read below
+    // rows read below: those past the last token are zero, not the next tokens
+    // (weight 0 times an infinite value is NaN)
+    const int n4 = (n + 3) & ~3;
     __syncthreads();                              // previous tile consumed (and q stored)
     if (packed) {
       pk.expand(g, 0, n4, sm.k, S::LDK);
@@ -270,11 +273,11 @@ attend_generic_kernel(Geom g, const void* q, int L, float scale, void* out,
         pv.load(g, 1, b, hkv, t0 + kTile, te - t0 - kTile, T, lg);
       }
     } else if (kvarn) {
-      kvarn_rows(g, 0, b, hkv, t0, n4, T, sm.k, S::LDK, inv_sqrt_d);
-      kvarn_rows(g, 1, b, hkv, t0, n4, T, sm.v, D, inv_sqrt_d);
+      kvarn_rows(g, 0, b, hkv, t0, n4, te, T, sm.k, S::LDK, inv_sqrt_d);
+      kvarn_rows(g, 1, b, hkv, t0, n4, te, T, sm.v, D, inv_sqrt_d);
     } else {
-      dequant_rows<D>(g, 0, b, hkv, t0, n4, T, tq, sm.k, S::LDK);
-      dequant_rows<D>(g, 1, b, hkv, t0, n4, T, tq, sm.v, D);
+      dequant_rows<D>(g, 0, b, hkv, t0, n4, te, tq, sm.k, S::LDK);
+      dequant_rows<D>(g, 1, b, hkv, t0, n4, te, tq, sm.v, D);
     }
     __syncthreads();
     if ((warp >> 2) * 32 < n4) {

@@ -76,3 +76,16 @@ def test_infinite_scale(decode):
     q = torch.from_numpy(synth.queries((1, 1, 1, D), seed=2)).cuda()
     got = (gc.attend_decode if decode else gc.attend_prefill)(q)[0, 0, 0]
     assert torch.isneginf(got[32:]).all() and torch.isfinite(got[:32]).all()
+
+
+@pytest.mark.parametrize("name", ["float", "kivi2"])
+def test_infinite_later_value(name):
+    """Queries whose CTA ends before a token do not read its value, also where the
+    number of keys they see is no multiple of 4."""
+    D, T, L, t_inf = 64, 207, 200, 135            # the 128th query is at position 134
+    gc = gpu_cache(FORMATS[name], 1, 1, 1, D, T, "f32")
+    kt, vt, _, _ = kv_pair(1, 1, T, D, "f32", seed=5)
+    vt[:, :, t_inf:] = float("inf")
+    gc.append(kt, vt)
+    q = torch.from_numpy(synth.queries((1, 1, L, D), seed=6)).cuda()
+    assert torch.isfinite(gc.attend_prefill(q)[:, :, :128]).all()
