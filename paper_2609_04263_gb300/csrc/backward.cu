@@ -454,7 +454,8 @@ bwd_softmax_ds_kernel(float* S, float* dP, int M, int T, int L, float scale) {
 #pragma unroll
     for (int i = 0; i < W; ++i)
       if (n + i < nvis) {
-        const float e = expf(scale * (s.x[i] - mx));
+        // (no finite score so far: an infinite one has weight 0, and -inf - -inf is NaN)
+        const float e = s.x[i] == -INFINITY ? 0.f : expf(scale * (s.x[i] - mx));
         sum += e;
         dot = fmaf(e, d.x[i], dot);
       }

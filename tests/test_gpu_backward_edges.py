@@ -68,3 +68,28 @@ def test_attend_backward_many_pairs():
     (s.softmax(-1) @ ref[2]).backward(do.double())
     for g, r, what in zip(got, ref, ("dq", "dk", "dv")):
         TB._close(g.cpu().numpy(), r.grad.cpu().numpy(), what)
+
+
+@pytest.mark.parametrize("T", [20, 21])
+def test_attend_backward_infinite_scores(T):
+    """Keys whose scores lie below fp32 (-9e38) have weight 0: they are the first of
+    a lane's keys, four at a time (T = 20) and one at a time."""
+    D, L, scale = 64, 16, 0.125
+    n = T - L
+    gc = TB.gpu_cache(TB.FORMATS["float"], 1, 1, 1, D, T, "f32")
+    gen = torch.Generator("cuda").manual_seed(T)
+    q, k, v, do = (torch.randn(1, 1, x, D, generator=gen, device="cuda") for x in (L, T, T, L))
+    k[..., 0] = 0
+    k[0, 0, :n] = 0
+    k[0, 0, :n, 0] = -3e19
+    q[..., 0] = 3e19
+    gc.append(k, v)
+    got = gc.attend_backward(q, do, scale=scale)
+    ref = [t.double().requires_grad_() for t in (q, k, v)]
+    s = ref[0] @ ref[1].transpose(-1, -2) * scale
+    s = s.masked_fill(torch.ones(L, T, dtype=torch.bool, device="cuda").triu(n + 1), float("-inf"))
+    (s.softmax(-1) @ ref[2]).backward(do.double())
+    # (d_k's channel 0 is a sum over the queries' 3e19)
+    for g, r, what in zip((got[0], got[1][..., 1:], got[2]),
+                          (ref[0].grad, ref[1].grad[..., 1:], ref[2].grad), ("dq", "dk", "dv")):
+        TB._close(g.cpu().numpy(), r.cpu().numpy(), what)
