@@ -45,7 +45,9 @@ namespace {
 // lie below 2^-24 of the product.  The tensor cores truncate as they
 // accumulate, so they sum 16 k at a time from zero (the products of the leading
 // parts last), added to the fp32 accumulator with a rounding addition: the error against
-// 64 bits is not above that of the fp32 chain this replaces.
+// 64 bits is not above that of the fp32 chain this replaces.  An infinite value has
+// no such parts (infinity times the other operand's zero parts is NaN): a 32-k step with
+// one runs in fp32.
 // What bounds it is the splitting and the fragment loads, not the MMAs (about 200
 // of 400 issue slots per warp and chunk at six products), which is why 64 x 64 tiles on
 // mma.sync, four CTAs per SM and no staging in tensor memory serve here.
@@ -143,7 +145,10 @@ struct Operand {
       }
     }
   }
-  static __device__ __forceinline__ void store(__nv_bfloat16* s, const V4 (&v)[4]) {
+  // True if a value has no parts: infinite, NaN, or beyond bf16's range.  (Its first
+  // part is then infinite or NaN and the others NaN.)
+  static __device__ __forceinline__ bool store(__nv_bfloat16* s, const V4 (&v)[4]) {
+    uint32_t top = 0;                // largest of the parts that are NaN (0x7FFF) in that case, as int16 pairs
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       int r, k;
@@ -151,6 +156,7 @@ struct Operand {
       __nv_bfloat16* d = s + (KMAJOR ? r * PITCH + k : k * PITCH + r);
       if constexpr (PARTS == 1) {
         *reinterpret_cast<uint2*>(d) = v[i];
+        top = __vmaxs2(top, __vmaxs2(v[i].x & 0x7FFF7FFFu, v[i].y & 0x7FFF7FFFu));
       } else {
         float x[4] = {v[i].x, v[i].y, v[i].z, v[i].w};
 #pragma unroll
@@ -166,9 +172,20 @@ struct Operand {
             x[2 * h + 1] -= f.y;
           }
           *reinterpret_cast<uint2*>(d + part * PART) = u;
+          if (part == 2) top = __vmaxs2(top, __vmaxs2(u.x, u.y));
         }
       }
     }
+    constexpr uint32_t kInf = 0x7F80u;
+    return (top & 0xFFFFu) >= kInf || (top >> 16) >= kInf;
+  }
+  // Element (r, k) of a stored tile.
+  static __device__ __forceinline__ float at(const __nv_bfloat16* s, int r, int k) {
+    const __nv_bfloat16* p = s + (KMAJOR ? r * PITCH + k : k * PITCH + r);
+    const float x = __bfloat162float(p[0]);
+    if (PARTS == 1) return x;
+    const float lo = __bfloat162float(p[PART]) + __bfloat162float(p[(PARTS - 1) * PART]);
+    return isnan(lo) ? x : x + lo;
   }
   // The 16 x 16 A fragment at rows r, k-step k.
   static __device__ __forceinline__ void frag_a(const __nv_bfloat16* s, int r, int k, int lane,
@@ -254,12 +271,26 @@ __global__ void __launch_bounds__(kGemmThreads) bgemm_kernel(const __grid_consta
   while (kt < kt1) {
     __nv_bfloat16* As = tiles + buf * kStage;
     __nv_bfloat16* Bs = As + PA * OA::PART;
-    OA::store(As, ra);
-    OB::store(Bs, rb);
-    __syncthreads();
+    bool odd = OA::store(As, ra);
+    odd |= OB::store(Bs, rb);
+    // (two bf16 operands multiply as they are)
+    if (PA + PB > 2) odd = __syncthreads_or(odd);
+    else __syncthreads();
     int nxt = kt + 1;
     while (nxt < kt1 && skip(nxt)) ++nxt;
     if (nxt < kt1) load(nxt);                  // prefetch the next tile into registers
+    if (PA + PB > 2 && odd) {                  // a value without parts: in fp32
+#pragma unroll 1
+      for (int k = 0; k < kBK; ++k)
+#pragma unroll
+        for (int m = 0; m < 2; ++m)
+#pragma unroll
+          for (int n = 0; n < 4; ++n)
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+              acc[m][n][i] = fmaf(OA::at(As, wm + 16 * m + 8 * (i >> 1) + (lane >> 2), k),
+                                  OB::at(Bs, wn + 8 * n + 2 * (lane & 3) + (i & 1), k), acc[m][n][i]);
+    } else
 #pragma unroll
     for (int ks = 0; ks < kBK; ks += 16) {
       float c[2][4][4] = {};                   // this step's sums

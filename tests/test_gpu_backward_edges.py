@@ -93,3 +93,23 @@ def test_attend_backward_infinite_scores(T):
     for g, r, what in zip((got[0], got[1][..., 1:], got[2]),
                           (ref[0].grad, ref[1].grad[..., 1:], ref[2].grad), ("dq", "dk", "dv")):
         TB._close(g.cpu().numpy(), r.cpu().numpy(), what)
+
+
+def test_attend_backward_infinite_key():
+    """A key with an infinite channel, of scores -inf, has weight 0: all gradients but
+    d_q's along that channel (0 times the key's infinity) are what they are for a
+    key of large scores.  Both of the last query's tiles of 32 keys hold others."""
+    D, T, L, scale = 64, 70, 66, 0.125
+    gen = torch.Generator("cuda").manual_seed(1)
+    q, k, v, do = (torch.randn(1, 1, x, D, generator=gen, device="cuda") for x in (L, T, T, L))
+    q[..., 5] = q[..., 5].abs() + 0.1
+    out = []
+    for big in (float("-inf"), -1e6):
+        k[0, 0, 2, 5] = big
+        gc = TB.gpu_cache(TB.FORMATS["float"], 1, 1, 1, D, T, "f32")
+        gc.append(k, v)
+        out.append(gc.attend_backward(q, do, scale=scale))
+    for g, r, what in zip(out[0], out[1], ("dq", "dk", "dv")):
+        if what == "dq":
+            g[..., 5] = r[..., 5] = 0
+        TB._close(g.cpu().numpy(), r.double().cpu().numpy(), what)
