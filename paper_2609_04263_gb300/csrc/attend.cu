@@ -716,7 +716,12 @@ cudaError_t launch_attend(const Geom& g, const void* q, int L, float scale, void
     if (!err) return cudaErrorInvalidDevice;
     return launch_prefill_m256(g, q, L, scale, out, err, s);
   }
-  if (!decode && prefill_kvarn_supported(g)) {
+  // (short calls stay with the mma.sync kernel, whose time grows with tokens and queries
+  // from 14 us on, where the tcgen05 pair takes 19-20 us to set up, rotate and store.  Four
+  // sequences, 8 kv heads of 2 query heads, mma.sync / tcgen05: 16 tokens and queries
+  // 17.4 / 19.7 us, 24 and 12 19.5 / 19.8, 32 and 4 18.6 / 19.9, 20 and 20 20.1 / 19.7,
+  // 32 and 12 20.7 / 19.8)
+  if (!decode && prefill_kvarn_supported(g) && t_hint + (int64_t)L > 36) {
     int* err = device_error_word();
     if (!err) return cudaErrorInvalidDevice;
     return launch_prefill_kvarn(g, q, L, scale, out, err, s);

@@ -25,6 +25,9 @@ def _gpu():
 
 CASES = [   # kb, vb, sinks, B, H, Hq, tokens, queries
     (4, 2, 128, 1, 1, 1, 1, 1),
+    (4, 2, 128, 1, 1, 2, 18, 18),       # the last call of the other kernel, the first of this one
+    (4, 2, 128, 1, 1, 2, 19, 18),
+    (4, 4, 0, 2, 1, 1, 66, 1),
     (4, 2, 128, 1, 1, 2, 32, 32),
     (4, 2, 128, 2, 1, 2, 129, 129),
     (4, 2, 128, 1, 2, 4, 192, 192),
@@ -68,16 +71,16 @@ def _one_query(gc, Q):
 def test_full_precision_key_bits():
     """A sink's key keeps 16 bits and more beside a bf16 high part that is rounded: its
     rotated channels are (1 +- b +- g) / 16 with b = 255 2^-15 and g = 2^-16, and a
-    query that sees g alone has the score 2^16 g = 1 against the zero key's 0.
+    query that sees g alone has the score 2^16 g = 1 against 0 of 39 zero keys.
     After a truncated high part the remainder b +- g needs nine bits, and the
     score comes out as 1.5.  The bound is bf16's of the output."""
     gc = gpu_cache(dict(fmt=O.FMT_KVARN, key_bits=4, value_bits=2, group_size=64, sink_tokens=128,
-                        norm_iters=8), 1, 1, 1, D, 8, "bf16")
-    k, v = torch.zeros(1, 1, 2, D), torch.zeros(1, 1, 2, D)
-    k[0, 0, 1, 0], k[0, 0, 1, 2], k[0, 0, 1, 1] = 1.0, 255 * 2.0 ** -15, 2.0 ** -16
-    v[0, 0, 1, 0] = 16.0
+                        norm_iters=8), 1, 1, 1, D, 40, "bf16")
+    k, v = torch.zeros(1, 1, 40, D), torch.zeros(1, 1, 40, D)
+    k[0, 0, 7, 0], k[0, 0, 7, 2], k[0, 0, 7, 1] = 1.0, 255 * 2.0 ** -15, 2.0 ** -16
+    v[0, 0, 7, 0] = 16.0
     gc.append(k.bfloat16().cuda(), v.bfloat16().cuda())
-    want = 1 / (1 + np.exp(-1.0))
+    want = 1 / (1 + 39 * np.exp(-1.0))
     assert abs(_one_query(gc, 2.0 ** 16) - want) <= 2 ** -8 * want
 
 
