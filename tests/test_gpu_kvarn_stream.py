@@ -2,7 +2,7 @@
 columns to a lane pair), tokens that end on a block and one past it (nothing
 staged, one staged token), caches whose heads span several CTAs, at both block
 shapes it takes; groups of odd size, whose partials end off a 16-byte boundary,
-and eight heads of 256, whose ring would hold one stage only.  Tolerance: the parity bound of the other bf16 attention tests."""
+and eight heads of 256, whose ring holds one stage only.  Tolerance: the parity bound of the other bf16 attention tests."""
 import pytest
 
 from oracle import kvq_oracle as O
@@ -22,7 +22,8 @@ CASES = [   # format, B, H, Hq, D, tokens
     ("kvarn", 16, 8, 8, 256, 128 + 64 * 10),        # group 1, nothing staged
     ("kvarn", 8, 8, 24, 256, 128 + 64 * 20 + 1),    # group 3, one staged token
     ("kvarn", 8, 8, 56, 256, 128 + 64 * 20 + 63),   # group 7, a full staging ring but one
-    ("kvarn", 8, 8, 64, 256, 128 + 64 * 20),        # group 8
+    ("kvarn", 8, 8, 64, 256, 128 + 64 * 20),        # group 8: a ring of one stage
+    ("kvarn", 3, 8, 64, 256, 128 + 64 * 61 + 5),    # its heads cut between CTAs
     ("kvarn_small", 16, 8, 8, 64, 40 + 32 * 20),
     ("kvarn_small", 16, 8, 40, 64, 40 + 32 * 20 + 1),
     ("kvarn_small", 16, 8, 64, 64, 40 + 32 * 21 - 1),
