@@ -802,7 +802,8 @@ cudaError_t launch_lora_backward(const void* x, int B, int L, int d_in, const vo
   }
   if (dx && e == cudaSuccess) {
     // dx = g W + sum_p (alpha/r) V_p A_p
-    if (dx_on_tc(act, d_in, ntot)) {
+    // (the tensor-core product stores 16 bytes at a time)
+    if (dx_on_tc(act, d_in, ntot) && (reinterpret_cast<uintptr_t>(dx) & 15) == 0) {
       // g W on tcgen05: g split into bf16 high and low parts in place (G is
       // not read again), [g_hi | g_lo] times [W^T | W^T] along K
       int* err = device_error_word();

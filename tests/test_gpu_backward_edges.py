@@ -113,3 +113,20 @@ def test_attend_backward_infinite_key():
         if what == "dq":
             g[..., 5] = r[..., 5] = 0
         TB._close(g.cpu().numpy(), r.double().cpu().numpy(), what)
+
+
+def test_lora_backward_unaligned_dx():
+    """d_x off a 16-byte boundary, at a shape whose d_x would go to the tensor cores."""
+    from paper_2609_04263_gb300 import kvq
+    L, d_in, Hq, Hkv, D = 70, 256, 2, 1, 64
+    gen = torch.Generator("cuda").manual_seed(3)
+    x, w = (torch.randn(*n, generator=gen, device="cuda").bfloat16() for n in ((L, d_in), (256, d_in)))
+    dq, dk, dv = (torch.randn(1, h, L, D, generator=gen, device="cuda") for h in (Hq, Hkv, Hkv))
+    n = kvq.kvq_lora_backward_workspace(1, L, d_in, Hq, Hkv, D, 0, 0, 0)
+    ws = torch.empty(n, dtype=torch.uint8, device="cuda")
+    dx = torch.empty(L * d_in + 1, device="cuda")[1:]
+    kvq.kvq_lora_backward(x.data_ptr(), 1, L, d_in, w.data_ptr(), *(None, None, 0) * 3, 1.0, Hq, Hkv, D, 0,
+                          0.0, kvq.KVQ_BF16, dq.data_ptr(), dk.data_ptr(), dv.data_ptr(), L, *(None,) * 6,
+                          dx.data_ptr(), ws.data_ptr(), n, torch.cuda.current_stream().cuda_stream)
+    g = torch.cat((dq, dk, dv), 1)[0].transpose(0, 1).reshape(L, -1).double()
+    TB._close(dx.view(1, 1, L, d_in).cpu().numpy(), (g @ w.double())[None, None].cpu().numpy(), "d_x")
