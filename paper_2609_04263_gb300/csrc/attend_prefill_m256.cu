@@ -72,6 +72,7 @@ struct M256Layout {
   static constexpr int NP = 32 * kProdWarps;        // producer threads
   static constexpr int KC = KT * D / NP;            // channels of K per thread
   static constexpr int CV = VC * 8 / NP;            // channels of V per thread
+  static_assert(KC == 32 && CV == 4, "build_tile: one group of K, one or two code bytes of V a token");
   // score tiles (TMEM) per query tile: what O (2 D columns) leaves of 512
   static constexpr int SB = 2;
   // Reconstructed K/V tile buffers.  A buffer is held from the start of its build to
@@ -255,16 +256,11 @@ __device__ __forceinline__ void build_tile(const Geom& g, int b, int h, int t0, 
       const uint2 u = *reinterpret_cast<const uint2*>(cp);
       kw[0] = u.x; kw[1] = u.y;
     }
-    uint32_t ks = 0, kz = 0;                      // affine/symmetric: the groups' metadata
+    uint32_t ks = 0, kz = 0;                      // affine/symmetric: the group's metadata
     if constexpr (!KIVI) {
       const unsigned char* sp = raw + S::RKS + tt * (D / 16) + hf * (S::KC / 16);
-      if constexpr (S::KC == 64) {
-        ks = *reinterpret_cast<const uint32_t*>(sp);
-        if (!SYM) kz = *reinterpret_cast<const uint32_t*>(sp + (S::RKZ - S::RKS));
-      } else {
-        ks = *reinterpret_cast<const unsigned short*>(sp);
-        if (!SYM) kz = *reinterpret_cast<const unsigned short*>(sp + (S::RKZ - S::RKS));
-      }
+      ks = *reinterpret_cast<const unsigned short*>(sp);
+      if (!SYM) kz = *reinterpret_cast<const unsigned short*>(sp + (S::RKZ - S::RKS));
     }
     const uint64_t bias2 = f2pack(-8388608.f, -8388608.f);
     constexpr int WT = BITS / 2;                  // code words per trip
@@ -292,11 +288,8 @@ __device__ __forceinline__ void build_tile(const Geom& g, int b, int h, int t0, 
                         : ffma2(c2, f2pack(sq.x, sq.y), f2pack(zq.x, zq.y));
         }
       } else {
-        const int gi = (c * 8) / 32;              // group of the thread's
-        const __half2 s2 = *reinterpret_cast<const __half2*>(&ks);
-        const __half2 z2 = *reinterpret_cast<const __half2*>(&kz);
-        const float s = gi ? __high2float(s2) : __low2float(s2);
-        const float m = SYM ? -(float)(1 << (BITS - 1)) * s : (gi ? __high2float(z2) : __low2float(z2));
+        const float s = __half2float(__ushort_as_half((unsigned short)ks));
+        const float m = SYM ? -(float)(1 << (BITS - 1)) * s : __half2float(__ushort_as_half((unsigned short)kz));
         const uint64_t ss = f2pack(s, s), mm = f2pack(m, m);
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
@@ -338,8 +331,7 @@ __device__ __forceinline__ void build_tile(const Geom& g, int b, int h, int t0, 
     for (int u = 0; u < 2; ++u) {
       const int tv = 8 * tb + 2 * p + u;          // token within the tile
       const unsigned char* cp = raw + S::RVC + tv * S::CROW + ch * BITS / 8;
-      if constexpr (CV * BITS == 32) w2[u] = *reinterpret_cast<const uint32_t*>(cp);
-      else if constexpr (CV * BITS == 16) w2[u] = *reinterpret_cast<const unsigned short*>(cp);
+      if constexpr (BITS == 4) w2[u] = *reinterpret_cast<const unsigned short*>(cp);
       else w2[u] = *cp;
     }
     {
@@ -355,20 +347,13 @@ __device__ __forceinline__ void build_tile(const Geom& g, int b, int h, int t0, 
         z2u = (uint32_t)zp[0] | ((uint32_t)zp[D / 32] << 16);
       }
     }
-    uint32_t pw[2];
-    if constexpr (CV * BITS == 32) {
-      pw[0] = __byte_perm(w2[0], w2[1], 0x5410);  // low halves of both tokens
-      pw[1] = __byte_perm(w2[0], w2[1], 0x7632);
-    } else {
-      pw[0] = (w2[0] & 0xFFFFu) | (w2[1] << 16);
-      pw[1] = 0;
-    }
+    const uint32_t pw = w2[0] | (w2[1] << 16);
     const __half2 s2 = *reinterpret_cast<const __half2*>(&s2u);
     const __half2 z2 = *reinterpret_cast<const __half2*>(&z2u);
 #pragma unroll
     for (int e = 0; e < CV; ++e) {
       constexpr uint32_t m2 = ((1u << BITS) - 1) * 0x00010001u;
-      const uint32_t x = ((pw[(e * BITS) / 16] >> ((e * BITS) % 16)) & m2) | 0x64006400u;
+      const uint32_t x = ((pw >> (e * BITS)) & m2) | 0x64006400u;
       const __half2 c2 = __hsub2(*reinterpret_cast<const __half2*>(&x), bias);
       const __half2 v2 = __hfma2(s2, c2, z2);
       out[e][pp] = *reinterpret_cast<const uint32_t*>(&v2);
@@ -384,13 +369,8 @@ __device__ __forceinline__ void build_tile(const Geom& g, int b, int h, int t0, 
       __nv_bfloat16 vals[CV];
       if (KIVI && tv < T) {
         const __nv_bfloat16* src = plane_ptr<__nv_bfloat16>(g, KVQ_PLANE_V_FULL, b, h, tv % g.ring, ch);
-        if constexpr (CV == 8) {
-          const uint4 u = *reinterpret_cast<const uint4*>(src);
-          memcpy(vals, &u, sizeof(vals));
-        } else {
-          const uint2 u = *reinterpret_cast<const uint2*>(src);
-          memcpy(vals, &u, sizeof(vals));
-        }
+        const uint2 u = *reinterpret_cast<const uint2*>(src);
+        memcpy(vals, &u, sizeof(vals));
       } else {
 #pragma unroll
         for (int e = 0; e < CV; ++e) vals[e] = __float2bfloat16_rn(0.f);

@@ -11,7 +11,6 @@
 namespace kvq {
 namespace tc {
 
-constexpr long kWaitLimit = 1L << 26;            // bounded polling loops without a barrier
 constexpr uint64_t kWaitNs = 1000000000ull;      // a bounded wait gives up after 1 s
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
@@ -66,14 +65,6 @@ __device__ __forceinline__ bool mbar_wait_or_abort(uint64_t* bar, uint32_t parit
 __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
-__device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, int c0, int c1,
-                                            uint64_t* bar) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
-      " [%0], [%1, {%2, %3}], [%4];"
-      ::"r"(smem_u32(dst)), "l"(map), "r"(c0), "r"(c1), "r"(smem_u32(bar)) : "memory");
-}
-
 // Shared-memory matrix descriptor: K-major operand in the 128-byte swizzle
 // layout (rows of 128 bytes, 8-row groups 1024 bytes apart).
 __device__ __forceinline__ uint64_t sw128_desc(const void* p) {
@@ -96,14 +87,7 @@ __host__ __device__ constexpr uint32_t idesc_bf16(int M, int N) {
 __host__ __device__ constexpr uint32_t idesc_f16(int M, int N) {
   return (1u << 4) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
-__device__ __forceinline__ void umma(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc,
-                                     uint32_t idesc, uint32_t accumulate) {
-  asm volatile(
-      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-      " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n"
-      ::"r"(tmem_d), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate));
-}
-// The same for two consecutive MMAs with one A operand: the first reads A
+// D (+)= A B, two consecutive MMAs with one A operand: the first reads A
 // from shared memory into the tensor core's collector buffer, the second
 // reads it from there (and releases it), so A crosses shared memory once.
 __device__ __forceinline__ void umma_a_fill(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc,
@@ -294,12 +278,18 @@ __device__ __forceinline__ void umma_commit_pair(uint64_t* bar) {
 }
 // Arrival on a barrier of either CTA of the pair for what this CTA's warp wrote to
 // its own shared memory (after fence.proxy.async) or TMEM (after
-// tcgen05.fence::before_thread_sync), where its own SM's tensor core reads it.
-// Nothing is handed to the other CTA's threads, so neither the arrival releases nor
-// the issuer's wait acquires at cluster scope.  A release that wide made the arrival
-// wait for the thread's global loads in flight, 1,200 of a dequantising warp's 2,100
-// cycles per slice (NF4 base, 2048 x 4096 -> 6144: 268 us with it, 225 passed on by
-// a thread without loads, 167 without).
+// tcgen05.wait::st and tcgen05.fence::before_thread_sync), where its own SM's tensor
+// core reads it.  Nothing is handed to the other CTA's threads, so neither the arrival
+// releases nor the issuer's wait acquires at cluster scope (the form's defaults are
+// release and acquire at CTA scope).  That an MMA which the first CTA's thread issues
+// afterwards finds the second CTA's writes is an assumption about the hardware that
+// the PTX memory model does not state; CUTLASS's ClusterBarrier::arrive to a remote
+// CTA, by which its pair kernels' transforming warps signal the MMA warp, is the same
+// instruction.  A release at cluster scope made the arrival wait for the thread's global
+// loads in flight, 1,200 of a dequantising warp's 2,100 cycles per slice (NF4 base,
+// 2048 x 4096 -> 6144: 268 us with it, 225 passed on by a thread without loads, 167
+// without); in the softmax warps alone, which have none, it takes the KIVI prefill of 2
+// x 8192 tokens from 1334 to 1367 us.
 __device__ __forceinline__ void mbar_arrive_pair(uint32_t bar) {
   asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
 }
