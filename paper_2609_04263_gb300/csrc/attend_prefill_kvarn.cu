@@ -564,7 +564,12 @@ attend_prefill_kvarn_kernel(Geom g, const __nv_bfloat16* __restrict__ q, int L, 
     bool ok = true;
     for (int j = 0; j < ntiles; ++j) {
       const int sb = j % kSBufs, t0 = j * kTok;
-      if (!warp_wait(&s_full[sb], (j / kSBufs) & 1, abort)) {
+      // the second CTA first for the P V that freed this buffer, so that the waits on s_free
+      // below skip none of its phases (a parity tells a phase only from its neighbours);
+      // the first CTA's issuer saw that phase end before it issued these scores, but that
+      // the second hears of it before it hears of them is not given
+      if ((rank == 1 && j >= kSBufs && !warp_wait(&s_free[sb], ((j - kSBufs) / kSBufs) & 1, abort)) ||
+          !warp_wait(&s_full[sb], (j / kSBufs) & 1, abort)) {
         ok = false;
         break;
       }

@@ -603,7 +603,12 @@ attend_prefill_m256_kernel(Geom g, const __nv_bfloat16* __restrict__ q, int L, f
     bool ok = true;
     for (int j = 0; j < ntiles; ++j) {
       const int bf = j % S::SB, t0 = j * kTok;
-      if (!warp_wait(&s_full[x][bf], (j / S::SB) & 1, abort)) {
+      // The second CTA of a pair first for the P V that freed this buffer, so that the waits
+      // on s_free below skip none of its phases (a parity tells a phase only from its
+      // neighbours).  The first CTA's issuer saw that phase end before it issued these
+      // scores; that the second hears of it before it hears of them is not given.
+      if ((rank == 1 && j >= S::SB && !warp_wait(&s_free[x][bf], ((j - S::SB) / S::SB) & 1, abort)) ||
+          !warp_wait(&s_full[x][bf], (j / S::SB) & 1, abort)) {
         ok = false;
         break;
       }

@@ -48,3 +48,26 @@ def test_prefill_tiles(fmt, D, B, H, Hq, T, L):
     got = gc.attend_prefill(q.cuda()).float().cpu().numpy()
     assert kvq.kvq_device_status(torch.cuda.current_stream().cuda_stream) == 0
     check_attention(got, O.attend(oc, q.float().numpy()), "bf16", fmt)
+
+
+@pytest.mark.parametrize("fmt,D,H,Hq", [("affine4", 128, 1, 2), ("kivi4", 128, 1, 4), ("sym4", 64, 1, 2),
+                                        ("kvarn", 256, 1, 2)])
+@pytest.mark.parametrize("grow", [(2, 5, 6, 9), (1, 2, 3, 4, 5, 6, 7, 8, 9), (3, 8)])
+def test_prefill_growing_maxima(fmt, D, H, Hq, grow):
+    """Keys whose scores grow at some tiles, at runs and gaps of odd and even length: the
+    rows' maxima jump there, O is rescaled, and the waits for the P V before it fall on
+    any of its barriers' phases."""
+    T, spec = 640, FORMATS[fmt]
+    gc = gpu_cache(spec, 1, H, Hq, D, T, "bf16")
+    oc = oracle_cache(spec, 1, H, D, T, "bf16")
+    kt, vt, _, _ = kv_pair(1, H, T, D, "bf16", seed=len(grow))
+    f = torch.ones(T // 64)
+    for i in grow:
+        f[i:] *= 2.0
+    kt = (kt * f.repeat_interleave(64).to(kt)[None, None, :, None]).contiguous()
+    gc.append(kt, vt)
+    oc.append(kt.float().cpu().numpy(), vt.float().cpu().numpy())
+    q = torch.from_numpy(synth.queries((1, Hq, T, D), seed=T)).to(torch.bfloat16) * (2.0 if len(grow) < 9 else 0.05)
+    got = gc.attend_prefill(q.cuda()).float().cpu().numpy()
+    assert kvq.kvq_device_status(torch.cuda.current_stream().cuda_stream) == 0
+    check_attention(got, O.attend(oc, q.float().numpy()), "bf16", fmt)
