@@ -1,8 +1,10 @@
-"""The straight-through backward's products at the edges of their 128-wide tiles and
-of its softmax's key ranges: one query, stacked rows a row short of and past a
-tile, key counts that no vector load divides, head_dim 64 to 256, adapters of
-unlike ranks (whose products share a launch) and rows short of a tile.  The
-checks and tolerances are those of the other backward tests."""
+"""The straight-through backward's products at the edges of their 64 x 64 tiles of 32
+k, and of its softmax's key ranges: one query; stacked rows and keys a row short
+of a tile, a whole one and a row past it; tiles that end with a head and tiles that
+hold two, over no earlier keys and some; key counts that no vector load divides;
+head_dim 64 to 256; adapters of unlike ranks (whose products share a launch); the
+workspace's size; infinite values.  The checks and tolerances are those of the
+other backward tests."""
 import pytest
 import torch
 
@@ -24,6 +26,15 @@ def _gpu():
     ("kivi2", "bf16", 1, 2, 2, 64, 126, 3),
     ("affine2", "f32", 2, 1, 2, 128, 0, 65),     # 130 stacked rows
     ("affine4", "bf16", 1, 1, 2, 256, 1, 130),
+    ("affine4", "f32", 1, 1, 1, 64, 0, 63),
+    ("affine4", "f32", 1, 1, 1, 64, 0, 64),      # one tile of rows, one of keys
+    ("sym2", "bf16", 1, 1, 1, 128, 0, 65),
+    ("affine4", "f32", 1, 2, 2, 64, 64, 64),     # 128 keys
+    ("affine4", "bf16", 1, 1, 2, 64, 0, 64),     # a head ends with its tile
+    ("affine4", "f32", 1, 1, 2, 64, 5, 64),      # the same past earlier keys
+    ("affine4", "bf16", 1, 1, 2, 64, 0, 32),     # two heads in a tile
+    ("affine4", "f32", 1, 1, 4, 64, 33, 32),
+    ("kivi2", "bf16", 1, 1, 2, 128, 32, 32),     # two heads in a tile, 64 keys
 ])
 def test_attend_backward_tiles(fmt, act, B, Hkv, Hq, D, T0, L):
     TB.test_attend_backward_parity(fmt, act, B, Hkv, Hq, D, T0, L)
