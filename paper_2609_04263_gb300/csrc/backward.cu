@@ -47,7 +47,7 @@ namespace {
 // parts last), added to the fp32 accumulator with a rounding addition: the error against
 // 64 bits is not above that of the fp32 chain this replaces.  An infinite value has
 // no such parts (infinity times the other operand's zero parts is NaN): a 32-k step with
-// one runs in fp32.
+// one runs in fp32 (out of line: unrolled in the loop it cost registers and 2 %).
 // What bounds it is the splitting and the fragment loads, not the MMAs (about 200
 // of 400 issue slots per warp and chunk at six products), which is why 64 x 64 tiles on
 // mma.sync, four CTAs per SM and no staging in tensor memory serve here.
@@ -202,6 +202,20 @@ struct Operand {
   }
 };
 
+// One 32-k step in fp32 into a thread's sums t[16 m + 4 n + i] (out of line: rare).
+template <typename OA, typename OB>
+__device__ __noinline__ void fp32_step(const __nv_bfloat16* As, const __nv_bfloat16* Bs, int row,
+                                       int col, float* t) {
+#pragma unroll 1
+  for (int j = 0; j < 32; ++j) {
+    const int r = row + 16 * (j >> 4) + 8 * ((j >> 1) & 1), c = col + 8 * ((j >> 2) & 3) + (j & 1);
+    float s = t[j];
+#pragma unroll 1
+    for (int k = 0; k < kBK; ++k) s = fmaf(OA::at(As, r, k), OB::at(Bs, c, k), s);
+    t[j] = s;
+  }
+}
+
 // A_KMAJOR: A(m, k) = a[m lda + k], else a[k lda + m].
 // B_KMAJOR: B(k, n) = b[n ldb + k], else b[k ldb + n].
 // CHAIN: the ops are one product, their K ranges behind one another (one batch entry,
@@ -280,16 +294,12 @@ __global__ void __launch_bounds__(kGemmThreads) bgemm_kernel(const __grid_consta
     while (nxt < kt1 && skip(nxt)) ++nxt;
     if (nxt < kt1) load(nxt);                  // prefetch the next tile into registers
     if (PA + PB > 2 && odd) {                  // a value without parts: in fp32
-#pragma unroll 1
-      for (int k = 0; k < kBK; ++k)
+      float t[32];
 #pragma unroll
-        for (int m = 0; m < 2; ++m)
+      for (int i = 0; i < 32; ++i) t[i] = acc[i >> 4][(i >> 2) & 3][i & 3];
+      fp32_step<OA, OB>(As, Bs, wm + (lane >> 2), wn + 2 * (lane & 3), t);
 #pragma unroll
-          for (int n = 0; n < 4; ++n)
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-              acc[m][n][i] = fmaf(OA::at(As, wm + 16 * m + 8 * (i >> 1) + (lane >> 2), k),
-                                  OB::at(Bs, wn + 8 * n + 2 * (lane & 3) + (i & 1), k), acc[m][n][i]);
+      for (int i = 0; i < 32; ++i) acc[i >> 4][(i >> 2) & 3][i & 3] = t[i];
     } else
 #pragma unroll
     for (int ks = 0; ks < kBK; ks += 16) {
