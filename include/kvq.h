@@ -371,7 +371,9 @@ kvq_status kvq_attend_decode_noalloc(kvq_cache* cache, const void* q, int n_q_he
  * workspace: caller-owned device memory, at least
  * kvq_attend_backward_workspace() bytes (one (sequence, kv head) pair's fp32
  * reconstruction, scores and score gradients); a larger workspace processes
- * that many pairs per pass.  Formats FLOAT, AFFINE, SYMMETRIC and KIVI;
+ * that many pairs per pass, and where T is no multiple of 4 is used faster with
+ * room for a pair's 2 (Hq / Hkv) L rows of scores and score gradients to be padded
+ * to one (the results are the same).  Formats FLOAT, AFFINE, SYMMETRIC and KIVI;
  * KVarN returns KVQ_ERR_UNSUPPORTED.  Too small a workspace returns
  * KVQ_ERR_CAPACITY.  The cache is not modified.
  */

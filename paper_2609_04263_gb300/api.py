@@ -155,6 +155,8 @@ class Cache:
         T = self.tokens
         per = kvq.kvq_attend_backward_workspace(self.handle, L, Hq)
         if workspace is None:
+            # with room to pad the rows of S and dP to a multiple of 4 keys
+            per += (2 * (Hq // d.kv_heads) * L * (-T % 4) * 4 + 255) // 256 * 256
             workspace = torch.empty(per * B * d.kv_heads, dtype=torch.uint8, device=q.device)
         scale = 1.0 / math.sqrt(D) if scale is None else scale
         f32 = dict(dtype=torch.float32, device=q.device)

@@ -454,38 +454,57 @@ __global__ void bwd_reconstruct_kernel(Geom g, int T, int p0, int npairs, float*
 // sum of P dP, one that rewrites the row, 16 bytes a lane where the row length allows.
 // Bound by HBM: S and dP are read twice (once from L2) and written once, the
 // visible half only: 32000 rows of 1000 keys in 62 us (137 us with a CTA per row).
-// Rows follow one another without padding, which would enlarge the workspace; where
-// T is no multiple of 4 this kernel and the products take them element by element:
-// the whole backward of 1000, 1001 tokens (32 / 8 heads of 128) takes 860, 942 us.
+// Where T is no multiple of 4, rows are padded to one if the workspace has room for
+// it and else taken element by element, here and in the products, with the same
+// results: 1001 tokens (32 / 8 heads of 128, whole backward) 858 and 888 us.
 // ---------------------------------------------------------------------------
 constexpr int kRowWarps = 8;
 
-// W: elements per access, 4 where rows start on 16-byte boundaries (T a multiple of 4).
-template <int W>
+// VEC: rows start on 16-byte boundaries (ld is a multiple of 4).
+template <bool VEC>
+__device__ __forceinline__ void row_load(const float* p, int left, float (&v)[4]) {
+  if (VEC) {
+    const float4 u = *reinterpret_cast<const float4*>(p);
+    v[0] = u.x; v[1] = u.y; v[2] = u.z; v[3] = u.w;
+  } else {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) v[i] = i < left ? p[i] : 0.f;
+  }
+}
+template <bool VEC>
+__device__ __forceinline__ void row_store(float* p, int left, const float (&v)[4]) {
+  if (VEC) {
+    *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
+  } else {
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      if (i < left) p[i] = v[i];
+  }
+}
+
+template <bool VEC>
 __global__ void __launch_bounds__(kRowWarps * 32)
-bwd_softmax_ds_kernel(float* S, float* dP, int M, int T, int L, float scale) {
+bwd_softmax_ds_kernel(float* S, float* dP, int M, int T, int ld, int L, float scale) {
   pdl_wait();
   pdl_trigger();
   const int m = blockIdx.x * kRowWarps + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (m >= M) return;
-  struct __align__(4 * W) Vec { float x[W]; };
-  const int64_t row = ((int64_t)blockIdx.y * M + m) * T;
-  Vec* sv = reinterpret_cast<Vec*>(S + row);
-  Vec* dv = reinterpret_cast<Vec*>(dP + row);
+  const int64_t row = ((int64_t)blockIdx.y * M + m) * ld;
+  float* sp = S + row;
+  float* dp = dP + row;
   const int nvis = T - L + m % L + 1;        // keys 0 .. T - L + l are visible
   const int tile = m / kBM * kBM;
   const int nend = min(T, (max_visible(tile, min(tile + kBM, M), L, T) / kBN + 1) * kBN);
   float mx = -INFINITY, sum = 0.f, dot = 0.f;
 #pragma unroll 4
-  for (int n = W * lane; n < nvis; n += 32 * W) {
-    Vec s = sv[n / W];
-    const Vec d = dv[n / W];
-    float top = -INFINITY;
+  for (int n = 4 * lane; n < nvis; n += 128) {
+    float s[4], d[4];
+    row_load<VEC>(sp + n, T - n, s);
+    row_load<VEC>(dp + n, T - n, d);
 #pragma unroll
-    for (int i = 0; i < W; ++i) {
-      if (n + i >= nvis) s.x[i] = -INFINITY;
-      top = fmaxf(top, s.x[i]);
-    }
+    for (int i = 0; i < 4; ++i)
+      if (n + i >= nvis) s[i] = -INFINITY;
+    const float top = fmaxf(fmaxf(s[0], s[1]), fmaxf(s[2], s[3]));
     if (top > mx) {
       const float f = expf(scale * (mx - top));
       sum *= f;
@@ -493,12 +512,12 @@ bwd_softmax_ds_kernel(float* S, float* dP, int M, int T, int L, float scale) {
       mx = top;
     }
 #pragma unroll
-    for (int i = 0; i < W; ++i)
+    for (int i = 0; i < 4; ++i)
       if (n + i < nvis) {
         // (no finite score so far: an infinite one has weight 0, and -inf - -inf is NaN)
-        const float e = s.x[i] == -INFINITY ? 0.f : expf(scale * (s.x[i] - mx));
+        const float e = s[i] == -INFINITY ? 0.f : expf(scale * (s[i] - mx));
         sum += e;
-        dot = fmaf(e, d.x[i], dot);
+        dot = fmaf(e, d[i], dot);
       }
   }
   float top = mx;
@@ -515,19 +534,20 @@ bwd_softmax_ds_kernel(float* S, float* dP, int M, int T, int L, float scale) {
   const float inv = 1.f / sum;
   const float delta = dot * inv;             // sum_n P dP
 #pragma unroll 4
-  for (int n = W * lane; n < nend; n += 32 * W) {
-    const Vec s = sv[n / W], d = dv[n / W];
-    Vec p, ds;
+  for (int n = 4 * lane; n < nend; n += 128) {
+    float s[4], d[4], p[4], ds[4];
+    row_load<VEC>(sp + n, T - n, s);
+    row_load<VEC>(dp + n, T - n, d);
 #pragma unroll
-    for (int i = 0; i < W; ++i) {
-      p.x[i] = ds.x[i] = 0.f;
+    for (int i = 0; i < 4; ++i) {
+      p[i] = ds[i] = 0.f;
       if (n + i < nvis) {
-        p.x[i] = expf(scale * (s.x[i] - top)) * inv;
-        ds.x[i] = p.x[i] * (d.x[i] - delta) * scale;
+        p[i] = expf(scale * (s[i] - top)) * inv;
+        ds[i] = p[i] * (d[i] - delta) * scale;
       }
     }
-    sv[n / W] = p;
-    dv[n / W] = ds;
+    row_store<VEC>(sp + n, T - n, p);
+    row_store<VEC>(dp + n, T - n, ds);
   }
 }
 
@@ -674,54 +694,57 @@ size_t a256(size_t x) { return (x + 255) & ~size_t(255); }
 
 }  // namespace
 
-size_t attend_backward_pair_bytes(const Geom& g, int T, int L) {
+// (rows of S and dP of ld floats)
+static size_t pair_bytes(const Geom& g, int T, int L, int ld) {
   const size_t gl = (size_t)(g.Hq / g.H) * L;
-  return a256((2 * (size_t)T * g.D + 2 * gl * T) * sizeof(float));
+  return a256((2 * (size_t)T * g.D + 2 * gl * ld) * sizeof(float));
 }
+size_t attend_backward_pair_bytes(const Geom& g, int T, int L) { return pair_bytes(g, T, L, T); }
 
 cudaError_t launch_attend_backward(const Geom& g, int T, const void* q, const void* d_out,
                                    int L, float scale, float* dq, float* dk, float* dv,
                                    void* ws, size_t ws_bytes, cudaStream_t s) {
   const int pairs = g.B * g.H, grp = g.Hq / g.H, D = g.D;
   const int M = grp * L;
-  const int act = g.act;
+  const int act = g.act, ld4 = (T + 3) & ~3;
   const size_t esz = act == KVQ_BF16 ? 2 : 4;
   // (two products of every pair share a launch: grid.z is at most 65,535)
   const int chunk = (int)std::min<size_t>(std::min(pairs, 65535 / 2),
-                                          ws_bytes / attend_backward_pair_bytes(g, T, L));
+                                          ws_bytes / pair_bytes(g, T, L, T));
+  const int ld = chunk * pair_bytes(g, T, L, ld4) <= ws_bytes ? ld4 : T;
   cudaError_t e = cudaSuccess;
   for (int p0 = 0; p0 < pairs && e == cudaSuccess; p0 += chunk) {
     const int np = std::min(chunk, pairs - p0);
     float* kh = static_cast<float*>(ws);
     float* vh = kh + (size_t)np * T * D;
     float* S = vh + (size_t)np * T * D;
-    float* dP = S + (size_t)np * M * T;
+    float* dP = S + (size_t)np * M * ld;
     const char* qp = static_cast<const char*>(q) + (size_t)p0 * M * D * esz;
     const char* op = static_cast<const char*>(d_out) + (size_t)p0 * M * D * esz;
     launch_pdl(bwd_reconstruct_kernel, dim3(grid_for((int64_t)np * T * D / 8, 256)), dim3(256),
                0, s, g, T, p0, np, kh, vh);
     e = cudaGetLastError();
     // S = Q K^T and dP = dO V^T (tiles above the causal edge skipped)
-    GemmArgs ga = gemm_args(1.f, np, (int64_t)M * D, (int64_t)T * D, (int64_t)M * T);
-    add_op(ga, qp, D, kh, D, S, T, M, T, D);
-    add_op(ga, op, D, vh, D, dP, T, M, T, D);
+    GemmArgs ga = gemm_args(1.f, np, (int64_t)M * D, (int64_t)T * D, (int64_t)M * ld);
+    add_op(ga, qp, D, kh, D, S, ld, M, T, D);
+    add_op(ga, op, D, vh, D, dP, ld, M, T, D);
     ga.mask = kMaskRowsQueriesColsKeys; ga.L = L; ga.T = T;
     if (e == cudaSuccess) e = gemm_act_a<true, true>(ga, act, s);
     if (e == cudaSuccess) {
-      launch_pdl(T % 4 == 0 ? bwd_softmax_ds_kernel<4> : bwd_softmax_ds_kernel<1>,
+      launch_pdl(ld % 4 == 0 ? bwd_softmax_ds_kernel<true> : bwd_softmax_ds_kernel<false>,
                  dim3((M + kRowWarps - 1) / kRowWarps, np), dim3(kRowWarps * 32), 0, s, S, dP, M, T,
-                 L, scale);
+                 ld, L, scale);
       e = cudaGetLastError();
     }
     // dQ = dS K
-    GemmArgs gq = gemm_args(1.f, np, (int64_t)M * T, (int64_t)T * D, (int64_t)M * D);
-    add_op(gq, dP, T, kh, D, dq + (size_t)p0 * M * D, D, M, D, T);
+    GemmArgs gq = gemm_args(1.f, np, (int64_t)M * ld, (int64_t)T * D, (int64_t)M * D);
+    add_op(gq, dP, ld, kh, D, dq + (size_t)p0 * M * D, D, M, D, T);
     gq.mask = kMaskRowsQueriesKKeys; gq.L = L; gq.T = T;
     if (e == cudaSuccess) e = run_gemm<float, float, true, false>(gq, s);
     // dK = dS^T Q and dV = P^T dO
-    GemmArgs gk = gemm_args(1.f, np, (int64_t)M * T, (int64_t)M * D, (int64_t)T * D);
-    add_op(gk, dP, T, qp, D, dk + (size_t)p0 * T * D, D, T, D, M);
-    add_op(gk, S, T, op, D, dv + (size_t)p0 * T * D, D, T, D, M);
+    GemmArgs gk = gemm_args(1.f, np, (int64_t)M * ld, (int64_t)M * D, (int64_t)T * D);
+    add_op(gk, dP, ld, qp, D, dk + (size_t)p0 * T * D, D, T, D, M);
+    add_op(gk, S, ld, op, D, dv + (size_t)p0 * T * D, D, T, D, M);
     gk.mask = kMaskRowsKeysKQueries; gk.L = L; gk.T = T;
     if (e == cudaSuccess) e = gemm_act_b<false, false>(gk, act, s);
   }

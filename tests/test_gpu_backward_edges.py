@@ -54,13 +54,19 @@ def test_lora_backward_tiles(act, B, L, d_in, Hq, Hkv, D, ranks, extra, pos0, ba
 @pytest.mark.parametrize("L", [44, 45, 46, 47])
 def test_attend_backward_workspace(L):
     """One pair's workspace is its K, V reconstruction and its S and dP, nothing more,
-    whatever the number of keys is a multiple of."""
+    whatever the number of keys is a multiple of; gradients in exactly that are those
+    in one with room for padded rows."""
     from paper_2609_04263_gb300 import kvq
     B, Hkv, Hq, D, T0 = 1, 1, 3, 64, 20
     gc, _ = TB._filled(TB.FORMATS["affine4"], "bf16", B, Hkv, Hq, D, T0, L, seed=L)
     T = T0 + L
     want = (2 * T * D + 2 * (Hq // Hkv) * L * T) * 4
-    assert kvq.kvq_attend_backward_workspace(gc.handle, L, Hq) == (want + 255) // 256 * 256
+    per = kvq.kvq_attend_backward_workspace(gc.handle, L, Hq)
+    assert per == (want + 255) // 256 * 256
+    gen = torch.Generator("cuda").manual_seed(L)
+    q, do = (torch.randn(B, Hq, L, D, generator=gen, device="cuda").bfloat16() for _ in range(2))
+    tight = gc.attend_backward(q, do, workspace=torch.empty(per, dtype=torch.uint8, device="cuda"))
+    assert all(torch.equal(a, b) for a, b in zip(tight, gc.attend_backward(q, do)))
     TB.test_attend_backward_parity("affine4", "bf16", B, Hkv, Hq, D, T0, L)
 
 
