@@ -596,18 +596,13 @@ def paged_decode_rates(run, peaks, flush):
             "l2": "flushed before each timed launch"}
 
 
-# fp32 FMA rate of the GB300: 152 SMs x 128 fp32 lanes x 2 flops x 2070 MHz
-FP32_FMA_TFLOPS = 152 * 128 * 2 * 2.070e9 / 1e12
-
-
 def ste_backward_rates(run, peaks, flush, max_len=2048):
     """The straight-through backward of one layer (kvq_attend_backward, then
     kvq_lora_backward with d_x) for one sequence of min(prefill, 2048) tokens
-    of the workload's shape and cache format: the adapter-training step.  The
-    attention products run on fp32 SIMT GEMMs (rated against the fp32 FMA
-    rate); with bf16 activations the adapters' dominant product, d_x = g W,
-    runs on the tensor cores (rated against the sustained bf16 peak).  None for
-    KVarN caches (no backward)."""
+    of the workload's shape and cache format: the adapter-training step.  Its
+    products run on the tensor cores with fp32 operands in bf16 parts, and are
+    rated, one product each, against the sustained bf16 peak.  None for KVarN
+    caches (no backward)."""
     from paper_2609_04263_gb300 import kvq
     wl, api = run.wl, run.api
     if wl.fmt == synth.FMT_KVARN:
@@ -655,16 +650,17 @@ def ste_backward_rates(run, peaks, flush, max_len=2048):
     lora_flops = (2 * L * d_in * 3 * r + 2 * 2 * L * r * n_out + 2 * L * r * 3 * d_in
                   + 2 * L * n_out * d_in + 2 * L * 3 * r * d_in)
     rate = lambda f, ms: round(f / ms / 1e9, 3)
-    fma = {"bound": "alu", "value": round(FP32_FMA_TFLOPS, 2), "unit": "TFLOP/s",
-           "what": "fp32 FMA: 152 SMs x 128 lanes x 2 flops x 2070 MHz"}
-    tensor = dt == torch.bfloat16 and d_in % 128 == 0 and n_out % 64 == 0
-    lpeak = ({"bound": "tensor", "value": peaks["bf16_tflops_sustained"], "unit": "TFLOP/s",
-              "what": "measured sustained bf16 (d_x = g W as bf16 high + low parts of g: "
-                      "twice the algorithmic MMA work)"} if tensor else fma)
+    parts = ("fp32 operands in three bf16 parts: three MMAs a product beside a bf16 operand, "
+             "six beside an fp32 one")
+    peak = {"bound": "tensor", "value": peaks["bf16_tflops_sustained"], "unit": "TFLOP/s",
+            "what": f"measured sustained bf16 ({parts})"}
+    dx_tc = dt == torch.bfloat16 and d_in % 128 == 0 and n_out % 64 == 0
+    lpeak = dict(peak, what=f"measured sustained bf16 (d_x = g W as bf16 high + low parts of g, "
+                            f"two MMAs a product; the others: {parts})") if dx_tc else peak
     return {"tokens": L, "sequences": 1,
             "attention": {"mean_ms": round(att_ms, 4), "flops": att_flops,
                           "achieved": rate(att_flops, att_ms), "unit": "TFLOP/s",
-                          "frac": round(att_flops / att_ms / 1e9 / fma["value"], 4), "peak": fma},
+                          "frac": round(att_flops / att_ms / 1e9 / peak["value"], 4), "peak": peak},
             "adapters": {"mean_ms": round(lora_ms, 4), "flops": lora_flops,
                          "achieved": rate(lora_flops, lora_ms), "unit": "TFLOP/s",
                          "frac": round(lora_flops / lora_ms / 1e9 / lpeak["value"], 4),

@@ -41,12 +41,13 @@
 // A CTA's start and end (rotating queries, sinks and output rows) take 50,000
 // cycles.  8192 tokens, 16 query heads, 8 kv heads, one sequence: 7667 us on
 // mma.sync (64 rows a CTA, 16-token tiles reconstructed by all its warps), 1526
-// with one CTA building 32-token tiles of K and V for 128 rows, 824 here: 1,480 as
+// with one CTA building 32-token tiles of K and V for 128 rows, 827 here: 1,480 as
 // a pair, 1,380 with arrivals that do not wait (mbar_arrive_pair), 1,100 with the
 // packed tile loaded without a branch that divides the warp (load_packed) and
 // rows of sinks, queries and outputs loaded together, 994 with K and V built by
 // warps of their own (no spills), 898 with four rows to a warp in the rotation,
-// 824 with the issuer blocking instead of polling.
+// 818 with the issuer blocking instead of polling, 827 with the second CTA's softmax
+// waiting for every phase.
 // Every wait is bounded and also gives up when another role has timed out;
 // the issuer drains its MMAs before TMEM is freed, and a timed-out CTA stores
 // nothing and sets the library's error word.

@@ -35,7 +35,7 @@
 // the softmax warps); D = 64, the chain from scores over softmax to P V and the buffers
 // it frees, about 2,000 cycles, 1,060 of them softmax.
 //   2 x 8192 tokens, 32 / 8 heads of 128, KIVI 2-bit: 2081 us with two tile
-// buffers, 1745 with three, 1335 here.  A thread's share of a tile is kept small
+// buffers, 1745 with three, 1338 here.  A thread's share of a tile is kept small
 // and the issuer holds one copy of each product: with 64 channels of K or V to a
 // thread unrolled and five copies the roles' code did not fit the instruction
 // cache (1.5 of 10 cycles an instruction went to fetching it), 1,800 us as a pair
