@@ -50,7 +50,7 @@ namespace {
 // one runs in fp32 (out of line: unrolled in the loop it cost registers and 2 %).
 // What bounds it is the splitting and the fragment loads, not the MMAs (about 200
 // of 400 issue slots per warp and chunk at six products), which is why 64 x 64 tiles on
-// mma.sync, four CTAs per SM and no staging in tensor memory serve here.
+// mma.sync, three or four CTAs per SM and no staging in tensor memory serve here.
 // All products of the attention backward of 1000 tokens, 32 / 8 heads of 128:
 // 1317 us in fp32 FMA, 548 us so.
 // ---------------------------------------------------------------------------
